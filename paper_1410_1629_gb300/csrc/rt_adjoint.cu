@@ -156,7 +156,7 @@ __device__ __forceinline__ int adjoint_exponent(unsigned long long bits) {
 // (units 2^ea).
 __device__ __forceinline__ float adj_weight(const AdjParams& A, int q, int lam, bool scattered, float3 x,
                                             float3& dW) {
-  const DevInstr& I = tr::S_INSTR[q];
+  const DevInstr& I = A.f.instr[q];
   dW = make_float3(0.0f, 0.0f, 0.0f);
   const float* img = A.adj_img[q];
   if (!img) return 0.0f;
@@ -252,7 +252,7 @@ __device__ __forceinline__ void fetch(const AdjParams& A, ALane& s, unsigned lon
   while (lam + 1 < P.n_lambda && (unsigned long long)(lam + 1) * P.n_per_lambda <= w) ++lam;
   s.lam = lam;
   s.pid = P.first_id + (w - (unsigned long long)lam * P.n_per_lambda);
-  s.kappa = tr::S_LAM[lam].kappa;
+  s.kappa = A.f.lam[lam].kappa;
   s.L = P.L0[lam];
   s.eL = A.e0[lam];
   s.eLA = s.eL + adjoint_exponent(*A.maxbits);
@@ -276,13 +276,13 @@ __device__ __forceinline__ void fetch(const AdjParams& A, ALane& s, unsigned lon
 template <bool kAbs>
 __device__ __forceinline__ void finish_path1(const AdjParams& A, ALane& s) {
   const FwdParams& P = A.f;
-  const double tau = tr::widen(s.th) + tr::widen(s.tl);
+  const double tau = widen(s.th) + widen(s.tl);
   if (!(tau > 0.0)) {  // escapes: there is no event s.event
     s.J = s.event - 1;
     s.phase = aSweep;
     return;
   }
-  const double albedo = tr::S_LAM[s.lam].albedo;
+  const double albedo = A.f.lam[s.lam].albedo;
   const double omE = -expm1(-tau);
   const uint4 rn = draw_block(s.pid, s.lam, s.event, 0, P.seed, P.model);
   const double u = u01(rn.x);
@@ -346,7 +346,7 @@ __device__ __forceinline__ void finish_path2(const AdjParams& A, ALane& s) {
 // xb); returns l (units 2^eLA).
 __device__ __forceinline__ float peel_values(const AdjParams& A, ALane& s, const DevInstr& I, float W, float3 dW) {
   float phase = 1.0f;
-  if (s.event > 0) phase = hg_phase(tr::S_LAM[s.lam].g, s.k.x * I.kobs[0] + s.k.y * I.kobs[1] + s.k.z * I.kobs[2]);
+  if (s.event > 0) phase = hg_phase(A.f.lam[s.lam].g, s.k.x * I.kobs[0] + s.k.y * I.kobs[1] + s.k.z * I.kobs[2]);
   const float pe = kInv4PiF * phase * expf(-s.th) * (1.0f - s.tl);
   const float V = (A.tape ? s.Lf : narrow(s.L, s.eL)) * pe;  // units 2^eL
   const float l = V * W;                   // units 2^eLA
@@ -363,7 +363,7 @@ __device__ __forceinline__ float peel_values(const AdjParams& A, ALane& s, const
 // A peel-off measuring walk ended: its values, then the depositing walk or
 // the next peel-off.
 __device__ __forceinline__ void finish_peel_measure(const AdjParams& A, ALane& s) {
-  const DevInstr& I = tr::S_INSTR[s.q];
+  const DevInstr& I = A.f.instr[s.q];
   float3 dW;
   const float W = adj_weight(A, s.q, s.lam, s.event > 0, s.x, dW);
   const float l = peel_values(A, s, I, W, dW);
@@ -432,7 +432,7 @@ __device__ __forceinline__ void peel_scan(const AdjParams& A, ALane& s, unsigned
     float3 dW;
     const float W = adj_weight(A, s.q, s.lam, s.event > 0, s.x, dW);
     if (W == 0.0f && dW.x == 0.0f && dW.y == 0.0f && dW.z == 0.0f) continue;  // contributes nothing
-    const DevInstr& I = tr::S_INSTR[s.q];
+    const DevInstr& I = A.f.instr[s.q];
     if (P.use_columns && I.column && column_peel(A, s, I, W, dW, n_cross, n_dep)) continue;
     request_walk(s, aPeelM, tr::instr_dir(I));
     return;
@@ -461,11 +461,11 @@ __device__ __forceinline__ void after_peels(const AdjParams& A, ALane& s) {
     request_path<kAbs>(s);
     return;
   }
-  const float mu = hg_sample(tr::S_LAM[s.lam].g, s.u_mu);
+  const float mu = hg_sample(A.f.lam[s.lam].g, s.u_mu);
   float sp, cp;
   sincospif(2.0f * s.u_phi, &sp, &cp);
   s.k = rotate_dir(s.k, mu, sp, cp);
-  if ((P.weight_cut && s.L < P.L_cut[s.lam]) || s.event >= P.max_events) {
+  if ((P.weight_cut && bits_of(s.L) < bits_of(P.L_cut[s.lam])) || s.event >= P.max_events) {
     s.J = s.event;
     s.phase = aSweep;
     return;
@@ -480,7 +480,7 @@ __device__ __forceinline__ void after_peels(const AdjParams& A, ALane& s) {
 // adjoints of the path's start weight and position.
 template <bool kAbs>
 __device__ __forceinline__ void sweep(const AdjParams& A, ALane& s) {
-  const float albedo = (float)tr::S_LAM[s.lam].albedo;
+  const float albedo = (float)A.f.lam[s.lam].albedo;
   float Lb = 0.0f, xb0 = 0.0f, xb1 = 0.0f, xb2 = 0.0f;
   for (int j = s.J; j >= 1; --j) {
     AdjRecord& r = s.rec[j];
@@ -580,7 +580,7 @@ __device__ __forceinline__ void step(const AdjParams& A, ALane& s, unsigned& n_c
     // prefix of the optical-depth adjoints wd e_i (a_i - a_{i+1}), i < m
     const double a = dt > 0.0f ? A.adj_abs[(size_t)s.lam * P.n_cells + cell] : 0.0;
     const double e_cur = (double)(expf(-nh) * (1.0f - nl));
-    const double wd = (1.0 - tr::S_LAM[s.lam].albedo) * s.L;
+    const double wd = (1.0 - A.f.lam[s.lam].albedo) * s.L;
     if (s.n_cross > 0) s.P += wd * s.e_prev * (s.a_prev - a);
     if (s.P != 0.0) grad_add(&A.grad[cell], -(double)(s.kappa * ds) * s.P);
     const double c = (double)kr * s.P;
@@ -605,11 +605,8 @@ __device__ __forceinline__ void step(const AdjParams& A, ALane& s, unsigned& n_c
 }
 
 template <bool kAbs, bool kTape>
-__global__ void __launch_bounds__(kAdjBlock, RT_ADJ_MIN_BLOCKS) k_adjoint(const AdjParams A) {
+__global__ void __launch_bounds__(kAdjBlock, RT_ADJ_MIN_BLOCKS) k_adjoint(const __grid_constant__ AdjParams A) {
   const FwdParams& P = A.f;
-  for (int i = threadIdx.x; i < P.n_instr; i += kAdjBlock) tr::S_INSTR[i] = P.instr[i];
-  for (int i = threadIdx.x; i < P.n_lambda; i += kAdjBlock) tr::S_LAM[i] = P.lam[i];
-  __syncthreads();
   const unsigned lane = threadIdx.x & 31u;
   const unsigned lt_mask = (1u << lane) - 1u;
   ALane s;

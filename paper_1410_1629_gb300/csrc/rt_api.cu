@@ -129,10 +129,10 @@ struct rt_ctx_s {
   std::vector<HostInstr> instr;
   // device tables and tallies
   double* d_absorption = nullptr;
-  DevLambda* d_lam = nullptr;
+  std::vector<DevLambda> lam_table;
+  std::vector<DevInstr> instr_table;
   DevSource* d_src = nullptr;
   double* d_src_cum = nullptr;
-  DevInstr* d_instr = nullptr;
   double* d_stats = nullptr;
   unsigned long long* d_counters = nullptr;
   unsigned long long* d_work = nullptr;
@@ -347,7 +347,8 @@ void frame_axes(const rt_instrument_desc& d, double kobs[3], double ex[3], doubl
   rtk::frame_axes(d.inclination, d.azimuth, d.position_angle, kobs, ex, ey);
 }
 
-// Rebuild the small device tables (per-wavelength optics, sources, instruments).
+// Rebuild the small tables: per-wavelength optics and instruments (they travel
+// with each launch) and the sources (device).
 rt_status upload_tables(rt_ctx c, cudaStream_t s) {
   if (!c->tables_dirty) return RT_OK;
   std::vector<DevLambda> lam((size_t)c->n_lambda);
@@ -413,16 +414,14 @@ rt_status upload_tables(rt_ctx c, cudaStream_t s) {
     if (I.column) c->columns_used[2 * I.axis + (I.dir > 0 ? 1 : 0)] = true;
     else c->n_walked_frames += 1;
   }
-  dfree(c->d_lam); dfree(c->d_src); dfree(c->d_src_cum); dfree(c->d_instr);
-  RT_CUDA(c, cudaMalloc(&c->d_lam, std::max<size_t>(1, lam.size()) * sizeof(DevLambda)));
+  dfree(c->d_src); dfree(c->d_src_cum);
   RT_CUDA(c, cudaMalloc(&c->d_src, std::max<size_t>(1, src.size()) * sizeof(DevSource)));
   RT_CUDA(c, cudaMalloc(&c->d_src_cum, std::max<size_t>(1, cum.size()) * sizeof(double)));
-  RT_CUDA(c, cudaMalloc(&c->d_instr, std::max<size_t>(1, ins.size()) * sizeof(DevInstr)));
   // synchronous copies: the host vectors go out of scope on return
-  if (!lam.empty()) RT_CUDA(c, cudaMemcpy(c->d_lam, lam.data(), lam.size() * sizeof(DevLambda), cudaMemcpyHostToDevice));
   if (!src.empty()) RT_CUDA(c, cudaMemcpy(c->d_src, src.data(), src.size() * sizeof(DevSource), cudaMemcpyHostToDevice));
   if (!cum.empty()) RT_CUDA(c, cudaMemcpy(c->d_src_cum, cum.data(), cum.size() * sizeof(double), cudaMemcpyHostToDevice));
-  if (!ins.empty()) RT_CUDA(c, cudaMemcpy(c->d_instr, ins.data(), ins.size() * sizeof(DevInstr), cudaMemcpyHostToDevice));
+  c->lam_table = std::move(lam);
+  c->instr_table = std::move(ins);
   (void)s;
   c->tables_dirty = false;
   return RT_OK;
@@ -607,7 +606,7 @@ rt_status rt_context_destroy(rt_ctx c) {
   free_problem(c);
   free_grid(c);
   pool_flush(c);
-  dfree(c->d_lam); dfree(c->d_src); dfree(c->d_src_cum); dfree(c->d_instr);
+  dfree(c->d_src); dfree(c->d_src_cum);
   dfree(c->d_stats); dfree(c->d_counters); dfree(c->d_work); dfree(c->d_flags);
   dfree(c->d_adj); dfree(c->d_adj_img); dfree(c->d_adj_max); dfree(c->d_tune_grad); dfree(c->d_tape);
   for (auto& p : c->d_line_dep) dfree(p);
@@ -1240,10 +1239,10 @@ rt_status rt_launch_packets(rt_ctx c, uint64_t n_per_lambda, uint64_t first_pack
   p.n_lambda = c->n_lambda;
   p.n_sources = (int)c->sources.size();
   p.n_instr = (int)c->instr.size();
-  p.lam = c->d_lam;
+  std::copy(c->lam_table.begin(), c->lam_table.end(), p.lam);
   p.src = c->d_src;
   p.src_cum = c->d_src_cum;
-  p.instr = c->d_instr;
+  std::copy(c->instr_table.begin(), c->instr_table.end(), p.instr);
   p.absorption = c->d_absorption;
   p.n_per_lambda = n_per_lambda;
   p.first_id = first_packet_id;
@@ -1419,10 +1418,10 @@ rt_status rt_adjoint(rt_ctx c, const double* const* adj_images, int32_t n_adj_im
   p.n_lambda = c->n_lambda;
   p.n_sources = (int)c->sources.size();
   p.n_instr = (int)c->instr.size();
-  p.lam = c->d_lam;
+  std::copy(c->lam_table.begin(), c->lam_table.end(), p.lam);
   p.src = c->d_src;
   p.src_cum = c->d_src_cum;
-  p.instr = c->d_instr;
+  std::copy(c->instr_table.begin(), c->instr_table.end(), p.instr);
   p.n_per_lambda = n_per_lambda;
   p.first_id = first_packet_id;
   p.n_total = n_total;

@@ -36,6 +36,13 @@ struct Tally {
   unsigned long long column_peels, column_crossings;  // the lane's, over the launch
 };
 
+__shared__ unsigned long long S_PID[kBatchBlock];
+__shared__ double S_WEIGHT[kBatchBlock];
+__shared__ float3 S_DIR[kBatchBlock];
+__shared__ float2 S_HG[kBatchBlock];
+__shared__ int S_EVENT[kBatchBlock], S_INSTR_Q[kBatchBlock], S_WPHASE[kBatchBlock];
+__shared__ bool S_HAS_CELL[kBatchBlock];
+__shared__ CartGrid::Cell S_CELL_CART[kBatchBlock];
 __shared__ Geo S_GEO[kBatchBlock];
 __shared__ Tally S_TALLY[kBatchBlock];
 
@@ -56,16 +63,16 @@ struct BLane {
   // for this event, the walk a kStart lane begins, weight, direction of
   // travel, the event's Henyey-Greenstein uniforms, the cell of x (valid when
   // has_cell)
-  __device__ __forceinline__ unsigned long long& pid() const { return tr::S_PID[threadIdx.x]; }
-  __device__ __forceinline__ int& event() const { return tr::S_EVENT[threadIdx.x]; }
-  __device__ __forceinline__ int& q() const { return tr::S_INSTR_Q[threadIdx.x]; }
-  __device__ __forceinline__ int& wphase() const { return tr::S_WPHASE[threadIdx.x]; }
-  __device__ __forceinline__ double& L() const { return tr::S_WEIGHT[threadIdx.x]; }
-  __device__ __forceinline__ float3& k() const { return tr::S_DIR[threadIdx.x]; }
-  __device__ __forceinline__ float& u_mu() const { return tr::S_HG[threadIdx.x].x; }
-  __device__ __forceinline__ float& u_phi() const { return tr::S_HG[threadIdx.x].y; }
-  __device__ __forceinline__ CartGrid::Cell& cell() const { return tr::S_CELL_CART[threadIdx.x]; }
-  __device__ __forceinline__ bool& has_cell() const { return tr::S_HAS_CELL[threadIdx.x]; }
+  __device__ __forceinline__ unsigned long long& pid() const { return S_PID[threadIdx.x]; }
+  __device__ __forceinline__ int& event() const { return S_EVENT[threadIdx.x]; }
+  __device__ __forceinline__ int& q() const { return S_INSTR_Q[threadIdx.x]; }
+  __device__ __forceinline__ int& wphase() const { return S_WPHASE[threadIdx.x]; }
+  __device__ __forceinline__ double& L() const { return S_WEIGHT[threadIdx.x]; }
+  __device__ __forceinline__ float3& k() const { return S_DIR[threadIdx.x]; }
+  __device__ __forceinline__ float& u_mu() const { return S_HG[threadIdx.x].x; }
+  __device__ __forceinline__ float& u_phi() const { return S_HG[threadIdx.x].y; }
+  __device__ __forceinline__ CartGrid::Cell& cell() const { return S_CELL_CART[threadIdx.x]; }
+  __device__ __forceinline__ bool& has_cell() const { return S_HAS_CELL[threadIdx.x]; }
   float3 d, id;
   CartGrid::Walk w;
   float rho;
@@ -102,7 +109,7 @@ __device__ __forceinline__ void deposit(const DevModel& M, const BLane& s, bool 
   float phase = 1.0f;
   if (scattered) phase = hg_phase(M.g, s.k().x * I.kobs[0] + s.k().y * I.kobs[1] + s.k().z * I.kobs[2]);
   const float tau = s.th;
-  const double value = tau < 80.0f ? s.L() * tr::widen(tr::kInv4PiF * phase * expf(-tau) * (1.0f - s.tl))
+  const double value = tau < 80.0f ? s.L() * widen(tr::kInv4PiF * phase * expf(-tau) * (1.0f - s.tl))
                                    : s.L() * kInv4PiD * (double)phase * exp(-((double)tau + (double)s.tl));
   const float fx = (s.x.x * I.ex[0] + s.x.y * I.ex[1] + s.x.z * I.ex[2] + I.off_x) * I.sx;
   const float fy = (s.x.x * I.ey[0] + s.x.y * I.ey[1] + s.x.z * I.ey[2] + I.off_y) * I.sy;
@@ -121,7 +128,7 @@ __device__ __forceinline__ void deposit(const DevModel& M, const BLane& s, bool 
     for (int dx = 0; dx < 2; ++dx) {
       const float fix = x0 + dx, fiy = y0 + dy;
       if (!(fix >= 0.0f && fiy >= 0.0f && fix < (float)I.nx && fiy < (float)I.ny)) continue;
-      const double v = value * tr::widen((dx ? tx : 1.0f - tx) * (dy ? ty : 1.0f - ty));
+      const double v = value * widen((dx ? tx : 1.0f - tx) * (dy ? ty : 1.0f - ty));
       atomicAdd(&I.image[(size_t)(int)fiy * I.nx + (int)fix], v);
     }
   }
@@ -204,7 +211,7 @@ __device__ __forceinline__ void begin(const BatchParams& P, BLane& s, Geo& G, Ta
 
 __device__ __forceinline__ void finish_path1(const BatchParams& P, BLane& s, Tally& T) {
   const DevModel& M = P.models[s.m];
-  const double tau = tr::widen(s.th) + tr::widen(s.tl);
+  const double tau = widen(s.th) + widen(s.tl);
   if (!(tau > 0.0)) {
     T.escaped += s.L();
     s.phase = tr::kFetch;

@@ -7,6 +7,7 @@
 #include <cuda_runtime.h>
 
 #include "rt_internal.h"
+#include "rt_math.cuh"
 
 namespace rtk {
 

@@ -5,7 +5,7 @@
 namespace rtk {
 
 namespace {
-__global__ void __launch_bounds__(tr::kBlock, RT_FWD_MIN_BLOCKS) k_forward_cartesian(const FwdParams P) {
+__global__ void __launch_bounds__(tr::kBlock, RT_FWD_MIN_BLOCKS) k_forward_cartesian(const __grid_constant__ FwdParams P) {
   tr::forward_body<tr::CartGrid>(P);
 }
 // The same launch recording the adjoint tape (P.tape): the tape's lane state
@@ -13,11 +13,11 @@ __global__ void __launch_bounds__(tr::kBlock, RT_FWD_MIN_BLOCKS) k_forward_carte
 #ifndef RT_TAPE_MIN_BLOCKS
 #define RT_TAPE_MIN_BLOCKS 3
 #endif
-__global__ void __launch_bounds__(tr::kBlock, RT_TAPE_MIN_BLOCKS) k_forward_cartesian_tape(const FwdParams P) {
+__global__ void __launch_bounds__(tr::kBlock, RT_TAPE_MIN_BLOCKS) k_forward_cartesian_tape(const __grid_constant__ FwdParams P) {
   tr::forward_body<tr::CartGrid, true>(P);
 }
 // The launch with execution counters (P.profile set, no tape).
-__global__ void __launch_bounds__(tr::kBlock, RT_FWD_MIN_BLOCKS) k_forward_cartesian_prof(const FwdParams P) {
+__global__ void __launch_bounds__(tr::kBlock, RT_FWD_MIN_BLOCKS) k_forward_cartesian_prof(const __grid_constant__ FwdParams P) {
   tr::forward_body<tr::CartGrid, false, true>(P);
 }
 }  // namespace
@@ -27,28 +27,9 @@ cudaError_t launch_forward(const FwdParams& p, int grid_kind, int num_sms, cudaS
   if (grid_kind == RT_GRID_RECTILINEAR) return launch_forward_rect(p, num_sms, stream);
   if (grid_kind == RT_GRID_BINTREE) return launch_forward_bintree(p, num_sms, stream);
   if (grid_kind == RT_GRID_VORONOI) return launch_forward_voronoi(p, num_sms, stream);
-  cudaError_t e = cudaMemsetAsync(p.work_counter, 0, sizeof(unsigned long long), stream);
-  if (e != cudaSuccess) return e;
-  int per_sm = 0;
-  const bool prof = p.profile != nullptr && !p.tape;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-      &per_sm, p.tape ? k_forward_cartesian_tape : (prof ? k_forward_cartesian_prof : k_forward_cartesian), tr::kBlock,
-      0);
-  if (e != cudaSuccess) return e;
-  per_sm = per_sm < 1 ? 1 : per_sm;
-  if (p.blocks_per_sm > 0 && p.blocks_per_sm < per_sm) per_sm = p.blocks_per_sm;
-  unsigned long long blocks = (unsigned long long)num_sms * per_sm;
-  const unsigned long long useful = (p.n_total + tr::kBlock - 1) / tr::kBlock;
-  if (blocks > useful) blocks = useful;
-  if (blocks < 1) blocks = 1;
-  if (p.tape) {
-    k_forward_cartesian_tape<<<(unsigned)blocks, tr::kBlock, 0, stream>>>(p);
-  } else if (prof) {
-    k_forward_cartesian_prof<<<(unsigned)blocks, tr::kBlock, 0, stream>>>(p);
-  } else {
-    k_forward_cartesian<<<(unsigned)blocks, tr::kBlock, 0, stream>>>(p);
-  }
-  return cudaGetLastError();
+  if (p.tape) return tr::launch_body<tr::CartGrid, true>(k_forward_cartesian_tape, p, num_sms, 0, stream);
+  return tr::launch_body<tr::CartGrid, false>(p.profile ? k_forward_cartesian_prof : k_forward_cartesian, p, num_sms, 0,
+                                              stream);
 }
 
 namespace {

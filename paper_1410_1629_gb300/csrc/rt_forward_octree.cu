@@ -15,30 +15,14 @@
 namespace rtk {
 
 namespace {
-__global__ void __launch_bounds__(tr::kBlock, RT_OCT_MIN_BLOCKS) k_forward_octree(const FwdParams P) {
+__global__ void __launch_bounds__(tr::kBlock, RT_OCT_MIN_BLOCKS) k_forward_octree(const __grid_constant__ FwdParams P) {
   tr::forward_body<tr::OctGrid>(P);
 }
 }  // namespace
 
 cudaError_t launch_forward_octree(const FwdParams& p, int num_sms, cudaStream_t stream) {
-  cudaError_t e = cudaMemsetAsync(p.work_counter, 0, sizeof(unsigned long long), stream);
-  if (e != cudaSuccess) return e;
-  const size_t stack_bytes = (size_t)tr::kBlock * (size_t)p.oct_levels * sizeof(int);
-  // static and dynamic shared memory together pass 48 KB: the launch needs
-  // the dynamic part allowed explicitly
-  e = cudaFuncSetAttribute(k_forward_octree, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)stack_bytes);
-  if (e != cudaSuccess) return e;
-  int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_forward_octree, tr::kBlock, stack_bytes);
-  if (e != cudaSuccess) return e;
-  per_sm = per_sm < 1 ? 1 : per_sm;
-  if (p.blocks_per_sm > 0 && p.blocks_per_sm < per_sm) per_sm = p.blocks_per_sm;
-  unsigned long long blocks = (unsigned long long)num_sms * per_sm;
-  const unsigned long long useful = (p.n_total + tr::kBlock - 1) / tr::kBlock;
-  if (blocks > useful) blocks = useful;
-  if (blocks < 1) blocks = 1;
-  k_forward_octree<<<(unsigned)blocks, tr::kBlock, stack_bytes, stream>>>(p);
-  return cudaGetLastError();
+  return tr::launch_body<tr::OctGrid, false>(k_forward_octree, p, num_sms, (size_t)tr::kBlock * (size_t)p.oct_levels * sizeof(int),
+                                            stream);
 }
 
 }  // namespace rtk

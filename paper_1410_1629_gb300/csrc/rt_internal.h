@@ -110,10 +110,12 @@ struct FwdParams {
   // problem
   int n_lambda, n_sources, n_instr;
   int pad1;
-  const DevLambda* lam;
+  // the small tables travel with the launch (constant bank: no copies to
+  // shared memory, which the packet slots and the L1 cache need)
+  DevLambda lam[kMaxLambda];
+  DevInstr instr[kMaxInstruments];
   const DevSource* src;
   const double* src_cum;  // [n_lambda][n_sources] cumulative luminosity fractions
-  const DevInstr* instr;
   double* absorption;     // [n_lambda][n_cells]
   // run
   unsigned long long n_per_lambda, first_id, n_total, n_norm;

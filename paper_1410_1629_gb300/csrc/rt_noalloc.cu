@@ -11,14 +11,14 @@
 // The working area is the file-scope array `g_noalloc_scratch` below, a
 // __device__ array of kNoallocScratchBytes bytes that every GPU which loads
 // this library holds until the process exits.  It carries the packet work
-// counter, the tallies and the device flags of one launch, and the small
-// per-launch tables (optics per wavelength, sources, instruments).  Host code
+// counter, the tallies and the device flags of one launch, and its source
+// tables (optics and instruments are launch parameters).  Host code
 // cannot use the array's name as a device address: every call looks the
 // address up with cudaGetSymbolAddress on the current device (a lookup that
 // allocates nothing, repeated per call so that a reset device never leaves a
 // stale address behind).  The first call on a device also loads the library's
 // device code there, so it should come before any stream capture on that
-// device.  The per-launch tables travel to the working area as the parameter
+// device.  The source tables travel to the working area as the parameter
 // of a small set-up kernel (by value), never as a copy from host memory, so
 // no queued work refers to the caller's stack.  Every call uses the same array
 // and the array keeps the last call's contents; a call clears the parts that
@@ -38,13 +38,11 @@ namespace {
 
 constexpr size_t kNoallocScratchBytes = 16384;
 
-// The per-launch tables, passed by value to the set-up kernel and kept in the
+// The source tables, passed by value to the set-up kernel and kept in the
 // working area after its first 256 bytes.
 struct NoallocTables {
-  DevLambda lam[kMaxLambda];
   DevSource src[kMaxSources];
   double cum[kMaxLambda * kMaxSources];  // [n_lambda][n_sources] cumulative luminosity fractions
-  DevInstr ins[kMaxInstruments];
 };
 
 // Byte offsets inside the working area.
@@ -53,10 +51,8 @@ constexpr size_t kOffStats = 16;     // 4 x f64
 constexpr size_t kOffCounters = 48;  // 8 x u64
 constexpr size_t kOffFlags = 112;    // 1 x i32
 constexpr size_t kOffTables = 256;   // NoallocTables
-constexpr size_t kOffLam = kOffTables + offsetof(NoallocTables, lam);
 constexpr size_t kOffSrc = kOffTables + offsetof(NoallocTables, src);
 constexpr size_t kOffCum = kOffTables + offsetof(NoallocTables, cum);
-constexpr size_t kOffInstr = kOffTables + offsetof(NoallocTables, ins);
 static_assert(kOffTables + sizeof(NoallocTables) <= kNoallocScratchBytes, "working area too small for its layout");
 // a kernel parameter may hold up to 32764 bytes (CUDA 12.1 and later)
 static_assert(sizeof(NoallocTables) <= 32000, "tables too large for a kernel parameter");
@@ -191,12 +187,12 @@ extern "C" rt_status rt_launch_packets_noalloc(const rt_grid_desc* grid, int32_t
   // ---- per-launch tables, handed to the set-up kernel by value
   NoallocTables t;
   std::memset(&t, 0, sizeof t);
-  DevLambda* lam = t.lam;
   DevSource* src = t.src;
   double* cum = t.cum;
-  DevInstr* ins = t.ins;
   FwdParams p;
   std::memset(&p, 0, sizeof p);
+  DevLambda* lam = p.lam;
+  DevInstr* ins = p.instr;
   const unsigned long long n_norm = o.n_norm ? o.n_norm : n_per_lambda;
   double emitted = 0.0;
   for (int l = 0; l < n_lambda; ++l) {
@@ -263,10 +259,8 @@ extern "C" rt_status rt_launch_packets_noalloc(const rt_grid_desc* grid, int32_t
   p.n_lambda = n_lambda;
   p.n_sources = n_sources;
   p.n_instr = n_instruments;
-  p.lam = reinterpret_cast<const DevLambda*>(scratch + kOffLam);
   p.src = reinterpret_cast<const DevSource*>(scratch + kOffSrc);
   p.src_cum = reinterpret_cast<const double*>(scratch + kOffCum);
-  p.instr = reinterpret_cast<const DevInstr*>(scratch + kOffInstr);
   p.absorption = absorption;
   p.n_per_lambda = n_per_lambda;
   p.first_id = first_packet_id;

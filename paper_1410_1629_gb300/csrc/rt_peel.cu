@@ -119,10 +119,7 @@ __global__ void __launch_bounds__(256) k_peel_scatter(const PeelRecord* __restri
 
 // The walks of the sorted records and their deposits; one record per thread,
 // consecutive threads on consecutive records of the order.
-__global__ void __launch_bounds__(256) k_peel_sorted(const FwdParams P, const unsigned* __restrict__ perm) {
-  for (int i = threadIdx.x; i < P.n_instr; i += blockDim.x) tr::S_INSTR[i] = P.instr[i];
-  for (int i = threadIdx.x; i < P.n_lambda; i += blockDim.x) tr::S_LAM[i] = P.lam[i];
-  __syncthreads();
+__global__ void __launch_bounds__(256) k_peel_sorted(const __grid_constant__ FwdParams P, const unsigned* __restrict__ perm) {
   const unsigned long long n = min(*P.peel_count, P.peel_cap);
   if (blockIdx.x == 0 && threadIdx.x == 0 && n) atomicAdd(&P.counters[8], n);
   const unsigned stride_k = (unsigned)(P.n_cells + 1);
@@ -140,13 +137,13 @@ __global__ void __launch_bounds__(256) k_peel_sorted(const FwdParams P, const un
     const bool known = (meta >> 31) != 0u;
     const double L = __hiloint2double(__float_as_int(b.y), __float_as_int(b.x));
     const float3 x = make_float3(a.x, a.y, a.z);
-    const DevInstr& I = tr::S_INSTR[q];
+    const DevInstr& I = P.instr[q];
     tr::CartGrid::Cell cell;
     cell.ix = (int)(c % (unsigned)P.nx);
     cell.iy = (int)((c / (unsigned)P.nx) % (unsigned)P.ny);
     cell.iz = (int)(c / ((unsigned)P.nx * (unsigned)P.ny));
     float th, tl;
-    crossings += tr::ray_tau(P, x, tr::instr_dir(I), known, cell, tr::S_LAM[lam].kappa, th, tl);
+    crossings += tr::ray_tau(P, x, tr::instr_dir(I), known, cell, P.lam[lam].kappa, th, tl);
     const ulonglong2 tag = P.peel_tag ? P.peel_tag[i] : make_ulonglong2(0ull, 0ull);
     tr::deposit_peel(P, q, lam, x, L, b.z, th, tl, (meta >> 30) & 1u, tag.x, (int)tag.y);
   }

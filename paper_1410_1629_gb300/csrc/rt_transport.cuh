@@ -3,21 +3,24 @@
 // Henyey-Greenstein scattering and termination for a stream of photon packets
 // (SKIRT paper, Sect. 1 and Sect. 2.2-2.4).
 //
-// Execution model.  A persistent grid of warps; every lane carries one packet
-// through a small state machine.  The expensive part of the method is the
-// straight cell walk: per packet a peel-off walk per instrument at emission and
-// at every scattering, and two walks of the forced path per scattering (the
-// first accumulates the optical depth to the boundary and deposits absorption,
-// the second stops at the interaction).  Peel-offs towards a frame along a grid
-// axis take their optical depth from per-line column sums; on cartesian grids
-// the other peel-offs become records for the sorted pass (rt_peel.cu), which
-// walks them after this kernel, ordered by start cell.  The main loop advances
-// every walking lane by exactly one cell crossing per iteration, whichever of
-// the remaining walks it is in, so the warp stays converged on the hot path.  The per-event work
-// (emission, forced-scattering inversion, weight update, deposits, the
-// Henyey-Greenstein draw, fetching the next packet) is deferred until enough
-// lanes of the warp need it and is then done for those lanes together;
-// packets are fetched with one atomic per warp.
+// Execution model.  A persistent grid of warps; every warp carries more packets
+// (G::kSlots, state in shared memory) than it has lanes, and a lane holds in
+// registers only the walk it is on.  The expensive part of the method is the
+// straight cell walk: two walks of the forced path per scattering (the first
+// accumulates the optical depth to the boundary and deposits absorption, the
+// second stops at the interaction) and the peel-offs that neither column sums
+// (frames along a grid axis) nor the sorted pass (rt_peel.cu) take.  The main
+// loop advances every walking lane by exactly one cell crossing per iteration,
+// whichever walk it is in.  A lane whose walk ended gets the next packet that
+// is ready to walk; the per-event work (emission, forced-scattering inversion,
+// weight update, deposits, the Henyey-Greenstein draw) runs in rounds over up
+// to 32 packets of the warp that all wait for the same kind of work.
+//
+// What bounds it: instruction issue and the latency of the dependent density
+// loads.  With one packet per lane (the warp's lanes waiting for one another)
+// 21 of 32 lanes walked per iteration and 40 % of the cycles went to rounds
+// serving 16 lanes in five stages; with the slots 27 walk and rounds take 9-25
+// % (2e6 packets of the disk galaxy, execution counters).
 //
 // Precision.  Geometry, the walk and the phase function are FP32.  The
 // cumulative optical depth of the forced path is held as an unevaluated sum
@@ -46,6 +49,42 @@ constexpr float kInv4PiF = 0.0795774715459476679f;
 #define RT_FWD_MIN_BLOCKS 4
 #endif
 
+#ifndef RT_ROUND_MIN
+#define RT_ROUND_MIN 20
+#endif
+#ifndef RT_IDLE_MAX
+#define RT_IDLE_MAX 12
+#endif
+// Rounds of per-event work: a queue of at least kRoundMin packets is served at
+// once, a shorter one when kIdleMax lanes have no walk.  Between (1, 0) and
+// (24, 16): 41.7 to 40.3 ms per 4e6 packets of the disk galaxy, 22.8 to 21.0
+// ms per 2e6 packets of an opaque 48^3 cube; flat around the values here.
+constexpr int kRoundMin = 20, kIdleMax = 12;
+// A launch of few packets uses fewer blocks, down to kSpread packets per warp:
+// 1e3 packets of a 32^3 cube 336 us at 4 per warp, 404 us at 16, 440 us at 32;
+// 1e4 416, 444, 489 us.
+constexpr int kSpread = 4;
+// Packet slots per warp, by grid (see Shared): as many as leave the shared
+// memory of four blocks at 164 KB on cartesian and rectilinear grids (92 KB of
+// the SM's 256 remain for L1; the next step, 196 KB, costs the disk galaxy
+// nothing at 52 slots of a larger layout, the last, 228 KB, 41 -> 50 ms per
+// 4e6 packets) and within reach of four blocks on the others.  48 / 56 / 60 /
+// 64 slots: disk galaxy 40.9 / 40.5 / 40.5 / 40.8 ms, opaque cube 21.5 / 20.2
+// / 19.7 / 19.6 ms; octree 36 / 48 / 56: 30.0 / 27.0 / 30.5 ms per 1e6 packets;
+// k-d tree 36 / 52 / 60: 39.4 / 36.6 / 37.1 ms.
+#ifndef RT_SLOTS_INDEXED
+#define RT_SLOTS_INDEXED 60
+#endif
+#ifndef RT_SLOTS_OCT
+#define RT_SLOTS_OCT 48
+#endif
+#ifndef RT_SLOTS_BIN
+#define RT_SLOTS_BIN 52
+#endif
+#ifndef RT_SLOTS_VOR
+#define RT_SLOTS_VOR 52
+#endif
+
 enum Phase : int {
   kFetch = 0,      // needs a new packet
   kPeelEmit = 1,   // peel-off walk at emission (instrument q)
@@ -67,18 +106,6 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
 }
 
 __device__ __forceinline__ float inv_or_zero(float d) { return d != 0.0f ? 1.0f / d : 0.0f; }
-
-// Exact widening of a positive normal FP32 value to FP64 with integer
-// operations (rebias the exponent by 1023 - 127 and shift the significand),
-// keeping the per-crossing path off GB300's low-rate FP64 pipe.  Zero,
-// subnormal and non-finite inputs take the ordinary conversion.
-__device__ __forceinline__ double widen(float f) {
-  const unsigned u = __float_as_uint(f);
-  const unsigned e = u & 0x7f800000u;
-  if (e == 0u || e == 0x7f800000u) return (double)f;
-  const unsigned hi = ((u & 0x7fffffffu) >> 3) + 0x38000000u;
-  return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)(u << 29));
-}
 
 // f 2^e in FP64 for a positive FP32 f, with integer operations (the widening
 // above with the exponent moved by e); zero for results below FP64's normal
@@ -104,17 +131,6 @@ __device__ __forceinline__ float split_exp(double v, int& e) {
   }
   e = be - 1022;  // v = (1.m / 2) 2^(be - 1022)
   return __uint_as_float((126u << 23) | ((unsigned)(b >> 29) & 0x7fffffu));
-}
-
-// FP64 to FP32 by cutting the significand to 24 bits, with integer
-// operations; zero and values outside the normal FP32 range take the
-// ordinary conversion.
-__device__ __forceinline__ float cut(double v) {
-  const long long b = __double_as_longlong(v);
-  const int be = (int)((b >> 52) & 0x7ff);
-  if (be < 1023 - 126 || be > 1023 + 127) return (float)v;
-  const unsigned top = (unsigned)((unsigned long long)b >> 32);
-  return __uint_as_float((top & 0x80000000u) | ((unsigned)(be - 896) << 23) | ((unsigned)(b >> 29) & 0x7fffffu));
 }
 
 // v as the unevaluated FP32 pair hi + lo: hi = v cut to 24 bits, lo = the
@@ -196,6 +212,7 @@ struct CartGrid {
   static constexpr bool kColumns = true;  // peel-offs along grid axes may use column sums
   static constexpr bool kIndexCells = true;  // cells indexed by (ix, iy, iz) between planes
   static constexpr bool kSortedPass = true;  // walked peel-offs may go to the sorted pass
+  static constexpr int kSlots = RT_SLOTS_INDEXED;
   struct Cell {
     int ix, iy, iz;
   };
@@ -281,6 +298,11 @@ struct CartGrid {
   template <class Geo>
   __device__ static __forceinline__ int id(const Geo& P, const Walk& w) { return w.ix + P.nx * (w.iy + P.ny * w.iz); }
 
+  // The row-major id of a carried cell.
+  __device__ static __forceinline__ int cell_id(const FwdParams& P, const Cell& c) {
+    return c.ix + P.nx * (c.iy + P.ny * c.iz);
+  }
+
   // Plane i of axis a.
   __device__ static __forceinline__ float plane(const FwdParams& P, int a, int i) {
     return fmaf((float)i, P.d[a], P.lo[a]);
@@ -314,6 +336,7 @@ struct RectGrid {
   static constexpr bool kColumns = true;
   static constexpr bool kIndexCells = true;
   static constexpr bool kSortedPass = false;
+  static constexpr int kSlots = RT_SLOTS_INDEXED;
   using Cell = CartGrid::Cell;
   using Walk = CartGrid::Walk;
   struct Scratch {};
@@ -390,6 +413,8 @@ struct RectGrid {
     return w.ix + P.nx * (w.iy + P.ny * w.iz);
   }
 
+  __device__ static __forceinline__ int cell_id(const FwdParams& P, const Cell& c) { return CartGrid::cell_id(P, c); }
+
   __device__ static __forceinline__ float plane(const FwdParams& P, int a, int i) { return edge(P, a, i); }
 
   __device__ static __forceinline__ void locate_cell(const FwdParams& P, float3 x, Cell& c) {
@@ -414,14 +439,12 @@ constexpr int kOctStack = kMaxOctreeDepth + 1;  // path stack: depths 0..21 (3 p
 constexpr int kChildCache = 1024;                // first child[] entries kept in shared memory
 
 __shared__ int S_CHILD[kChildCache];
-// the octree kernel's per-lane ancestor stacks, P.oct_levels entries each
-// (dynamic shared memory sized by the tree's depth)
-extern __shared__ int S_OCT_STACK[];
 
 struct OctGrid {
   static constexpr bool kColumns = false;
   static constexpr bool kIndexCells = false;
   static constexpr bool kSortedPass = false;
+  static constexpr int kSlots = RT_SLOTS_OCT;
   struct Cell {
     int leaf;
     float lo[3], hi[3];
@@ -435,8 +458,12 @@ struct OctGrid {
     float lo[3], hi[3];
     unsigned long long path;
   };
+  // the lane's ancestor stack: entry l at stack[l kBlock] (dynamic shared
+  // memory of P.oct_levels rows; consecutive lanes on consecutive words, so
+  // lanes at different levels never meet in a bank)
   struct Scratch {
     int* stack;
+    __device__ __forceinline__ int& operator[](int level) const { return stack[level * kBlock]; }
   };
 
   __device__ static __forceinline__ int child(const FwdParams& P, int node) {
@@ -461,7 +488,7 @@ struct OctGrid {
 
   // Descend from node stack[depth] (box w.lo/hi) to the leaf containing p.
   __device__ static __forceinline__ bool descend(const FwdParams& P, float3 p, float3 d, Walk& w, Scratch& sc) {
-    int node = sc.stack[w.depth];
+    int node = sc[w.depth];
     while (true) {
       const int c = child(P, node);
       if (c < 0) {
@@ -477,7 +504,7 @@ struct OctGrid {
       w.path |= (unsigned long long)oct << (3 * w.depth);
       node = c + oct;
       w.depth += 1;
-      sc.stack[w.depth] = node;
+      sc[w.depth] = node;
     }
   }
 
@@ -487,7 +514,7 @@ struct OctGrid {
     for (int a = 0; a < 3; ++a) { w.lo[a] = P.lo[a]; w.hi[a] = P.hi[a]; }
     w.depth = 0;
     w.path = 0ull;
-    sc.stack[0] = 0;
+    sc[0] = 0;
     return descend(P, p, d, w, sc);
   }
 
@@ -579,7 +606,7 @@ struct OctGrid {
         // leaf above it.  The box: the old leaf's, moved across the face, then
         // doubled on the side away from each octant up to the level reached.
         const int flip = 1 << axis;
-        int node = sc.stack[part];
+        int node = sc[part];
         int c = child(P, node);
         unsigned long long path = part > 0 ? (old_path & ((1ull << (3 * part)) - 1ull)) : 0ull;
         depth = part;
@@ -588,7 +615,7 @@ struct OctGrid {
           path |= (unsigned long long)oct << (3 * depth);
           node = c + oct;
           depth += 1;
-          sc.stack[depth] = node;
+          sc[depth] = node;
           c = child(P, node);
         }
 #pragma unroll
@@ -657,6 +684,7 @@ struct OctGrid {
   __device__ static __forceinline__ int cell(const Walk& w) { return w.leaf; }
 
   __device__ static __forceinline__ int id(const FwdParams&, const Walk& w) { return w.leaf; }
+  __device__ static __forceinline__ int cell_id(const FwdParams&, const Cell& c) { return c.leaf; }
 
   __device__ static __forceinline__ Cell carried(const Walk& w) {
     Cell c;
@@ -691,6 +719,7 @@ struct BinGrid {
   static constexpr bool kColumns = false;
   static constexpr bool kIndexCells = false;
   static constexpr bool kSortedPass = false;
+  static constexpr int kSlots = RT_SLOTS_BIN;
   using Cell = OctGrid::Cell;  // the leaf and its box
   struct Walk {
     int leaf;
@@ -810,6 +839,7 @@ struct BinGrid {
 
   __device__ static __forceinline__ int cell(const Walk& w) { return w.leaf; }
   __device__ static __forceinline__ int id(const FwdParams&, const Walk& w) { return w.leaf; }
+  __device__ static __forceinline__ int cell_id(const FwdParams&, const Cell& c) { return c.leaf; }
 
   __device__ static __forceinline__ Cell carried(const Walk& w) {
     Cell c;
@@ -843,6 +873,7 @@ struct VorGrid {
   static constexpr bool kColumns = false;
   static constexpr bool kIndexCells = false;
   static constexpr bool kSortedPass = false;
+  static constexpr int kSlots = RT_SLOTS_VOR;
   using Cell = OctGrid::Cell;  // the cell id in .leaf (the box is not used)
   struct Walk {
     int leaf;   // current cell
@@ -965,6 +996,7 @@ struct VorGrid {
 
   __device__ static __forceinline__ int cell(const Walk& w) { return w.leaf; }
   __device__ static __forceinline__ int id(const FwdParams&, const Walk& w) { return w.leaf; }
+  __device__ static __forceinline__ int cell_id(const FwdParams&, const Cell& c) { return c.leaf; }
 
   __device__ static __forceinline__ Cell carried(const Walk& w) {
     Cell c;
@@ -982,109 +1014,134 @@ struct VorGrid {
   }
 };
 
-// ---------------------------------------------------------------- lane state
-// The lane state that only the per-event work touches lives in per-thread
-// slots of shared memory (structure of arrays: the lanes of a warp hit
-// distinct banks), so that the walk's own state fits the registers of four
-// resident blocks per SM.
-__shared__ unsigned long long S_PID[kBlock];
-__shared__ double S_WEIGHT[kBlock];
-__shared__ float3 S_DIR[kBlock];
-__shared__ float2 S_HG[kBlock];
-__shared__ int S_EVENT[kBlock], S_INSTR_Q[kBlock], S_WPHASE[kBlock];
-// binary exponent of a path-1 deposit weight outside [1e-30, 1e30] (aux1 < 0)
-__shared__ int S_DEPEXP[kBlock];
-__shared__ bool S_HAS_CELL[kBlock];
-__shared__ CartGrid::Cell S_CELL_CART[kBlock];
-__shared__ OctGrid::Cell S_CELL_OCT[kBlock];
+// ---------------------------------------------------------------- packet slots
+// A warp carries more packets than it has lanes: G::kSlots slots of shared
+// memory per warp (structure of arrays) hold the packets' state between
+// walks, a lane holds in registers only the walk it is on.  A packet is either
+// walked by a lane or waits in one of the warp's queues: for a lane (kQReady)
+// or for per-event work of one kind (kQPath1: its first walk ended; kQEvent:
+// its second walk or a peel-off walk ended; kQFetch: the slot is free and
+// takes a new packet).  Lanes whose walk ended are given the next ready packet,
+// so walking lanes stay near the full warp, and per-event work runs as rounds
+// over up to 32 packets that all need the same work.
+enum Queue : int { kQPath1 = 0, kQEvent = 1, kQFetch = 2, kQReady = 3, kQueues = 4 };
+constexpr int kWarps = kBlock / 32;
+constexpr int kRing = 64;  // entries of a queue's ring buffer; slots per warp are at most this
 
-template <class G>
-__device__ __forceinline__ typename G::Cell& cell_slot();
-template <>
-__device__ __forceinline__ CartGrid::Cell& cell_slot<CartGrid>() { return S_CELL_CART[threadIdx.x]; }
-template <>
-__device__ __forceinline__ OctGrid::Cell& cell_slot<OctGrid>() { return S_CELL_OCT[threadIdx.x]; }
-template <>
-__device__ __forceinline__ RectGrid::Cell& cell_slot<RectGrid>() { return S_CELL_CART[threadIdx.x]; }
-template <>
-__device__ __forceinline__ BinGrid::Cell& cell_slot<BinGrid>() { return S_CELL_OCT[threadIdx.x]; }
-template <>
-__device__ __forceinline__ VorGrid::Cell& cell_slot<VorGrid>() { return S_CELL_OCT[threadIdx.x]; }
+// Counts of one warp, kept by its first lane.
+struct WarpTally {
+  unsigned long long crossings, path_crossings, column_crossings;
+  unsigned long long events, peeloffs, packets, column_peels;
+};
 
+// Luminosity tallies of one lane, in its local memory.
+struct LaneTally {
+  double escaped, absorbed, truncated;
+};
+
+template <class G, bool kTape>
+struct Shared {
+  static constexpr int kN = kWarps * G::kSlots;
+  unsigned long long pid[kN];   // packet id
+  double L[kN];                 // weight
+  float2 hg[kN];                // the event's Henyey-Greenstein uniforms
+  // what a walk starts with (path 1: the deposit weight, path 2: tau* as a
+  // pair) and what it ended with (the optical depth pair; path 2: s*)
+  float2 res[kN];
+  float3 x[kN], k[kN];          // position, direction of travel
+  typename G::Cell cell[kN];    // the cell of x (valid with the has-cell bit)
+  int event[kN];                // event index
+  unsigned pack[kN];            // see Pack
+  float3 g[kTape ? kN : 1];     // tape: plane sums of the first walk
+  WarpTally tally[kWarps];
+  LaneTally lum[kWarps];        // the warps' luminosity tallies, at the end
+  uint2 queues[kWarps];         // each warp's queue counts and heads (see Queues)
+  unsigned char ring[kWarps][kQueues][kRing];
+};
+
+// The small fields of a slot in one word: phase (4 bits), wavelength (6),
+// instrument of the next peel-off (5), has-cell (1), exponent of the deposit
+// weight (16, signed).
+struct Pack {
+  __device__ static __forceinline__ unsigned make(int phase, int lam, int q, bool has_cell, int e) {
+    return (unsigned)phase | ((unsigned)lam << 4) | ((unsigned)q << 10) | (has_cell ? 1u << 15 : 0u) |
+           ((unsigned)e << 16);
+  }
+  __device__ static __forceinline__ int phase(unsigned p) { return (int)(p & 15u); }
+  __device__ static __forceinline__ int lam(unsigned p) { return (int)((p >> 4) & 63u); }
+  __device__ static __forceinline__ int q(unsigned p) { return (int)((p >> 10) & 31u); }
+  __device__ static __forceinline__ bool has_cell(unsigned p) { return (p >> 15) & 1u; }
+  __device__ static __forceinline__ int exponent(unsigned p) { return (int)p >> 16; }
+};
+
+// the kernel's Shared (and, for octrees, the ancestor stacks behind it)
+extern __shared__ __align__(16) unsigned char S_RAW[];
+template <class G, bool kTape>
+__device__ __forceinline__ Shared<G, kTape>& shared_state() {
+  return *reinterpret_cast<Shared<G, kTape>*>(S_RAW);
+}
+
+// The walk a lane is on.
 template <class G>
-struct Lane {
-  int lam, phase;
-  float kappa;          // extinction per unit density at this wavelength
-  float3 x;             // position
+struct Walker {
+  int slot;             // the packet's slot (index in the block's arrays), -1: none
+  int phase;            // kPath1, kPath2, kPeelEmit or kPeelScat
+  double* absorption;   // the tallies of this wavelength
   bool walking;
-  // in shared memory: packet id, event index, instrument of the next
-  // peel-off, the walk a kStart lane begins, weight, direction of travel,
-  // the event's Henyey-Greenstein uniforms, the cell of x (valid when
-  // has_cell)
-  __device__ __forceinline__ unsigned long long& pid() const { return S_PID[threadIdx.x]; }
-  __device__ __forceinline__ int& event() const { return S_EVENT[threadIdx.x]; }
-  __device__ __forceinline__ int& q() const { return S_INSTR_Q[threadIdx.x]; }
-  __device__ __forceinline__ int& wphase() const { return S_WPHASE[threadIdx.x]; }
-  __device__ __forceinline__ double& L() const { return S_WEIGHT[threadIdx.x]; }
-  __device__ __forceinline__ float3& k() const { return S_DIR[threadIdx.x]; }
-  __device__ __forceinline__ float& u_mu() const { return S_HG[threadIdx.x].x; }
-  __device__ __forceinline__ float& u_phi() const { return S_HG[threadIdx.x].y; }
-  __device__ __forceinline__ typename G::Cell& cell() const { return cell_slot<G>(); }
-  __device__ __forceinline__ bool& has_cell() const { return S_HAS_CELL[threadIdx.x]; }
-  float3 d, id;         // direction of the current walk and its inverse
-  typename G::Walk w;   // the walk: its current cell and exit data
-  float rho;            // density of the walk's current cell (loaded one crossing ahead)
-  float th, tl;         // optical depth of the current walk (pair sum)
+  float kappa;          // extinction per unit density at this wavelength
+  float3 x;             // start of the walk
+  float3 d, id;         // its direction and inverse
+  typename G::Walk w;   // its current cell and exit data
+  float rho;            // density of the current cell (loaded one crossing ahead)
+  float th, tl;         // optical depth so far (pair sum)
+  unsigned n;           // crossings so far
   // path 1: the deposit weight (1 - albedo) L as aux0 2^e: aux0 the FP32
   // weight (e = 0) while that lies in [1e-30, 1e30], with aux1 = 64, the
   // optical depth below which a deposit takes the plain FP32 product; else
-  // aux0 in [1/2, 1) and e in S_DEPEXP, aux1 = -1 (every deposit carries the
+  // aux0 in [1/2, 1) and e in the slot's word, aux1 = -1 (every deposit carries the
   // exponent), so that deposits keep FP64's range whatever the weight;
   // path 2: tau* as a float pair, then s*
   float aux0, aux1;
-  // adjoint tape (launches that record one): plane sums of the current path
-  // walk, entry axis of its segment, crossings so far, the interaction's
-  // crossing index, kappa rho and remainder, the unit exponent of weights
+  // adjoint tape (launches that record one): plane sums of the walk, entry
+  // axis of its segment, the interaction's crossing index, kappa rho and
+  // remainder
   float3 g;
-  int axis_in, n_cross, h, eL;
+  int axis_in, h;
   float kr_h, rem;
-  AdjRecord* rec;
 };
 
-// Small per-launch tables (instruments, per-wavelength optics) copied to
-// shared memory at kernel start.
-__shared__ DevInstr S_INSTR[kMaxInstruments];
-__shared__ DevLambda S_LAM[kMaxLambda];
-
-// Per-lane tallies, one slot per thread in shared memory (no atomics).
-struct LaneTally {
-  double escaped, absorbed, truncated;
-  unsigned long long crossings, path_crossings, column_crossings;
-  unsigned events, peeloffs, packets, column_peels;
+// A packet in per-event work: its slot and the fields in registers.
+template <class G, bool kTape>
+struct Task {
+  Shared<G, kTape>& sh;
+  LaneTally& tally;
+  int i;             // slot
+  int phase, wphase; // kStart: the walk to start
+  int lam, q, event;
+  bool has_cell;
+  int dep_exp;
+  float th, tl;      // optical depth of the walk that ended (path 2: th = s*)
+  unsigned n_peel, n_col, c_col;  // peel-offs, of which by column sums, and their crossings
+  __device__ __forceinline__ unsigned long long& pid() const { return sh.pid[i]; }
+  __device__ __forceinline__ double& L() const { return sh.L[i]; }
+  __device__ __forceinline__ float3& x() const { return sh.x[i]; }
+  __device__ __forceinline__ float3& k() const { return sh.k[i]; }
+  __device__ __forceinline__ float2& hg() const { return sh.hg[i]; }
+  __device__ __forceinline__ float2& res() const { return sh.res[i]; }
+  __device__ __forceinline__ typename G::Cell& cell() const { return sh.cell[i]; }
 };
 
-template <class G>
-__device__ __forceinline__ void trace_row(const FwdParams& P, const Lane<G>& s, int event, int cell, double L,
+template <class G, bool kTape>
+__device__ __forceinline__ void trace_row(const FwdParams& P, const Task<G, kTape>& s, int event, int cell, double L,
                                           double tau_path, double tau_star) {
   if (!P.trace || s.pid() != P.trace_packet || s.lam != P.trace_lambda || event >= P.trace_cap) return;
   rt_trace_row r;
+  const float3 x = s.x(), k = s.k();
   r.event = event; r.reserved = 0; r.cell = cell;
-  r.x[0] = s.x.x; r.x[1] = s.x.y; r.x[2] = s.x.z;
-  r.k[0] = s.k().x; r.k[1] = s.k().y; r.k[2] = s.k().z;
+  r.x[0] = x.x; r.x[1] = x.y; r.x[2] = x.z;
+  r.k[0] = k.x; r.k[1] = k.y; r.k[2] = k.z;
   r.L = L; r.tau_path = tau_path; r.tau_star = tau_star;
   P.trace[event] = r;
-}
-
-// Start a walk from the lane's position along d; the first cell's density
-// load is issued here.
-template <class G>
-__device__ __forceinline__ void start_walk(const FwdParams& P, Lane<G>& s, float3 d, typename G::Scratch& sc) {
-  s.d = d;
-  s.id = make_float3(inv_or_zero(d.x), inv_or_zero(d.y), inv_or_zero(d.z));
-  s.th = 0.0f;
-  s.tl = 0.0f;
-  s.walking = G::init(P, s.x, d, s.id, s.has_cell(), s.cell(), s.w, sc);
-  if (s.walking) s.rho = load_density(&P.density[G::cell(s.w)]);
 }
 
 __device__ __forceinline__ float3 instr_dir(const DevInstr& I) { return make_float3(I.kobs[0], I.kobs[1], I.kobs[2]); }
@@ -1121,15 +1178,13 @@ __device__ __forceinline__ bool column_tau(const FwdParams& P, float3 x, bool kn
   return true;
 }
 
-template <class G>
-__device__ __forceinline__ bool column_peel(const FwdParams& P, Lane<G>& s, const DevInstr& I, LaneTally* bt) {
+template <class G, bool kTape>
+__device__ __forceinline__ bool column_peel(const FwdParams& P, Task<G, kTape>& s, const DevInstr& I) {
   unsigned long long nc;
-  if (!column_tau<G>(P, s.x, s.has_cell(), s.cell(), I, s.kappa, s.th, nc)) return false;
+  if (!column_tau<G>(P, s.x(), s.has_cell, s.cell(), I, P.lam[s.lam].kappa, s.th, nc)) return false;
   s.tl = 0.0f;
-  s.walking = false;
-  bt->crossings += nc;
-  bt->column_crossings += nc;
-  bt->column_peels += 1u;
+  s.c_col += (unsigned)nc;
+  s.n_col += 1u;
   return true;
 }
 
@@ -1167,8 +1222,8 @@ __device__ __forceinline__ unsigned ray_tau(const FwdParams& P, float3 x, float3
 }
 
 // Phase-function value of a scattering peel-off towards instrument I.
-__device__ __forceinline__ float peel_phase(int lam, float3 k, const DevInstr& I) {
-  return hg_phase(S_LAM[lam].g, k.x * I.kobs[0] + k.y * I.kobs[1] + k.z * I.kobs[2]);
+__device__ __forceinline__ float peel_phase(const FwdParams& P, int lam, float3 k, const DevInstr& I) {
+  return hg_phase(P.lam[lam].g, k.x * I.kobs[0] + k.y * I.kobs[1] + k.z * I.kobs[2]);
 }
 
 // Deposit a finished peel-off from x (weight L, phase-function value phase,
@@ -1176,7 +1231,7 @@ __device__ __forceinline__ float peel_phase(int lam, float3 k, const DevInstr& I
 // label debug records.
 __device__ __forceinline__ void deposit_peel(const FwdParams& P, int q, int lam, float3 x, double L, float phase,
                                              float th, float tl, bool scattered, unsigned long long pid, int event) {
-  const DevInstr& I = S_INSTR[q];
+  const DevInstr& I = P.instr[q];
   // exp(-(th + tl)) with the walk's compensated optical depth: the low word
   // enters as the first-order factor (1 - tl)
   const float tau = th;
@@ -1185,14 +1240,25 @@ __device__ __forceinline__ void deposit_peel(const FwdParams& P, int q, int lam,
   const int ch = scattered ? 2 : 1;
   if (I.sed) {
     // an SED instrument has one bin per wavelength and channel: the lanes of
-    // the warp that deposit into the same bin add their values first (in lane
-    // order) and one of them issues the atomics
+    // the warp that deposit into the same bin add their values first and one of
+    // them issues the atomics; consecutive lanes (nearly always the case) by
+    // halving steps, 5 FP64 additions instead of up to 31
     const unsigned act = __activemask();
     const unsigned key = ((unsigned)q << 20) | ((unsigned)lam << 1) | (scattered ? 1u : 0u);
     const unsigned grp = __match_any_sync(act, key);
-    double sum = 0.0;
-    for (unsigned m = grp; m; m &= m - 1u) sum += __shfl_sync(grp, value, __ffs(m) - 1);
-    if ((int)(threadIdx.x & 31u) == __ffs(grp) - 1) {
+    const int first = __ffs(grp) - 1, last = 31 - __clz(grp), lane = (int)(threadIdx.x & 31u);
+    double sum = value;
+    if (__popc(grp) == last - first + 1) {
+      for (int o = 16; o > 0; o >>= 1) {
+        if (o > last - first) continue;  // the same for the whole group
+        const double v = __shfl_sync(grp, sum, min(lane + o, last));
+        if (lane + o <= last) sum += v;
+      }
+    } else {
+      sum = 0.0;
+      for (unsigned m = grp; m; m &= m - 1u) sum += __shfl_sync(grp, value, __ffs(m) - 1);
+    }
+    if (lane == first) {
       atomicAdd(&I.image[lam], sum);
       if (I.channels == 3) atomicAdd(&I.image[(size_t)ch * P.n_lambda + lam], sum);
     }
@@ -1244,10 +1310,10 @@ __device__ __forceinline__ void deposit_peel(const FwdParams& P, int q, int lam,
   }
 }
 
-template <class G>
-__device__ __forceinline__ void peel_deposit(const FwdParams& P, const Lane<G>& s, bool scattered) {
-  const float phase = scattered ? peel_phase(s.lam, s.k(), S_INSTR[s.q()]) : 1.0f;
-  deposit_peel(P, s.q(), s.lam, s.x, s.L(), phase, s.th, s.tl, scattered, s.pid(), s.event());
+template <class G, bool kTape>
+__device__ __forceinline__ void peel_deposit(const FwdParams& P, const Task<G, kTape>& s, int q, bool scattered) {
+  const float phase = scattered ? peel_phase(P, s.lam, s.k(), P.instr[q]) : 1.0f;
+  deposit_peel(P, q, s.lam, s.x(), s.L(), phase, s.th, s.tl, scattered, s.pid(), s.event);
 }
 
 // Hand the peel-off towards instrument q from x to the sorted pass: a
@@ -1286,10 +1352,10 @@ __device__ __forceinline__ bool defer_record(const FwdParams& P, int q, int lam,
   return true;
 }
 
-template <class G>
-__device__ __forceinline__ bool defer_peel(const FwdParams& P, const Lane<G>& s, const DevInstr& I, bool emission) {
-  const float phase = emission ? 1.0f : peel_phase(s.lam, s.k(), I);
-  return defer_record(P, s.q(), s.lam, s.x, s.L(), phase, s.has_cell(), s.cell(), emission, s.pid(), s.event());
+template <class G, bool kTape>
+__device__ __forceinline__ bool defer_peel(const FwdParams& P, const Task<G, kTape>& s, int q, bool emission) {
+  const float phase = emission ? 1.0f : peel_phase(P, s.lam, s.k(), P.instr[q]);
+  return defer_record(P, q, s.lam, s.x(), s.L(), phase, s.has_cell, s.cell(), emission, s.pid(), s.event);
 }
 
 // Emission (Sect. 3.4): source component by luminosity (FP64 comparison of
@@ -1371,29 +1437,29 @@ __device__ __forceinline__ void emit_dust(const FwdParams& P, unsigned long long
   }
 }
 
-// Ask for walk `phase` from the lane's position along d; walks start in the
-// last stage of a control round, from one place in the code.
-template <class G>
-__device__ __forceinline__ void request_walk(Lane<G>& s, int phase, float3 d) {
-  s.wphase() = phase;
-  s.d = d;
+// Ask for walk `phase` (towards instrument s.q for a peel-off, else along the
+// direction of travel); a lane starts it when it is free.
+template <class G, bool kTape>
+__device__ __forceinline__ void request_walk(Task<G, kTape>& s, int phase) {
+  s.wphase = phase;
   s.phase = kStart;
 }
 
-// The forced path of event s.event(): its first walk carries the deposit
+// The forced path of event s.event: its first walk carries the deposit
 // weight (1 - albedo) L.
-template <class G>
-__device__ __forceinline__ void request_path(Lane<G>& s) {
-  const double wdep = S_LAM[s.lam].one_minus_albedo * s.L();
-  const bool plain = wdep >= 1e-30 && wdep <= 1e30;
+template <class G, bool kTape>
+__device__ __forceinline__ void request_path(const FwdParams& P, Task<G, kTape>& s) {
+  const double wdep = P.lam[s.lam].one_minus_albedo * s.L();
+  // integer comparisons: positive doubles order like their bit patterns
+  const bool plain = bits_of(wdep) >= bits_of(1e-30) && bits_of(wdep) <= bits_of(1e30);
   int e = 0;
-  s.aux0 = plain ? cut(wdep) : split_exp(wdep, e);
-  s.aux1 = plain ? 64.0f : -1.0f;
-  S_DEPEXP[threadIdx.x] = e;
-  request_walk(s, kPath1, s.k());
+  const float a = plain ? cut(wdep) : split_exp(wdep, e);
+  s.res() = make_float2(a, plain ? 64.0f : -1.0f);
+  s.dep_exp = e;
+  request_walk(s, kPath1);
 }
 
-// ---- the stages of a control round (each for the lanes in that phase)
+// ---- the stages of a control round (each for the packets in that phase)
 
 // ---- the adjoint tape (cartesian grids; records as the adjoint's replay writes them)
 
@@ -1408,151 +1474,156 @@ __device__ __forceinline__ float tape_units(double v, int e) {
   return __uint_as_float((top & 0x80000000u) | ((unsigned)fe << 23) | ((unsigned)(b >> 29) & 0x7fffffu));
 }
 
-template <class G>
-__device__ __forceinline__ int tape_cell(const FwdParams& P, const Lane<G>& s) {
+// The unit exponent of weights: L0 = m 2^e, m in [1/2, 1).
+__device__ __forceinline__ int tape_exponent(const FwdParams& P, int lam) {
+  const int be = (int)((__double_as_longlong(P.L0[lam]) >> 52) & 0x7ff);
+  return be == 0 ? 0 : be - 1022;
+}
+
+// The packet's records on the tape.
+__device__ __forceinline__ AdjRecord* tape_records(const FwdParams& P, int lam, unsigned long long pid) {
+  return P.tape + (size_t)((unsigned long long)lam * P.n_per_lambda + (pid - P.first_id)) * (size_t)P.tape_stride;
+}
+
+template <class G, bool kTape>
+__device__ __forceinline__ int tape_cell(const FwdParams& P, const Task<G, kTape>& s) {
   if constexpr (G::kColumns) {
-    return s.has_cell() ? s.cell().ix + P.nx * (s.cell().iy + P.ny * s.cell().iz) : -1;
+    return s.has_cell ? s.cell().ix + P.nx * (s.cell().iy + P.ny * s.cell().iz) : -1;
   } else {
     return -1;
   }
 }
 
 // The packet ends after event J: record 0 holds J and the last position.
-template <class G>
-__device__ __forceinline__ void tape_end(const FwdParams& P, const Lane<G>& s, int J) {
-  AdjRecord& r = s.rec[0];
+template <class G, bool kTape>
+__device__ __forceinline__ void tape_end(const FwdParams& P, const Task<G, kTape>& s, int J) {
+  AdjRecord& r = tape_records(P, s.lam, s.pid())[0];
+  const float3 x = s.x();
   r.h = J;
-  r.x[0] = s.x.x; r.x[1] = s.x.y; r.x[2] = s.x.z;
+  r.x[0] = x.x; r.x[1] = x.y; r.x[2] = x.z;
   r.cell = tape_cell(P, s);
-  r.L = tape_units(s.L(), s.eL);
+  r.L = tape_units(s.L(), tape_exponent(P, s.lam));
 }
 
 // A new packet (index w of the launch): wavelength, weight, emission.
 template <class G, bool kTape>
-__device__ __forceinline__ void fetch(const FwdParams& P, Lane<G>& s, unsigned long long w, LaneTally* bt) {
+__device__ __forceinline__ void fetch(const FwdParams& P, Task<G, kTape>& s, unsigned long long w) {
   if (w >= P.n_total) { s.phase = kExit; return; }
   int lam = min((int)(__ull2float_rz(w) * P.inv_n_per_lambda), P.n_lambda - 1);
   while (lam > 0 && (unsigned long long)lam * P.n_per_lambda > w) --lam;
   while (lam + 1 < P.n_lambda && (unsigned long long)(lam + 1) * P.n_per_lambda <= w) ++lam;
   s.lam = lam;
-  s.pid() = P.first_id + (w - (unsigned long long)lam * P.n_per_lambda);
+  const unsigned long long pid = P.first_id + (w - (unsigned long long)lam * P.n_per_lambda);
+  s.pid() = pid;
   const double L0 = P.L0[lam];
   if (L0 == 0.0) {  // no emission at this wavelength (dust that emits nothing here)
-    bt->packets += 1u;
     s.phase = kFetch;
     return;
   }
-  s.kappa = S_LAM[lam].kappa;
   s.L() = L0;
-  s.event() = 0;
-  s.has_cell() = false;
+  s.event = 0;
+  s.has_cell = false;
+  float3 x, k;
   if constexpr (G::kIndexCells) {
     if (P.dust_cum) {
-      emit_dust<G>(P, s.pid(), s.lam, s.x, s.k(), s.cell());
-      s.has_cell() = true;
+      emit_dust<G>(P, pid, lam, x, k, s.cell());
+      s.has_cell = true;
     } else {
-      emit(P, s.pid(), s.lam, s.x, s.k());
+      emit(P, pid, lam, x, k);
     }
   } else {
-    emit(P, s.pid(), s.lam, s.x, s.k());
+    emit(P, pid, lam, x, k);
   }
-  bt->packets += 1u;
+  s.x() = x;
+  s.k() = k;
   trace_row(P, s, 0, -1, L0, 0.0, 0.0);
-  if (kTape) {
-    s.rec = P.tape + (size_t)w * (size_t)P.tape_stride;
-    const int be = (int)((__double_as_longlong(L0) >> 52) & 0x7ff);
-    s.eL = be == 0 ? 0 : be - 1022;  // L0 = m 2^eL, m in [1/2, 1)
-  }
-  s.q() = 0;
+  s.q = 0;
   s.phase = kPeelScan;
 }
 
 // Path 1 ended: escape, or the deposit bookkeeping and the forced-scattering
 // inversion (FP64); then the second walk.
 template <class G, bool kTape>
-__device__ __forceinline__ void finish_path1(const FwdParams& P, Lane<G>& s, LaneTally* bt) {
+__device__ __forceinline__ void finish_path1(const FwdParams& P, Task<G, kTape>& s) {
   const double tau = widen(s.th) + widen(s.tl);
   if (!(tau > 0.0)) {
-    trace_row(P, s, s.event(), -1, s.L(), 0.0, 0.0);
-    bt->escaped += s.L();
-    if (kTape) tape_end(P, s, s.event() - 1);
+    trace_row(P, s, s.event, -1, s.L(), 0.0, 0.0);
+    s.tally.escaped += s.L();
+    if (kTape) tape_end(P, s, s.event - 1);
     s.phase = kFetch;
     return;
   }
   const double one_minus_E = -expm1(-tau);
   const double E = 1.0 - one_minus_E;
-  bt->escaped += s.L() * E;
-  bt->absorbed += S_LAM[s.lam].one_minus_albedo * s.L() * one_minus_E;
-  const uint4 r = draw_block(s.pid(), s.lam, s.event(), 0, P.seed, P.model);
+  const double L = s.L();
+  s.tally.escaped += L * E;
+  s.tally.absorbed += P.lam[s.lam].one_minus_albedo * L * one_minus_E;
+  const uint4 r = draw_block(s.pid(), s.lam, s.event, 0, P.seed, P.model);
   const double tau_star = -log1p(-u01(r.x) * one_minus_E);
-  s.u_mu() = u01f(r.y);
-  s.u_phi() = u01f(r.z);
-  split_pair(tau_star, s.aux0, s.aux1);
+  s.hg() = make_float2(u01f(r.y), u01f(r.z));
   if (kTape) {
     // the record's first two sectors, whole, with 16-byte stores
-    float4* t = reinterpret_cast<float4*>(&s.rec[s.event()]);
-    t[0] = make_float4(s.x.x, s.x.y, s.x.z, s.k().x);
-    t[1] = make_float4(s.k().y, s.k().z, __int_as_float(tape_cell(P, s)), tape_units(s.L(), s.eL));
-    t[2] = make_float4((float)one_minus_E, (float)E, u01f(r.x), s.g.x);
-    t[3] = make_float4(s.g.y, s.g.z, 0.0f, 0.0f);
-    s.h = -1;
+    const float3 x = s.x(), k = s.k(), g = s.sh.g[s.i];
+    float4* t = reinterpret_cast<float4*>(&tape_records(P, s.lam, s.pid())[s.event]);
+    t[0] = make_float4(x.x, x.y, x.z, k.x);
+    t[1] = make_float4(k.y, k.z, __int_as_float(tape_cell(P, s)), tape_units(L, tape_exponent(P, s.lam)));
+    t[2] = make_float4((float)one_minus_E, (float)E, u01f(r.x), g.x);
+    t[3] = make_float4(g.y, g.z, 0.0f, 0.0f);
   }
-  s.L() = S_LAM[s.lam].albedo * s.L() * one_minus_E;  // weight after the scattering
-  request_walk(s, kPath2, s.k());
+  s.L() = P.lam[s.lam].albedo * L * one_minus_E;  // weight after the scattering
+  float2 a;
+  split_pair(tau_star, a.x, a.y);
+  s.res() = a;
+  request_walk(s, kPath2);
 }
 
-// Path 2 ended in the interaction cell (aux0 holds s*): move the packet,
-// then the scattering peel-offs.
+// Path 2 ended in the interaction cell (th holds s*, the slot the cell): move
+// the packet, then the scattering peel-offs.
 template <class G, bool kTape>
-__device__ __forceinline__ void finish_path2(const FwdParams& P, Lane<G>& s, LaneTally* bt) {
-  if (kTape) {
-    // the record's third sector, whole
-    float4* t = reinterpret_cast<float4*>(&s.rec[s.event()]);
-    t[4] = make_float4(__int_as_float(s.h), __int_as_float(s.axis_in), __int_as_float(G::id(P, s.w)), s.kr_h);
-    t[5] = make_float4(s.rem, s.g.x, s.g.y, s.g.z);
-  }
-  const float s_star = s.aux0;
-  float3 x = make_float3(fmaf(s_star, s.k().x, s.x.x), fmaf(s_star, s.k().y, s.x.y), fmaf(s_star, s.k().z, s.x.z));
-  s.cell() = G::carried(s.w);
+__device__ __forceinline__ void finish_path2(const FwdParams& P, Task<G, kTape>& s) {
+  const float s_star = s.th;
+  const float3 x0 = s.x(), k = s.k();
+  float3 x = make_float3(fmaf(s_star, k.x, x0.x), fmaf(s_star, k.y, x0.y), fmaf(s_star, k.z, x0.z));
   G::clamp(P, s.cell(), x);
-  s.x = x;
-  s.has_cell() = true;
-  bt->events += 1u;
-  trace_row(P, s, s.event(), G::id(P, s.w), s.L(), 0.0, 0.0);
-  s.q() = 0;
+  s.x() = x;
+  s.has_cell = true;
+  trace_row(P, s, s.event, G::cell_id(P, s.cell()), s.L(), 0.0, 0.0);
+  s.q = 0;
   s.phase = kPeelScan;
 }
 
-// The peel-off towards instrument s.q(), or the end of the event's peel-offs:
-// along a frame that looks along a grid axis the optical depth comes from
-// the column sums at once (the lane then waits for the deposit stage);
-// otherwise a record for the sorted pass, or (no pass, or its buffer full)
-// its walk.  After the last instrument: the first forced path (emission) or
-// the scattering (kAfter).
-template <class G>
-__device__ __forceinline__ void peel_scan(const FwdParams& P, Lane<G>& s, LaneTally* bt) {
-  const bool emission = s.event() == 0;
-  if ((emission ? P.peel_emission : P.peel_scatter) && s.q() < P.n_instr) {
-    const DevInstr& I = S_INSTR[s.q()];
-    const int phase = emission ? kPeelEmit : kPeelScat;
-    if constexpr (G::kColumns) {
-      if (P.use_columns && I.column && column_peel(P, s, I, bt)) {
-        s.phase = phase;
-        return;
-      }
-      if (P.peel && G::kSortedPass && defer_peel(P, s, I, emission)) {
-        // walked and deposited by the sorted pass; on to the next instrument
-        bt->peeloffs += 1u;
-        s.q() += 1;
-        return;
-      }
+// The peel-off of the event towards instrument q (the same for the whole warp,
+// so its table is read as uniform values): along a frame that looks along a
+// grid axis the optical depth comes from the column sums and is deposited at
+// once; otherwise a record for the sorted pass, or (no pass, or its buffer
+// full) its walk.
+template <class G, bool kTape>
+__device__ __forceinline__ void peel_off(const FwdParams& P, Task<G, kTape>& s, int q) {
+  const DevInstr& I = P.instr[q];
+  const bool emission = s.event == 0;
+  s.q = q + 1;
+  if constexpr (G::kColumns) {
+    if (P.use_columns && I.column && column_peel(P, s, I)) {
+      peel_deposit(P, s, q, !emission);
+      s.n_peel += 1u;
+      return;
     }
-    request_walk(s, phase, instr_dir(I));
-    return;
+    if (G::kSortedPass && P.peel && defer_peel(P, s, q, emission)) {
+      s.n_peel += 1u;  // walked and deposited by the sorted pass
+      return;
+    }
   }
-  if (emission) {
-    s.event() = 1;
-    request_path(s);
+  s.q = q;
+  request_walk(s, emission ? kPeelEmit : kPeelScat);
+}
+
+// After the last instrument: the first forced path (emission) or the
+// scattering (kAfter).
+template <class G, bool kTape>
+__device__ __forceinline__ void peels_done(const FwdParams& P, Task<G, kTape>& s) {
+  if (s.event == 0) {
+    s.event = 1;
+    request_path(P, s);
   } else {
     s.phase = kAfter;
   }
@@ -1561,76 +1632,196 @@ __device__ __forceinline__ void peel_scan(const FwdParams& P, Lane<G>& s, LaneTa
 // After the scattering peel-offs: new direction, then termination or the
 // next forced path.
 template <class G, bool kTape>
-__device__ __forceinline__ void after_scattering(const FwdParams& P, Lane<G>& s, LaneTally* bt) {
-  const float mu = hg_sample(S_LAM[s.lam].g, s.u_mu());
+__device__ __forceinline__ void after_scattering(const FwdParams& P, Task<G, kTape>& s) {
+  const float2 u = s.hg();
+  const float mu = hg_sample(P.lam[s.lam].g, u.x);
   float sp, cp;
-  sincospif(2.0f * s.u_phi(), &sp, &cp);
+  sincospif(2.0f * u.y, &sp, &cp);
   s.k() = rotate_dir(s.k(), mu, sp, cp);
-  if ((P.weight_cut && s.L() < P.L_cut[s.lam]) || s.event() >= P.max_events) {
-    bt->truncated += s.L();
-    if (kTape) tape_end(P, s, s.event());
+  const double L = s.L();
+  if ((P.weight_cut && bits_of(L) < bits_of(P.L_cut[s.lam])) || s.event >= P.max_events) {
+    s.tally.truncated += L;
+    if (kTape) tape_end(P, s, s.event);
     s.phase = kFetch;
     return;
   }
-  s.event() += 1;
-  request_path(s);
+  s.event += 1;
+  request_path(P, s);
 }
 
-// One control round for the warp: every stage runs for the lanes in its
-// phase together, and a stage hands lanes on to later stages (the peel-off
-// loop repeats deposit and scan while any lane has a peel-off ready, which
-// column sums complete without a walk; lanes whose packet ended fetch the
-// next one and go round once more).
+// The warp's queues: entries and heads of the four rings, one byte each (the
+// same values in every lane).
+struct Queues {
+  unsigned count, head;
+  unsigned char (*ring)[kRing];  // the warp's rings
+  __device__ __forceinline__ int size(int q) const { return (int)((count >> (8 * q)) & 255u); }
+  // The fullest of the queues of per-event work.
+  __device__ __forceinline__ int fullest() const {
+    const int a = size(kQPath1), b = size(kQEvent), c = size(kQFetch);
+    return a >= b && a >= c ? kQPath1 : (b >= c ? kQEvent : kQFetch);
+  }
+  // Whether a round should run for n_idle lanes without a walk.
+  __device__ __forceinline__ bool round_due(int n_idle) const {
+    const int n = size(fullest());
+    return n >= kRoundMin || (n > 0 && n_idle - size(kQReady) >= kIdleMax);
+  }
+  // Append `slot` of the lanes where pred holds.
+  __device__ __forceinline__ int push(int q, bool pred, int slot, unsigned lt_mask) {
+    const unsigned m = __ballot_sync(0xffffffffu, pred);
+    if (pred) ring[q][((head >> (8 * q)) + (count >> (8 * q)) + __popc(m & lt_mask)) & (kRing - 1)] = (unsigned char)slot;
+    const int n = __popc(m);
+    count += (unsigned)n << (8 * q);
+    return n;
+  }
+  // Entry r of queue q (r below its size).
+  __device__ __forceinline__ int at(int q, int r) const { return ring[q][((head >> (8 * q)) + r) & (kRing - 1)]; }
+  __device__ __forceinline__ void drop(int q, int n) {
+    const unsigned sh = 8 * q;
+    head = (head & ~(255u << sh)) | ((((head >> sh) + n) & (kRing - 1)) << sh);
+    count -= (unsigned)n << sh;
+  }
+};
+
+// One control round: up to 32 packets of queue `cls` (packet r of it in lane
+// r) go through the per-event work they wait for, until each needs a walk, a
+// new packet or nothing more; they are queued accordingly.  Returns the packets
+// served.
 template <class G, bool kTape>
-__device__ __forceinline__ void control_round(const FwdParams& P, Lane<G>& s, LaneTally* bt,
-                                              typename G::Scratch& sc, unsigned lane, unsigned lt_mask) {
-  if (!s.walking) {
-    if (s.phase == kPath1) finish_path1<G, kTape>(P, s, bt);
-    if (s.phase == kPath2) finish_path2<G, kTape>(P, s, bt);
-  }
-  // Peel-offs, the scattering and new packets, repeated while a lane has
-  // just finished its packet: such a lane starts its next packet in the same
-  // round (at most two passes: a new packet never ends before its first walk).
-  while (true) {
-    while (true) {
-      const bool ready = !s.walking && (s.phase == kPeelEmit || s.phase == kPeelScat);
-      if (!__any_sync(0xffffffffu, ready || s.phase == kPeelScan)) break;
-      if (ready) {
-        peel_deposit(P, s, s.phase == kPeelScat);
-        bt->peeloffs += 1u;
-        s.q() += 1;
-        s.phase = kPeelScan;
+__device__ __forceinline__ int control_round(const FwdParams& P, Queues& Q, LaneTally& tally, int cls, unsigned lane,
+                                              unsigned lt_mask) {
+  Shared<G, kTape>& sh = shared_state<G, kTape>();
+  const unsigned warp = threadIdx.x >> 5;
+  const int n = min(32, Q.size(cls));
+  const bool on = (int)lane < n;
+  const int local = on ? Q.at(cls, (int)lane) : 0;
+  Q.drop(cls, n);
+  Task<G, kTape> s{sh, tally};
+  s.i = (int)warp * G::kSlots + local;
+  const unsigned pk = sh.pack[s.i];
+  s.phase = on ? Pack::phase(pk) : kExit;
+  s.wphase = 0;
+  s.lam = Pack::lam(pk);
+  s.q = Pack::q(pk);
+  s.has_cell = Pack::has_cell(pk);
+  s.dep_exp = 0;
+  s.event = sh.event[s.i];
+  const float2 res = sh.res[s.i];
+  s.th = res.x;
+  s.tl = res.y;
+  s.n_peel = s.n_col = s.c_col = 0u;
+  int n_events = 0, n_packets = 0;
+  if (cls == kQPath1) {
+    if (on) finish_path1(P, s);
+  } else {
+    if (cls == kQFetch) {
+      // one atomic for the round
+      unsigned long long base = 0;
+      if (lane == 0) base = atomicAdd(P.work_counter, (unsigned long long)n);
+      base = __shfl_sync(0xffffffffu, base, 0);
+      if (on) fetch(P, s, base + lane);
+      n_packets = base >= P.n_total ? 0 : (int)min((unsigned long long)n, P.n_total - base);
+    } else {
+      const bool ended = on && s.phase == kPath2;
+      n_events = __popc(__ballot_sync(0xffffffffu, ended));
+      if (ended) finish_path2(P, s);
+    }
+    // a peel-off walk that ended, then the event's next peel-offs, instrument
+    // by instrument for the packets that have reached it
+    if (s.phase == kPeelEmit || s.phase == kPeelScat) {
+      peel_deposit(P, s, s.q, s.phase == kPeelScat);
+      s.n_peel += 1u;
+      s.q += 1;
+      s.phase = kPeelScan;
+    }
+    if (s.phase == kPeelScan && !(s.event == 0 ? P.peel_emission : P.peel_scatter)) s.q = P.n_instr;
+    for (int q = 0; q < P.n_instr; ++q) {
+      const bool here = s.phase == kPeelScan && s.q == q;
+      if (__any_sync(0xffffffffu, here)) {
+        if (here) peel_off(P, s, q);
       }
-      if (s.phase == kPeelScan) peel_scan(P, s, bt);
     }
-    if (s.phase == kAfter) after_scattering<G, kTape>(P, s, bt);
-    // packets for every lane that needs one: one atomic per warp
-    const bool wants = !s.walking && s.phase == kFetch;
-    const unsigned fetchers = __ballot_sync(0xffffffffu, wants);
-    if (!fetchers) break;
-    unsigned long long base = 0;
-    const int leader = __ffs(fetchers) - 1;
-    if ((int)lane == leader) base = atomicAdd(P.work_counter, (unsigned long long)__popc(fetchers));
-    base = __shfl_sync(0xffffffffu, base, leader);
-    if (wants) fetch<G, kTape>(P, s, base + __popc(fetchers & lt_mask), bt);
+    if (s.phase == kPeelScan) peels_done(P, s);
+    if (s.phase == kAfter) after_scattering(P, s);
   }
-  if (s.phase == kStart) {
-    s.phase = s.wphase();
-    if (kTape) {
-      s.g = make_float3(0.0f, 0.0f, 0.0f);
-      s.axis_in = -1;
-      s.n_cross = 0;
+  const bool start = on && s.phase == kStart, again = on && s.phase == kFetch;
+  if (start) {
+    sh.pack[s.i] = Pack::make(s.wphase, s.lam, s.q, s.has_cell, s.dep_exp);
+    sh.event[s.i] = s.event;
+  }
+  Q.push(kQReady, start, local, lt_mask);
+  Q.push(kQFetch, again, local, lt_mask);
+  if (cls != kQPath1) {
+    const unsigned np = __reduce_add_sync(0xffffffffu, s.n_peel);
+    const unsigned nc = __reduce_add_sync(0xffffffffu, s.n_col);
+    const unsigned cc = __reduce_add_sync(0xffffffffu, s.c_col);
+    if (lane == 0) {
+      WarpTally& t = sh.tally[warp];
+      t.events += (unsigned long long)n_events;
+      t.packets += (unsigned long long)n_packets;
+      t.peeloffs += np;
+      t.column_peels += nc;
+      t.column_crossings += cc;
+      t.crossings += cc;
     }
-    start_walk(P, s, s.d, sc);
+  }
+  __syncwarp();
+  return n;
+}
+
+// Start the ready packet in slot i on this lane; the first cell's density
+// load is issued here.
+template <class G, bool kTape>
+__device__ __forceinline__ void start_walk(const FwdParams& P, Walker<G>& s, int i, typename G::Scratch& sc) {
+  Shared<G, kTape>& sh = shared_state<G, kTape>();
+  const unsigned pk = sh.pack[i];
+  s.slot = i;
+  s.phase = Pack::phase(pk);
+  const int lam = Pack::lam(pk);
+  s.absorption = P.absorption + (size_t)lam * P.n_cells;
+  s.kappa = P.lam[lam].kappa;
+  s.x = sh.x[i];
+  s.d = s.phase == kPath1 || s.phase == kPath2 ? sh.k[i] : instr_dir(P.instr[Pack::q(pk)]);
+  s.id = make_float3(inv_or_zero(s.d.x), inv_or_zero(s.d.y), inv_or_zero(s.d.z));
+  const float2 a = sh.res[i];
+  s.aux0 = a.x;
+  s.aux1 = a.y;
+  s.th = 0.0f;
+  s.tl = 0.0f;
+  s.n = 0u;
+  if (kTape) {
+    s.g = make_float3(0.0f, 0.0f, 0.0f);
+    s.axis_in = -1;
+    s.h = -1;
+  }
+  s.walking = G::init(P, s.x, s.d, s.id, Pack::has_cell(pk), sh.cell[i], s.w, sc);
+  if (s.walking) s.rho = load_density(&P.density[G::cell(s.w)]);
+}
+
+// A lane's walk ended: its result goes to the packet's slot.
+template <class G, bool kTape>
+__device__ __forceinline__ void end_walk(const FwdParams& P, const Walker<G>& s) {
+  Shared<G, kTape>& sh = shared_state<G, kTape>();
+  const int i = s.slot;
+  if (s.phase == kPath2) {
+    sh.res[i] = make_float2(s.aux0, 0.0f);
+    sh.cell[i] = G::carried(s.w);
+    if (kTape) {
+      // the record's third sector, whole
+      float4* t = reinterpret_cast<float4*>(&tape_records(P, Pack::lam(sh.pack[i]), sh.pid[i])[sh.event[i]]);
+      t[4] = make_float4(__int_as_float(s.h), __int_as_float(s.axis_in), __int_as_float(G::id(P, s.w)), s.kr_h);
+      t[5] = make_float4(s.rem, s.g.x, s.g.y, s.g.z);
+    }
+  } else {
+    sh.res[i] = make_float2(s.th, s.tl);
+    if (kTape && s.phase == kPath1) sh.g[i] = s.g;
   }
 }
 
-// One cell crossing of the lane's current walk.  Written with selects rather
-// than branches where lanes in different walks (peel-off, forced path 1 or 2)
+// One cell crossing of the lane's walk.  Written with selects rather than
+// branches where lanes in different walks (peel-off, forced path 1 or 2)
 // share the step, so the warp issues it once.
 template <class G, bool kTape>
-__device__ __forceinline__ void walk_step(const FwdParams& P, Lane<G>& s, unsigned& n_path, unsigned& n_peel,
-                                          typename G::Scratch& sc) {
+__device__ __forceinline__ void walk_step(const FwdParams& P, Walker<G>& s, typename G::Scratch& sc) {
   typename G::Walk& w = s.w;
   int axis;
   const float te = G::exit(w, s.x, s.id, axis);
@@ -1653,7 +1844,7 @@ __device__ __forceinline__ void walk_step(const FwdParams& P, Lane<G>& s, unsign
     if (kTape) {
       s.kr_h = kr;
       s.rem = rem;
-      s.h = s.n_cross;
+      s.h = (int)s.n;
     }
     return;
   }
@@ -1663,11 +1854,10 @@ __device__ __forceinline__ void walk_step(const FwdParams& P, Lane<G>& s, unsign
     s.g.y += (axis == 1 ? kr : 0.0f) - (s.axis_in == 1 ? kr : 0.0f);
     s.g.z += (axis == 2 ? kr : 0.0f) - (s.axis_in == 2 ? kr : 0.0f);
     s.axis_in = axis;
-    ++s.n_cross;
   }
   if (path1 && dt > 0.0f) {
     // continuous absorption: (1 - albedo) L exp(-tau_before) (1 - exp(-dtau))
-    double* const a = &P.absorption[(size_t)s.lam * P.n_cells + G::cell(w)];
+    double* const a = &s.absorption[G::cell(w)];
     if (s.th < s.aux1) {
       add_absorption(a, widen(s.aux0 * __expf(-s.th) * one_minus_exp_neg(dt)));
     } else {
@@ -1675,13 +1865,13 @@ __device__ __forceinline__ void walk_step(const FwdParams& P, Lane<G>& s, unsign
       // part joins the weight's exponent, so deep deposits do not underflow
       const float y = s.th * 1.44269504f;
       const float k = floorf(y);
-      add_absorption(a, widen_exp(s.aux0 * exp2f(k - y) * one_minus_exp_neg(dt), S_DEPEXP[threadIdx.x] - (int)k));
+      add_absorption(a, widen_exp(s.aux0 * exp2f(k - y) * one_minus_exp_neg(dt),
+                                  Pack::exponent(shared_state<G, kTape>().pack[s.slot]) - (int)k));
     }
   }
   s.th = nh;
   s.tl = nl;
-  n_path += path1 ? 1u : 0u;
-  n_peel += (path1 || path2) ? 0u : 1u;
+  s.n += 1u;
   w.t = texit;
   if (G::advance(P, s.x, s.d, s.id, axis, w, sc)) {
     s.rho = load_density(&P.density[G::cell(w)]);  // consumed by the next crossing
@@ -1697,28 +1887,16 @@ __device__ __forceinline__ void walk_step(const FwdParams& P, Lane<G>& s, unsign
 }
 
 template <class G>
-__device__ __forceinline__ typename G::Scratch lane_scratch(const FwdParams& P);
+__device__ __forceinline__ typename G::Scratch lane_scratch(size_t) {
+  return typename G::Scratch{};
+}
 template <>
-__device__ __forceinline__ CartGrid::Scratch lane_scratch<CartGrid>(const FwdParams&) { return CartGrid::Scratch{}; }
-template <>
-__device__ __forceinline__ RectGrid::Scratch lane_scratch<RectGrid>(const FwdParams&) { return RectGrid::Scratch{}; }
-template <>
-__device__ __forceinline__ BinGrid::Scratch lane_scratch<BinGrid>(const FwdParams&) { return BinGrid::Scratch{}; }
-template <>
-__device__ __forceinline__ VorGrid::Scratch lane_scratch<VorGrid>(const FwdParams&) { return VorGrid::Scratch{}; }
-template <>
-__device__ __forceinline__ OctGrid::Scratch lane_scratch<OctGrid>(const FwdParams& P) {
-  return OctGrid::Scratch{&S_OCT_STACK[threadIdx.x * P.oct_levels]};
+__device__ __forceinline__ OctGrid::Scratch lane_scratch<OctGrid>(size_t offset) {
+  return OctGrid::Scratch{reinterpret_cast<int*>(S_RAW + offset) + threadIdx.x};
 }
 
 template <class G>
-__device__ __forceinline__ void load_grid_cache(const FwdParams& P);
-template <>
-__device__ __forceinline__ void load_grid_cache<CartGrid>(const FwdParams&) {}
-template <>
-__device__ __forceinline__ void load_grid_cache<RectGrid>(const FwdParams&) {}
-template <>
-__device__ __forceinline__ void load_grid_cache<VorGrid>(const FwdParams&) {}
+__device__ __forceinline__ void load_grid_cache(const FwdParams&) {}
 template <>
 __device__ __forceinline__ void load_grid_cache<BinGrid>(const FwdParams& P) {
   const int n = P.n_nodes < kChildCache ? (int)P.n_nodes : kChildCache;
@@ -1735,94 +1913,169 @@ __device__ __forceinline__ void load_grid_cache<OctGrid>(const FwdParams& P) {
 // plain kernel ~4 % of its time).
 template <class G, bool kTape = false, bool kProf = false>
 __device__ __forceinline__ void forward_body(const FwdParams& P) {
-  __shared__ LaneTally tally[kBlock];
-  for (int i = threadIdx.x; i < P.n_instr; i += kBlock) S_INSTR[i] = P.instr[i];
-  for (int i = threadIdx.x; i < P.n_lambda; i += kBlock) S_LAM[i] = P.lam[i];
+  static_assert(G::kSlots <= kRing, "a queue holds every slot of its warp");
+  Shared<G, kTape>& sh = shared_state<G, kTape>();
   load_grid_cache<G>(P);
-  __syncthreads();
-  typename G::Scratch sc = lane_scratch<G>(P);
-  LaneTally* bt = &tally[threadIdx.x];
-  bt->escaped = bt->absorbed = bt->truncated = 0.0;
-  bt->crossings = bt->path_crossings = bt->column_crossings = 0ull;
-  bt->events = bt->peeloffs = bt->packets = bt->column_peels = 0u;
-  const unsigned lane = threadIdx.x & 31u;
+  typename G::Scratch sc = lane_scratch<G>(sizeof(Shared<G, kTape>));
+  const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
   const unsigned lt_mask = (1u << lane) - 1u;
-  Lane<G> s;
-  s.phase = kFetch;
-  s.walking = false;
-  unsigned n_path = 0, n_peel = 0;
+  LaneTally tally{0.0, 0.0, 0.0};
+  asm volatile("" ::"l"(&tally) : "memory");  // kept in memory, not in registers
+  if (lane == 0) {
+    WarpTally& t = sh.tally[warp];
+    t.crossings = t.path_crossings = t.column_crossings = 0ull;
+    t.events = t.peeloffs = t.packets = t.column_peels = 0ull;
+  }
+  // the warp's slots, all free; a launch with fewer packets than the grid has
+  // slots spreads them over the warps
+  const unsigned n_warps = gridDim.x * (unsigned)kWarps;
+  const unsigned long long share = (P.n_total + n_warps - 1) / n_warps;
+  const int n_slots = share < (unsigned long long)G::kSlots ? (int)share : G::kSlots;
+  // when all of them are resident at once nothing refills the lanes, few warps
+  // share an SM and a round's latency counts: the warp then waits for all its
+  // walks (1e4 packets of a 32^3 cube 611 -> 416 us, 2e5 1548 -> 1313 us; from
+  // 80 packets per warp on it loses: 4e5 packets of the spiral example 5.3
+  // against 7.7 ms)
+  const bool lockstep = n_slots < G::kSlots;
+  if (lane == 0) sh.queues[warp] = make_uint2((unsigned)n_slots << (8 * kQFetch), 0u);
+  for (int i = (int)lane; i < n_slots; i += 32) sh.ring[warp][kQFetch][i] = (unsigned char)i;
+  for (int i = (int)lane; i < G::kSlots; i += 32) sh.pack[(int)warp * G::kSlots + i] = 0u;
+  __syncthreads();
+  Walker<G> s{};
+  s.slot = -1;
+  s.phase = kExit;
+  int wait = 0;  // ended walks the warp waits for before it serves them
   // optional execution counters (warp leader only)
   const bool prof = kProf && P.profile != nullptr && lane == 0;
   // iterations, walking lanes, rounds, lanes served, cycles in control, in
   // the walk: per warp in shared memory (no registers held across the loop)
-  __shared__ unsigned long long prof_c[kBlock / 32][6];
-  unsigned long long* pc = prof_c[threadIdx.x >> 5];
+  __shared__ unsigned long long prof_c[kProf ? kWarps : 1][6];
+  unsigned long long* pc = prof_c[kProf ? warp : 0];
   if (prof)
     for (int i = 0; i < 6; ++i) pc[i] = 0ull;
   while (true) {
-    const bool idle = !s.walking && s.phase != kExit;
-    const unsigned need = __ballot_sync(0xffffffffu, idle);
-    const unsigned walkers = __ballot_sync(0xffffffffu, s.walking);
-    if (need == 0u && walkers == 0u) break;
-    long long t0 = 0;
-    if (prof) { pc[0] += 1ull; t0 = clock64(); }
-    if (walkers == 0u || __popc(need) >= P.control_min) {
-      if (prof) { pc[2] += 1ull; pc[3] += __popc(need); }
-      control_round<G, kTape>(P, s, bt, sc, lane, lt_mask);
-      if ((n_path | n_peel) & 0xC0000000u) {  // keep the 32-bit lane counters far from overflow
-        bt->crossings += (unsigned long long)n_path + n_peel;
-        bt->path_crossings += n_path;
-        n_path = n_peel = 0;
+    const bool ended = !s.walking && s.slot >= 0;
+    if (__popc(__ballot_sync(0xffffffffu, ended)) >= wait) {
+      long long t0 = 0;
+      if (prof) t0 = clock64();
+      const uint2 qs = sh.queues[warp];
+      Queues Q{qs.x, qs.y, sh.ring[warp]};
+      // the ended walks' packets to their queues
+      {
+        const bool p1 = ended && s.phase == kPath1;
+        const unsigned np = __reduce_add_sync(0xffffffffu, p1 ? s.n : 0u);
+        const unsigned nq = __reduce_add_sync(0xffffffffu, ended && !p1 && s.phase != kPath2 ? s.n : 0u);
+        if (ended) end_walk<G, kTape>(P, s);
+        if (lane == 0) {
+          sh.tally[warp].path_crossings += np;
+          sh.tally[warp].crossings += (unsigned long long)np + nq;
+        }
+        const int local = s.slot - (int)warp * G::kSlots;
+        Q.push(kQPath1, p1, local, lt_mask);
+        Q.push(kQEvent, ended && !p1, local, lt_mask);
+        if (ended) s.slot = -1;
+        __syncwarp();
       }
+      const unsigned idle = __ballot_sync(0xffffffffu, !s.walking);
+      const int n_idle = __popc(idle);
+      // rounds, the fullest queue first, until every idle lane has a packet; a
+      // queue of few packets waits for more while few lanes are idle
+      if (Q.size(kQReady) < n_idle && Q.round_due(n_idle)) {
+        // the walks go to local memory for the rounds: left to itself the
+        // compiler keeps part of them there for the whole loop, at 14 local
+        // loads per crossing (27.2 against 18.8 ms per 2e6 packets, disk galaxy)
+        Walker<G> saved = s;
+        asm volatile("" ::"l"(&saved) : "memory");
+        do {
+          const int served = control_round<G, kTape>(P, Q, tally, Q.fullest(), lane, lt_mask);
+          if (prof) { pc[2] += 1ull; pc[3] += (unsigned long long)served; }
+        } while (Q.size(kQReady) < n_idle && Q.round_due(n_idle));
+        asm volatile("" ::"l"(&saved) : "memory");
+        s = saved;
+      }
+      // idle lanes take the ready packets
+      const int n_start = min(n_idle, Q.size(kQReady));
+      const int r = __popc(idle & lt_mask);
+      if (!s.walking && r < n_start)
+        start_walk<G, kTape>(P, s, (int)warp * G::kSlots + Q.at(kQReady, r), sc);
+      Q.drop(kQReady, n_start);
+      __syncwarp();
+      if (lane == 0) sh.queues[warp] = make_uint2(Q.count, Q.head);
+      __syncwarp();
+      const int busy = 32 - n_idle + n_start;  // lanes with a packet
+      if (busy == 0) break;                    // no packets left
+      wait = lockstep ? busy : max(1, (P.control_min * busy) >> 5);
+      if (prof) pc[4] += clock64() - t0;
     }
     long long t1 = 0;
-    if (prof) { t1 = clock64(); pc[4] += t1 - t0; }
+    if (prof) { t1 = clock64(); pc[0] += 1ull; }
     const unsigned stepping = kProf ? __ballot_sync(0xffffffffu, s.walking) : 0u;
-    if (s.walking) walk_step<G, kTape>(P, s, n_path, n_peel, sc);
+    if (s.walking) walk_step<G, kTape>(P, s, sc);
     if (prof) { pc[1] += __popc(stepping); pc[5] += clock64() - t1; }
   }
   if (prof) {
     for (int i = 0; i < 6; ++i) atomicAdd(&P.profile[i], pc[i]);
   }
-  bt->crossings += (unsigned long long)n_path + n_peel;
-  bt->path_crossings += n_path;
+  // the block's sums: lanes of a warp, then the warps
+  double esc = tally.escaped, ab = tally.absorbed, trc = tally.truncated;
+  for (int o = 16; o > 0; o >>= 1) {
+    esc += __shfl_down_sync(0xffffffffu, esc, o);
+    ab += __shfl_down_sync(0xffffffffu, ab, o);
+    trc += __shfl_down_sync(0xffffffffu, trc, o);
+  }
+  if (lane == 0) sh.lum[warp] = LaneTally{esc, ab, trc};
   __syncthreads();
-  if (threadIdx.x < 32) {
-    double esc = 0.0, ab = 0.0, trc = 0.0;
-    unsigned long long cr = 0, pc = 0, ev = 0, pe = 0, pk = 0, cc = 0, cp = 0;
-    for (int t = threadIdx.x; t < kBlock; t += 32) {
-      esc += tally[t].escaped; ab += tally[t].absorbed; trc += tally[t].truncated;
-      cr += tally[t].crossings; pc += tally[t].path_crossings;
-      ev += tally[t].events; pe += tally[t].peeloffs; pk += tally[t].packets;
-      cc += tally[t].column_crossings; cp += tally[t].column_peels;
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-      esc += __shfl_down_sync(0xffffffffu, esc, o);
-      ab += __shfl_down_sync(0xffffffffu, ab, o);
-      trc += __shfl_down_sync(0xffffffffu, trc, o);
-      cr += __shfl_down_sync(0xffffffffu, cr, o);
-      pc += __shfl_down_sync(0xffffffffu, pc, o);
-      ev += __shfl_down_sync(0xffffffffu, ev, o);
-      pe += __shfl_down_sync(0xffffffffu, pe, o);
-      pk += __shfl_down_sync(0xffffffffu, pk, o);
-      cc += __shfl_down_sync(0xffffffffu, cc, o);
-      cp += __shfl_down_sync(0xffffffffu, cp, o);
-    }
+  {
     if (threadIdx.x == 0) {
-      atomicAdd(&P.stats[1], esc);
-      atomicAdd(&P.stats[2], ab);
-      atomicAdd(&P.stats[3], trc);
-      atomicAdd(&P.counters[0], cr);
-      atomicAdd(&P.counters[1], ev);
-      atomicAdd(&P.counters[2], pe);
-      atomicAdd(&P.counters[3], pk);
-      atomicAdd(&P.counters[5], pc);
-      if (cp) {
-        atomicAdd(&P.counters[6], cp);
-        atomicAdd(&P.counters[7], cc);
+      WarpTally a = sh.tally[0];
+      for (int w = 1; w < kWarps; ++w) {
+        const WarpTally& b = sh.tally[w];
+        a.crossings += b.crossings; a.path_crossings += b.path_crossings; a.column_crossings += b.column_crossings;
+        a.events += b.events; a.peeloffs += b.peeloffs; a.packets += b.packets; a.column_peels += b.column_peels;
+        esc += sh.lum[w].escaped; ab += sh.lum[w].absorbed; trc += sh.lum[w].truncated;
+      }
+      if (a.packets) {  // a block that found no packets has nothing to add
+        atomicAdd(&P.stats[1], esc);
+        atomicAdd(&P.stats[2], ab);
+        atomicAdd(&P.stats[3], trc);
+        atomicAdd(&P.counters[0], a.crossings);
+        atomicAdd(&P.counters[1], a.events);
+        atomicAdd(&P.counters[2], a.peeloffs);
+        atomicAdd(&P.counters[3], a.packets);
+        atomicAdd(&P.counters[5], a.path_crossings);
+        if (a.column_peels) {
+          atomicAdd(&P.counters[6], a.column_peels);
+          atomicAdd(&P.counters[7], a.column_crossings);
+        }
       }
     }
   }
+}
+
+// Launch a forward kernel: a persistent grid of as many resident blocks per
+// SM as fit (at most p.blocks_per_sm when set), fewer when the packets do not
+// give every warp one.  `extra`: dynamic shared memory beyond the packet state.
+template <class G, bool kTape>
+cudaError_t launch_body(void (*kernel)(const FwdParams), const FwdParams& p, int num_sms, size_t extra,
+                        cudaStream_t stream) {
+  cudaError_t e = cudaMemsetAsync(p.work_counter, 0, sizeof(unsigned long long), stream);
+  if (e != cudaSuccess) return e;
+  const size_t bytes = sizeof(Shared<G, kTape>) + extra;
+  // static and dynamic shared memory together pass 48 KB: the launch needs
+  // the dynamic part allowed explicitly
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e != cudaSuccess) return e;
+  int per_sm = 0;
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kBlock, bytes);
+  if (e != cudaSuccess) return e;
+  per_sm = per_sm < 1 ? 1 : per_sm;
+  if (p.blocks_per_sm > 0 && p.blocks_per_sm < per_sm) per_sm = p.blocks_per_sm;
+  unsigned long long blocks = (unsigned long long)num_sms * per_sm;
+  const unsigned long long useful = (p.n_total + kWarps * kSpread - 1) / (kWarps * kSpread);
+  if (blocks > useful) blocks = useful;
+  if (blocks < 1) blocks = 1;
+  kernel<<<(unsigned)blocks, kBlock, bytes, stream>>>(p);
+  return cudaGetLastError();
 }
 
 }  // namespace tr
