@@ -283,10 +283,10 @@ __device__ __forceinline__ void finish_path1(const AdjParams& A, ALane& s) {
     return;
   }
   const double albedo = A.f.lam[s.lam].albedo;
-  const double omE = -expm1(-tau);
+  const double omE = one_minus_exp(tau);
   const uint4 rn = draw_block(s.pid, s.lam, s.event, 0, P.seed, P.model);
   const double u = u01(rn.x);
-  const double tau_star = -log1p(-u * omE);
+  const double tau_star = neg_log_one_minus(u * omE);
   s.u_mu = tr::u01f(rn.y);
   s.u_phi = tr::u01f(rn.z);
   AdjRecord& r = s.rec[s.event];

@@ -218,12 +218,12 @@ __device__ __forceinline__ void finish_path1(const BatchParams& P, BLane& s, Tal
     return;
   }
   const double albedo = M.albedo;
-  const double one_minus_E = -expm1(-tau);
+  const double one_minus_E = one_minus_exp(tau);
   const double E = 1.0 - one_minus_E;
   T.escaped += s.L() * E;
   T.absorbed += (1.0 - albedo) * s.L() * one_minus_E;
   const uint4 r = draw_block(s.pid(), 0, s.event(), 0, P.seed, (unsigned)s.m);
-  const double tau_star = -log1p(-u01(r.x) * one_minus_E);
+  const double tau_star = neg_log_one_minus(u01(r.x) * one_minus_E);
   s.u_mu() = tr::u01f(r.y);
   s.u_phi() = tr::u01f(r.z);
   tr::split_pair(tau_star, s.aux0, s.aux1);

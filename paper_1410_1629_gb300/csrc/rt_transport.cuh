@@ -1553,13 +1553,13 @@ __device__ __forceinline__ void finish_path1(const FwdParams& P, Task<G, kTape>&
     s.phase = kFetch;
     return;
   }
-  const double one_minus_E = -expm1(-tau);
+  const double one_minus_E = one_minus_exp(tau);
   const double E = 1.0 - one_minus_E;
   const double L = s.L();
   s.tally.escaped += L * E;
   s.tally.absorbed += P.lam[s.lam].one_minus_albedo * L * one_minus_E;
   const uint4 r = draw_block(s.pid(), s.lam, s.event, 0, P.seed, P.model);
-  const double tau_star = -log1p(-u01(r.x) * one_minus_E);
+  const double tau_star = neg_log_one_minus(u01(r.x) * one_minus_E);
   s.hg() = make_float2(u01f(r.y), u01f(r.z));
   if (kTape) {
     // the record's first two sectors, whole, with 16-byte stores
