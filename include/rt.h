@@ -225,16 +225,19 @@ typedef struct {
                            of the same packets (same n_per_lambda, first_packet_id, seed and
                            options, density unchanged, no absorption adjoint) needs no
                            replay of the forced paths                                       */
-  int32_t inline_peels; /* 0 (default): on cartesian grids, the peel-offs that walk (frames not
-                           along a grid axis, or all with walk_peels) run in a second pass after
+  int32_t inline_peels; /* 0 (default): the peel-offs that walk (frames not along an axis of a
+                           cartesian or rectilinear grid, all frames on other grids, or all with
+                           walk_peels) run in a second pass after
                            the transport kernel, ordered by instrument and start cell so that
                            the walks of a warp share cache lines (skipped with the tape, and
                            while its buffer, sized from the last launch's count within 40 % of
-                           free device memory, cannot be had); 1: each walks inside the
+                           free device memory, cannot be had; except on cartesian grids a launch
+                           of more than 2^28 records goes part by part); 1: each walks inside the
                            transport kernel.  The two give the same optical depths, crossings
                            and deposits; only the order of the FP64 image additions differs.   */
   int32_t time_parts;   /* 1: record CUDA events around the parts of this launch on its stream,
-                           read back by rt_read_launch_times                               */
+                           read back by rt_read_launch_times (a launch that goes part by part:
+                           all but the last part's sorted pass counts as transport)         */
   int32_t emitter;      /* RT_EMITTER_SOURCES (0): the sources emit; RT_EMITTER_DUST (1): the dust
                            cells emit their thermal luminosity (rt_set_dust_emission), a cell
                            drawn in proportion to its luminosity at the packet's wavelength, a

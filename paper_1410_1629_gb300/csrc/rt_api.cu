@@ -99,6 +99,9 @@ struct rt_ctx_s {
   int vb_n[3] = {1, 1, 1};
   bool oct_exact = false;  // octree boxes exact binary fractions (FwdParams::oct_exact)
   int oct_depth = 0;       // octrees: the deepest leaf's depth
+  // trees and Voronoi grids: the sorted pass's order of the cells (FwdParams)
+  int* d_cell_rank = nullptr;
+  float4* d_rank_cell = nullptr;
   // k-d trees: leaf ropes [n_cells][6] and node boxes [n_nodes][2] (FwdParams)
   int32_t* d_rope = nullptr;
   float4* d_node_box = nullptr;
@@ -278,6 +281,8 @@ void free_grid(rt_ctx c) {
     pool_release(c, c->d_rope, (size_t)c->n_cells * 6 * sizeof(int32_t));
     pool_release(c, c->d_node_box, (size_t)c->n_nodes * 2 * sizeof(float4));
   }
+  pool_release(c, c->d_cell_rank, (size_t)c->n_cells * sizeof(int));
+  pool_release(c, c->d_rank_cell, (size_t)c->n_cells * sizeof(float4));
   pool_release(c, c->d_edges, (size_t)(c->nx + c->ny + c->nz + 3) * sizeof(float));
   if (c->grid_kind == RT_GRID_VORONOI) {
     pool_release(c, c->d_site, (size_t)c->n_cells * sizeof(float4));
@@ -797,6 +802,42 @@ rt_status rt_create_grid(rt_ctx c, const rt_grid_desc* d, int32_t* grid_id) {
           vor_seed[(size_t)i + (size_t)vb_n[0] * ((size_t)j + (size_t)vb_n[1] * k)] = (int)cur;
         }
   }
+  // trees and Voronoi grids: the sorted pass's order of the cells
+  const bool unordered = !indexed_cells(d->kind);
+  std::vector<int> cell_rank(unordered ? (size_t)n_cells : 0, -1);
+  std::vector<float4> rank_cell;
+  rank_cell.reserve(cell_rank.size());
+  bool one_place = true;  // no cell met twice (a tree's nodes each have one parent)
+  auto next_cell = [&](long long cell, float x, float y, float z) {
+    if (cell_rank[(size_t)cell] >= 0) {
+      one_place = false;
+      return;
+    }
+    cell_rank[(size_t)cell] = (int)rank_cell.size();
+    float id;
+    const int cell_i = (int)cell;
+    std::memcpy(&id, &cell_i, sizeof id);
+    rank_cell.push_back(make_float4(x, y, z, id));
+  };
+  if (d->kind == RT_GRID_VORONOI) {
+    // Morton order of the sites, 10 bits per axis
+    std::vector<std::pair<unsigned, int>> order((size_t)n_cells);
+    for (long long i = 0; i < n_cells; ++i) {
+      const float p[3] = {vor_site[(size_t)i].x, vor_site[(size_t)i].y, vor_site[(size_t)i].z};
+      unsigned key = 0;
+      for (int a = 0; a < 3; ++a) {
+        const double u = (p[a] - d->bounds[2 * a]) / (d->bounds[2 * a + 1] - d->bounds[2 * a]);
+        const unsigned v = (unsigned)std::min(1023.0, std::max(0.0, 1024.0 * u));
+        for (int bit = 0; bit < 10; ++bit) key |= ((v >> bit) & 1u) << (3 * bit + a);
+      }
+      order[(size_t)i] = {key, (int)i};
+    }
+    std::sort(order.begin(), order.end());
+    for (const auto& o : order) {
+      const float4 p = vor_site[(size_t)o.second];
+      next_cell(o.second, p.x, p.y, p.z);
+    }
+  }
   std::vector<int32_t> child_host;
   std::vector<int32_t> rope_host;     // k-d trees: leaf ropes
   std::vector<float4> node_box_host;  // k-d trees: node boxes
@@ -874,6 +915,8 @@ rt_status rt_create_grid(rt_ctx c, const rt_grid_desc* d, int32_t* grid_id) {
         const int32_t v = child_host[(size_t)it.node];
         if (v < 0) {
           for (int f = 0; f < 6; ++f) rope_host[(size_t)(-(long long)v - 1) * 6 + f] = it.r[f];
+          next_cell(-(long long)v - 1, 0.5f * (it.lo[0] + it.hi[0]), 0.5f * (it.lo[1] + it.hi[1]),
+                    0.5f * (it.lo[2] + it.hi[2]));
           continue;
         }
         const int a = v & 3;
@@ -889,7 +932,40 @@ rt_status rt_create_grid(rt_ctx c, const rt_grid_desc* d, int32_t* grid_id) {
         stack.push_back(lower);
         stack.push_back(upper);
       }
+    } else {
+      // depth-first, boxes with the device's FP32 halving
+      struct Item {
+        int32_t node;
+        float lo[3], hi[3];
+      };
+      std::vector<Item> stack(1);
+      stack[0].node = 0;
+      for (int a = 0; a < 3; ++a) {
+        stack[0].lo[a] = (float)d->bounds[2 * a];
+        stack[0].hi[a] = (float)d->bounds[2 * a + 1];
+      }
+      while (!stack.empty() && one_place) {
+        const Item it = stack.back();
+        stack.pop_back();
+        const int32_t v = child_host[(size_t)it.node];
+        const float mid[3] = {0.5f * (it.lo[0] + it.hi[0]), 0.5f * (it.lo[1] + it.hi[1]), 0.5f * (it.lo[2] + it.hi[2])};
+        if (v < 0) {
+          next_cell(-(long long)v - 1, mid[0], mid[1], mid[2]);
+          continue;
+        }
+        for (int o = 7; o >= 0; --o) {
+          Item k = it;
+          k.node = v + o;
+          for (int a = 0; a < 3; ++a) {
+            if ((o >> a) & 1) k.lo[a] = mid[a]; else k.hi[a] = mid[a];
+          }
+          stack.push_back(k);
+        }
+      }
     }
+    // (leaves of nodes that no parent names come last: no walk starts there)
+    for (long long leaf = 0; one_place && leaf < n_cells; ++leaf)
+      if (cell_rank[(size_t)leaf] < 0) next_cell(leaf, (float)d->bounds[0], (float)d->bounds[2], (float)d->bounds[4]);
   }
   if (set_device(c) != RT_OK) return RT_ERR_CUDA;
   free_problem(c);
@@ -904,6 +980,12 @@ rt_status rt_create_grid(rt_ctx c, const rt_grid_desc* d, int32_t* grid_id) {
   if (d->kind == RT_GRID_OCTREE || d->kind == RT_GRID_BINTREE) {
     RT_CUDA(c, pool_alloc(c, &c->d_child, (size_t)n_nodes * sizeof(int32_t)));
     RT_CUDA(c, cudaMemcpy(c->d_child, child_host.data(), (size_t)n_nodes * sizeof(int32_t), cudaMemcpyHostToDevice));
+  }
+  if (unordered && one_place) {
+    RT_CUDA(c, pool_alloc(c, &c->d_cell_rank, cell_rank.size() * sizeof(int)));
+    RT_CUDA(c, cudaMemcpy(c->d_cell_rank, cell_rank.data(), cell_rank.size() * sizeof(int), cudaMemcpyHostToDevice));
+    RT_CUDA(c, pool_alloc(c, &c->d_rank_cell, rank_cell.size() * sizeof(float4)));
+    RT_CUDA(c, cudaMemcpy(c->d_rank_cell, rank_cell.data(), rank_cell.size() * sizeof(float4), cudaMemcpyHostToDevice));
   }
   if (d->kind == RT_GRID_BINTREE) {
     RT_CUDA(c, pool_alloc(c, &c->d_rope, rope_host.size() * sizeof(int32_t)));
@@ -1082,8 +1164,12 @@ namespace {
 // Buffers of the sorted peel-off pass for a launch of n_total packets with
 // `walked` instruments whose peel-offs walk; on success p.peel is set (left
 // null when the pass does not fit: the kernel then walks every peel-off).
+// part: packets whose records the buffer holds by that estimate; on trees,
+// Voronoi and rectilinear grids a launch of more goes part by part, with at
+// most kPeelPart records (10 GB) each.
+constexpr unsigned long long kPeelPart = 1ull << 28;
 rt_status prepare_peel_pass(rt_ctx c, FwdParams& p, unsigned long long n_total, int walked, bool tags,
-                            cudaStream_t s) {
+                            unsigned long long* part) {
   const unsigned long long keys = (unsigned long long)c->instr.size() * (unsigned long long)(c->n_cells + 1);
   if (keys >= 0xffffffffull) return RT_OK;
   if (!c->peel_event) {
@@ -1106,7 +1192,8 @@ rt_status prepare_peel_pass(rt_ctx c, FwdParams& p, unsigned long long n_total, 
   // records per packet: what the last launch asked for plus a quarter, else
   // eight per walked instrument (a packet peels off once per event)
   const double per = c->peel_per_packet > 0.0 ? 1.25 * c->peel_per_packet + 0.05 : 8.0 * walked;
-  unsigned long long want = (unsigned long long)std::min(per * (double)n_total, 4.0e9);
+  const bool parts = c->grid_kind != RT_GRID_CARTESIAN;
+  unsigned long long want = (unsigned long long)std::min(per * (double)n_total, parts ? (double)kPeelPart : 4.0e9);
   want = std::max(want, 4096ull);
   if (want > c->peel_cap) {
     dfree(c->d_peel);
@@ -1145,8 +1232,7 @@ rt_status prepare_peel_pass(rt_ctx c, FwdParams& p, unsigned long long n_total, 
     RT_CUDA(c, cudaMalloc(&c->d_peel_tiles, ((keys + 4095) / 4096) * sizeof(unsigned)));
     c->peel_keys = keys;
   }
-  RT_CUDA(c, cudaMemsetAsync(c->d_peel_hist, 0, keys * sizeof(unsigned), s));
-  RT_CUDA(c, cudaMemsetAsync(c->d_peel_count, 0, sizeof(unsigned long long), s));
+  if (parts) *part = std::max(1ull, std::min(n_total, (unsigned long long)((double)c->peel_cap / per)));
   p.peel = c->d_peel;
   p.peel_cap = c->peel_cap;
   p.peel_count = c->d_peel_count;
@@ -1219,6 +1305,8 @@ rt_status rt_launch_packets(rt_ctx c, uint64_t n_per_lambda, uint64_t first_pack
   p.oct_levels = c->oct_depth + 1;
   p.rope = c->d_rope;
   p.node_box = c->d_node_box;
+  p.cell_rank = c->d_cell_rank;
+  p.rank_cell = c->d_rank_cell;
   if (c->grid_kind == RT_GRID_VORONOI) {
     p.site = c->d_site;
     p.face_off = c->d_face_off;
@@ -1318,27 +1406,37 @@ rt_status rt_launch_packets(rt_ctx c, uint64_t n_per_lambda, uint64_t first_pack
   }
   if (ev) RT_CUDA(c, cudaEventRecord(ev[1], s));
   const int walked = o.walk_peels ? (int)c->instr.size() : c->n_walked_frames;
-  if (c->grid_kind == RT_GRID_CARTESIAN && !o.tape && !o.inline_peels && walked > 0 &&
-      (o.peel_emission || o.peel_scatter)) {
-    st = prepare_peel_pass(c, p, n_total, walked, o.records != nullptr, s);
+  unsigned long long part = n_total;  // packets per transport kernel
+  const bool ordered = indexed_cells(c->grid_kind) || c->d_rank_cell;
+  if (ordered && !o.tape && !o.inline_peels && walked > 0 && (o.peel_emission || o.peel_scatter)) {
+    st = prepare_peel_pass(c, p, n_total, walked, o.records != nullptr, &part);
     if (st != RT_OK) return st;
   }
-  cudaError_t e = launch_forward(p, c->grid_kind, c->num_sms, s);
-  if (e != cudaSuccess) return cuda_fail(c, e, "forward launch");
-  if (ev) RT_CUDA(c, cudaEventRecord(ev[2], s));
-  if (p.peel) {
-    e = launch_peel_pass(p, (unsigned long long)c->instr.size() * (unsigned long long)(c->n_cells + 1),
-                         c->d_peel_tiles, c->d_peel_perm, c->num_sms, s, ev ? ev[3] : nullptr);
-    if (e != cudaSuccess) return cuda_fail(c, e, "peel-off pass");
-    if (!c->peel_pending) {
-      RT_CUDA(c, cudaMemcpyAsync(c->h_peel_count, c->d_peel_count, sizeof(unsigned long long),
-                                 cudaMemcpyDeviceToHost, s));
-      RT_CUDA(c, cudaEventRecord(c->peel_event, s));
-      c->peel_pending = true;
-      c->peel_last_packets = n_total;
+  const unsigned long long keys = (unsigned long long)c->instr.size() * (unsigned long long)(c->n_cells + 1);
+  cudaError_t e = cudaSuccess;
+  for (unsigned long long first = 0; first < n_total; first += part) {
+    p.w_first = first;
+    p.n_total = std::min(n_total, first + part);
+    if (p.peel) {
+      RT_CUDA(c, cudaMemsetAsync(c->d_peel_hist, 0, keys * sizeof(unsigned), s));
+      RT_CUDA(c, cudaMemsetAsync(c->d_peel_count, 0, sizeof(unsigned long long), s));
     }
-  } else if (ev) {
-    RT_CUDA(c, cudaEventRecord(ev[3], s));
+    e = launch_forward(p, c->grid_kind, c->num_sms, s);
+    if (e != cudaSuccess) return cuda_fail(c, e, "forward launch");
+    if (ev) RT_CUDA(c, cudaEventRecord(ev[2], s));
+    if (p.peel) {
+      e = launch_peel_pass(p, c->grid_kind, keys, c->d_peel_tiles, c->d_peel_perm, c->num_sms, s, ev ? ev[3] : nullptr);
+      if (e != cudaSuccess) return cuda_fail(c, e, "peel-off pass");
+      if (!c->peel_pending) {
+        RT_CUDA(c, cudaMemcpyAsync(c->h_peel_count, c->d_peel_count, sizeof(unsigned long long),
+                                   cudaMemcpyDeviceToHost, s));
+        RT_CUDA(c, cudaEventRecord(c->peel_event, s));
+        c->peel_pending = true;
+        c->peel_last_packets = p.n_total - p.w_first;
+      }
+    } else if (ev) {
+      RT_CUDA(c, cudaEventRecord(ev[3], s));
+    }
   }
   if (ev) {
     RT_CUDA(c, cudaEventRecord(ev[4], s));

@@ -56,8 +56,8 @@ struct AdjRecord;
 
 // A peel-off whose walk runs in the sorted pass after the transport kernel
 // (one 32-byte sector): the position it starts from; its sort key, the
-// instrument q times (n_cells + 1) plus the cell of the position (n_cells
-// when it lies outside the grid); the packet weight; the phase-function value
+// instrument q times (n_cells + 1) plus the place of the position's cell in
+// the sort order (n_cells when it lies outside the grid); the packet weight; the phase-function value
 // towards the instrument (1 at emission); the wavelength in the low 16 bits
 // of meta, bit 30 set for a scattering, bit 31 when the walk starts from the
 // packet's known cell.
@@ -101,6 +101,12 @@ struct FwdParams {
   int vb_n[3];
   float vb_inv[3];  // buckets per unit length per axis
   int max_walk;     // cells one Voronoi walk or point location may visit before the walk flag
+  // trees and Voronoi grids, sorted pass: the place of every cell in an order
+  // that keeps neighbouring cells together (depth-first over a tree's leaves,
+  // Morton order of Voronoi sites), and per place a point strictly inside the
+  // cell with the cell id in .w (other grids sort by the row-major index)
+  const int* cell_rank;
+  const float4* rank_cell;
   // storage strides of the cell index (cartesian and rectilinear grids): the
   // density and absorption of cell (ix, iy, iz) sit at ix stride[0] +
   // iy stride[1] + iz stride[2]; row-major is (1, nx, nx ny).  Cell ids seen
@@ -119,6 +125,7 @@ struct FwdParams {
   double* absorption;     // [n_lambda][n_cells]
   // run
   unsigned long long n_per_lambda, first_id, n_total, n_norm;
+  unsigned long long w_first;     // first packet of this part of the launch (see peel_cap), n_total its end
   unsigned int seed, model;
   double w_min;
   int max_events, weight_cut, peel_emission, peel_scatter;
@@ -143,7 +150,7 @@ struct FwdParams {
   int use_columns;              // peel-offs along grid axes use the instruments' column sums
   AdjRecord* tape;              // adjoint tape: [packets][tape_stride] event records, or null
   int tape_stride;              // records per packet (max_events + 1)
-  // peel-off walks deferred to the sorted pass (cartesian grids), or peel null
+  // peel-off walks deferred to the sorted pass, or peel null
   PeelRecord* peel;
   unsigned long long peel_cap;     // records peel holds
   unsigned long long* peel_count;  // records asked for (beyond peel_cap the kernel walks them itself)
@@ -241,7 +248,7 @@ cudaError_t launch_forward_voronoi(const FwdParams& p, int num_sms, cudaStream_t
 // records by key (perm: p.peel_cap entries), and the walks and deposits.
 // `mid`, if not null, is recorded on the stream between the ordering and the
 // walks.
-cudaError_t launch_peel_pass(const FwdParams& p, unsigned long long n_keys, unsigned* tile_sum, unsigned* perm,
+cudaError_t launch_peel_pass(const FwdParams& p, int grid_kind, unsigned long long n_keys, unsigned* tile_sum, unsigned* perm,
                              int num_sms, cudaStream_t stream, cudaEvent_t mid);
 // One forced path of a packet in the adjoint (rt_adjoint.cu): what the
 // backward sweep and the path's depositing walk need.  Adjoint quantities are

@@ -1,6 +1,5 @@
-// The sorted peel-off pass of the cartesian forward launch: the walks of the
-// peel-offs that the transport kernel (rt_forward.cu) recorded, ordered by
-// instrument and start cell.
+// The sorted peel-off pass of the forward launch: the walks of the peel-offs
+// that the transport kernels recorded, ordered by instrument and start cell.
 #include "rt_transport.cuh"
 
 namespace rtk {
@@ -11,13 +10,27 @@ namespace {
 //
 // The transport kernel hands each walked peel-off to this pass as a record
 // (start point, weight, phase-function value) counted under its sort key
-// (instrument, cell of the start point).  Ordered by key, the records of a
-// warp start in the same or neighbouring cells and walk parallel rays
-// towards one instrument, so their density loads fall on the same cache
-// lines; in the transport kernel the lanes of a warp walk unrelated rays.
-// Each walk is the transport kernel's own (same arithmetic, same optical
-// depth pair, same deposit), so only the order of the FP64 image additions
-// differs from walking the peel-off in place.
+// (instrument, place of the start point's cell in an order that keeps
+// neighbouring cells together).  Ordered by key, the records of a warp start in
+// the same or neighbouring cells and walk parallel rays towards one
+// instrument, so they cross the same cells together; in the transport kernel
+// the lanes of a warp walk unrelated rays.  Each walk is the transport kernel's
+// own (same arithmetic, same optical depth pair, same deposit), so only the
+// order of the FP64 image additions differs from walking the peel-off in place.
+//
+// On trees and Voronoi grids every frame's peel-offs walk (80 % of the
+// crossings): clumpy octree 52.0 -> 44.2 ms per 2e6 packets, k-d tree 70.0 ->
+// 50.0 ms, Voronoi disk 52.8 -> 38.3 ms per 1.5e6; 16, 10 and 14 lanes active
+// per instruction of the sorted walks against 9, 7 and 6 in place.  Bound by
+// instruction issue (63-68 % of cycles), trees in the descent to the next leaf.
+
+// Resident blocks per SM that the walks' register allocation aims at (disk
+// galaxy and panchromatic disk flat between 4 and 6; octree 3 / 4 / 5: 31.7 /
+// 27.8 / 29.2 ms, k-d tree 31.5 / 30.0 / 32.7, Voronoi 29.4 / 25.6 / 26.2).
+template <class G>
+constexpr int kPeelBlocks = 4;
+template <>
+constexpr int kPeelBlocks<tr::CartGrid> = 5;
 
 constexpr int kScanTile = 4096;  // keys per block of the scan (256 threads x 16)
 
@@ -119,7 +132,12 @@ __global__ void __launch_bounds__(256) k_peel_scatter(const PeelRecord* __restri
 
 // The walks of the sorted records and their deposits; one record per thread,
 // consecutive threads on consecutive records of the order.
-__global__ void __launch_bounds__(256) k_peel_sorted(const __grid_constant__ FwdParams P, const unsigned* __restrict__ perm) {
+template <class G>
+__global__ void __launch_bounds__(tr::kBlock, kPeelBlocks<G>) k_peel_sorted(const __grid_constant__ FwdParams P,
+                                                                            const unsigned* __restrict__ perm) {
+  tr::load_grid_cache<G>(P);
+  __syncthreads();
+  typename G::Scratch sc = tr::lane_scratch<G>(0);
   const unsigned long long n = min(*P.peel_count, P.peel_cap);
   if (blockIdx.x == 0 && threadIdx.x == 0 && n) atomicAdd(&P.counters[8], n);
   const unsigned stride_k = (unsigned)(P.n_cells + 1);
@@ -137,13 +155,10 @@ __global__ void __launch_bounds__(256) k_peel_sorted(const __grid_constant__ Fwd
     const bool known = (meta >> 31) != 0u;
     const double L = __hiloint2double(__float_as_int(b.y), __float_as_int(b.x));
     const float3 x = make_float3(a.x, a.y, a.z);
-    const DevInstr& I = P.instr[q];
-    tr::CartGrid::Cell cell;
-    cell.ix = (int)(c % (unsigned)P.nx);
-    cell.iy = (int)((c / (unsigned)P.nx) % (unsigned)P.ny);
-    cell.iz = (int)(c / ((unsigned)P.nx * (unsigned)P.ny));
+    typename G::Cell cell;
+    if (known) cell = G::sorted_cell(P, c);
     float th, tl;
-    crossings += tr::ray_tau(P, x, tr::instr_dir(I), known, cell, P.lam[lam].kappa, th, tl);
+    crossings += tr::ray_tau<G>(P, x, tr::instr_dir(P.instr[q]), known, cell, P.lam[lam].kappa, th, tl, sc);
     const ulonglong2 tag = P.peel_tag ? P.peel_tag[i] : make_ulonglong2(0ull, 0ull);
     tr::deposit_peel(P, q, lam, x, L, b.z, th, tl, (meta >> 30) & 1u, tag.x, (int)tag.y);
   }
@@ -151,10 +166,23 @@ __global__ void __launch_bounds__(256) k_peel_sorted(const __grid_constant__ Fwd
   if ((threadIdx.x & 31u) == 0 && crossings) atomicAdd(&P.counters[0], crossings);
 }
 
+template <class G>
+cudaError_t launch_walks(const FwdParams& p, const unsigned* perm, int num_sms, size_t smem, cudaStream_t stream) {
+  cudaError_t e = cudaSuccess;
+  if (smem) e = cudaFuncSetAttribute(k_peel_sorted<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  int per_sm = 0;
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_peel_sorted<G>, tr::kBlock, smem);
+  if (e != cudaSuccess) return e;
+  per_sm = per_sm < 1 ? 1 : per_sm;
+  k_peel_sorted<G><<<(unsigned)num_sms * (unsigned)per_sm, tr::kBlock, smem, stream>>>(p, perm);
+  return cudaGetLastError();
+}
+
 }  // namespace
 
-cudaError_t launch_peel_pass(const FwdParams& p, unsigned long long n_keys, unsigned* tile_sum, unsigned* perm,
-                             int num_sms, cudaStream_t stream, cudaEvent_t mid) {
+cudaError_t launch_peel_pass(const FwdParams& p, int grid_kind, unsigned long long n_keys, unsigned* tile_sum,
+                             unsigned* perm, int num_sms, cudaStream_t stream, cudaEvent_t mid) {
   const unsigned long long n_tiles = (n_keys + kScanTile - 1) / kScanTile;
   k_peel_scan_tiles<<<(unsigned)n_tiles, 256, 0, stream>>>(p.peel_hist, n_keys, tile_sum);
   k_peel_scan_sums<<<1, 1024, 0, stream>>>(tile_sum, n_tiles);
@@ -164,12 +192,14 @@ cudaError_t launch_peel_pass(const FwdParams& p, unsigned long long n_keys, unsi
     const cudaError_t em = cudaEventRecord(mid, stream);
     if (em != cudaSuccess) return em;
   }
-  int per_sm = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_peel_sorted, 256, 0);
-  if (e != cudaSuccess) return e;
-  per_sm = per_sm < 1 ? 1 : per_sm;
-  k_peel_sorted<<<(unsigned)num_sms * (unsigned)per_sm, 256, 0, stream>>>(p, perm);
-  return cudaGetLastError();
+  switch (grid_kind) {
+    case RT_GRID_RECTILINEAR: return launch_walks<tr::RectGrid>(p, perm, num_sms, 0, stream);
+    case RT_GRID_OCTREE:
+      return launch_walks<tr::OctGrid>(p, perm, num_sms, (size_t)tr::kBlock * (size_t)p.oct_levels * sizeof(int), stream);
+    case RT_GRID_BINTREE: return launch_walks<tr::BinGrid>(p, perm, num_sms, 0, stream);
+    case RT_GRID_VORONOI: return launch_walks<tr::VorGrid>(p, perm, num_sms, 0, stream);
+    default: return launch_walks<tr::CartGrid>(p, perm, num_sms, 0, stream);
+  }
 }
 
 }  // namespace rtk
