@@ -32,6 +32,19 @@ constexpr int kPeelBlocks = 4;
 template <>
 constexpr int kPeelBlocks<tr::CartGrid> = 5;
 
+// Whether the walks of a warp are kept together crossing by crossing
+// (k_peel_together) or only start together (k_peel_sorted): trees.  On the other
+// grids the plain loop stays converged by itself and the ballot and the state
+// across deposits cost more than they give (disk galaxy 7.6 against 11.6 ms per
+// 4e6 packets, Voronoi disk 25.6 against 28.0 ms per 1.5e6; with ended rays
+// replaced a warp's rays are no longer in the same cell: 33 ms).
+template <class G>
+constexpr bool kPeelTogether = false;
+template <>
+constexpr bool kPeelTogether<tr::OctGrid> = true;
+template <>
+constexpr bool kPeelTogether<tr::BinGrid> = true;
+
 constexpr int kScanTile = 4096;  // keys per block of the scan (256 threads x 16)
 
 // Exclusive scan of each tile of 4096 key counts in place; tile totals out.
@@ -154,28 +167,117 @@ __global__ void __launch_bounds__(tr::kBlock, kPeelBlocks<G>) k_peel_sorted(cons
     const int lam = (int)(meta & 0xffffu);
     const bool known = (meta >> 31) != 0u;
     const double L = __hiloint2double(__float_as_int(b.y), __float_as_int(b.x));
-    const float3 x = make_float3(a.x, a.y, a.z);
     typename G::Cell cell;
     if (known) cell = G::sorted_cell(P, c);
-    float th, tl;
-    crossings += tr::ray_tau<G>(P, x, tr::instr_dir(P.instr[q]), known, cell, P.lam[lam].kappa, th, tl, sc);
+    tr::Ray<G> ray;
+    ray.x = make_float3(a.x, a.y, a.z);
+    ray.d = tr::instr_dir(P.instr[q]);
+    ray.kappa = P.lam[lam].kappa;
+    if (tr::ray_start<G>(P, ray, known, cell, sc)) {
+      do {
+        ++crossings;
+      } while (tr::ray_step<G>(P, ray, sc));
+    }
     const ulonglong2 tag = P.peel_tag ? P.peel_tag[i] : make_ulonglong2(0ull, 0ull);
-    tr::deposit_peel(P, q, lam, x, L, b.z, th, tl, (meta >> 30) & 1u, tag.x, (int)tag.y);
+    tr::deposit_peel(P, q, lam, ray.x, L, b.z, ray.th, ray.tl, (meta >> 30) & 1u, tag.x, (int)tag.y);
   }
   for (int o = 16; o > 0; o >>= 1) crossings += __shfl_down_sync(0xffffffffu, crossings, o);
   if ((threadIdx.x & 31u) == 0 && crossings) atomicAdd(&P.counters[0], crossings);
 }
 
+// Consecutive records that one warp walks, and the ended rays for which it stops
+// to deposit them and start others (12 / 16 / 24 / 32: octree 18.9 / 19.6 / 18.5 /
+// 18.7 ms, k-d tree 18.2 / 18.0 / 18.2 / 19.1 ms).
+constexpr int kSegment = 256, kRefill = 24;
+
+// The walks of the sorted records and their deposits.  A warp takes kSegment
+// consecutive records of the order and keeps its lanes walking: ended rays are
+// deposited and replaced by the segment's next records, kRefill at a time.  The
+// ballot at the loop's head brings the lanes together again after every
+// crossing: in k_peel_sorted the lanes of a tree walk drift apart in the
+// branches of the descent (octree 27.8 -> 18.5 ms per 2e6 packets of the clumpy
+// medium, k-d tree 30.1 -> 18.2 ms).
+template <class G>
+__global__ void __launch_bounds__(tr::kBlock, kPeelBlocks<G>) k_peel_together(const __grid_constant__ FwdParams P,
+                                                                            const unsigned* __restrict__ perm) {
+  tr::load_grid_cache<G>(P);
+  __syncthreads();
+  typename G::Scratch sc = tr::lane_scratch<G>(0);
+  const unsigned long long n = min(*P.peel_count, P.peel_cap);
+  if (blockIdx.x == 0 && threadIdx.x == 0 && n) atomicAdd(&P.counters[8], n);
+  const unsigned stride_k = (unsigned)(P.n_cells + 1);
+  const unsigned lt_mask = (1u << (threadIdx.x & 31u)) - 1u;
+  const unsigned long long n_warps = (unsigned long long)gridDim.x * (blockDim.x >> 5);
+  unsigned crossings = 0;
+  unsigned long long total = 0;
+  for (unsigned long long seg = blockIdx.x * (unsigned long long)(blockDim.x >> 5) + (threadIdx.x >> 5);
+       seg * kSegment < n; seg += n_warps) {
+    unsigned long long next = seg * kSegment;
+    const unsigned long long end = min(n, next + kSegment);
+    tr::Ray<G> ray;
+    bool walking = false, held = false;
+    unsigned rec = 0;  // the lane's record
+    int wait = 0;
+    while (true) {
+      const unsigned idle = __ballot_sync(0xffffffffu, !walking);
+      if (__popc(idle) >= wait) {
+        if (held && !walking) {
+          const float4* r = reinterpret_cast<const float4*>(&P.peel[rec]);
+          const float4 a = r[0], b = r[1];
+          const unsigned meta = __float_as_uint(b.w);
+          const ulonglong2 tag = P.peel_tag ? P.peel_tag[rec] : make_ulonglong2(0ull, 0ull);
+          tr::deposit_peel(P, (int)(__float_as_uint(a.w) / stride_k), (int)(meta & 0xffffu),
+                           make_float3(a.x, a.y, a.z), __hiloint2double(__float_as_int(b.y), __float_as_int(b.x)), b.z,
+                           ray.th, ray.tl, (meta >> 30) & 1u, tag.x, (int)tag.y);
+          held = false;
+        }
+        const unsigned long long j = next + __popc(idle & lt_mask);
+        if (!walking && j < end) {
+          rec = perm[j];
+          const float4* r = reinterpret_cast<const float4*>(&P.peel[rec]);
+          const float4 a = r[0];
+          const unsigned key = __float_as_uint(a.w), meta = __float_as_uint(r[1].w);
+          const unsigned q = key / stride_k;
+          const bool known = (meta >> 31) != 0u;
+          typename G::Cell cell;
+          if (known) cell = G::sorted_cell(P, key - q * stride_k);
+          ray.x = make_float3(a.x, a.y, a.z);
+          ray.d = tr::instr_dir(P.instr[q]);
+          ray.kappa = P.lam[meta & 0xffffu].kappa;
+          walking = tr::ray_start<G>(P, ray, known, cell, sc);
+          held = true;
+        }
+        next = min(end, next + __popc(idle));
+        const int busy = __popc(__ballot_sync(0xffffffffu, held));
+        if (busy == 0) break;
+        // at the segment's end the remaining rays all finish first
+        wait = next < end ? 32 - busy + kRefill : 32;
+      }
+      if (walking) {
+        walking = tr::ray_step<G>(P, ray, sc);
+        crossings += 1u;
+      }
+    }
+    total += crossings;
+    crossings = 0;
+  }
+  for (int o = 16; o > 0; o >>= 1) total += __shfl_down_sync(0xffffffffu, total, o);
+  if ((threadIdx.x & 31u) == 0 && total) atomicAdd(&P.counters[0], total);
+}
+
 template <class G>
 cudaError_t launch_walks(const FwdParams& p, const unsigned* perm, int num_sms, size_t smem, cudaStream_t stream) {
+  void (*kernel)(const FwdParams, const unsigned*);
+  if constexpr (kPeelTogether<G>) kernel = k_peel_together<G>;
+  else kernel = k_peel_sorted<G>;
   cudaError_t e = cudaSuccess;
-  if (smem) e = cudaFuncSetAttribute(k_peel_sorted<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (smem) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_peel_sorted<G>, tr::kBlock, smem);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, tr::kBlock, smem);
   if (e != cudaSuccess) return e;
   per_sm = per_sm < 1 ? 1 : per_sm;
-  k_peel_sorted<G><<<(unsigned)num_sms * (unsigned)per_sm, tr::kBlock, smem, stream>>>(p, perm);
+  kernel<<<(unsigned)num_sms * (unsigned)per_sm, tr::kBlock, smem, stream>>>(p, perm);
   return cudaGetLastError();
 }
 

@@ -1233,38 +1233,44 @@ __device__ __forceinline__ bool column_peel(const FwdParams& P, Task<G, kTape>& 
   return true;
 }
 
-// The optical depth th + tl from x along d to the grid boundary (FP32 pair
-// sum, the transport kernel's walk arithmetic); known: x lies in cell cc.
-// Returns the crossings.
+// A peel-off ray of the sorted pass: the optical depth th + tl from x along d
+// (FP32 pair sum, the transport kernel's walk arithmetic).
 template <class G>
-__device__ __forceinline__ unsigned ray_tau(const FwdParams& P, float3 x, float3 d, bool known,
-                                            const typename G::Cell& cc, float kappa, float& th, float& tl,
-                                            typename G::Scratch& sc) {
-  const float3 id = make_float3(inv_or_zero(d.x), inv_or_zero(d.y), inv_or_zero(d.z));
+struct Ray {
+  float3 x, d, id;
   typename G::Walk w;
-  th = 0.0f;
-  tl = 0.0f;
-  unsigned n = 0;
-  if (G::init(P, x, d, id, known, cc, w, sc)) {
-    float rho = load_density(&P.density[G::cell(w)]);
-    while (true) {
-      int axis;
-      const float te = G::exit(w, x, id, axis);
-      const float texit = fmaxf(te, w.t);
-      const float ds = texit - w.t;
-      const float kr = kappa * rho;
-      const float dt = kr * ds;
-      float nh, e;
-      two_sum(th, dt, nh, e);
-      tl = tl + e;
-      th = nh;
-      ++n;
-      w.t = texit;
-      if (!G::advance(P, x, d, id, axis, w, sc)) break;
-      rho = load_density(&P.density[G::cell(w)]);
-    }
-  }
-  return n;
+  float kappa, rho, th, tl;
+};
+
+// Start the ray at x, which lies in cell cc if known; false if it misses the grid.
+template <class G>
+__device__ __forceinline__ bool ray_start(const FwdParams& P, Ray<G>& r, bool known, const typename G::Cell& cc,
+                                          typename G::Scratch& sc) {
+  r.id = make_float3(inv_or_zero(r.d.x), inv_or_zero(r.d.y), inv_or_zero(r.d.z));
+  r.th = 0.0f;
+  r.tl = 0.0f;
+  if (!G::init(P, r.x, r.d, r.id, known, cc, r.w, sc)) return false;
+  r.rho = load_density(&P.density[G::cell(r.w)]);
+  return true;
+}
+
+// One cell crossing; false when the ray leaves the grid.
+template <class G>
+__device__ __forceinline__ bool ray_step(const FwdParams& P, Ray<G>& r, typename G::Scratch& sc) {
+  int axis;
+  const float te = G::exit(r.w, r.x, r.id, axis);
+  const float texit = fmaxf(te, r.w.t);
+  const float ds = texit - r.w.t;
+  const float kr = r.kappa * r.rho;
+  const float dt = kr * ds;
+  float nh, e;
+  two_sum(r.th, dt, nh, e);
+  r.tl = r.tl + e;
+  r.th = nh;
+  r.w.t = texit;
+  if (!G::advance(P, r.x, r.d, r.id, axis, r.w, sc)) return false;
+  r.rho = load_density(&P.density[G::cell(r.w)]);
+  return true;
 }
 
 // Phase-function value of a scattering peel-off towards instrument I.
