@@ -122,6 +122,7 @@ struct rt_ctx_s {
   double* d_dust_cum = nullptr;
   double* d_dust_tiles = nullptr;
   unsigned* d_dust_clamped = nullptr;
+  double* d_dust_table = nullptr;  // working table of rt_dust_temperature (250 KB)
   std::vector<double> dust_total;
   bool dust_ready = false;
   // optics
@@ -615,6 +616,7 @@ rt_status rt_context_destroy(rt_ctx c) {
   dfree(c->d_stats); dfree(c->d_counters); dfree(c->d_work); dfree(c->d_flags);
   dfree(c->d_adj); dfree(c->d_adj_img); dfree(c->d_adj_max); dfree(c->d_tune_grad); dfree(c->d_tape);
   for (auto& p : c->d_line_dep) dfree(p);
+  dfree(c->d_dust_clamped); dfree(c->d_dust_table);
   dfree(c->d_peel); dfree(c->d_peel_perm); dfree(c->d_peel_hist); dfree(c->d_peel_tiles); dfree(c->d_peel_count);
   dfree(c->d_peel_tag);
   if (c->h_peel_count) cudaFreeHost(c->h_peel_count);
@@ -1875,6 +1877,7 @@ rt_status rt_dust_temperature(rt_ctx c, double emission_scale, double t_min, dou
   const size_t nc = (size_t)c->n_cells, nl = (size_t)c->n_lambda;
   if (!c->d_dust_T) RT_CUDA(c, pool_alloc(c, &c->d_dust_T, nc * sizeof(double)));
   if (!c->d_dust_clamped) RT_CUDA(c, cudaMalloc(&c->d_dust_clamped, sizeof(unsigned)));
+  if (!c->d_dust_table) RT_CUDA(c, cudaMalloc(&c->d_dust_table, dust_table_bytes()));
   RT_CUDA(c, cudaMemsetAsync(c->d_dust_clamped, 0, sizeof(unsigned), s));
   const double* src = c->d_absorption;
   int stored = 1;
@@ -1895,8 +1898,8 @@ rt_status rt_dust_temperature(rt_ctx c, double emission_scale, double t_min, dou
     }
   }
   cudaError_t e = launch_dust_temperature(c->n_lambda, c->nx, c->ny, c->nz, c->stride, c->d_planes64, c->d_density,
-                                          w.data(), c->lambda_um.data(), src, stored, t_min, t_max, c->d_dust_T,
-                                          c->d_dust_clamped, s);
+                                          w.data(), c->lambda_um.data(), src, stored, t_min, t_max, c->d_dust_table,
+                                          c->d_dust_T, c->d_dust_clamped, s);
   unsigned clamped = 0;
   if (e == cudaSuccess) e = cudaMemcpyAsync(&clamped, c->d_dust_clamped, sizeof(unsigned), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess)

@@ -223,8 +223,9 @@ cudaError_t launch_from_storage(const double* src, double* dst, int n_lambda, in
 // cell planes x, y, z; w: S kappa_l (1 - albedo_l) dlambda_l; lambda in um.
 cudaError_t launch_dust_temperature(int n_lambda, int nx, int ny, int nz, const int stride[3], const double* planes,
                                     const float* density, const double* w, const double* lambda,
-                                    const double* absorbed, int stored, double t_min, double t_max, double* T,
-                                    unsigned* clamped, cudaStream_t s);
+                                    const double* absorbed, int stored, double t_min, double t_max, double* table,
+                                    double* T, unsigned* clamped, cudaStream_t s);
+size_t dust_table_bytes();  // of the working table
 cudaError_t launch_dust_emission(int n_lambda, int nx, int ny, int nz, const int stride[3], const double* planes,
                                  const float* density, const double* w, const double* lambda, const double* T,
                                  double* lum, double* cum, double* tile_sum, cudaStream_t s);

@@ -365,6 +365,28 @@ RT_FN double one_minus_exp(double x) {
   return big ? 1.0 : A + fma(T, p, m > 0 ? 0.0 : e.a_lo);
 }
 
+// exp(-x) / (1 - exp(-x)) = 1 / (exp(x) - 1) for x > 0 (zero above 709.78, where
+// exp(x) - 1 overflows), with the reduction of one_minus_exp.
+RT_FN double bose(double x) {
+  if (bits_of(x) > 0x40862e42fefa39efll) return 0.0;
+  const float kf = rintf(cut(x) * 184.664965f);
+  const int k = (int)kf;
+  const double kd = widen(kf);
+  const double r = fma(-kd, kLn2Over128Lo, fma(-kd, kLn2Over128Hi, x));
+  const float rf = cut(r);
+  const float tail = fmaf(rf, fmaf(rf, -1.0f / 720.0f, 1.0f / 120.0f), -1.0f / 24.0f);
+  double q = fma(r, widen(tail), 1.0 / 6.0);
+  q = fma(r, q, -0.5);
+  const double p = fma(r, r * q, r);
+  const ExpEntry e = kExpTable[k & 127];
+  const int m = k >> 7, big = m > 960 ? m - 960 : 0;  // 2^-m in two normal factors
+  const double T = double_of(bits_of(e.t) - ((long long)(m - big) << 52));
+  const double A = m > 0 ? 1.0 - T : e.a;
+  const double one_minus = m > 64 ? 1.0 : A + fma(T, p, m > 0 ? 0.0 : e.a_lo);
+  const double z = fma(-T, p, T) / one_minus;
+  return big ? z * double_of((long long)(1023 - big) << 52) : z;
+}
+
 // -ln(1 - v) for 0 <= v < 1.  y = 1 - v rounded, its rounding error kept; y =
 // 2^-m z with z in (1/2, 1]; z rc = 1 + r, |r| <= 2^-8: -ln(1 - v) = m ln 2 +
 // ln rc - ln(1 + r).  On the last interval of z with m = 0, rc = 1 and r = -v

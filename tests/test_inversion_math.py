@@ -19,6 +19,8 @@ def math_lib(tmp_path_factory):
     d = tmp_path_factory.mktemp("math")
     src = d / "shim.cpp"
     src.write_text(f'#include "{CSRC}/rt_math.cuh"\n'
+                   'extern "C" void run_bose(const double* x, double* y, long n) {\n'
+                   "  for (long i = 0; i < n; ++i) y[i] = rtk::bose(x[i]);\n}\n"
                    'extern "C" void run(const double* x, double* e, double* l, long n) {\n'
                    "  for (long i = 0; i < n; ++i) {\n"
                    "    if (e) e[i] = rtk::one_minus_exp(x[i]);\n"
@@ -26,6 +28,7 @@ def math_lib(tmp_path_factory):
     so = d / "shim.so"
     subprocess.run(["g++", "-O1", "-std=c++17", "-ffp-contract=off", "-shared", "-fPIC", str(src), "-o", str(so)], check=True)
     lib = ctypes.CDLL(str(so))
+    lib.run_bose.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_long]
     lib.run.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_long]
     return lib
 
@@ -53,3 +56,19 @@ def test_against_extended_precision(math_lib, which, lo, hi):
     got = _call(math_lib, x, which)
     err = np.abs(got.astype(np.longdouble) - ref) / np.spacing(np.maximum(ref.astype(np.float64), 1e-300))
     assert np.all(np.isfinite(got)) and float(err.max()) <= ULP
+
+
+def test_bose_against_extended_precision(math_lib):
+    """1 / (exp(x) - 1): the leading roundings are those of 1 - exp(-x) and
+    exp(-x) (2 ulp each) and of the quotient; zero where exp(x) overflows."""
+    rng = np.random.default_rng(12)
+    x = np.concatenate([np.exp(rng.uniform(np.log(1e-9), np.log(700.0), 200_000)), np.arange(1, 4000) * (np.log(2.0) / 256.0)])
+    y = np.empty_like(x)
+    math_lib.run_bose(x.ctypes.data, y.ctypes.data, x.size)
+    ref = 1.0 / np.expm1(x.astype(np.longdouble))
+    assert float((np.abs(y.astype(np.longdouble) - ref) / ref).max()) <= 5.0 * 2.0 ** -53
+    ends = np.array([709.0, 709.7, 709.79, 1e4, np.inf, np.nan])
+    y = np.empty_like(ends)
+    math_lib.run_bose(ends.ctypes.data, y.ctypes.data, ends.size)
+    np.testing.assert_allclose(y[:2], 1.0 / np.expm1(ends[:2]), rtol=1e-15)
+    assert np.all(y[2:] == 0.0)
