@@ -10,12 +10,18 @@
 //
 // Work list: runs of packets of one model (chunks), sorted by estimated cost,
 // largest first, so that the long runs start early and the short ones fill
-// the tail.  A warp takes a chunk with one atomic and hands its packets to
-// its lanes as they need them; lanes of a warp may hold packets of different
-// models.  A lane keeps its model's grid geometry in its own shared-memory
-// slot (the cell walk reads it there), and the model's escaped / absorbed /
-// truncated luminosity in another, flushed to the model's FP64 tallies when
-// the lane moves to another model.
+// the tail.  A warp takes a chunk with one atomic and hands its packets to its
+// slots as they become free; the slots of a warp may hold packets of different
+// models.
+//
+// The execution model is the transport kernels' (rt_transport.cuh): more packets
+// than lanes per warp in shared-memory slots, lanes that only walk, rounds of
+// per-event work over packets that wait for the same kind of work.  A lane keeps
+// the geometry its walk reads in its own shared-memory words (nine: an odd
+// count, so that the lanes of a warp meet no bank conflicts; at 64 bytes apart
+// they met 16-way ones, half of the kernel's shared-memory cycles).  The
+// luminosity tallies of a lane are flushed to the model's when it serves
+// another model.
 #include "rt_transport.cuh"
 
 namespace rtk {
@@ -24,61 +30,54 @@ namespace {
 
 using tr::CartGrid;
 
-// Grid geometry of a lane's model, in the shape CartGrid reads.
+// Packet slots per warp (256 models: 40 / 48 / 52 / 56 / 60 / 64 slots 128 / 114 /
+// 110 / 107 / 108 / 106 ms).
+#ifndef RT_BATCH_SLOTS
+#define RT_BATCH_SLOTS 56
+#endif
+constexpr int kBatchSlots = RT_BATCH_SLOTS;
+constexpr int kBatchWarps = kBatchBlock / 32;
+static_assert(kBatchSlots <= tr::kRing, "a queue holds every slot of its warp");
+
+// What a walk reads of its model's grid, in the shape CartGrid reads.
 struct Geo {
-  int nx, ny, nz, pad;
-  float lo[3], hi[3], d[3], inv_d[3];
+  int nx, ny, nz;
+  float lo[3], d[3];
 };
 
-struct Tally {
-  double escaped, absorbed, truncated;
-  int model, pad;
-  unsigned long long column_peels, column_crossings;  // the lane's, over the launch
+// A warp's current chunk, and its counts.
+struct WarpState {
+  uint2 queues;
+  unsigned long long next, end;  // packet ids left of the chunk
+  int model, drained;
+  unsigned long long crossings, events, peeloffs, packets, column_peels, column_crossings;
 };
 
-__shared__ unsigned long long S_PID[kBatchBlock];
-__shared__ double S_WEIGHT[kBatchBlock];
-__shared__ float3 S_DIR[kBatchBlock];
-__shared__ float2 S_HG[kBatchBlock];
-__shared__ int S_EVENT[kBatchBlock], S_INSTR_Q[kBatchBlock], S_WPHASE[kBatchBlock];
-__shared__ bool S_HAS_CELL[kBatchBlock];
-__shared__ CartGrid::Cell S_CELL_CART[kBatchBlock];
-__shared__ Geo S_GEO[kBatchBlock];
-__shared__ Tally S_TALLY[kBatchBlock];
+struct BShared {
+  static constexpr int kN = kBatchWarps * kBatchSlots;
+  unsigned long long pid[kN];
+  double L[kN];
+  float2 hg[kN];     // the event's Henyey-Greenstein uniforms
+  float2 res[kN];    // what a walk starts with (path 2: tau* as a pair) and ended with
+  float3 x[kN], k[kN];
+  CartGrid::Cell cell[kN];
+  int event[kN], model[kN];
+  unsigned pack[kN];  // phase, has-cell (tr::Pack)
+  Geo geo[kBatchBlock];
+  WarpState warp[kBatchWarps];
+  unsigned char ring[kBatchWarps][tr::kQueues][tr::kRing];
+};
+__device__ __forceinline__ BShared& state() { return *reinterpret_cast<BShared*>(tr::S_RAW); }
 
-// The lane state that only the per-event work touches sits in the transport
-// kernels' per-thread shared-memory slots, so that the walk's state fits the
-// registers of four resident blocks per SM.
+// Resident blocks per SM the register allocation aims at.
 #ifndef RT_BATCH_MIN_BLOCKS
 #define RT_BATCH_MIN_BLOCKS 4
 #endif
-static_assert(kBatchBlock == tr::kBlock, "per-thread slots are sized for the transport block");
 
-struct BLane {
-  int m, phase;
-  float kappa;
-  float3 x;
-  bool walking;
-  // in shared memory: packet id, event index, peel-off done (1) or not (0)
-  // for this event, the walk a kStart lane begins, weight, direction of
-  // travel, the event's Henyey-Greenstein uniforms, the cell of x (valid when
-  // has_cell)
-  __device__ __forceinline__ unsigned long long& pid() const { return S_PID[threadIdx.x]; }
-  __device__ __forceinline__ int& event() const { return S_EVENT[threadIdx.x]; }
-  __device__ __forceinline__ int& q() const { return S_INSTR_Q[threadIdx.x]; }
-  __device__ __forceinline__ int& wphase() const { return S_WPHASE[threadIdx.x]; }
-  __device__ __forceinline__ double& L() const { return S_WEIGHT[threadIdx.x]; }
-  __device__ __forceinline__ float3& k() const { return S_DIR[threadIdx.x]; }
-  __device__ __forceinline__ float& u_mu() const { return S_HG[threadIdx.x].x; }
-  __device__ __forceinline__ float& u_phi() const { return S_HG[threadIdx.x].y; }
-  __device__ __forceinline__ CartGrid::Cell& cell() const { return S_CELL_CART[threadIdx.x]; }
-  __device__ __forceinline__ bool& has_cell() const { return S_HAS_CELL[threadIdx.x]; }
-  float3 d, id;
-  CartGrid::Walk w;
-  float rho;
-  float th, tl;
-  float aux0, aux1;   // path 1: deposit weight (unused here); path 2: tau* pair, then s*
-  const float* dens;  // the model's densities
+// Luminosity of one model gathered by one lane (in its local memory).
+struct Tally {
+  double escaped, absorbed, truncated;
+  int model;
 };
 
 __device__ __forceinline__ void flush(const BatchParams& P, Tally& t) {
@@ -91,28 +90,40 @@ __device__ __forceinline__ void flush(const BatchParams& P, Tally& t) {
   t.escaped = t.absorbed = t.truncated = 0.0;
 }
 
-__device__ __forceinline__ void start_walk(BLane& s, const Geo& G, float3 d) {
-  s.d = d;
-  s.id = make_float3(tr::inv_or_zero(d.x), tr::inv_or_zero(d.y), tr::inv_or_zero(d.z));
-  s.th = 0.0f;
-  s.tl = 0.0f;
-  CartGrid::Scratch sc;
-  s.walking = CartGrid::init(G, s.x, d, s.id, s.has_cell(), s.cell(), s.w, sc);
-  if (s.walking) s.rho = tr::load_density(&s.dens[s.w.cell]);
-}
+// The walk a lane is on.
+struct BWalker {
+  int slot, phase;
+  bool walking;
+  float kappa;
+  float3 x, id;
+  CartGrid::Walk w;
+  float rho, th, tl;
+  unsigned n;
+  float aux0, aux1;   // path 2: tau* pair, then s*
+  const float* dens;  // the model's densities
+};
 
-__device__ __forceinline__ float3 kobs(const DevInstr& I) { return make_float3(I.kobs[0], I.kobs[1], I.kobs[2]); }
+// A packet in per-event work.
+struct BTask {
+  Tally& tally;
+  int i, phase, wphase, m, event;
+  bool has_cell;
+  float th, tl;
+  unsigned n_peel, n_col, c_col;
+};
 
 // The forward kernel's peel-off deposit for a single-channel frame.
-__device__ __forceinline__ void deposit(const DevModel& M, const BLane& s, bool scattered) {
+__device__ __forceinline__ void deposit(const DevModel& M, const BTask& s, bool scattered) {
   const DevInstr& I = M.instr;
+  const float3 x = state().x[s.i], k = state().k[s.i];
+  const double L = state().L[s.i];
   float phase = 1.0f;
-  if (scattered) phase = hg_phase(M.g, s.k().x * I.kobs[0] + s.k().y * I.kobs[1] + s.k().z * I.kobs[2]);
+  if (scattered) phase = hg_phase(M.g, k.x * I.kobs[0] + k.y * I.kobs[1] + k.z * I.kobs[2]);
   const float tau = s.th;
-  const double value = tau < 80.0f ? s.L() * widen(tr::kInv4PiF * phase * expf(-tau) * (1.0f - s.tl))
-                                   : s.L() * kInv4PiD * (double)phase * exp(-((double)tau + (double)s.tl));
-  const float fx = (s.x.x * I.ex[0] + s.x.y * I.ex[1] + s.x.z * I.ex[2] + I.off_x) * I.sx;
-  const float fy = (s.x.x * I.ey[0] + s.x.y * I.ey[1] + s.x.z * I.ey[2] + I.off_y) * I.sy;
+  const double value = tau < 80.0f ? L * widen(tr::kInv4PiF * phase * expf(-tau) * (1.0f - s.tl))
+                                   : L * kInv4PiD * (double)phase * exp(-((double)tau + (double)s.tl));
+  const float fx = (x.x * I.ex[0] + x.y * I.ex[1] + x.z * I.ex[2] + I.off_x) * I.sx;
+  const float fy = (x.x * I.ey[0] + x.y * I.ey[1] + x.z * I.ey[2] + I.off_y) * I.sy;
   if (!I.bilinear) {
     const float fix = floorf(fx), fiy = floorf(fy);
     if (!(fix >= 0.0f && fiy >= 0.0f && fix < (float)I.nx && fiy < (float)I.ny)) return;
@@ -135,153 +146,277 @@ __device__ __forceinline__ void deposit(const DevModel& M, const BLane& s, bool 
 }
 
 // The forward kernel's column shortcut for a frame along a grid axis (see
-// column_peel there); false when the position is outside the grid.
-__device__ __forceinline__ bool column_peel(const DevInstr& I, BLane& s, const Geo& G, Tally& T,
-                                            unsigned& n_cross) {
+// column_tau there); false when the position is outside the grid.
+__device__ __forceinline__ bool column_peel(const BatchParams& P, const DevModel& M, BTask& s) {
+  const DevInstr& I = M.instr;
+  const float3 x = state().x[s.i];
   CartGrid::Cell c;
-  if (s.has_cell()) {
-    c = s.cell();
+  if (s.has_cell) {
+    c = state().cell[s.i];
   } else {
-    if (!inside_box(G, s.x)) return false;
-    c.ix = min(max(__float2int_rd((s.x.x - G.lo[0]) * G.inv_d[0]), 0), G.nx - 1);
-    c.iy = min(max(__float2int_rd((s.x.y - G.lo[1]) * G.inv_d[1]), 0), G.ny - 1);
-    c.iz = min(max(__float2int_rd((s.x.z - G.lo[2]) * G.inv_d[2]), 0), G.nz - 1);
+    if (!inside_box(M, x)) return false;
+    c.ix = min(max(__float2int_rd((x.x - M.lo[0]) * M.inv_d[0]), 0), M.nx - 1);
+    c.iy = min(max(__float2int_rd((x.y - M.lo[1]) * M.inv_d[1]), 0), M.ny - 1);
+    c.iz = min(max(__float2int_rd((x.z - M.lo[2]) * M.inv_d[2]), 0), M.nz - 1);
   }
   const int a = I.axis;
   const bool up = I.dir > 0;
   const int i = a == 0 ? c.ix : (a == 1 ? c.iy : c.iz);
-  const int n = a == 0 ? G.nx : (a == 1 ? G.ny : G.nz);
-  const float xa = a == 0 ? s.x.x : (a == 1 ? s.x.y : s.x.z);
-  const float plane = fmaf((float)(i + (up ? 1 : 0)), G.d[a], G.lo[a]);
+  const int n = a == 0 ? M.nx : (a == 1 ? M.ny : M.nz);
+  const float xa = a == 0 ? x.x : (a == 1 ? x.y : x.z);
+  const float plane = fmaf((float)(i + (up ? 1 : 0)), M.d[a], M.lo[a]);
   const float ds0 = fmaxf(up ? plane - xa : xa - plane, 0.0f);
-  const int cell = c.ix + G.nx * (c.iy + G.ny * c.iz);
-  s.th = s.kappa * fmaf(tr::load_density(&s.dens[cell]), ds0, __ldg(&I.column[cell]));
+  const int cell = c.ix + M.nx * (c.iy + M.ny * c.iz);
+  s.th = M.kappa * fmaf(tr::load_density(&P.density[M.density + cell]), ds0, __ldg(&I.column[cell]));
   s.tl = 0.0f;
-  s.walking = false;
-  const unsigned nc = (unsigned)(up ? n - i : i + 1);
-  n_cross += nc;
-  T.column_peels += 1ull;
-  T.column_crossings += nc;
+  s.n_col += 1u;
+  s.c_col += (unsigned)(up ? n - i : i + 1);
   return true;
 }
 
-// Ask for walk `phase` from the lane's position along d (started in the last
-// stage of a control round, from one place in the code).
-__device__ __forceinline__ void request_walk(BLane& s, int phase, float3 d) {
-  s.wphase() = phase;
-  s.d = d;
+__device__ __forceinline__ void request_walk(BTask& s, int phase) {
+  s.wphase = phase;
   s.phase = tr::kStart;
 }
 
 // ---- the stages of a control round (the forward kernel's, for one frame
 // per model and no absorption field)
 
-// A new packet (model m, packet id pid): the model's geometry, emission from
-// its point source (the forward kernel's event-0 draws).
-__device__ __forceinline__ void begin(const BatchParams& P, BLane& s, Geo& G, Tally& T, int m,
-                                      unsigned long long pid) {
-  const DevModel& M = P.models[m];
-  if (T.model != m) {
-    flush(P, T);
-    T.model = m;
-  }
-  G.nx = M.nx; G.ny = M.ny; G.nz = M.nz;
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    G.lo[a] = M.lo[a]; G.hi[a] = M.hi[a]; G.d[a] = M.d[a]; G.inv_d[a] = M.inv_d[a];
-  }
-  s.m = m;
-  s.pid() = pid;
-  s.dens = P.density + M.density;
-  s.kappa = M.kappa;
-  s.L() = M.L0;
-  s.event() = 0;
-  s.has_cell() = false;
+// A new packet (model m, packet id pid): emission from its point source (the
+// forward kernel's event-0 draws).
+__device__ __forceinline__ void begin(const BatchParams& P, BTask& s, unsigned long long pid) {
+  const DevModel& M = P.models[s.m];
+  state().pid[s.i] = pid;
+  state().model[s.i] = s.m;
+  state().L[s.i] = M.L0;
+  s.event = 0;
+  s.has_cell = false;
   // one point source: the position draws of block 0 are not needed
-  const uint4 r1 = draw_block(pid, 0, 0, 1, P.seed, (unsigned)m);
-  s.x = make_float3(M.src[0], M.src[1], M.src[2]);
+  const uint4 r1 = draw_block(pid, 0, 0, 1, P.seed, (unsigned)s.m);
+  state().x[s.i] = make_float3(M.src[0], M.src[1], M.src[2]);
   const float mu = tr::u01f_signed(r1.z);
   const float st = sqrtf(fmaxf(0.0f, 1.0f - mu * mu));
   float sp, cp;
   sincospif(2.0f * tr::u01f(r1.w), &sp, &cp);
-  s.k() = make_float3(st * cp, st * sp, mu);
-  s.q() = 0;
+  state().k[s.i] = make_float3(st * cp, st * sp, mu);
   s.phase = tr::kPeelScan;
 }
 
-__device__ __forceinline__ void finish_path1(const BatchParams& P, BLane& s, Tally& T) {
+// The tally of the packet's model.
+__device__ __forceinline__ Tally& tally_of(const BatchParams& P, BTask& s) {
+  if (s.tally.model != s.m) {
+    flush(P, s.tally);
+    s.tally.model = s.m;
+  }
+  return s.tally;
+}
+
+__device__ __forceinline__ void finish_path1(const BatchParams& P, BTask& s) {
   const DevModel& M = P.models[s.m];
   const double tau = widen(s.th) + widen(s.tl);
+  const double L = state().L[s.i];
+  Tally& T = tally_of(P, s);
   if (!(tau > 0.0)) {
-    T.escaped += s.L();
+    T.escaped += L;
     s.phase = tr::kFetch;
     return;
   }
   const double albedo = M.albedo;
   const double one_minus_E = one_minus_exp(tau);
   const double E = 1.0 - one_minus_E;
-  T.escaped += s.L() * E;
-  T.absorbed += (1.0 - albedo) * s.L() * one_minus_E;
-  const uint4 r = draw_block(s.pid(), 0, s.event(), 0, P.seed, (unsigned)s.m);
+  T.escaped += L * E;
+  T.absorbed += (1.0 - albedo) * L * one_minus_E;
+  const uint4 r = draw_block(state().pid[s.i], 0, s.event, 0, P.seed, (unsigned)s.m);
   const double tau_star = neg_log_one_minus(u01(r.x) * one_minus_E);
-  s.u_mu() = tr::u01f(r.y);
-  s.u_phi() = tr::u01f(r.z);
-  tr::split_pair(tau_star, s.aux0, s.aux1);
-  s.L() = albedo * s.L() * one_minus_E;
-  request_walk(s, tr::kPath2, s.k());
+  state().hg[s.i] = make_float2(tr::u01f(r.y), tr::u01f(r.z));
+  float2 a;
+  tr::split_pair(tau_star, a.x, a.y);
+  state().res[s.i] = a;
+  state().L[s.i] = albedo * L * one_minus_E;
+  request_walk(s, tr::kPath2);
 }
 
-__device__ __forceinline__ void finish_path2(const Geo& G, BLane& s, unsigned& n_events) {
-  const float s_star = s.aux0;
-  float3 x = make_float3(fmaf(s_star, s.k().x, s.x.x), fmaf(s_star, s.k().y, s.x.y), fmaf(s_star, s.k().z, s.x.z));
-  s.cell() = CartGrid::carried(s.w);
-  CartGrid::clamp(G, s.cell(), x);
-  s.x = x;
-  s.has_cell() = true;
-  n_events += 1u;
-  s.q() = 0;
+// Path 2 ended (th holds s*, the slot the cell).
+__device__ __forceinline__ void finish_path2(const BatchParams& P, BTask& s) {
+  const float s_star = s.th;
+  const float3 x0 = state().x[s.i], k = state().k[s.i];
+  float3 x = make_float3(fmaf(s_star, k.x, x0.x), fmaf(s_star, k.y, x0.y), fmaf(s_star, k.z, x0.z));
+  CartGrid::clamp(P.models[s.m], state().cell[s.i], x);
+  state().x[s.i] = x;
+  s.has_cell = true;
   s.phase = tr::kPeelScan;
 }
 
-// The model's one peel-off of this event, or what follows it.
-__device__ __forceinline__ void peel_scan(const BatchParams& P, BLane& s, const Geo& G, Tally& T,
-                                          unsigned& n_cross) {
-  const bool emission = s.event() == 0;
-  if ((emission ? P.peel_emission : P.peel_scatter) && s.q() == 0) {
-    const DevInstr& I = P.models[s.m].instr;
-    const int phase = emission ? tr::kPeelEmit : tr::kPeelScat;
-    if (P.use_columns && I.column && column_peel(I, s, G, T, n_cross)) {
-      s.phase = phase;
-      return;
-    }
-    request_walk(s, phase, kobs(I));
-    return;
-  }
-  if (emission) {
-    s.event() = 1;
-    request_walk(s, tr::kPath1, s.k());
-  } else {
-    s.phase = tr::kAfter;
-  }
-}
-
-__device__ __forceinline__ void after_scattering(const BatchParams& P, BLane& s, Tally& T) {
+__device__ __forceinline__ void after_scattering(const BatchParams& P, BTask& s) {
   const DevModel& M = P.models[s.m];
-  const float mu = hg_sample(M.g, s.u_mu());
+  const float2 u = state().hg[s.i];
+  const float mu = hg_sample(M.g, u.x);
   float sp, cp;
-  sincospif(2.0f * s.u_phi(), &sp, &cp);
-  s.k() = rotate_dir(s.k(), mu, sp, cp);
-  if ((P.weight_cut && s.L() < P.w_min * M.L0) || s.event() >= P.max_events) {
-    T.truncated += s.L();
+  sincospif(2.0f * u.y, &sp, &cp);
+  state().k[s.i] = rotate_dir(state().k[s.i], mu, sp, cp);
+  const double L = state().L[s.i];
+  if ((P.weight_cut && L < P.w_min * M.L0) || s.event >= P.max_events) {
+    tally_of(P, s).truncated += L;
     s.phase = tr::kFetch;
     return;
   }
-  s.event() += 1;
-  request_walk(s, tr::kPath1, s.k());
+  s.event += 1;
+  request_walk(s, tr::kPath1);
+}
+
+// Hand packets of the warp's chunk to the lanes below n, taking new chunks as
+// needed: model and id of the lane's, or model -1 (no packets left).
+__device__ __forceinline__ void take_packets(const BatchParams& P, WarpState& ws, int n, int lane, int& model,
+                                             unsigned long long& pid) {
+  unsigned long long next = ws.next, end = ws.end;
+  int m = ws.model, drained = ws.drained, done = 0;
+  model = -1;
+  pid = 0ull;
+  __syncwarp();
+  while (done < n && !drained) {
+    if (next >= end) {
+      unsigned long long ci = 0;
+      if (lane == 0) ci = atomicAdd(P.chunk_counter, 1ull);
+      ci = __shfl_sync(0xffffffffu, ci, 0);
+      if (ci >= (unsigned long long)P.n_chunks) {
+        drained = 1;
+        break;
+      }
+      const BatchChunk ch = P.chunks[ci];
+      m = ch.model;
+      next = ch.first;
+      end = ch.first + ch.count;
+    }
+    const unsigned long long avail = end - next;
+    const int take = avail < (unsigned long long)(n - done) ? (int)avail : n - done;
+    if (lane >= done && lane < done + take) {
+      model = m;
+      pid = next + (unsigned long long)(lane - done);
+    }
+    next += (unsigned long long)take;
+    done += take;
+  }
+  if (lane == 0) {
+    ws.next = next;
+    ws.end = end;
+    ws.model = m;
+    ws.drained = drained;
+  }
+}
+
+// One control round (see the forward kernel's).
+__device__ __forceinline__ void control_round(const BatchParams& P, tr::Queues& Q, WarpState& ws, Tally& tally, int cls,
+                                              unsigned lane, unsigned lt_mask) {
+  const int n = min(32, Q.size(cls));
+  const bool on = (int)lane < n;
+  const int local = on ? Q.at(cls, (int)lane) : 0;
+  Q.drop(cls, n);
+  BTask s{tally};
+  s.i = (int)(threadIdx.x >> 5) * kBatchSlots + local;
+  const unsigned pk = state().pack[s.i];
+  s.phase = on ? tr::Pack::phase(pk) : tr::kExit;
+  s.wphase = 0;
+  s.has_cell = tr::Pack::has_cell(pk);
+  s.m = state().model[s.i];
+  s.event = state().event[s.i];
+  const float2 res = state().res[s.i];
+  s.th = res.x;
+  s.tl = res.y;
+  s.n_peel = s.n_col = s.c_col = 0u;
+  int n_events = 0, n_packets = 0;
+  if (cls == tr::kQPath1) {
+    if (on) finish_path1(P, s);
+  } else {
+    if (cls == tr::kQFetch) {
+      unsigned long long pid;
+      take_packets(P, ws, n, (int)lane, s.m, pid);
+      const bool got = on && s.m >= 0;
+      n_packets = __popc(__ballot_sync(0xffffffffu, got));
+      if (got) begin(P, s, pid);
+      else s.phase = tr::kExit;
+    } else {
+      const bool ended = on && s.phase == tr::kPath2;
+      n_events = __popc(__ballot_sync(0xffffffffu, ended));
+      if (ended) finish_path2(P, s);
+    }
+    // the model's one peel-off of this event: along a grid axis by the column
+    // sums, else by a walk; deposited here when it is known
+    const bool walked = s.phase == tr::kPeelEmit || s.phase == tr::kPeelScat;
+    if (walked || s.phase == tr::kPeelScan) {
+      const DevModel& M = P.models[s.m];
+      bool known = walked;
+      if (!walked && (s.event == 0 ? P.peel_emission : P.peel_scatter)) {
+        known = P.use_columns && M.instr.column && column_peel(P, M, s);
+        if (!known) request_walk(s, s.event == 0 ? tr::kPeelEmit : tr::kPeelScat);
+      }
+      if (known) {
+        deposit(M, s, s.event != 0);
+        s.n_peel += 1u;
+      }
+      if (s.phase != tr::kStart) {
+        if (s.event == 0) {
+          s.event = 1;
+          request_walk(s, tr::kPath1);
+        } else {
+          s.phase = tr::kAfter;
+        }
+      }
+    }
+    if (s.phase == tr::kAfter) after_scattering(P, s);
+  }
+  const bool start = on && s.phase == tr::kStart, again = on && s.phase == tr::kFetch;
+  if (start) {
+    state().pack[s.i] = tr::Pack::make(s.wphase, 0, 0, s.has_cell, 0);
+    state().event[s.i] = s.event;
+  }
+  Q.push(tr::kQReady, start, local, lt_mask);
+  Q.push(tr::kQFetch, again, local, lt_mask);
+  if (cls != tr::kQPath1) {
+    const unsigned np = __reduce_add_sync(0xffffffffu, s.n_peel);
+    const unsigned nc = __reduce_add_sync(0xffffffffu, s.n_col);
+    const unsigned cc = __reduce_add_sync(0xffffffffu, s.c_col);
+    if (lane == 0) {
+      ws.events += (unsigned long long)n_events;
+      ws.packets += (unsigned long long)n_packets;
+      ws.peeloffs += np;
+      ws.column_peels += nc;
+      ws.column_crossings += cc;
+      ws.crossings += cc;
+    }
+  }
+  __syncwarp();
+}
+
+// Start the ready packet in slot i on this lane.
+__device__ __forceinline__ void start_walk(const BatchParams& P, BWalker& s, int i) {
+  const DevModel& M = P.models[state().model[i]];
+  const unsigned pk = state().pack[i];
+  s.slot = i;
+  s.phase = tr::Pack::phase(pk);
+  s.kappa = M.kappa;
+  s.dens = P.density + M.density;
+  s.x = state().x[i];
+  float3 d = state().k[i];
+  if (s.phase == tr::kPeelEmit || s.phase == tr::kPeelScat) d = tr::instr_dir(M.instr);
+  s.id = make_float3(tr::inv_or_zero(d.x), tr::inv_or_zero(d.y), tr::inv_or_zero(d.z));
+  const float2 a = state().res[i];
+  s.aux0 = a.x;
+  s.aux1 = a.y;
+  s.th = 0.0f;
+  s.tl = 0.0f;
+  s.n = 0u;
+  Geo& G = state().geo[threadIdx.x];
+  G.nx = M.nx; G.ny = M.ny; G.nz = M.nz;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) { G.lo[c] = M.lo[c]; G.d[c] = M.d[c]; }
+  CartGrid::Scratch sc;
+  s.walking = CartGrid::init(M, s.x, d, s.id, tr::Pack::has_cell(pk), state().cell[i], s.w, sc);
+  if (s.walking) s.rho = tr::load_density(&s.dens[s.w.cell]);
 }
 
 // One cell crossing (the forward kernel's step without the absorption field).
-__device__ __forceinline__ void step(const BatchParams& P, BLane& s, const Geo& G, unsigned& n_cross) {
+__device__ __forceinline__ void step(const BatchParams& P, BWalker& s) {
+  const Geo& G = state().geo[threadIdx.x];
   CartGrid::Walk& w = s.w;
   int axis;
   const float te = CartGrid::exit(w, s.x, s.id, axis);
@@ -301,10 +436,10 @@ __device__ __forceinline__ void step(const BatchParams& P, BLane& s, const Geo& 
   }
   s.th = nh;
   s.tl = nl;
-  n_cross += path2 ? 0u : 1u;
+  s.n += 1u;
   w.t = texit;
   CartGrid::Scratch sc;
-  if (CartGrid::advance(G, s.x, s.d, s.id, axis, w, sc)) {
+  if (CartGrid::advance(G, s.x, s.x, s.id, axis, w, sc)) {
     s.rho = tr::load_density(&s.dens[w.cell]);
   } else {
     s.walking = false;
@@ -316,120 +451,84 @@ __device__ __forceinline__ void step(const BatchParams& P, BLane& s, const Geo& 
 }
 
 __global__ void __launch_bounds__(kBatchBlock, RT_BATCH_MIN_BLOCKS) k_batch(const BatchParams P) {
-  const unsigned lane = threadIdx.x & 31u;
+  const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
   const unsigned lt_mask = (1u << lane) - 1u;
-  Geo& G = S_GEO[threadIdx.x];
-  Tally& T = S_TALLY[threadIdx.x];
-  T.escaped = T.absorbed = T.truncated = 0.0;
-  T.model = -1;
-  T.column_peels = T.column_crossings = 0ull;
-  BLane s;
-  s.phase = tr::kFetch;
-  s.walking = false;
-  s.m = 0;
-  unsigned n_cross = 0, n_events = 0, n_peel = 0, n_packets = 0;
-  unsigned long long tot_cross = 0;
-  // the warp's current chunk (the same in every lane)
-  unsigned long long c_next = 0, c_end = 0;
-  int c_model = 0;
-  bool drained = false;
-  while (true) {
-    const bool idle = !s.walking && s.phase != tr::kExit;
-    const unsigned need = __ballot_sync(0xffffffffu, idle);
-    const unsigned walkers = __ballot_sync(0xffffffffu, s.walking);
-    if (need == 0u && walkers == 0u) break;
-    if (walkers == 0u || __popc(need) >= P.control_min) {
-      // per-event work in stages, each run by the lanes in its phase together
-      if (!s.walking) {
-        if (s.phase == tr::kPath1) finish_path1(P, s, T);
-        if (s.phase == tr::kPath2) finish_path2(G, s, n_events);
-      }
-      // peel-offs, the scattering and new packets, repeated while a lane has
-      // just finished its packet (at most two passes)
-      while (true) {
-        while (true) {
-          const bool ready = !s.walking && (s.phase == tr::kPeelEmit || s.phase == tr::kPeelScat);
-          if (!__any_sync(0xffffffffu, ready || s.phase == tr::kPeelScan)) break;
-          if (ready) {
-            deposit(P.models[s.m], s, s.phase == tr::kPeelScat);
-            n_peel += 1u;
-            s.q() = 1;
-            s.phase = tr::kPeelScan;
-          }
-          if (s.phase == tr::kPeelScan) peel_scan(P, s, G, T, n_cross);
-        }
-        if (s.phase == tr::kAfter) after_scattering(P, s, T);
-        const bool wants = !s.walking && s.phase == tr::kFetch;
-        const unsigned fetchers = __ballot_sync(0xffffffffu, wants);
-        if (!fetchers) break;
-        // hand out packets of the warp's chunk, taking new chunks as needed
-        const int rank = __popc(fetchers & lt_mask);
-        int remaining = __popc(fetchers), done = 0;
-        int my_model = -1;
-        unsigned long long my_pid = 0;
-        while (remaining > 0 && !drained) {
-          if (c_next >= c_end) {
-            unsigned long long ci = 0;
-            if (lane == 0) ci = atomicAdd(P.chunk_counter, 1ull);
-            ci = __shfl_sync(0xffffffffu, ci, 0);
-            if (ci >= (unsigned long long)P.n_chunks) {
-              drained = true;
-              break;
-            }
-            const BatchChunk ch = P.chunks[ci];
-            c_model = ch.model;
-            c_next = ch.first;
-            c_end = ch.first + ch.count;
-          }
-          const unsigned long long avail = c_end - c_next;
-          const int take = avail < (unsigned long long)remaining ? (int)avail : remaining;
-          if (wants && rank >= done && rank < done + take) {
-            my_model = c_model;
-            my_pid = c_next + (unsigned long long)(rank - done);
-          }
-          c_next += (unsigned long long)take;
-          done += take;
-          remaining -= take;
-        }
-        if (wants) {
-          if (my_model >= 0) {
-            begin(P, s, G, T, my_model, my_pid);
-            n_packets += 1u;
-          } else {
-            s.phase = tr::kExit;
-          }
-        }
-      }
-      if (s.phase == tr::kStart) {
-        s.phase = s.wphase();
-        start_walk(s, G, s.d);
-      }
-      if (n_cross & 0xC0000000u) {
-        tot_cross += n_cross;
-        n_cross = 0;
-      }
-    }
-    if (s.walking) step(P, s, G, n_cross);
-  }
-  flush(P, T);
-  tot_cross += n_cross;
-  unsigned long long ev = n_events, pe = n_peel, pk = n_packets, cp = T.column_peels, cc = T.column_crossings;
-  for (int o = 16; o > 0; o >>= 1) {
-    cp += __shfl_down_sync(0xffffffffu, cp, o);
-    cc += __shfl_down_sync(0xffffffffu, cc, o);
-    tot_cross += __shfl_down_sync(0xffffffffu, tot_cross, o);
-    ev += __shfl_down_sync(0xffffffffu, ev, o);
-    pe += __shfl_down_sync(0xffffffffu, pe, o);
-    pk += __shfl_down_sync(0xffffffffu, pk, o);
-  }
+  WarpState& ws = state().warp[warp];
   if (lane == 0) {
-    atomicAdd(&P.counters[0], tot_cross);
-    atomicAdd(&P.counters[1], ev);
-    atomicAdd(&P.counters[2], pe);
-    atomicAdd(&P.counters[3], pk);
-    if (cp) {
-      atomicAdd(&P.counters[4], cp);
-      atomicAdd(&P.counters[5], cc);
+    ws.queues = make_uint2((unsigned)kBatchSlots << (8 * tr::kQFetch), 0u);
+    ws.next = ws.end = 0ull;
+    ws.model = ws.drained = 0;
+    ws.crossings = ws.events = ws.peeloffs = ws.packets = ws.column_peels = ws.column_crossings = 0ull;
+  }
+  for (int i = (int)lane; i < kBatchSlots; i += 32) {
+    state().ring[warp][tr::kQFetch][i] = (unsigned char)i;
+    state().pack[(int)warp * kBatchSlots + i] = 0u;
+    state().model[(int)warp * kBatchSlots + i] = 0;
+  }
+  __syncwarp();
+  Tally tally{0.0, 0.0, 0.0, -1};
+  asm volatile("" ::"l"(&tally) : "memory");  // kept in memory, not in registers
+  BWalker s{};
+  s.slot = -1;
+  s.phase = tr::kExit;
+  int wait = 0;  // ended walks the warp waits for before it serves them
+  while (true) {
+    const bool ended = !s.walking && s.slot >= 0;
+    if (__popc(__ballot_sync(0xffffffffu, ended)) >= wait) {
+      const uint2 qs = ws.queues;
+      tr::Queues Q{qs.x, qs.y, state().ring[warp]};
+      {
+        const bool p1 = ended && s.phase == tr::kPath1;
+        const unsigned nc = __reduce_add_sync(0xffffffffu, ended && s.phase != tr::kPath2 ? s.n : 0u);
+        if (ended) {
+          if (s.phase == tr::kPath2) {
+            state().res[s.slot] = make_float2(s.aux0, 0.0f);
+            state().cell[s.slot] = CartGrid::carried(s.w);
+          } else {
+            state().res[s.slot] = make_float2(s.th, s.tl);
+          }
+        }
+        if (lane == 0) ws.crossings += nc;
+        const int local = s.slot - (int)warp * kBatchSlots;
+        Q.push(tr::kQPath1, p1, local, lt_mask);
+        Q.push(tr::kQEvent, ended && !p1, local, lt_mask);
+        if (ended) s.slot = -1;
+        __syncwarp();
+      }
+      const unsigned idle = __ballot_sync(0xffffffffu, !s.walking);
+      const int n_idle = __popc(idle);
+      if (Q.size(tr::kQReady) < n_idle && Q.round_due(n_idle)) {
+        // the walks go to local memory for the rounds (see the forward kernel)
+        BWalker saved = s;
+        asm volatile("" ::"l"(&saved) : "memory");
+        do {
+          control_round(P, Q, ws, tally, Q.fullest(), lane, lt_mask);
+        } while (Q.size(tr::kQReady) < n_idle && Q.round_due(n_idle));
+        asm volatile("" ::"l"(&saved) : "memory");
+        s = saved;
+      }
+      const int n_start = min(n_idle, Q.size(tr::kQReady));
+      const int r = __popc(idle & lt_mask);
+      if (!s.walking && r < n_start) start_walk(P, s, (int)warp * kBatchSlots + Q.at(tr::kQReady, r));
+      Q.drop(tr::kQReady, n_start);
+      __syncwarp();
+      if (lane == 0) ws.queues = make_uint2(Q.count, Q.head);
+      __syncwarp();
+      const int busy = 32 - n_idle + n_start;
+      if (busy == 0) break;
+      wait = max(1, (P.control_min * busy) >> 5);
+    }
+    if (s.walking) step(P, s);
+  }
+  flush(P, tally);
+  if (lane == 0 && ws.packets) {
+    atomicAdd(&P.counters[0], ws.crossings);
+    atomicAdd(&P.counters[1], ws.events);
+    atomicAdd(&P.counters[2], ws.peeloffs);
+    atomicAdd(&P.counters[3], ws.packets);
+    if (ws.column_peels) {
+      atomicAdd(&P.counters[4], ws.column_peels);
+      atomicAdd(&P.counters[5], ws.column_crossings);
     }
   }
 }
@@ -484,12 +583,17 @@ cudaError_t launch_batch_columns(const DevModel* models, int n_models, const flo
 }
 
 cudaError_t launch_batch(const BatchParams& p, unsigned blocks, cudaStream_t stream) {
-  k_batch<<<blocks, kBatchBlock, 0, stream>>>(p);
+  k_batch<<<blocks, kBatchBlock, batch_shared_bytes(), stream>>>(p);
   return cudaGetLastError();
 }
 
+size_t batch_shared_bytes() { return sizeof(BShared); }
+
 cudaError_t batch_blocks_per_sm(int* blocks) {
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, k_batch, kBatchBlock, 0);
+  const cudaError_t e =
+      cudaFuncSetAttribute(k_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)batch_shared_bytes());
+  if (e != cudaSuccess) return e;
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, k_batch, kBatchBlock, batch_shared_bytes());
 }
 
 }  // namespace rtk

@@ -333,6 +333,7 @@ const void* batch_emitted_kernel();
 // k_batch_columns(const DevModel* models, int n_models, const float* density):
 // the column sums of every model whose frame looks along a grid axis.
 const void* batch_columns_kernel();
+size_t batch_shared_bytes();  // dynamic shared memory of the batch kernel (allowed by batch_blocks_per_sm)
 cudaError_t batch_blocks_per_sm(int* blocks);
 cudaError_t launch_batch(const BatchParams& p, unsigned blocks, cudaStream_t stream);
 cudaError_t launch_batch_columns(const DevModel* models, int n_models, const float* density, cudaStream_t stream);
