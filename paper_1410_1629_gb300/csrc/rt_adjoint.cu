@@ -49,7 +49,9 @@ namespace {
 using tr::CartGrid;
 
 constexpr int kAdjBlock = 256;
-// Resident blocks per SM the register allocation aims at.
+// Resident blocks per SM the register allocation aims at (2 / 3 / 4, forward and
+// adjoint: image target 46.1 / 32.1 / 33.1 ms, absorption target 20.5 / 20.3 /
+// 22.2 ms).
 #ifndef RT_ADJ_MIN_BLOCKS
 #define RT_ADJ_MIN_BLOCKS 3
 #endif
@@ -88,17 +90,46 @@ struct AdjParams {
   AdjRecord* tape;                        // the forward launch's tape ([packets][rec_stride]) or null: replay
 };
 
+// Lane state that only the per-event work touches, in per-thread slots of shared
+// memory (structure of arrays), so that the walk's state fits the registers:
+// packet id, wavelength, event index, the walk an aStart lane begins, the next
+// instrument, the last event, weight and its unit exponent, the event's
+// Henyey-Greenstein uniforms, direction of travel, the cell of x (valid when
+// has_cell), the lane's or packet's event records, the weight at the current
+// event from the tape (units 2^eL), kappa rho of the interaction cell.
+__shared__ unsigned long long A_PID[kAdjBlock];
+__shared__ double A_WEIGHT[kAdjBlock];
+__shared__ AdjRecord* A_REC[kAdjBlock];
+__shared__ float3 A_DIR[kAdjBlock];
+__shared__ CartGrid::Cell A_CELL[kAdjBlock];
+__shared__ int A_LAM[kAdjBlock], A_EVENT[kAdjBlock], A_WPHASE[kAdjBlock], A_Q[kAdjBlock], A_LAST[kAdjBlock],
+    A_UNIT[kAdjBlock];
+__shared__ float A_U_MU[kAdjBlock], A_U_PHI[kAdjBlock], A_TAPE_WEIGHT[kAdjBlock], A_HIT[kAdjBlock];
+__shared__ bool A_HAS_CELL[kAdjBlock];
+
 // The lane: one packet.
 struct ALane {
-  unsigned long long pid;
-  int lam, event, phase, wphase, q, J;
-  int eL, eLA;          // 2^eL: unit of weights; 2^eLA: unit of position and tau adjoints
-  double L;             // weight (as in the forward kernel)
+  int phase;
+  bool walking;
+  __device__ __forceinline__ unsigned long long& pid() const { return A_PID[threadIdx.x]; }
+  __device__ __forceinline__ double& L() const { return A_WEIGHT[threadIdx.x]; }
+  __device__ __forceinline__ AdjRecord*& rec() const { return A_REC[threadIdx.x]; }
+  __device__ __forceinline__ float3& k() const { return A_DIR[threadIdx.x]; }
+  __device__ __forceinline__ CartGrid::Cell& cell() const { return A_CELL[threadIdx.x]; }
+  __device__ __forceinline__ int& lam() const { return A_LAM[threadIdx.x]; }
+  __device__ __forceinline__ int& event() const { return A_EVENT[threadIdx.x]; }
+  __device__ __forceinline__ int& wphase() const { return A_WPHASE[threadIdx.x]; }
+  __device__ __forceinline__ int& q() const { return A_Q[threadIdx.x]; }
+  __device__ __forceinline__ int& J() const { return A_LAST[threadIdx.x]; }
+  __device__ __forceinline__ int& eL() const { return A_UNIT[threadIdx.x]; }
+  __device__ __forceinline__ float& u_mu() const { return A_U_MU[threadIdx.x]; }
+  __device__ __forceinline__ float& u_phi() const { return A_U_PHI[threadIdx.x]; }
+  __device__ __forceinline__ float& Lf() const { return A_TAPE_WEIGHT[threadIdx.x]; }
+  __device__ __forceinline__ float& kr_h() const { return A_HIT[threadIdx.x]; }
+  __device__ __forceinline__ bool& has_cell() const { return A_HAS_CELL[threadIdx.x]; }
+  int eLA;              // 2^eLA: unit of position and tau adjoints
   float kappa;
-  float u_mu, u_phi;    // the event's Henyey-Greenstein uniforms
-  float3 x, k;          // position, direction of travel
-  CartGrid::Cell cell;  // cell of x (valid when has_cell)
-  bool has_cell, walking;
+  float3 x;             // position
   float3 d, id;         // the walk's direction and its inverse (0 for a zero component)
   CartGrid::Walk w;
   float rho;            // density of the walk's current cell
@@ -108,13 +139,12 @@ struct ALane {
   int axis_in;          // axis of the plane the current segment was entered by (-1: none)
   int n_cross;          // crossings of the walk so far
   int h;                // path 2: crossing index of the interaction (-1: none); deposits: split index
-  float kr_h;           // path 2: kappa rho of the interaction cell
   float c0, c1;         // depositing walks: coefficient before / from crossing h (units 2^eLA)
-  // absorption adjoint, path 1 (FP64, true units)
-  double P, D, a_prev, e_prev;
+  // absorption adjoint, path 1 (FP64, true units); wd: (1 - albedo) L, adj: the
+  // wavelength's adjoint field
+  double P, D, a_prev, e_prev, wd;
   double3 g0;
-  AdjRecord* rec;
-  float Lf;             // tape: the weight at the current event, units 2^eL
+  const double* adj;
 };
 
 __device__ __forceinline__ void grad_add(double* p, double v) {
@@ -188,20 +218,20 @@ __device__ __forceinline__ float adj_weight(const AdjParams& A, int q, int lam, 
 // Ask for walk `phase` from the lane's position along d; walks start in the
 // last stage of a control round, from one place in the code.
 __device__ __forceinline__ void request_walk(ALane& s, int phase, float3 d) {
-  s.wphase = phase;
+  s.wphase() = phase;
   s.d = d;
   s.phase = aStart;
 }
 
 __device__ __forceinline__ void start_walk(const FwdParams& P, ALane& s) {
-  s.phase = s.wphase;
+  s.phase = s.wphase();
   s.id = make_float3(tr::inv_or_zero(s.d.x), tr::inv_or_zero(s.d.y), tr::inv_or_zero(s.d.z));
   s.th = s.tl = 0.0f;
   s.g = make_float3(0.0f, 0.0f, 0.0f);
   s.axis_in = -1;
   s.n_cross = 0;
   CartGrid::Scratch sc;
-  s.walking = CartGrid::init(P, s.x, s.d, s.id, s.has_cell, s.cell, s.w, sc);
+  s.walking = CartGrid::init(P, s.x, s.d, s.id, s.has_cell(), s.cell(), s.w, sc);
   if (s.walking) s.rho = tr::load_density(&P.density[s.w.cell]);
 }
 
@@ -210,9 +240,11 @@ __device__ __forceinline__ int linear_cell(const FwdParams& P, const CartGrid::C
 }
 
 template <bool kAbs>
-__device__ __forceinline__ void request_path(ALane& s) {
-  request_walk(s, aPath1, s.k);
+__device__ __forceinline__ void request_path(const AdjParams& A, ALane& s) {
+  request_walk(s, aPath1, s.k());
   if (kAbs) {
+    s.wd = (1.0 - A.f.lam[s.lam()].albedo) * s.L();
+    s.adj = A.adj_abs + (size_t)s.lam() * A.f.n_cells;
     s.P = s.D = s.a_prev = 0.0;
     s.e_prev = 1.0;
     s.g0 = make_double3(0.0, 0.0, 0.0);
@@ -221,23 +253,23 @@ __device__ __forceinline__ void request_path(ALane& s) {
 
 // ---- the stages of a control round (each for the lanes in that phase)
 
-// Tape: the lane's position, cell and weight at event s.event (records
+// Tape: the lane's position, cell and weight at event s.event() (records
 // event+1 for events before the last, record 0 for the last), and the
-// direction of travel into it (that of path s.event, for the phase function).
+// direction of travel into it (that of path s.event(), for the phase function).
 __device__ __forceinline__ void tape_event(const AdjParams& A, ALane& s) {
-  const AdjRecord& r = s.rec[s.event < s.J ? s.event + 1 : 0];
+  const AdjRecord& r = s.rec()[s.event() < s.J() ? s.event() + 1 : 0];
   s.x = make_float3(r.x[0], r.x[1], r.x[2]);
-  s.Lf = r.L;
-  s.has_cell = r.cell >= 0;
-  if (s.has_cell) {
+  s.Lf() = r.L;
+  s.has_cell() = r.cell >= 0;
+  if (s.has_cell()) {
     const FwdParams& P = A.f;
-    s.cell.ix = r.cell % P.nx;
-    s.cell.iy = (r.cell / P.nx) % P.ny;
-    s.cell.iz = r.cell / (P.nx * P.ny);
+    s.cell().ix = r.cell % P.nx;
+    s.cell().iy = (r.cell / P.nx) % P.ny;
+    s.cell().iz = r.cell / (P.nx * P.ny);
   }
-  if (s.event > 0) {
-    AdjRecord& pj = s.rec[s.event];
-    s.k = make_float3(pj.k[0], pj.k[1], pj.k[2]);
+  if (s.event() > 0) {
+    AdjRecord& pj = s.rec()[s.event()];
+    s.k() = make_float3(pj.k[0], pj.k[1], pj.k[2]);
     pj.dLb = 0.0f;  // the peel-offs at this event accumulate here
     pj.dxb[0] = pj.dxb[1] = pj.dxb[2] = 0.0f;
   }
@@ -250,24 +282,24 @@ __device__ __forceinline__ void fetch(const AdjParams& A, ALane& s, unsigned lon
   int lam = min((int)(__ull2float_rz(w) * P.inv_n_per_lambda), P.n_lambda - 1);
   while (lam > 0 && (unsigned long long)lam * P.n_per_lambda > w) --lam;
   while (lam + 1 < P.n_lambda && (unsigned long long)(lam + 1) * P.n_per_lambda <= w) ++lam;
-  s.lam = lam;
-  s.pid = P.first_id + (w - (unsigned long long)lam * P.n_per_lambda);
+  s.lam() = lam;
+  s.pid() = P.first_id + (w - (unsigned long long)lam * P.n_per_lambda);
   s.kappa = A.f.lam[lam].kappa;
-  s.L = P.L0[lam];
-  s.eL = A.e0[lam];
-  s.eLA = s.eL + adjoint_exponent(*A.maxbits);
-  s.event = 0;
-  s.J = 0;
-  s.has_cell = false;
-  s.q = 0;
+  s.L() = P.L0[lam];
+  s.eL() = A.e0[lam];
+  s.eLA = s.eL() + adjoint_exponent(*A.maxbits);
+  s.event() = 0;
+  s.J() = 0;
+  s.has_cell() = false;
+  s.q() = 0;
   s.phase = aPeelScan;
   if constexpr (kTape) {
     // the forward launch recorded this packet's events: no replay
-    s.rec = A.tape + (size_t)w * (size_t)A.rec_stride;
-    s.J = s.rec[0].h;
+    s.rec() = A.tape + (size_t)w * (size_t)A.rec_stride;
+    s.J() = s.rec()[0].h;
     tape_event(A, s);
   } else {
-    tr::emit(P, s.pid, s.lam, s.x, s.k);
+    tr::emit(P, s.pid(), s.lam(), s.x, s.k());
   }
 }
 
@@ -277,38 +309,38 @@ template <bool kAbs>
 __device__ __forceinline__ void finish_path1(const AdjParams& A, ALane& s) {
   const FwdParams& P = A.f;
   const double tau = widen(s.th) + widen(s.tl);
-  if (!(tau > 0.0)) {  // escapes: there is no event s.event
-    s.J = s.event - 1;
+  if (!(tau > 0.0)) {  // escapes: there is no event s.event()
+    s.J() = s.event() - 1;
     s.phase = aSweep;
     return;
   }
-  const double albedo = A.f.lam[s.lam].albedo;
+  const double albedo = A.f.lam[s.lam()].albedo;
   const double omE = one_minus_exp(tau);
-  const uint4 rn = draw_block(s.pid, s.lam, s.event, 0, P.seed, P.model);
+  const uint4 rn = draw_block(s.pid(), s.lam(), s.event(), 0, P.seed, P.model);
   const double u = u01(rn.x);
   const double tau_star = neg_log_one_minus(u * omE);
-  s.u_mu = tr::u01f(rn.y);
-  s.u_phi = tr::u01f(rn.z);
-  AdjRecord& r = s.rec[s.event];
+  s.u_mu() = tr::u01f(rn.y);
+  s.u_phi() = tr::u01f(rn.z);
+  AdjRecord& r = s.rec()[s.event()];
   r.x[0] = s.x.x; r.x[1] = s.x.y; r.x[2] = s.x.z;
-  r.k[0] = s.k.x; r.k[1] = s.k.y; r.k[2] = s.k.z;
-  r.cell = s.has_cell ? linear_cell(P, s.cell) : -1;
-  r.L = narrow(s.L, s.eL);
+  r.k[0] = s.k().x; r.k[1] = s.k().y; r.k[2] = s.k().z;
+  r.cell = s.has_cell() ? linear_cell(P, s.cell()) : -1;
+  r.L = narrow(s.L(), s.eL());
   r.omE = (float)omE;
   r.E = (float)(1.0 - omE);
   r.u = tr::u01f(rn.x);
   r.g1[0] = s.g.x; r.g1[1] = s.g.y; r.g1[2] = s.g.z;
   if (kAbs) {
-    const double wd = (1.0 - albedo) * s.L;
-    const int ea = s.eLA - s.eL;
+    const double wd = (1.0 - albedo) * s.L();
+    const int ea = s.eLA - s.eL();
     r.Tdep = narrow(s.P + wd * s.e_prev * s.a_prev, s.eLA);  // the last index: a_n = 0
     r.D = narrow(s.D, ea);
     r.g0[0] = narrow(s.g0.x, s.eLA); r.g0[1] = narrow(s.g0.y, s.eLA); r.g0[2] = narrow(s.g0.z, s.eLA);
   }
-  s.L = albedo * s.L * omE;  // weight after the scattering
+  s.L() = albedo * s.L() * omE;  // weight after the scattering
   tr::split_pair(tau_star, s.a0, s.a1);  // as the forward kernel
   s.h = -1;
-  request_walk(s, aPath2, s.k);
+  request_walk(s, aPath2, s.k());
 }
 
 // Path 2 ended at the interaction: record it, move the packet, then the
@@ -317,27 +349,27 @@ __device__ __forceinline__ void finish_path2(const AdjParams& A, ALane& s) {
   const FwdParams& P = A.f;
   if (s.h < 0) {  // not reachable: identical pair sums in both walks and tau* < tau_path
     atomicOr(P.flags, kFlagNoInteraction);
-    s.J = s.event - 1;
+    s.J() = s.event() - 1;
     s.phase = aSweep;
     return;
   }
-  AdjRecord& r = s.rec[s.event];
+  AdjRecord& r = s.rec()[s.event()];
   r.h = s.h;
   r.hit_axis = s.axis_in;
   r.hit_cell = s.w.cell;
-  r.kr_h = s.kr_h;
+  r.kr_h = s.kr_h();
   r.rem = s.a1;
   // segments h.. with the entry of h counted: all segments minus those before h
   r.gp[0] = s.g.x; r.gp[1] = s.g.y; r.gp[2] = s.g.z;
   r.dLb = 0.0f;
   r.dxb[0] = r.dxb[1] = r.dxb[2] = 0.0f;
   const float s_star = s.a0;
-  float3 x = make_float3(fmaf(s_star, s.k.x, s.x.x), fmaf(s_star, s.k.y, s.x.y), fmaf(s_star, s.k.z, s.x.z));
-  s.cell = CartGrid::carried(s.w);
-  CartGrid::clamp(P, s.cell, x);
+  float3 x = make_float3(fmaf(s_star, s.k().x, s.x.x), fmaf(s_star, s.k().y, s.x.y), fmaf(s_star, s.k().z, s.x.z));
+  s.cell() = CartGrid::carried(s.w);
+  CartGrid::clamp(P, s.cell(), x);
   s.x = x;
-  s.has_cell = true;
-  s.q = 0;
+  s.has_cell() = true;
+  s.q() = 0;
   s.phase = aPeelScan;
 }
 
@@ -346,12 +378,12 @@ __device__ __forceinline__ void finish_path2(const AdjParams& A, ALane& s) {
 // xb); returns l (units 2^eLA).
 __device__ __forceinline__ float peel_values(const AdjParams& A, ALane& s, const DevInstr& I, float W, float3 dW) {
   float phase = 1.0f;
-  if (s.event > 0) phase = hg_phase(A.f.lam[s.lam].g, s.k.x * I.kobs[0] + s.k.y * I.kobs[1] + s.k.z * I.kobs[2]);
+  if (s.event() > 0) phase = hg_phase(A.f.lam[s.lam()].g, s.k().x * I.kobs[0] + s.k().y * I.kobs[1] + s.k().z * I.kobs[2]);
   const float pe = kInv4PiF * phase * expf(-s.th) * (1.0f - s.tl);
-  const float V = (A.tape ? s.Lf : narrow(s.L, s.eL)) * pe;  // units 2^eL
+  const float V = (A.tape ? s.Lf() : narrow(s.L(), s.eL())) * pe;  // units 2^eL
   const float l = V * W;                   // units 2^eLA
-  if (s.event > 0) {
-    AdjRecord& r = s.rec[s.event];
+  if (s.event() > 0) {
+    AdjRecord& r = s.rec()[s.event()];
     r.dLb += pe * W;
     r.dxb[0] += V * dW.x + l * s.g.x * s.id.x;
     r.dxb[1] += V * dW.y + l * s.g.y * s.id.y;
@@ -363,9 +395,9 @@ __device__ __forceinline__ float peel_values(const AdjParams& A, ALane& s, const
 // A peel-off measuring walk ended: its values, then the depositing walk or
 // the next peel-off.
 __device__ __forceinline__ void finish_peel_measure(const AdjParams& A, ALane& s) {
-  const DevInstr& I = A.f.instr[s.q];
+  const DevInstr& I = A.f.instr[s.q()];
   float3 dW;
-  const float W = adj_weight(A, s.q, s.lam, s.event > 0, s.x, dW);
+  const float W = adj_weight(A, s.q(), s.lam(), s.event() > 0, s.x, dW);
   const float l = peel_values(A, s, I, W, dW);
   if (l != 0.0f && s.n_cross > 0) {
     s.c0 = s.c1 = -l * s.kappa;
@@ -373,7 +405,7 @@ __device__ __forceinline__ void finish_peel_measure(const AdjParams& A, ALane& s
     request_walk(s, aPeelD, s.d);
     return;
   }
-  s.q += 1;
+  s.q() += 1;
   s.phase = aPeelScan;
 }
 
@@ -387,8 +419,8 @@ __device__ __forceinline__ bool column_peel(const AdjParams& A, ALane& s, const 
                                             unsigned& n_cross, unsigned& n_dep) {
   const FwdParams& P = A.f;
   CartGrid::Cell c;
-  if (s.has_cell) {
-    c = s.cell;
+  if (s.has_cell()) {
+    c = s.cell();
   } else {
     if (!inside_box(P, s.x)) return false;
     c.ix = min(max(__float2int_rd((s.x.x - P.lo[0]) * P.inv_d[0]), 0), P.nx - 1);
@@ -422,17 +454,17 @@ __device__ __forceinline__ bool column_peel(const AdjParams& A, ALane& s, const 
   return true;
 }
 
-// The next instrument from s.q whose adjoint weight at the lane's position
+// The next instrument from s.q() whose adjoint weight at the lane's position
 // is not zero: its peel-off walk (frames along grid axes are done here
 // without walks); after the last one, aAfter.
 __device__ __forceinline__ void peel_scan(const AdjParams& A, ALane& s, unsigned& n_cross, unsigned& n_dep) {
   const FwdParams& P = A.f;
-  const bool on = s.event == 0 ? P.peel_emission : P.peel_scatter;
-  for (; on && s.q < P.n_instr; ++s.q) {
+  const bool on = s.event() == 0 ? P.peel_emission : P.peel_scatter;
+  for (; on && s.q() < P.n_instr; ++s.q()) {
     float3 dW;
-    const float W = adj_weight(A, s.q, s.lam, s.event > 0, s.x, dW);
+    const float W = adj_weight(A, s.q(), s.lam(), s.event() > 0, s.x, dW);
     if (W == 0.0f && dW.x == 0.0f && dW.y == 0.0f && dW.z == 0.0f) continue;  // contributes nothing
-    const DevInstr& I = A.f.instr[s.q];
+    const DevInstr& I = A.f.instr[s.q()];
     if (P.use_columns && I.column && column_peel(A, s, I, W, dW, n_cross, n_dep)) continue;
     request_walk(s, aPeelM, tr::instr_dir(I));
     return;
@@ -440,15 +472,15 @@ __device__ __forceinline__ void peel_scan(const AdjParams& A, ALane& s, unsigned
   s.phase = aAfter;
 }
 
-// After the peel-offs of event s.event: the first forced path, or the new
+// After the peel-offs of event s.event(): the first forced path, or the new
 // direction and then termination (the sweep) or the next forced path.
 template <bool kAbs, bool kTape>
 __device__ __forceinline__ void after_peels(const AdjParams& A, ALane& s) {
   const FwdParams& P = A.f;
   if constexpr (kTape) {  // the next recorded event, or the sweep
-    if (s.event < s.J) {
-      s.event += 1;
-      s.q = 0;
+    if (s.event() < s.J()) {
+      s.event() += 1;
+      s.q() = 0;
       tape_event(A, s);
       s.phase = aPeelScan;
     } else {
@@ -456,22 +488,22 @@ __device__ __forceinline__ void after_peels(const AdjParams& A, ALane& s) {
     }
     return;
   }
-  if (s.event == 0) {
-    s.event = 1;
-    request_path<kAbs>(s);
+  if (s.event() == 0) {
+    s.event() = 1;
+    request_path<kAbs>(A, s);
     return;
   }
-  const float mu = hg_sample(A.f.lam[s.lam].g, s.u_mu);
+  const float mu = hg_sample(A.f.lam[s.lam()].g, s.u_mu());
   float sp, cp;
-  sincospif(2.0f * s.u_phi, &sp, &cp);
-  s.k = rotate_dir(s.k, mu, sp, cp);
-  if ((P.weight_cut && bits_of(s.L) < bits_of(P.L_cut[s.lam])) || s.event >= P.max_events) {
-    s.J = s.event;
+  sincospif(2.0f * s.u_phi(), &sp, &cp);
+  s.k() = rotate_dir(s.k(), mu, sp, cp);
+  if ((P.weight_cut && bits_of(s.L()) < bits_of(P.L_cut[s.lam()])) || s.event() >= P.max_events) {
+    s.J() = s.event();
     s.phase = aSweep;
     return;
   }
-  s.event += 1;
-  request_path<kAbs>(s);
+  s.event() += 1;
+  request_path<kAbs>(A, s);
 }
 
 // Backward sweep over the packet's events J..1 (no walks): per forced path
@@ -480,10 +512,10 @@ __device__ __forceinline__ void after_peels(const AdjParams& A, ALane& s) {
 // adjoints of the path's start weight and position.
 template <bool kAbs>
 __device__ __forceinline__ void sweep(const AdjParams& A, ALane& s) {
-  const float albedo = (float)A.f.lam[s.lam].albedo;
+  const float albedo = (float)A.f.lam[s.lam()].albedo;
   float Lb = 0.0f, xb0 = 0.0f, xb1 = 0.0f, xb2 = 0.0f;
-  for (int j = s.J; j >= 1; --j) {
-    AdjRecord& r = s.rec[j];
+  for (int j = s.J(); j >= 1; --j) {
+    AdjRecord& r = s.rec()[j];
     Lb += r.dLb;
     xb0 += r.dxb[0]; xb1 += r.dxb[1]; xb2 += r.dxb[2];
     const float k0 = r.k[0], k1 = r.k[1], k2 = r.k[2];
@@ -514,26 +546,26 @@ __device__ __forceinline__ void sweep(const AdjParams& A, ALane& s) {
     r.T = T;
     r.tbh = tbh;
   }
-  s.event = 1;
+  s.event() = 1;
   s.phase = aDepScan;
 }
 
-// The depositing walk of forced path s.event or of a later one; after the
+// The depositing walk of forced path s.event() or of a later one; after the
 // last, the lane needs a new packet.
 __device__ __forceinline__ void dep_scan(const AdjParams& A, ALane& s) {
   const FwdParams& P = A.f;
-  for (; s.event <= s.J; ++s.event) {
-    const AdjRecord& r = s.rec[s.event];
+  for (; s.event() <= s.J(); ++s.event()) {
+    const AdjRecord& r = s.rec()[s.event()];
     s.c0 = s.kappa * r.T;
     s.c1 = s.kappa * (r.T - r.tbh);
     if (s.c0 == 0.0f && s.c1 == 0.0f) continue;
     s.h = r.h;
     s.x = make_float3(r.x[0], r.x[1], r.x[2]);
-    s.has_cell = r.cell >= 0;
-    if (s.has_cell) {
-      s.cell.ix = r.cell % P.nx;
-      s.cell.iy = (r.cell / P.nx) % P.ny;
-      s.cell.iz = r.cell / (P.nx * P.ny);
+    s.has_cell() = r.cell >= 0;
+    if (s.has_cell()) {
+      s.cell().ix = r.cell % P.nx;
+      s.cell().iy = (r.cell / P.nx) % P.ny;
+      s.cell().iz = r.cell / (P.nx * P.ny);
     }
     request_walk(s, aDep, make_float3(r.k[0], r.k[1], r.k[2]));
     return;
@@ -561,7 +593,7 @@ __device__ __forceinline__ void step(const AdjParams& A, ALane& s, unsigned& n_c
     const float rem = ((s.a0 - s.th) + s.a1) - s.tl;
     s.a0 = w.t + rem / kr;
     s.a1 = rem;
-    s.kr_h = kr;
+    s.kr_h() = kr;
     s.h = s.n_cross;
     s.walking = false;
     return;
@@ -577,16 +609,26 @@ __device__ __forceinline__ void step(const AdjParams& A, ALane& s, unsigned& n_c
   }
   if (kAbs && s.phase == aPath1) {
     // deposits (1 - albedo) L (e_{m-1} - e_m) with adjoints a_m: P is the
-    // prefix of the optical-depth adjoints wd e_i (a_i - a_{i+1}), i < m
-    const double a = dt > 0.0f ? A.adj_abs[(size_t)s.lam * P.n_cells + cell] : 0.0;
-    const double e_cur = (double)(expf(-nh) * (1.0f - nl));
-    const double wd = (1.0 - A.f.lam[s.lam].albedo) * s.L;
-    if (s.n_cross > 0) s.P += wd * s.e_prev * (s.a_prev - a);
-    if (s.P != 0.0) grad_add(&A.grad[cell], -(double)(s.kappa * ds) * s.P);
-    const double c = (double)kr * s.P;
-    s.g0.x += (axis == 0 ? c : 0.0) - (s.axis_in == 0 ? c : 0.0);
-    s.g0.y += (axis == 1 ? c : 0.0) - (s.axis_in == 1 ? c : 0.0);
-    s.g0.z += (axis == 2 ? c : 0.0) - (s.axis_in == 2 ? c : 0.0);
+    // prefix of the optical-depth adjoints wd e_i (a_i - a_{i+1}), i < m.  Eleven
+    // FP64 operations per crossing: conversions by integer operations, and of
+    // the three plane sums only the exit and entry planes' change
+    const double a = dt > 0.0f ? s.adj[cell] : 0.0;
+    const double e_cur = widen(expf(-nh) * (1.0f - nl));
+    if (s.n_cross > 0) s.P += s.wd * s.e_prev * (s.a_prev - a);
+    if (s.P != 0.0) {
+      grad_add(&A.grad[cell], -widen(s.kappa * ds) * s.P);
+      const double c = widen(kr) * s.P;
+      if (axis != s.axis_in) {
+        const double out = (axis == 0 ? s.g0.x : (axis == 1 ? s.g0.y : s.g0.z)) + c;
+        s.g0.x = axis == 0 ? out : s.g0.x;
+        s.g0.y = axis == 1 ? out : s.g0.y;
+        s.g0.z = axis == 2 ? out : s.g0.z;
+        const double in = (s.axis_in == 0 ? s.g0.x : (s.axis_in == 1 ? s.g0.y : s.g0.z)) - c;
+        s.g0.x = s.axis_in == 0 ? in : s.g0.x;
+        s.g0.y = s.axis_in == 1 ? in : s.g0.y;
+        s.g0.z = s.axis_in == 2 ? in : s.g0.z;
+      }
+    }
     s.D += a * (s.e_prev - e_cur);
     s.e_prev = e_cur;
     s.a_prev = a;
@@ -609,10 +651,10 @@ __global__ void __launch_bounds__(kAdjBlock, RT_ADJ_MIN_BLOCKS) k_adjoint(const 
   const FwdParams& P = A.f;
   const unsigned lane = threadIdx.x & 31u;
   const unsigned lt_mask = (1u << lane) - 1u;
-  ALane s;
+  ALane s{};
   s.phase = aFetch;
   s.walking = false;
-  s.rec = A.recs + ((size_t)blockIdx.x * kAdjBlock + threadIdx.x) * (size_t)A.rec_stride;
+  s.rec() = A.recs + ((size_t)blockIdx.x * kAdjBlock + threadIdx.x) * (size_t)A.rec_stride;
   unsigned n_cross = 0, n_dep = 0;
   unsigned long long tot_cross = 0, tot_dep = 0;
   while (true) {
@@ -629,8 +671,8 @@ __global__ void __launch_bounds__(kAdjBlock, RT_ADJ_MIN_BLOCKS) k_adjoint(const 
           if (s.phase == aPath2) finish_path2(A, s);
         }
         if (s.phase == aPeelM) finish_peel_measure(A, s);
-        if (s.phase == aPeelD) { s.q += 1; s.phase = aPeelScan; }
-        if (s.phase == aDep) { s.event += 1; s.phase = aDepScan; }
+        if (s.phase == aPeelD) { s.q() += 1; s.phase = aPeelScan; }
+        if (s.phase == aDep) { s.event() += 1; s.phase = aDepScan; }
       }
       // new packets, their peel-offs, scatterings, sweeps and deposit scans,
       // repeated while a lane has just finished its packet (at most two passes)
@@ -647,7 +689,7 @@ __global__ void __launch_bounds__(kAdjBlock, RT_ADJ_MIN_BLOCKS) k_adjoint(const 
         if (s.phase == aPeelScan) peel_scan(A, s, n_cross, n_dep);
         if (s.phase == aAfter) after_peels<kAbs, kTape>(A, s);
         if (s.phase == aSweep) {
-          if (s.J >= 1) sweep<kAbs>(A, s); else s.phase = aFetch;
+          if (s.J() >= 1) sweep<kAbs>(A, s); else s.phase = aFetch;
         }
         if (s.phase == aDepScan) dep_scan(A, s);
         // a fetched lane never returns to aFetch within the round
