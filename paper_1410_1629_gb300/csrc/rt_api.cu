@@ -414,6 +414,16 @@ rt_status upload_tables(rt_ctx c, cudaStream_t s) {
       I.dir = dir;
     }
   }
+  // instruments that share walks: no column sums, the same direction
+  for (size_t q = 0; q < ins.size(); ++q) {
+    ins[q].leader = -1;
+    for (size_t p = 0; p < q && !ins[q].column; ++p) {
+      if (ins[p].column || ins[p].leader >= 0 || std::memcmp(ins[p].kobs, ins[q].kobs, sizeof ins[q].kobs) != 0) continue;
+      ins[q].leader = (int)p;
+      ins[p].followers |= 1u << q;
+      break;
+    }
+  }
   for (int k = 0; k < 6; ++k) c->columns_used[k] = false;
   c->n_walked_frames = 0;
   for (const DevInstr& I : ins) {

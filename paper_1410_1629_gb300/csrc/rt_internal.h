@@ -50,6 +50,11 @@ struct DevInstr {
   // boundary, sum of rho d_axis over the cells beyond c (or null: walk)
   const float* column;
   int axis, dir;
+  // instruments without column sums that look along the same direction (a frame
+  // and an SED of one view) share the walks of the sorted pass: the first of
+  // them (or -1), and for that one the others as bits
+  int leader;
+  unsigned followers;
 };
 
 struct AdjRecord;

@@ -143,6 +143,18 @@ __global__ void __launch_bounds__(256) k_peel_scatter(const PeelRecord* __restri
   }
 }
 
+// A warp's crossings and the peel-offs that shared another's record.
+__device__ __forceinline__ void add_counts(const FwdParams& P, unsigned long long crossings, unsigned long long shared) {
+  for (int o = 16; o > 0; o >>= 1) {
+    crossings += __shfl_down_sync(0xffffffffu, crossings, o);
+    shared += __shfl_down_sync(0xffffffffu, shared, o);
+  }
+  if ((threadIdx.x & 31u) == 0) {
+    if (crossings) atomicAdd(&P.counters[0], crossings);
+    if (shared) atomicAdd(&P.counters[8], shared);
+  }
+}
+
 // The walks of the sorted records and their deposits; one record per thread,
 // consecutive threads on consecutive records of the order.
 template <class G>
@@ -154,7 +166,7 @@ __global__ void __launch_bounds__(tr::kBlock, kPeelBlocks<G>) k_peel_sorted(cons
   const unsigned long long n = min(*P.peel_count, P.peel_cap);
   if (blockIdx.x == 0 && threadIdx.x == 0 && n) atomicAdd(&P.counters[8], n);
   const unsigned stride_k = (unsigned)(P.n_cells + 1);
-  unsigned long long crossings = 0;
+  unsigned long long crossings = 0, shared = 0;
   for (unsigned long long j = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; j < n;
        j += (unsigned long long)gridDim.x * blockDim.x) {
     const unsigned i = perm[j];
@@ -173,16 +185,23 @@ __global__ void __launch_bounds__(tr::kBlock, kPeelBlocks<G>) k_peel_sorted(cons
     ray.x = make_float3(a.x, a.y, a.z);
     ray.d = tr::instr_dir(P.instr[q]);
     ray.kappa = P.lam[lam].kappa;
+    unsigned steps = 0;
     if (tr::ray_start<G>(P, ray, known, cell, sc)) {
       do {
-        ++crossings;
+        ++steps;
       } while (tr::ray_step<G>(P, ray, sc));
     }
     const ulonglong2 tag = P.peel_tag ? P.peel_tag[i] : make_ulonglong2(0ull, 0ull);
     tr::deposit_peel(P, q, lam, ray.x, L, b.z, ray.th, ray.tl, (meta >> 30) & 1u, tag.x, (int)tag.y);
+    // the instruments that share the record, one crossing and one peel-off each
+    crossings += steps;
+    for (unsigned m = P.instr[q].followers; m; m &= m - 1u) {
+      tr::deposit_peel(P, __ffs(m) - 1, lam, ray.x, L, b.z, ray.th, ray.tl, (meta >> 30) & 1u, tag.x, (int)tag.y);
+      crossings += steps;
+      ++shared;
+    }
   }
-  for (int o = 16; o > 0; o >>= 1) crossings += __shfl_down_sync(0xffffffffu, crossings, o);
-  if ((threadIdx.x & 31u) == 0 && crossings) atomicAdd(&P.counters[0], crossings);
+  add_counts(P, crossings, shared);
 }
 
 // Consecutive records that one warp walks, and the ended rays for which it stops
@@ -208,8 +227,8 @@ __global__ void __launch_bounds__(tr::kBlock, kPeelBlocks<G>) k_peel_together(co
   const unsigned stride_k = (unsigned)(P.n_cells + 1);
   const unsigned lt_mask = (1u << (threadIdx.x & 31u)) - 1u;
   const unsigned long long n_warps = (unsigned long long)gridDim.x * (blockDim.x >> 5);
-  unsigned crossings = 0;
-  unsigned long long total = 0;
+  unsigned crossings = 0;  // of the lane's ray
+  unsigned long long total = 0, shared = 0;
   for (unsigned long long seg = blockIdx.x * (unsigned long long)(blockDim.x >> 5) + (threadIdx.x >> 5);
        seg * kSegment < n; seg += n_warps) {
     unsigned long long next = seg * kSegment;
@@ -226,9 +245,15 @@ __global__ void __launch_bounds__(tr::kBlock, kPeelBlocks<G>) k_peel_together(co
           const float4 a = r[0], b = r[1];
           const unsigned meta = __float_as_uint(b.w);
           const ulonglong2 tag = P.peel_tag ? P.peel_tag[rec] : make_ulonglong2(0ull, 0ull);
-          tr::deposit_peel(P, (int)(__float_as_uint(a.w) / stride_k), (int)(meta & 0xffffu),
-                           make_float3(a.x, a.y, a.z), __hiloint2double(__float_as_int(b.y), __float_as_int(b.x)), b.z,
-                           ray.th, ray.tl, (meta >> 30) & 1u, tag.x, (int)tag.y);
+          const int q = (int)(__float_as_uint(a.w) / stride_k);
+          unsigned m = P.instr[q].followers | 1u << q;
+          shared += (unsigned)__popc(m) - 1u;
+          total += (unsigned long long)crossings * (unsigned)__popc(m);
+          crossings = 0;
+          for (; m; m &= m - 1u)
+            tr::deposit_peel(P, __ffs(m) - 1, (int)(meta & 0xffffu), make_float3(a.x, a.y, a.z),
+                             __hiloint2double(__float_as_int(b.y), __float_as_int(b.x)), b.z, ray.th, ray.tl,
+                             (meta >> 30) & 1u, tag.x, (int)tag.y);
           held = false;
         }
         const unsigned long long j = next + __popc(idle & lt_mask);
@@ -258,11 +283,8 @@ __global__ void __launch_bounds__(tr::kBlock, kPeelBlocks<G>) k_peel_together(co
         crossings += 1u;
       }
     }
-    total += crossings;
-    crossings = 0;
   }
-  for (int o = 16; o > 0; o >>= 1) total += __shfl_down_sync(0xffffffffu, total, o);
-  if ((threadIdx.x & 31u) == 0 && total) atomicAdd(&P.counters[0], total);
+  add_counts(P, total, shared);
 }
 
 template <class G>

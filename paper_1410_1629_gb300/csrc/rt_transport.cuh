@@ -1105,7 +1105,7 @@ struct Shared {
 
 // The small fields of a slot in one word: phase (4 bits), wavelength (6),
 // instrument of the next peel-off (5), has-cell (1), exponent of the deposit
-// weight (16, signed).
+// weight or the deferred peel-offs (16).
 struct Pack {
   __device__ static __forceinline__ unsigned make(int phase, int lam, int q, bool has_cell, int e) {
     return (unsigned)phase | ((unsigned)lam << 4) | ((unsigned)q << 10) | (has_cell ? 1u << 15 : 0u) |
@@ -1163,7 +1163,8 @@ struct Task {
   int phase, wphase; // kStart: the walk to start
   int lam, q, event;
   bool has_cell;
-  int dep_exp;
+  int dep_exp;       // exponent of the deposit weight; peel-off walks: `deferred`
+  unsigned deferred; // instruments whose peel-off of this event is a record of the sorted pass
   int place;         // of the position's cell in the sorted pass's order, once asked for (else -1)
   float th, tl;      // optical depth of the walk that ended (path 2: th = s*)
   unsigned n_peel, n_col, c_col;  // peel-offs, of which by column sums, and their crossings
@@ -1662,11 +1663,21 @@ __device__ __forceinline__ void peel_off(const FwdParams& P, Task<G, kTape>& s, 
       return;
     }
   }
-  if (P.peel && defer_peel(P, s, q, emission)) {
-    s.n_peel += 1u;  // walked and deposited by the sorted pass
-    return;
+  if (P.peel) {
+    // walked and deposited by the sorted pass, along with another's when that is
+    // a record
+    if (I.leader >= 0 && (s.deferred >> I.leader & 1u)) {
+      s.n_peel += 1u;
+      return;
+    }
+    if (defer_peel(P, s, q, emission)) {
+      s.deferred |= 1u << q;
+      s.n_peel += 1u;
+      return;
+    }
   }
   s.q = q;
+  s.dep_exp = (int)s.deferred;
   request_walk(s, emission ? kPeelEmit : kPeelScat);
 }
 
@@ -1757,6 +1768,7 @@ __device__ __forceinline__ int control_round(const FwdParams& P, Queues& Q, Lane
   s.q = Pack::q(pk);
   s.has_cell = Pack::has_cell(pk);
   s.dep_exp = 0;
+  s.deferred = cls == kQEvent && s.phase != kPath2 ? (unsigned)Pack::exponent(pk) & 0xffffu : 0u;
   s.place = -1;
   s.event = sh.event[s.i];
   const float2 res = sh.res[s.i];
