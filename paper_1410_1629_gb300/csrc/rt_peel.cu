@@ -23,6 +23,12 @@ namespace {
 // 50.0 ms, Voronoi disk 52.8 -> 38.3 ms per 1.5e6; 16, 10 and 14 lanes active
 // per instruction of the sorted walks against 9, 7 and 6 in place.  Bound by
 // instruction issue (63-68 % of cycles), trees in the descent to the next leaf.
+//
+// Instruments that look along the same direction (a frame and an SED of one
+// view) see the same optical depth and phase-function value: one record and one
+// walk serve all of them, and only the deposits differ.  Panchromatic disk
+// (frame and SED; the whole calculation) 10.3 -> 8.8 ms, ragged disk 2.53 ->
+// 2.44 ms.
 
 // Resident blocks per SM that the walks' register allocation aims at (disk
 // galaxy and panchromatic disk flat between 4 and 6; octree 3 / 4 / 5: 31.7 /
@@ -143,8 +149,14 @@ __global__ void __launch_bounds__(256) k_peel_scatter(const PeelRecord* __restri
   }
 }
 
-// A warp's crossings and the peel-offs that shared another's record.
-__device__ __forceinline__ void add_counts(const FwdParams& P, unsigned long long crossings, unsigned long long shared) {
+// A lane's crossings and the peel-offs that shared another's record, kept in
+// local memory: touched once per ray.
+struct Counts {
+  unsigned long long crossings, shared;
+};
+
+__device__ __forceinline__ void add_counts(const FwdParams& P, const Counts& sum) {
+  unsigned long long crossings = sum.crossings, shared = sum.shared;
   for (int o = 16; o > 0; o >>= 1) {
     crossings += __shfl_down_sync(0xffffffffu, crossings, o);
     shared += __shfl_down_sync(0xffffffffu, shared, o);
@@ -166,7 +178,8 @@ __global__ void __launch_bounds__(tr::kBlock, kPeelBlocks<G>) k_peel_sorted(cons
   const unsigned long long n = min(*P.peel_count, P.peel_cap);
   if (blockIdx.x == 0 && threadIdx.x == 0 && n) atomicAdd(&P.counters[8], n);
   const unsigned stride_k = (unsigned)(P.n_cells + 1);
-  unsigned long long crossings = 0, shared = 0;
+  Counts sum{0ull, 0ull};
+  asm volatile("" ::"l"(&sum) : "memory");
   for (unsigned long long j = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; j < n;
        j += (unsigned long long)gridDim.x * blockDim.x) {
     const unsigned i = perm[j];
@@ -194,14 +207,14 @@ __global__ void __launch_bounds__(tr::kBlock, kPeelBlocks<G>) k_peel_sorted(cons
     const ulonglong2 tag = P.peel_tag ? P.peel_tag[i] : make_ulonglong2(0ull, 0ull);
     tr::deposit_peel(P, q, lam, ray.x, L, b.z, ray.th, ray.tl, (meta >> 30) & 1u, tag.x, (int)tag.y);
     // the instruments that share the record, one crossing and one peel-off each
-    crossings += steps;
+    sum.crossings += steps;
     for (unsigned m = P.instr[q].followers; m; m &= m - 1u) {
       tr::deposit_peel(P, __ffs(m) - 1, lam, ray.x, L, b.z, ray.th, ray.tl, (meta >> 30) & 1u, tag.x, (int)tag.y);
-      crossings += steps;
-      ++shared;
+      sum.crossings += steps;
+      sum.shared += 1ull;
     }
   }
-  add_counts(P, crossings, shared);
+  add_counts(P, sum);
 }
 
 // Consecutive records that one warp walks, and the ended rays for which it stops
@@ -216,7 +229,12 @@ constexpr int kSegment = 256, kRefill = 24;
 // crossing: in k_peel_sorted the lanes of a tree walk drift apart in the
 // branches of the descent (octree 27.8 -> 18.5 ms per 2e6 packets of the clumpy
 // medium, k-d tree 30.1 -> 18.2 ms).
-template <class G>
+//
+// kShare: some records serve several instruments.  Their deposits are a loop, for
+// which the walking lanes' rays go to local memory (left in registers, the tree
+// walks spill: octree 18.7 -> 20.7 ms; saved 19.9 ms).  Without any the plain
+// kernel runs.
+template <class G, bool kShare>
 __global__ void __launch_bounds__(tr::kBlock, kPeelBlocks<G>) k_peel_together(const __grid_constant__ FwdParams P,
                                                                             const unsigned* __restrict__ perm) {
   tr::load_grid_cache<G>(P);
@@ -227,8 +245,9 @@ __global__ void __launch_bounds__(tr::kBlock, kPeelBlocks<G>) k_peel_together(co
   const unsigned stride_k = (unsigned)(P.n_cells + 1);
   const unsigned lt_mask = (1u << (threadIdx.x & 31u)) - 1u;
   const unsigned long long n_warps = (unsigned long long)gridDim.x * (blockDim.x >> 5);
-  unsigned crossings = 0;  // of the lane's ray
-  unsigned long long total = 0, shared = 0;
+  unsigned crossings = 0;  // of the lane's segment (kShare: of its ray)
+  Counts sum{0ull, 0ull};
+  asm volatile("" ::"l"(&sum) : "memory");
   for (unsigned long long seg = blockIdx.x * (unsigned long long)(blockDim.x >> 5) + (threadIdx.x >> 5);
        seg * kSegment < n; seg += n_warps) {
     unsigned long long next = seg * kSegment;
@@ -240,21 +259,34 @@ __global__ void __launch_bounds__(tr::kBlock, kPeelBlocks<G>) k_peel_together(co
     while (true) {
       const unsigned idle = __ballot_sync(0xffffffffu, !walking);
       if (__popc(idle) >= wait) {
+        tr::Ray<G> saved;
+        if constexpr (kShare) {
+          saved = ray;
+          asm volatile("" ::"l"(&saved) : "memory");
+        }
         if (held && !walking) {
           const float4* r = reinterpret_cast<const float4*>(&P.peel[rec]);
           const float4 a = r[0], b = r[1];
           const unsigned meta = __float_as_uint(b.w);
           const ulonglong2 tag = P.peel_tag ? P.peel_tag[rec] : make_ulonglong2(0ull, 0ull);
           const int q = (int)(__float_as_uint(a.w) / stride_k);
-          unsigned m = P.instr[q].followers | 1u << q;
-          shared += (unsigned)__popc(m) - 1u;
-          total += (unsigned long long)crossings * (unsigned)__popc(m);
-          crossings = 0;
-          for (; m; m &= m - 1u)
-            tr::deposit_peel(P, __ffs(m) - 1, (int)(meta & 0xffffu), make_float3(a.x, a.y, a.z),
+          unsigned m = kShare ? P.instr[q].followers | 1u << q : 1u << q;
+          do {
+            tr::deposit_peel(P, kShare ? __ffs(m) - 1 : q, (int)(meta & 0xffffu), make_float3(a.x, a.y, a.z),
                              __hiloint2double(__float_as_int(b.y), __float_as_int(b.x)), b.z, ray.th, ray.tl,
                              (meta >> 30) & 1u, tag.x, (int)tag.y);
+            if constexpr (kShare) {
+              sum.crossings += crossings;
+              m &= m - 1u;
+              if (m) sum.shared += 1ull;
+            }
+          } while (kShare && m);
+          if constexpr (kShare) crossings = 0;
           held = false;
+        }
+        if constexpr (kShare) {
+          asm volatile("" ::"l"(&saved) : "memory");
+          ray = saved;
         }
         const unsigned long long j = next + __popc(idle & lt_mask);
         if (!walking && j < end) {
@@ -283,15 +315,22 @@ __global__ void __launch_bounds__(tr::kBlock, kPeelBlocks<G>) k_peel_together(co
         crossings += 1u;
       }
     }
+    sum.crossings += crossings;
+    crossings = 0;
   }
-  add_counts(P, total, shared);
+  add_counts(P, sum);
 }
 
 template <class G>
 cudaError_t launch_walks(const FwdParams& p, const unsigned* perm, int num_sms, size_t smem, cudaStream_t stream) {
   void (*kernel)(const FwdParams, const unsigned*);
-  if constexpr (kPeelTogether<G>) kernel = k_peel_together<G>;
-  else kernel = k_peel_sorted<G>;
+  if constexpr (kPeelTogether<G>) {
+    unsigned shared = 0;
+    for (int q = 0; q < p.n_instr; ++q) shared |= p.instr[q].followers;
+    kernel = shared ? k_peel_together<G, true> : k_peel_together<G, false>;
+  } else {
+    kernel = k_peel_sorted<G>;
+  }
   cudaError_t e = cudaSuccess;
   if (smem) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
