@@ -833,8 +833,9 @@ rt_status rt_create_grid(rt_ctx c, const rt_grid_desc* d, int32_t* grid_id) {
     rank_cell.push_back(make_float4(x, y, z, id));
   };
   if (d->kind == RT_GRID_VORONOI) {
-    // Morton order of the sites, 10 bits per axis
-    std::vector<std::pair<unsigned, int>> order((size_t)n_cells);
+    // Morton order of the sites, 10 bits per axis, sites of equal keys by
+    // index: a counting sort by ten key bits at a time
+    std::vector<std::pair<unsigned, int>> order((size_t)n_cells), sorted((size_t)n_cells);
     for (long long i = 0; i < n_cells; ++i) {
       const float p[3] = {vor_site[(size_t)i].x, vor_site[(size_t)i].y, vor_site[(size_t)i].z};
       unsigned key = 0;
@@ -845,7 +846,13 @@ rt_status rt_create_grid(rt_ctx c, const rt_grid_desc* d, int32_t* grid_id) {
       }
       order[(size_t)i] = {key, (int)i};
     }
-    std::sort(order.begin(), order.end());
+    for (int shift = 0; shift < 30; shift += 10) {
+      std::vector<size_t> at(1025, 0);
+      for (const auto& o : order) ++at[((o.first >> shift) & 1023u) + 1];
+      for (size_t k = 1; k < at.size(); ++k) at[k] += at[k - 1];
+      for (const auto& o : order) sorted[at[(o.first >> shift) & 1023u]++] = o;
+      order.swap(sorted);
+    }
     for (const auto& o : order) {
       const float4 p = vor_site[(size_t)o.second];
       next_cell(o.second, p.x, p.y, p.z);
@@ -946,34 +953,51 @@ rt_status rt_create_grid(rt_ctx c, const rt_grid_desc* d, int32_t* grid_id) {
         stack.push_back(upper);
       }
     } else {
-      // depth-first, boxes with the device's FP32 halving
+      // depth-first, boxes with the device's FP32 halving; an inner node's leaves
+      // are placed from its own entry of the stack
       struct Item {
-        int32_t node;
-        float lo[3], hi[3];
+        int32_t first;  // of its children
+        int next;       // the child to visit
+        float lo[3], mid[3], hi[3];
       };
-      std::vector<Item> stack(1);
-      stack[0].node = 0;
+      std::vector<Item> stack;
+      stack.reserve(kMaxOctreeDepth + 1);
+      const auto enter = [&](int32_t first, const float (&lo)[3], const float (&hi)[3]) {
+        Item it;
+        it.first = first;
+        it.next = 0;
+        for (int a = 0; a < 3; ++a) {
+          it.lo[a] = lo[a];
+          it.hi[a] = hi[a];
+          it.mid[a] = 0.5f * (lo[a] + hi[a]);
+        }
+        stack.push_back(it);
+      };
+      float lo[3], hi[3];
       for (int a = 0; a < 3; ++a) {
-        stack[0].lo[a] = (float)d->bounds[2 * a];
-        stack[0].hi[a] = (float)d->bounds[2 * a + 1];
+        lo[a] = (float)d->bounds[2 * a];
+        hi[a] = (float)d->bounds[2 * a + 1];
       }
+      if (child_host[0] < 0)
+        next_cell(-(long long)child_host[0] - 1, 0.5f * (lo[0] + hi[0]), 0.5f * (lo[1] + hi[1]), 0.5f * (lo[2] + hi[2]));
+      else
+        enter(child_host[0], lo, hi);
       while (!stack.empty() && one_place) {
-        const Item it = stack.back();
-        stack.pop_back();
-        const int32_t v = child_host[(size_t)it.node];
-        const float mid[3] = {0.5f * (it.lo[0] + it.hi[0]), 0.5f * (it.lo[1] + it.hi[1]), 0.5f * (it.lo[2] + it.hi[2])};
-        if (v < 0) {
-          next_cell(-(long long)v - 1, mid[0], mid[1], mid[2]);
+        Item& it = stack.back();
+        if (it.next == 8) {
+          stack.pop_back();
           continue;
         }
-        for (int o = 7; o >= 0; --o) {
-          Item k = it;
-          k.node = v + o;
-          for (int a = 0; a < 3; ++a) {
-            if ((o >> a) & 1) k.lo[a] = mid[a]; else k.hi[a] = mid[a];
-          }
-          stack.push_back(k);
+        const int o = it.next++;
+        const int32_t v = child_host[(size_t)(it.first + o)];
+        for (int a = 0; a < 3; ++a) {
+          lo[a] = (o >> a) & 1 ? it.mid[a] : it.lo[a];
+          hi[a] = (o >> a) & 1 ? it.hi[a] : it.mid[a];
         }
+        if (v < 0)
+          next_cell(-(long long)v - 1, 0.5f * (lo[0] + hi[0]), 0.5f * (lo[1] + hi[1]), 0.5f * (lo[2] + hi[2]));
+        else
+          enter(v, lo, hi);
       }
     }
     // (leaves of nodes that no parent names come last: no walk starts there)
