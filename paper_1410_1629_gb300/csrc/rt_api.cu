@@ -1265,8 +1265,13 @@ rt_status prepare_peel_pass(rt_ctx c, FwdParams& p, unsigned long long n_total, 
     dfree(c->d_peel_hist);
     dfree(c->d_peel_tiles);
     c->peel_keys = 0;
-    RT_CUDA(c, cudaMalloc(&c->d_peel_hist, keys * sizeof(unsigned)));
-    RT_CUDA(c, cudaMalloc(&c->d_peel_tiles, ((keys + 4095) / 4096) * sizeof(unsigned)));
+    if (cudaMalloc(&c->d_peel_hist, keys * sizeof(unsigned)) != cudaSuccess ||
+        cudaMalloc(&c->d_peel_tiles, ((keys + 4095) / 4096) * sizeof(unsigned)) != cudaSuccess) {
+      cudaGetLastError();
+      dfree(c->d_peel_hist);
+      dfree(c->d_peel_tiles);
+      return RT_OK;
+    }
     c->peel_keys = keys;
   }
   if (parts) *part = std::max(1ull, std::min(n_total, (unsigned long long)((double)c->peel_cap / per)));
@@ -1444,7 +1449,14 @@ rt_status rt_launch_packets(rt_ctx c, uint64_t n_per_lambda, uint64_t first_pack
   if (ev) RT_CUDA(c, cudaEventRecord(ev[1], s));
   const int walked = o.walk_peels ? (int)c->instr.size() : c->n_walked_frames;
   unsigned long long part = n_total;  // packets per transport kernel
-  const bool ordered = indexed_cells(c->grid_kind) || c->d_rank_cell;
+  bool ordered = indexed_cells(c->grid_kind) || c->d_rank_cell;
+  if (ordered && c->grid_kind != RT_GRID_CARTESIAN) {
+    // a launch being captured into a graph can neither size the pass's buffers nor
+    // read its count: its peel-offs walk in place
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) cudaGetLastError();
+    else if (capture != cudaStreamCaptureStatusNone) ordered = false;
+  }
   if (ordered && !o.tape && !o.inline_peels && walked > 0 && (o.peel_emission || o.peel_scatter)) {
     st = prepare_peel_pass(c, p, n_total, walked, o.records != nullptr, &part);
     if (st != RT_OK) return st;

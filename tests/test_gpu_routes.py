@@ -78,6 +78,39 @@ def test_sorted_pass_equals_inline_walks(grid, views):
         sim.close()
 
 
+@pytest.mark.parametrize("grid", ["rectilinear", "octree", "bintree", "voronoi"])
+def test_launches_captured_into_a_graph(grid):
+    """A launch recorded into a CUDA graph walks its peel-offs in place: two
+    replays add up to two launches, and a plain launch afterwards takes the
+    sorted pass again."""
+    prob = _grid_problem(grid)
+    n = 700
+    ref = PAR.gpu_run(prob, n, walk_peels=1)
+    sim = rt.Simulation(prob)
+    try:
+        sim.launch(n, walk_peels=1)  # the first launch of a problem makes its tables
+        sim.reset()
+        graph = torch.cuda.CUDAGraph()
+        torch.cuda.synchronize()
+        with torch.cuda.graph(graph):
+            sim.launch(n, 0, None, stream=torch.cuda.current_stream().cuda_stream, walk_peels=1)
+        for k in range(2):
+            graph.replay()
+        torch.cuda.synchronize()
+        st = sim.stats()
+        assert st["device_flags"] == 0 and st["sorted_peels"] == 0
+        assert st["peeloffs"] == 2 * ref["raw_stats"]["peeloffs"] and st["crossings"] == 2 * ref["raw_stats"]["crossings"]
+        for x, y in zip(sim.images(), ref["images"]):
+            np.testing.assert_allclose(x.cpu().numpy(), 2.0 * y, rtol=_order_bound(st["peeloffs"]), atol=0)
+        sim.reset()
+        again = PAR.gpu_run(prob, n, sim=sim, walk_peels=1)
+        assert again["raw_stats"]["sorted_peels"] > 0
+        for x, y in zip(again["images"], ref["images"]):
+            np.testing.assert_allclose(x, y, rtol=_order_bound(st["peeloffs"]), atol=0)
+    finally:
+        sim.close()
+
+
 @pytest.mark.parametrize("grid", ["cartesian", "octree"])
 def test_launch_sizes_around_the_slots(grid):
     """Packets per wavelength from one to beyond every slot of the device: one
