@@ -20,8 +20,7 @@
 #include "rt_internal.h"
 
 namespace rtk {
-// Zero entries after the Voronoi neighbour and face arrays (the walk reads
-// lists in batches of three).
+// Zero entries after the Voronoi neighbour and face arrays.
 constexpr long long kVorPad = 2;
 // rt_layout.cu: n doubles from device memory to memory the device addresses.
 cudaError_t launch_copy_f64(const double* src, double* dst, long long n, cudaStream_t stream);
@@ -93,7 +92,7 @@ struct rt_ctx_s {
   // Voronoi grids: sites, face offsets, face planes (neighbour ids in
   // d_child, n_nodes faces), bucket seeds
   float4* d_site = nullptr;
-  int* d_face_off = nullptr;
+  unsigned* d_face_off = nullptr;
   float4* d_face = nullptr;
   int* d_bucket_seed = nullptr;
   int vb_n[3] = {1, 1, 1};
@@ -287,7 +286,7 @@ void free_grid(rt_ctx c) {
   pool_release(c, c->d_edges, (size_t)(c->nx + c->ny + c->nz + 3) * sizeof(float));
   if (c->grid_kind == RT_GRID_VORONOI) {
     pool_release(c, c->d_site, (size_t)c->n_cells * sizeof(float4));
-    pool_release(c, c->d_face_off, (size_t)(c->n_cells + 1) * sizeof(int));
+    pool_release(c, c->d_face_off, (size_t)(c->n_cells + 1) * sizeof(unsigned));
     pool_release(c, c->d_face, (size_t)c->n_nodes * sizeof(float4));
     pool_release(c, c->d_bucket_seed, (size_t)c->vb_n[0] * c->vb_n[1] * c->vb_n[2] * sizeof(int));
   }
@@ -736,7 +735,8 @@ rt_status rt_create_grid(rt_ctx c, const rt_grid_desc* d, int32_t* grid_id) {
   // from the site (FP64, stored FP32); per bucket the nearest site to its
   // centre, by greedy descent from the previous bucket's
   std::vector<float4> vor_site, vor_face;
-  std::vector<int> vor_off, vor_seed;
+  std::vector<unsigned> vor_off;  // first pair of a cell's faces
+  std::vector<int> vor_nbr, vor_seed;
   int vb_n[3] = {1, 1, 1};
   if (d->kind == RT_GRID_VORONOI) {
     std::vector<double> site((size_t)n_cells * 3);
@@ -768,9 +768,17 @@ rt_status rt_create_grid(rt_ctx c, const rt_grid_desc* d, int32_t* grid_id) {
       vor_site[(size_t)i] = make_float4((float)site[(size_t)(3 * i)], (float)site[(size_t)(3 * i + 1)],
                                         (float)site[(size_t)(3 * i + 2)], 0.0f);
     vor_off.resize((size_t)n_cells + 1);
-    vor_face.resize((size_t)n_nodes);
+    // every list in pairs: an odd one ends with a zero plane and the cell itself
+    size_t pairs = 0;
     for (long long i = 0; i < n_cells; ++i) {
-      vor_off[(size_t)i] = (int)off[(size_t)i];
+      vor_off[(size_t)i] = (unsigned)pairs;
+      pairs += (size_t)((off[(size_t)i + 1] - off[(size_t)i] + 1) / 2);
+    }
+    vor_off[(size_t)n_cells] = (unsigned)pairs;
+    vor_face.assign(2 * pairs, make_float4(0.0f, 0.0f, 0.0f, 0.0f));
+    vor_nbr.resize(2 * pairs);
+    for (long long i = 0; i < n_cells; ++i) {
+      size_t at = 2 * (size_t)vor_off[(size_t)i];
       const double* si = &site[(size_t)(3 * i)];
       for (int64_t f = off[(size_t)i]; f < off[(size_t)i + 1]; ++f) {
         const long long j = nbr[(size_t)f];
@@ -780,11 +788,11 @@ rt_status rt_create_grid(rt_ctx c, const rt_grid_desc* d, int32_t* grid_id) {
         const double v[3] = {sj[0] - si[0], sj[1] - si[1], sj[2] - si[2]};
         const double len = std::sqrt(v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
         if (!(len > 0.0)) return fail(c, RT_ERR_ARG, "rt_create_grid: Voronoi sites %lld and %lld coincide", i, j);
-        vor_face[(size_t)f] = make_float4((float)(v[0] / len), (float)(v[1] / len), (float)(v[2] / len),
-                                          (float)(0.5 * len));
+        vor_nbr[at] = (int)j;
+        vor_face[at++] = make_float4((float)(v[0] / len), (float)(v[1] / len), (float)(v[2] / len), (float)(0.5 * len));
       }
+      if (at < 2 * (size_t)vor_off[(size_t)i + 1]) vor_nbr[at] = (int)i;
     }
-    vor_off[(size_t)n_cells] = (int)n_nodes;
     // buckets: about one per two sites, cubic in shape, at most 256 per axis
     const double ext[3] = {d->bounds[1] - d->bounds[0], d->bounds[3] - d->bounds[2], d->bounds[5] - d->bounds[4]};
     const double h = std::cbrt(ext[0] * ext[1] * ext[2] / std::max(1.0, 0.5 * (double)n_cells));
@@ -1032,17 +1040,17 @@ rt_status rt_create_grid(rt_ctx c, const rt_grid_desc* d, int32_t* grid_id) {
                           cudaMemcpyHostToDevice));
   }
   if (d->kind == RT_GRID_VORONOI) {
-    // neighbour ids and face planes with kVorPad zero entries after the last
-    // list: the walk loads a cell's list three entries at a time (entries
-    // past its end are masked, and the padding keeps them inside the arrays)
-    const size_t n_alloc = (size_t)n_nodes + kVorPad;
+    // neighbour ids and face planes in pairs, with kVorPad zero entries after
+    // the last list
+    const size_t n_alloc = vor_face.size() + kVorPad;
     RT_CUDA(c, pool_alloc(c, &c->d_child, n_alloc * sizeof(int32_t)));
     RT_CUDA(c, cudaMemset(c->d_child, 0, n_alloc * sizeof(int32_t)));
-    if (n_nodes > 0) RT_CUDA(c, cudaMemcpy(c->d_child, d->child, (size_t)n_nodes * sizeof(int32_t), kind));
+    if (n_nodes > 0)
+      RT_CUDA(c, cudaMemcpy(c->d_child, vor_nbr.data(), vor_nbr.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
     RT_CUDA(c, pool_alloc(c, &c->d_site, vor_site.size() * sizeof(float4)));
     RT_CUDA(c, cudaMemcpy(c->d_site, vor_site.data(), vor_site.size() * sizeof(float4), cudaMemcpyHostToDevice));
-    RT_CUDA(c, pool_alloc(c, &c->d_face_off, vor_off.size() * sizeof(int)));
-    RT_CUDA(c, cudaMemcpy(c->d_face_off, vor_off.data(), vor_off.size() * sizeof(int), cudaMemcpyHostToDevice));
+    RT_CUDA(c, pool_alloc(c, &c->d_face_off, vor_off.size() * sizeof(unsigned)));
+    RT_CUDA(c, cudaMemcpy(c->d_face_off, vor_off.data(), vor_off.size() * sizeof(unsigned), cudaMemcpyHostToDevice));
     RT_CUDA(c, pool_alloc(c, &c->d_face, n_alloc * sizeof(float4)));
     RT_CUDA(c, cudaMemset(c->d_face, 0, n_alloc * sizeof(float4)));
     if (n_nodes > 0)
@@ -1091,7 +1099,7 @@ rt_status rt_create_grid(rt_ctx c, const rt_grid_desc* d, int32_t* grid_id) {
   }
   std::memcpy(c->bounds, d->bounds, sizeof c->bounds);
   c->n_cells = n_cells;
-  c->n_nodes = d->kind == RT_GRID_VORONOI ? n_nodes + kVorPad : n_nodes;  // as allocated
+  c->n_nodes = d->kind == RT_GRID_VORONOI ? (long long)vor_face.size() + kVorPad : n_nodes;  // as allocated
   c->has_grid = true;
   c->tables_dirty = true;
   c->tape_valid = false;

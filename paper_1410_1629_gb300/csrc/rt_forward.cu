@@ -1,4 +1,4 @@
-// Forward transport on cartesian grids: the state-machine kernel of
+// Forward transport on cartesian grids: the transport engine of
 // rt_transport.cuh instantiated with the cartesian cell walk.
 #include "rt_transport.cuh"
 

@@ -1,5 +1,5 @@
 // Forward transport on k-d tree grids (the BinTree grid of the SKIRT paper,
-// Table 1(d)): the state-machine kernel of rt_transport.cuh instantiated with
+// Table 1(d)): the transport engine of rt_transport.cuh instantiated with
 // the k-d tree cell walk.
 #include "rt_transport.cuh"
 

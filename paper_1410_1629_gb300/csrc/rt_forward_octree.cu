@@ -1,5 +1,5 @@
 // Forward transport on octree grids (SKIRT paper, Sect. 2.4): the
-// state-machine kernel of rt_transport.cuh instantiated with the octree cell
+// transport engine of rt_transport.cuh instantiated with the octree cell
 // walk (ancestor stack per lane in shared memory, top of the tree cached in
 // shared memory).
 #include "rt_transport.cuh"

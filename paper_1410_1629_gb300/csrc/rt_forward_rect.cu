@@ -1,6 +1,6 @@
 // Forward transport on rectilinear grids (cells between arbitrary edges per
-// axis; the PowCub grid of the SKIRT paper, Table 1(d)): the state-machine
-// kernel of rt_transport.cuh instantiated with the rectilinear cell walk.
+// axis; the PowCub grid of the SKIRT paper, Table 1(d)): the transport engine
+// of rt_transport.cuh instantiated with the rectilinear cell walk.
 #include "rt_transport.cuh"
 
 namespace rtk {

@@ -1,10 +1,10 @@
 // Forward transport on Voronoi grids (the VoronoiDustGrid of the SKIRT paper,
-// Table 1(d) and Sect. 2.4): the state-machine kernel of rt_transport.cuh
+// Table 1(d) and Sect. 2.4): the transport engine of rt_transport.cuh
 // instantiated with the walk across the cells' bisecting planes.
 #include "rt_transport.cuh"
 
-// four resident blocks of 256 fit the Voronoi walk in 64 registers without
-// spills: more warps to hide the L2 latency of the face-plane loads
+// four resident blocks of 256 (64 registers; 16 B of spills): more warps to
+// hide the latency of the face-plane loads
 #ifndef RT_VOR_MIN_BLOCKS
 #define RT_VOR_MIN_BLOCKS 4
 #endif

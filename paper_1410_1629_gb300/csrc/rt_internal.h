@@ -94,13 +94,14 @@ struct FwdParams {
   int oct_exact;
   int oct_levels;  // octrees: ancestor-stack entries per lane (the deepest leaf's depth + 1)
   const float* edge[3];  // rectilinear only: cell edges per axis, n + 1 each
-  // Voronoi grids: sites (x, y, z, 0), the faces of cell c at
-  // [face_off[c], face_off[c + 1]) as (unit normal towards the neighbour,
+  // Voronoi grids: sites (x, y, z, 0), the faces of cell c as
+  // pairs [face_off[c], face_off[c + 1]) of (unit normal towards the neighbour,
   // distance of the bisecting plane from the site) with the neighbour's id in
-  // child[], and per bucket of a uniform bucket grid the site nearest to its
+  // child[]; an odd list ends with a zero normal (no ray leaves through it) and
+  // the cell's own id; and per bucket of a uniform bucket grid the site nearest to its
   // centre (bucket (i, j, k) at i + vb_n[0] (j + vb_n[1] k))
   const float4* site;
-  const int* face_off;
+  const unsigned* face_off;
   const float4* face;
   const int* bucket_seed;
   int vb_n[3];

@@ -49,12 +49,6 @@ constexpr float kInv4PiF = 0.0795774715459476679f;
 #define RT_FWD_MIN_BLOCKS 4
 #endif
 
-#ifndef RT_ROUND_MIN
-#define RT_ROUND_MIN 20
-#endif
-#ifndef RT_IDLE_MAX
-#define RT_IDLE_MAX 12
-#endif
 // Rounds of per-event work: a queue of at least kRoundMin packets is served at
 // once, a shorter one when kIdleMax lanes have no walk.  Between (1, 0) and
 // (24, 16): 41.7 to 40.3 ms per 4e6 packets of the disk galaxy, 22.8 to 21.0
@@ -161,6 +155,13 @@ __device__ __forceinline__ float load_density(const float* p) {
       : "=f"(v)
       : "l"(p));
   return v;
+}
+
+// Two float4 at p (32-byte aligned) with one load.
+__device__ __forceinline__ void load_pair(const float4* p, float4& a, float4& b) {
+  asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
+      : "l"(p));
 }
 
 __device__ __forceinline__ void add_absorption(double* p, double v) {
@@ -943,10 +944,10 @@ struct VorGrid {
     for (int it = 0; it < P.max_walk; ++it) {
       float best = dist2(p, __ldg(&P.site[c]));
       int move = -1;
-      const int f1 = __ldg(&P.face_off[c + 1]);
-      // three neighbours at once, as in the face loop of the walk (past the
-      // last face the cell itself, never nearer than itself)
-      for (int f = __ldg(&P.face_off[c]); f < f1; f += 3) {
+      const unsigned f1 = 2u * __ldg(&P.face_off[c + 1]);
+      // three neighbours at once (past the last face, and in place of a padded
+      // one, the cell itself, never nearer than itself)
+      for (unsigned f = 2u * __ldg(&P.face_off[c]); f < f1; f += 3) {
         int j[3];
 #pragma unroll
         for (int k = 0; k < 3; ++k) j[k] = f + k < f1 ? __ldg(&P.child[f + k]) : c;
@@ -968,32 +969,40 @@ struct VorGrid {
 
   __device__ static __forceinline__ void locate_cell(const FwdParams& P, float3 x, Cell& c) { c.leaf = locate(P, x); }
 
+  // Pairs of face planes in flight per lane.  The walk waits on the planes'
+  // loads and on the L1 wavefronts they take (lanes in different cells: one per
+  // lane and load), so two planes come with one 32-byte load, and two pairs at
+  // once: 25.5 + 12.2 ms (sorted walks + transport, Voronoi disk, 1.5e6 packets)
+  // with three 16-byte loads in flight, 29.1 + 15.3 with one pair, 23.8 + 11.3
+  // with two.
+  static constexpr int kPairs = 2;
+
   // The exit of the current cell along x + t d: parameter and next cell.
   __device__ static __forceinline__ void find_exit(const FwdParams& P, float3 x, float3 d, Walk& w) {
     const float4 s = __ldg(&P.site[w.leaf]);
     const float rx = x.x - s.x, ry = x.y - s.y, rz = x.z - s.z;
     float best = w.t_box;
-    int face = -1;
-    const int f1 = __ldg(&P.face_off[w.leaf + 1]);
-    // three face planes loaded at once (a plane past the last face reads as
-    // zero: d.n = 0, never an exit), tested in face order: three L2 loads in
-    // flight per lane instead of one (190 -> 142 ms on the 1e5-site disk; four
-    // spill at 64 registers)
-    for (int f = __ldg(&P.face_off[w.leaf]); f < f1; f += 3) {
-      float4 n[3];
+    constexpr unsigned kNoFace = 0xffffffffu;
+    unsigned face = kNoFace;
+    const unsigned p1 = __ldg(&P.face_off[w.leaf + 1]);
+    for (unsigned p = __ldg(&P.face_off[w.leaf]); p < p1; p += kPairs) {
+      float4 n[2 * kPairs];
 #pragma unroll
-      for (int k = 0; k < 3; ++k) n[k] = f + k < f1 ? __ldg(&P.face[f + k]) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      for (int k = 0; k < kPairs; ++k) {
+        if (k == 0 || p + k < p1) load_pair(&P.face[2 * (size_t)(p + k)], n[2 * k], n[2 * k + 1]);
+        else n[2 * k] = n[2 * k + 1] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      }
 #pragma unroll
-      for (int k = 0; k < 3; ++k) {
+      for (int k = 0; k < 2 * kPairs; ++k) {
         const float den = fmaf(d.x, n[k].x, fmaf(d.y, n[k].y, d.z * n[k].z));
         if (den > 0.0f) {
           const float tf = (n[k].w - fmaf(rx, n[k].x, fmaf(ry, n[k].y, rz * n[k].z))) / den;
-          if (tf < best) { best = tf; face = f + k; }
+          if (tf < best) { best = tf; face = 2u * p + (unsigned)k; }
         }
       }
     }
     w.te = best;
-    w.next = face >= 0 ? __ldg(&P.child[face]) : -1;
+    w.next = face != kNoFace ? __ldg(&P.child[face]) : -1;
   }
 
   __device__ static __forceinline__ bool init(const FwdParams& P, float3 x, float3 d, float3 id, bool known,
