@@ -573,7 +573,7 @@ rt_status rt_batch_read_stats(rt_ctx ctx, int32_t batch_id, rt_stats* out);
 /* Choose control_lanes and the packets per work-list run by timing launches
  * of a fraction (0 < fraction <= 1) of every model's packets for each
  * candidate (control_lanes 8, 12, ..., 32; runs of 64, 256, 1024, 4096
- * packets); the choice is kept for later launches with control_lanes 0 and
+ * packets, without those far too short for the whole batch); the choice is kept for later launches with control_lanes 0 and
  * written to *control_lanes and *run_packets if not NULL.  The images and
  * tallies are zeroed afterwards.  Synchronous.  Errors: RT_ERR_ARG,
  * RT_ERR_CUDA. */

@@ -2066,6 +2066,17 @@ rt_status rt_synchronize(rt_ctx c, void* stream) {
   return RT_OK;
 }
 
+// Packets per run of a batch's work list: four runs per resident warp on
+// average, so that a batch of few models still fills the grid, at most 1024 (16 /
+// 48 / 128 / 256 models: 21.0 / 39.3 / 92.2 / 206 ms in runs of 32, 13.8 / 22.5 /
+// 46.9 / 110 ms by this rule, 128 models 52.2 ms in runs of up to 4096).
+static unsigned default_run(const Batch& b) {
+  unsigned long long total = 0;
+  for (unsigned long long n : b.n_packets) total += n;
+  const unsigned long long warps = (unsigned long long)b.blocks * (kBatchBlock / 32);
+  return (unsigned)std::min(1024ull, std::max(64ull, total / (warps * 4) / 32 * 32));
+}
+
 rt_status rt_batch_create(rt_ctx c, int32_t n_models, const rt_model_desc* models, int32_t* batch_id) {
   if (!c) return RT_ERR_ARG;
   c->err.clear();
@@ -2195,15 +2206,7 @@ rt_status rt_batch_create(rt_ctx c, int32_t n_models, const rt_model_desc* model
   e = batch_blocks_per_sm(&per_sm);
   if (e != cudaSuccess) return bail(cuda_fail(c, e, "rt_batch_create: occupancy"));
   b->blocks = (unsigned)(c->num_sms * std::max(1, per_sm));
-  // runs of packets: four per resident warp on average, so that a batch of few
-  // models still fills the grid, at most 1024 (16 / 48 / 128 / 256 models: 21.0 /
-  // 39.3 / 92.2 / 206 ms in runs of 32, 13.8 / 22.5 / 46.9 / 110 ms by this rule,
-  // 128 models 52.2 ms in runs of up to 4096)
-  unsigned long long total = 0;
-  for (unsigned long long n : b->n_packets) total += n;
-  const unsigned long long warps = (unsigned long long)b->blocks * (kBatchBlock / 32);
-  const unsigned run = (unsigned)std::min(1024ull, std::max(64ull, total / (warps * 4) / 32 * 32));
-  rt_status st = upload_chunks(c, b, run);
+  rt_status st = upload_chunks(c, b, default_run(*b));
   if (st != RT_OK) return bail(st);
   c->batches.push_back(b);
   *batch_id = (int32_t)(c->batches.size() - 1);
@@ -2339,7 +2342,11 @@ rt_status rt_batch_tune(rt_ctx c, int32_t id, uint64_t seed, double fraction, in
   unsigned best_run = 1024;
   BatchChunk* d_ch = nullptr;
   cudaError_t e = cudaSuccess;
+  const unsigned whole = default_run(*b);
   for (unsigned run : runs_c) {
+    // the sample's tail favours runs too short for the whole batch (4096 models
+    // tuned on 2 %: runs of 64 and 2.69 s, against 1.68 s in runs of 1024)
+    if (4 * run < whole) continue;
     const std::vector<BatchChunk> ch = batch_chunks(*b, run, fraction);
     dfree(d_ch);
     e = cudaMalloc(&d_ch, std::max<size_t>(1, ch.size()) * sizeof(BatchChunk));
