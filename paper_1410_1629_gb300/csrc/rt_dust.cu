@@ -17,10 +17,9 @@
 // rate, when every cell was solved by itself): so E(T), the emission per unit
 // mass, is one function for all cells of a launch and its inverse is tabulated
 // once per call and looked up per cell, and the thermal emission uses the
-// library's own 1 / (exp(x) - 1) (rt_math.cuh, 24 instead of 44 FP64
-// instructions per value with its argument and scale).  192 x 192 x 128 cells,
-// 24 wavelengths: temperatures 44.9 ms, emission and running sums 10.3 ms; now
-// 7.1 ms together with the read-out (56.0 before).
+// library's own a / (exp(x) - 1) (rt_math.cuh).  192 x 192 x 128 cells, 24
+// wavelengths: temperatures 44.9 ms, emission and running sums 10.3 ms; now 7.6
+// ms together with the read-out (56.0 before).
 #include <algorithm>
 #include <cmath>
 
@@ -251,7 +250,7 @@ __global__ void k_dust_luminosity(const DustArgs A, const double* __restrict__ T
       double x = b * inv;
       const double rem = fma(-x, t, b);
       if ((bits_of(rem) >> 52 & 0x7ff) != 0x7ff) x = fma(rem, inv, x);
-      lum[(size_t)l * A.n_cells + c] = warm ? m * (A.a[l] * bose(x)) : 0.0;
+      lum[(size_t)l * A.n_cells + c] = warm ? m * bose(x, A.a[l]) : 0.0;
     }
   }
 }
