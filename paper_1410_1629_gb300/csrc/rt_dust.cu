@@ -114,12 +114,17 @@ __device__ __forceinline__ double solve_temperature(const DustArgs& A, double x,
 // is analytic well beyond it where the wavelengths are dense (its nearest
 // singularities lie a distance of order 1 away in ln x), so the coefficients fall
 // by about 60 per degree and the series ends below 1e-16 of T.  Where they fall
-// more slowly (two wavelengths far apart: the last coefficient above 4e-16) the
-// row is marked by a negative T_mid and its values take one Newton step on E
-// itself; a row whose last coefficient is above 1e-9, on which a node had no
-// root, or an x beyond the table (E(t_min) to E(t_max), at most kTableOctaves
-// down from the top) is solved by itself.
+// more slowly (two wavelengths far apart) the row is marked by a negative T_mid
+// and its values take one Newton step on E itself, or it is not used: a row
+// that does not fall fast enough for the step, on which a node had no root, or an
+// x beyond the table (E(t_min) to E(t_max), at most kTableOctaves down from the
+// top) is solved by itself.  How far the series has fallen is judged by its last
+// three coefficients, those before the last at 64 and 64^2 of it (kTableFall):
+// where two terms of E meet, the coefficients change sign from degree to degree
+// and the last alone can vanish while the series is far from its end (by the last
+// alone 2e-7 of T on such a row).
 constexpr int kTableNodes = 9, kTableRow = 10;  // T_mid and nine coefficients
+constexpr double kTableFall = 1.0 / 64.0;
 
 // Row i of the table from its nodes' roots (one thread per node, solved as a
 // cell would be over a wider range, then one Newton step in T itself, whose
@@ -129,7 +134,7 @@ __global__ void __launch_bounds__(kRowsPerBlock * kTableNodes) k_dust_table(cons
                                                                             int first, int rows,
                                                                             double* __restrict__ table,
                                                                             double* __restrict__ limits) {
-  __shared__ double T[kRowsPerBlock][kTableNodes];
+  __shared__ double T[kRowsPerBlock][kTableNodes], C[kRowsPerBlock][kTableNodes];
   const int r = threadIdx.x / kTableNodes, j = threadIdx.x % kTableNodes;
   const int row = blockIdx.x * kRowsPerBlock + r;
   if (row < rows) {
@@ -150,7 +155,14 @@ __global__ void __launch_bounds__(kRowsPerBlock * kTableNodes) k_dust_table(cons
     double* out = table + (size_t)row * kTableRow;
     c *= (j ? 2.0 : 1.0) / kTableNodes;
     out[1 + j] = c;
-    if (j == kTableNodes - 1) out[0] = fabs(c) <= 4e-16 * mid ? mid : (fabs(c) <= 1e-9 * mid ? -mid : nan(""));
+    C[r][j] = fabs(c);  // not a number on all degrees if a node had no root
+  }
+  __syncthreads();
+  if (row < rows && j == 0) {
+    const double mid = T[r][kTableNodes / 2];
+    const double* c = &C[r][kTableNodes - 3];
+    const double left = fmax(fmax(c[0] * kTableFall, c[1]) * kTableFall, c[2]);
+    table[(size_t)row * kTableRow] = left <= 4e-16 * mid ? mid : (left <= 1e-9 * mid ? -mid : nan(""));
   }
   if (blockIdx.x == 0 && threadIdx.x < 2) limits[threadIdx.x] = emission(A.n_lambda, A.a, A.b, threadIdx.x ? t_max : t_min);
 }
