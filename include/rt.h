@@ -231,9 +231,9 @@ typedef struct {
                            the transport kernel, ordered by instrument and start cell so that
                            the walks of a warp share cache lines (skipped with the tape, and
                            while its buffer, sized from the last launch's count within 40 % of
-                           free device memory, cannot be had; except on cartesian grids a launch
-                           of more than 2^28 records goes part by part, and one that is being
-                           captured into a CUDA graph skips the pass); 1: each walks inside the
+                           free device memory, cannot be had; a launch that is being captured
+                           into a CUDA graph skips the pass; except on cartesian grids a launch
+                           of more than 2^28 records goes part by part); 1: each walks inside the
                            transport kernel.  The two give the same optical depths, crossings
                            and deposits; only the order of the FP64 image additions differs.   */
   int32_t time_parts;   /* 1: record CUDA events around the parts of this launch on its stream,

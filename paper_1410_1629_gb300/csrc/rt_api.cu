@@ -1458,7 +1458,7 @@ rt_status rt_launch_packets(rt_ctx c, uint64_t n_per_lambda, uint64_t first_pack
   const int walked = o.walk_peels ? (int)c->instr.size() : c->n_walked_frames;
   unsigned long long part = n_total;  // packets per transport kernel
   bool ordered = indexed_cells(c->grid_kind) || c->d_rank_cell;
-  if (ordered && c->grid_kind != RT_GRID_CARTESIAN) {
+  if (ordered) {
     // a launch being captured into a graph can neither size the pass's buffers nor
     // read its count: its peel-offs walk in place
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
