@@ -229,11 +229,9 @@ typedef struct {
                            cartesian or rectilinear grid, all frames on other grids, or all with
                            walk_peels) run in a second pass after
                            the transport kernel, ordered by instrument and start cell so that
-                           the walks of a warp share cache lines (skipped with the tape, and
-                           while its buffer, sized from the last launch's count within 40 % of
-                           free device memory, cannot be had; a launch that is being captured
-                           into a CUDA graph skips the pass; except on cartesian grids a launch
-                           of more than 2^28 records goes part by part); 1: each walks inside the
+                           the walks of a warp share cache lines (skipped with the tape, for
+                           launches that are being captured into a CUDA graph, and while its
+                           buffer cannot be had, see part_records); 1: each walks inside the
                            transport kernel.  The two give the same optical depths, crossings
                            and deposits; only the order of the FP64 image additions differs.   */
   int32_t time_parts;   /* 1: record CUDA events around the parts of this launch on its stream,
@@ -248,7 +246,13 @@ typedef struct {
                             (0 = the value rt_tune chose, else as many as fit: 4, or 3 for
                             octrees deeper than 10 levels); the grid is this
                             times the SM count */
-  int32_t reserved;
+  int32_t part_records; /* the most records of the sorted peel-off pass's buffer (36 bytes each, 16
+                           more with debug records): beyond it a launch goes part by part, on
+                           cartesian grids its last peel-offs walk in place.  0 (default): 4e9 on
+                           cartesian grids, else 2^28 (9.7 GB), or in place when memory is too
+                           short for the records of 2^20 packets.  The buffer is sized from the
+                           last launch's count, takes at most 40 % of the free device memory,
+                           and is kept until the context is destroyed                         */
 } rt_launch_opts;
 
 /* Tallies since the last rt_reset_tallies. */

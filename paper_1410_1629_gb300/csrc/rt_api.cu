@@ -1209,12 +1209,22 @@ namespace {
 // Buffers of the sorted peel-off pass for a launch of n_total packets with
 // `walked` instruments whose peel-offs walk; on success p.peel is set (left
 // null when the pass does not fit: the kernel then walks every peel-off).
-// part: packets whose records the buffer holds by that estimate; on trees,
-// Voronoi and rectilinear grids a launch of more goes part by part, with at
-// most kPeelPart records (10 GB) each.
+// limit: the most records of the buffer (0: kPeelPart, 10 GB with the order, on
+// trees, Voronoi and rectilinear grids, where a launch of more goes part by
+// part; else what the order's 32-bit indices allow).  part: packets whose
+// records the buffer holds by the estimate.
 constexpr unsigned long long kPeelPart = 1ull << 28;
+constexpr unsigned long long kPeelMost = 4000000000ull;
+// The fewest packets of a part: each part clears and scans the counts of all
+// keys and ends with its last packets' walks.  When memory is too short for that
+// many packets' records, the launch walks its peel-offs in place.  2e6 packets
+// whole / in parts of 2^20, 2^19, 2^18, 2^16 / in place: octree of 4e5 leaves 35 /
+// 47, 61, 102, 299 / 51 ms, of 3e6 leaves 69 / 99, 135, 223, 657 / 95 ms, k-d tree
+// of 2e5 leaves 38 / 54, 71, 125, 379 / 69 ms, 3e4 Voronoi cells (1.5e6 packets)
+// 36 / 39, 45, 66, 125 / 48 ms.
+constexpr unsigned long long kMinPart = 1ull << 20;
 rt_status prepare_peel_pass(rt_ctx c, FwdParams& p, unsigned long long n_total, int walked, bool tags,
-                            unsigned long long* part) {
+                            unsigned long long limit, unsigned long long* part) {
   const unsigned long long keys = (unsigned long long)c->instr.size() * (unsigned long long)(c->n_cells + 1);
   if (keys >= 0xffffffffull) return RT_OK;
   if (!c->peel_event) {
@@ -1238,18 +1248,22 @@ rt_status prepare_peel_pass(rt_ctx c, FwdParams& p, unsigned long long n_total, 
   // eight per walked instrument (a packet peels off once per event)
   const double per = c->peel_per_packet > 0.0 ? 1.25 * c->peel_per_packet + 0.05 : 8.0 * walked;
   const bool parts = c->grid_kind != RT_GRID_CARTESIAN;
-  unsigned long long want = (unsigned long long)std::min(per * (double)n_total, parts ? (double)kPeelPart : 4.0e9);
-  want = std::max(want, 4096ull);
+  const unsigned long long least = parts && !limit ? std::min(n_total, kMinPart) : 1;  // packets of a part
+  if (!limit) limit = parts ? kPeelPart : kPeelMost;
+  unsigned long long want = std::min((unsigned long long)std::min(per * (double)n_total, (double)kPeelMost), limit);
+  want = std::max(want, std::min(4096ull, limit));
+  if (want > c->peel_cap) {
+    size_t free_b = 0, total_b = 0;
+    RT_CUDA(c, cudaMemGetInfo(&free_b, &total_b));
+    // at most 40 % of the device memory that is free without the present buffer
+    const size_t record = sizeof(PeelRecord) + sizeof(unsigned);
+    want = std::min(want, (unsigned long long)(0.4 * ((double)free_b + (double)(c->peel_cap * record))) / record);
+  }
+  if (std::max(want, c->peel_cap) < (unsigned long long)std::min(per * (double)least, (double)kPeelMost)) return RT_OK;
   if (want > c->peel_cap) {
     dfree(c->d_peel);
     dfree(c->d_peel_perm);
     c->peel_cap = 0;
-    size_t free_b = 0, total_b = 0;
-    RT_CUDA(c, cudaMemGetInfo(&free_b, &total_b));
-    // at most 40 % of the free device memory
-    const unsigned long long fit = (unsigned long long)(0.4 * (double)free_b) / (sizeof(PeelRecord) + sizeof(unsigned));
-    want = std::min(want, fit);
-    if (want < 4096) return RT_OK;
     if (cudaMalloc(&c->d_peel, want * sizeof(PeelRecord)) != cudaSuccess ||
         cudaMalloc(&c->d_peel_perm, want * sizeof(unsigned)) != cudaSuccess) {
       cudaGetLastError();
@@ -1259,6 +1273,7 @@ rt_status prepare_peel_pass(rt_ctx c, FwdParams& p, unsigned long long n_total, 
     }
     c->peel_cap = want;
   }
+  const unsigned long long cap = std::min(c->peel_cap, limit);
   if (tags && c->peel_tag_cap < c->peel_cap) {
     dfree(c->d_peel_tag);
     c->peel_tag_cap = 0;
@@ -1282,9 +1297,9 @@ rt_status prepare_peel_pass(rt_ctx c, FwdParams& p, unsigned long long n_total, 
     }
     c->peel_keys = keys;
   }
-  if (parts) *part = std::max(1ull, std::min(n_total, (unsigned long long)((double)c->peel_cap / per)));
+  if (parts) *part = std::max(1ull, std::min(n_total, (unsigned long long)((double)cap / per)));
   p.peel = c->d_peel;
-  p.peel_cap = c->peel_cap;
+  p.peel_cap = cap;
   p.peel_count = c->d_peel_count;
   p.peel_hist = c->d_peel_hist;
   p.peel_tag = tags ? c->d_peel_tag : nullptr;
@@ -1466,7 +1481,8 @@ rt_status rt_launch_packets(rt_ctx c, uint64_t n_per_lambda, uint64_t first_pack
     else if (capture != cudaStreamCaptureStatusNone) ordered = false;
   }
   if (ordered && !o.tape && !o.inline_peels && walked > 0 && (o.peel_emission || o.peel_scatter)) {
-    st = prepare_peel_pass(c, p, n_total, walked, o.records != nullptr, &part);
+    st = prepare_peel_pass(c, p, n_total, walked, o.records != nullptr,
+                           o.part_records > 0 ? (unsigned long long)o.part_records : 0, &part);
     if (st != RT_OK) return st;
   }
   const unsigned long long keys = (unsigned long long)c->instr.size() * (unsigned long long)(c->n_cells + 1);
