@@ -10,6 +10,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <new>
 #include <string>
 #include <utility>
@@ -17,6 +18,7 @@
 
 #include <cuda_runtime.h>
 
+#include "rt_cells.h"
 #include "rt_internal.h"
 
 namespace rtk {
@@ -98,9 +100,15 @@ struct rt_ctx_s {
   int vb_n[3] = {1, 1, 1};
   bool oct_exact = false;  // octree boxes exact binary fractions (FwdParams::oct_exact)
   int oct_depth = 0;       // octrees: the deepest leaf's depth
-  // trees and Voronoi grids: the sorted pass's order of the cells (FwdParams)
+  // trees and Voronoi grids: the sorted pass's order of the cells (FwdParams), made
+  // when the grid gets its first instrument, and what it is made from until then:
+  // an octree's nodes, Voronoi sites, or the order itself, a by-product of the
+  // k-d tree's ropes
   int* d_cell_rank = nullptr;
   float4* d_rank_cell = nullptr;
+  std::vector<int32_t> order_child;
+  std::vector<float4> order_site;
+  std::unique_ptr<CellOrder> order;
   // k-d trees: leaf ropes [n_cells][6] and node boxes [n_nodes][2] (FwdParams)
   int32_t* d_rope = nullptr;
   float4* d_node_box = nullptr;
@@ -272,6 +280,12 @@ rt_status set_device(rt_ctx ctx) {
   return RT_OK;
 }
 
+void drop_order(rt_ctx c) {
+  std::vector<int32_t>().swap(c->order_child);
+  std::vector<float4>().swap(c->order_site);
+  c->order.reset();
+}
+
 void free_grid(rt_ctx c) {
   c->tape_valid = false;
   cudaDeviceSynchronize();  // no kernel may still read the released buffers
@@ -283,6 +297,7 @@ void free_grid(rt_ctx c) {
   }
   pool_release(c, c->d_cell_rank, (size_t)c->n_cells * sizeof(int));
   pool_release(c, c->d_rank_cell, (size_t)c->n_cells * sizeof(float4));
+  drop_order(c);
   pool_release(c, c->d_edges, (size_t)(c->nx + c->ny + c->nz + 3) * sizeof(float));
   if (c->grid_kind == RT_GRID_VORONOI) {
     pool_release(c, c->d_site, (size_t)c->n_cells * sizeof(float4));
@@ -823,52 +838,10 @@ rt_status rt_create_grid(rt_ctx c, const rt_grid_desc* d, int32_t* grid_id) {
           vor_seed[(size_t)i + (size_t)vb_n[0] * ((size_t)j + (size_t)vb_n[1] * k)] = (int)cur;
         }
   }
-  // trees and Voronoi grids: the sorted pass's order of the cells
-  const bool unordered = !indexed_cells(d->kind);
-  std::vector<int> cell_rank(unordered ? (size_t)n_cells : 0, -1);
-  std::vector<float4> rank_cell;
-  rank_cell.reserve(cell_rank.size());
-  bool one_place = true;  // no cell met twice (a tree's nodes each have one parent)
-  auto next_cell = [&](long long cell, float x, float y, float z) {
-    if (cell_rank[(size_t)cell] >= 0) {
-      one_place = false;
-      return;
-    }
-    cell_rank[(size_t)cell] = (int)rank_cell.size();
-    float id;
-    const int cell_i = (int)cell;
-    std::memcpy(&id, &cell_i, sizeof id);
-    rank_cell.push_back(make_float4(x, y, z, id));
-  };
-  if (d->kind == RT_GRID_VORONOI) {
-    // Morton order of the sites, 10 bits per axis, sites of equal keys by
-    // index: a counting sort by ten key bits at a time
-    std::vector<std::pair<unsigned, int>> order((size_t)n_cells), sorted((size_t)n_cells);
-    for (long long i = 0; i < n_cells; ++i) {
-      const float p[3] = {vor_site[(size_t)i].x, vor_site[(size_t)i].y, vor_site[(size_t)i].z};
-      unsigned key = 0;
-      for (int a = 0; a < 3; ++a) {
-        const double u = (p[a] - d->bounds[2 * a]) / (d->bounds[2 * a + 1] - d->bounds[2 * a]);
-        const unsigned v = (unsigned)std::min(1023.0, std::max(0.0, 1024.0 * u));
-        for (int bit = 0; bit < 10; ++bit) key |= ((v >> bit) & 1u) << (3 * bit + a);
-      }
-      order[(size_t)i] = {key, (int)i};
-    }
-    for (int shift = 0; shift < 30; shift += 10) {
-      std::vector<size_t> at(1025, 0);
-      for (const auto& o : order) ++at[((o.first >> shift) & 1023u) + 1];
-      for (size_t k = 1; k < at.size(); ++k) at[k] += at[k - 1];
-      for (const auto& o : order) sorted[at[(o.first >> shift) & 1023u]++] = o;
-      order.swap(sorted);
-    }
-    for (const auto& o : order) {
-      const float4 p = vor_site[(size_t)o.second];
-      next_cell(o.second, p.x, p.y, p.z);
-    }
-  }
   std::vector<int32_t> child_host;
   std::vector<int32_t> rope_host;     // k-d trees: leaf ropes
-  std::vector<float4> node_box_host;  // k-d trees: node boxes
+  std::vector<float> node_box_host;   // k-d trees: node boxes
+  std::unique_ptr<CellOrder> order;   // k-d trees: the sorted pass's order of the cells
   int oct_depth = 0;  // octrees: the deepest leaf's depth
   if (d->kind == RT_GRID_OCTREE || d->kind == RT_GRID_BINTREE) {
     // validate the tree on the host: every child block in range (after its
@@ -916,101 +889,10 @@ rt_status rt_create_grid(rt_ctx c, const rt_grid_desc* d, int32_t* grid_id) {
     if (!bin && oct_depth > kMaxOctreeDepth)
       return fail(c, RT_ERR_ARG, "rt_create_grid: octree depth %d above %d", oct_depth, kMaxOctreeDepth);
     if (bin) {
-      // node boxes with the device's FP32 halving, and the ropes: going down,
-      // the lower child's rope across its upper face on the split axis is the
-      // upper child and the other way round; the other faces inherit
-      rope_host.assign((size_t)n_cells * 6, -1);
-      node_box_host.resize((size_t)n_nodes * 2);
-      struct Item {
-        long long node;
-        float lo[3], hi[3];
-        int32_t r[6];
-      };
-      std::vector<Item> stack;
-      Item root;
-      root.node = 0;
-      for (int a = 0; a < 3; ++a) {
-        root.lo[a] = (float)d->bounds[2 * a];
-        root.hi[a] = (float)d->bounds[2 * a + 1];
-      }
-      for (int f = 0; f < 6; ++f) root.r[f] = -1;
-      stack.push_back(root);
-      while (!stack.empty()) {
-        const Item it = stack.back();
-        stack.pop_back();
-        node_box_host[2 * (size_t)it.node] = make_float4(it.lo[0], it.lo[1], it.lo[2], 0.0f);
-        node_box_host[2 * (size_t)it.node + 1] = make_float4(it.hi[0], it.hi[1], it.hi[2], 0.0f);
-        const int32_t v = child_host[(size_t)it.node];
-        if (v < 0) {
-          for (int f = 0; f < 6; ++f) rope_host[(size_t)(-(long long)v - 1) * 6 + f] = it.r[f];
-          next_cell(-(long long)v - 1, 0.5f * (it.lo[0] + it.hi[0]), 0.5f * (it.lo[1] + it.hi[1]),
-                    0.5f * (it.lo[2] + it.hi[2]));
-          continue;
-        }
-        const int a = v & 3;
-        const long long first = (long long)(v >> 2);
-        const float mid = 0.5f * (it.lo[a] + it.hi[a]);
-        Item lower = it, upper = it;
-        lower.node = first;
-        lower.hi[a] = mid;
-        lower.r[2 * a + 1] = (int32_t)(first + 1);
-        upper.node = first + 1;
-        upper.lo[a] = mid;
-        upper.r[2 * a] = (int32_t)first;
-        stack.push_back(lower);
-        stack.push_back(upper);
-      }
-    } else {
-      // depth-first, boxes with the device's FP32 halving; an inner node's leaves
-      // are placed from its own entry of the stack
-      struct Item {
-        int32_t first;  // of its children
-        int next;       // the child to visit
-        float lo[3], mid[3], hi[3];
-      };
-      std::vector<Item> stack;
-      stack.reserve(kMaxOctreeDepth + 1);
-      const auto enter = [&](int32_t first, const float (&lo)[3], const float (&hi)[3]) {
-        Item it;
-        it.first = first;
-        it.next = 0;
-        for (int a = 0; a < 3; ++a) {
-          it.lo[a] = lo[a];
-          it.hi[a] = hi[a];
-          it.mid[a] = 0.5f * (lo[a] + hi[a]);
-        }
-        stack.push_back(it);
-      };
-      float lo[3], hi[3];
-      for (int a = 0; a < 3; ++a) {
-        lo[a] = (float)d->bounds[2 * a];
-        hi[a] = (float)d->bounds[2 * a + 1];
-      }
-      if (child_host[0] < 0)
-        next_cell(-(long long)child_host[0] - 1, 0.5f * (lo[0] + hi[0]), 0.5f * (lo[1] + hi[1]), 0.5f * (lo[2] + hi[2]));
-      else
-        enter(child_host[0], lo, hi);
-      while (!stack.empty() && one_place) {
-        Item& it = stack.back();
-        if (it.next == 8) {
-          stack.pop_back();
-          continue;
-        }
-        const int o = it.next++;
-        const int32_t v = child_host[(size_t)(it.first + o)];
-        for (int a = 0; a < 3; ++a) {
-          lo[a] = (o >> a) & 1 ? it.mid[a] : it.lo[a];
-          hi[a] = (o >> a) & 1 ? it.hi[a] : it.mid[a];
-        }
-        if (v < 0)
-          next_cell(-(long long)v - 1, 0.5f * (lo[0] + hi[0]), 0.5f * (lo[1] + hi[1]), 0.5f * (lo[2] + hi[2]));
-        else
-          enter(v, lo, hi);
-      }
+      order.reset(new CellOrder(n_cells));
+      if (!bintree_walk_arrays(child_host.data(), n_nodes, n_cells, d->bounds, rope_host, node_box_host, *order))
+        order.reset();
     }
-    // (leaves of nodes that no parent names come last: no walk starts there)
-    for (long long leaf = 0; one_place && leaf < n_cells; ++leaf)
-      if (cell_rank[(size_t)leaf] < 0) next_cell(leaf, (float)d->bounds[0], (float)d->bounds[2], (float)d->bounds[4]);
   }
   if (set_device(c) != RT_OK) return RT_ERR_CUDA;
   free_problem(c);
@@ -1026,17 +908,11 @@ rt_status rt_create_grid(rt_ctx c, const rt_grid_desc* d, int32_t* grid_id) {
     RT_CUDA(c, pool_alloc(c, &c->d_child, (size_t)n_nodes * sizeof(int32_t)));
     RT_CUDA(c, cudaMemcpy(c->d_child, child_host.data(), (size_t)n_nodes * sizeof(int32_t), cudaMemcpyHostToDevice));
   }
-  if (unordered && one_place) {
-    RT_CUDA(c, pool_alloc(c, &c->d_cell_rank, cell_rank.size() * sizeof(int)));
-    RT_CUDA(c, cudaMemcpy(c->d_cell_rank, cell_rank.data(), cell_rank.size() * sizeof(int), cudaMemcpyHostToDevice));
-    RT_CUDA(c, pool_alloc(c, &c->d_rank_cell, rank_cell.size() * sizeof(float4)));
-    RT_CUDA(c, cudaMemcpy(c->d_rank_cell, rank_cell.data(), rank_cell.size() * sizeof(float4), cudaMemcpyHostToDevice));
-  }
   if (d->kind == RT_GRID_BINTREE) {
     RT_CUDA(c, pool_alloc(c, &c->d_rope, rope_host.size() * sizeof(int32_t)));
     RT_CUDA(c, cudaMemcpy(c->d_rope, rope_host.data(), rope_host.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
-    RT_CUDA(c, pool_alloc(c, &c->d_node_box, node_box_host.size() * sizeof(float4)));
-    RT_CUDA(c, cudaMemcpy(c->d_node_box, node_box_host.data(), node_box_host.size() * sizeof(float4),
+    RT_CUDA(c, pool_alloc(c, &c->d_node_box, node_box_host.size() * sizeof(float)));
+    RT_CUDA(c, cudaMemcpy(c->d_node_box, node_box_host.data(), node_box_host.size() * sizeof(float),
                           cudaMemcpyHostToDevice));
   }
   if (d->kind == RT_GRID_VORONOI) {
@@ -1100,6 +976,9 @@ rt_status rt_create_grid(rt_ctx c, const rt_grid_desc* d, int32_t* grid_id) {
   std::memcpy(c->bounds, d->bounds, sizeof c->bounds);
   c->n_cells = n_cells;
   c->n_nodes = d->kind == RT_GRID_VORONOI ? (long long)vor_face.size() + kVorPad : n_nodes;  // as allocated
+  if (d->kind == RT_GRID_OCTREE) c->order_child = std::move(child_host);
+  c->order_site = std::move(vor_site);
+  c->order = std::move(order);
   c->has_grid = true;
   c->tables_dirty = true;
   c->tape_valid = false;
@@ -1167,6 +1046,43 @@ rt_status rt_add_sources(rt_ctx c, int32_t n, const rt_source_desc* s) {
   return RT_OK;
 }
 
+namespace {
+
+// The sorted pass's order of the cells (trees and Voronoi grids), made once per
+// grid.  Without it (a leaf with two parents, no memory) peel-offs walk in place.
+rt_status prepare_cell_order(rt_ctx c) {
+  const size_t n = (size_t)c->n_cells;
+  try {
+    if (!c->order_child.empty()) {
+      c->order.reset(new CellOrder(c->n_cells));
+      if (!order_octree(c->order_child.data(), c->bounds, *c->order)) c->order.reset();
+    } else if (!c->order_site.empty()) {
+      c->order.reset(new CellOrder(c->n_cells));
+      order_voronoi(&c->order_site[0].x, c->bounds, *c->order);
+    }
+  } catch (const std::bad_alloc&) {
+    c->order.reset();
+  }
+  static_assert(sizeof(CellPoint) == sizeof(float4), "rank_cell is read as float4");
+  cudaError_t e = cudaSuccess;
+  if (c->order) {
+    e = pool_alloc(c, &c->d_cell_rank, n * sizeof(int));
+    if (e == cudaSuccess) e = pool_alloc(c, &c->d_rank_cell, n * sizeof(float4));
+    if (e == cudaSuccess) e = cudaMemcpy(c->d_cell_rank, c->order->rank.data(), n * sizeof(int), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess)
+      e = cudaMemcpy(c->d_rank_cell, c->order->cell.get(), n * sizeof(float4), cudaMemcpyHostToDevice);
+  }
+  drop_order(c);
+  if (e == cudaSuccess) return RT_OK;
+  dfree(c->d_cell_rank);
+  dfree(c->d_rank_cell);
+  if (e != cudaErrorMemoryAllocation) return cuda_fail(c, e, "order of the cells");
+  cudaGetLastError();
+  return RT_OK;
+}
+
+}  // namespace
+
 rt_status rt_add_instruments(rt_ctx c, int32_t n, const rt_instrument_desc* q, int32_t* ids) {
   if (!c) return RT_ERR_ARG;
   c->err.clear();
@@ -1190,6 +1106,10 @@ rt_status rt_add_instruments(rt_ctx c, int32_t n, const rt_instrument_desc* q, i
       return fail(c, RT_ERR_ARG, "instrument %d: non-finite angle or centre", i);
   }
   if (set_device(c) != RT_OK) return RT_ERR_CUDA;
+  if (n > 0) {
+    const rt_status so = prepare_cell_order(c);
+    if (so != RT_OK) return so;
+  }
   for (int i = 0; i < n; ++i) {
     HostInstr h;
     h.desc = q[i];
@@ -1472,18 +1392,17 @@ rt_status rt_launch_packets(rt_ctx c, uint64_t n_per_lambda, uint64_t first_pack
   if (ev) RT_CUDA(c, cudaEventRecord(ev[1], s));
   const int walked = o.walk_peels ? (int)c->instr.size() : c->n_walked_frames;
   unsigned long long part = n_total;  // packets per transport kernel
-  bool ordered = indexed_cells(c->grid_kind) || c->d_rank_cell;
-  if (ordered) {
+  const bool ordered = indexed_cells(c->grid_kind) || c->d_rank_cell;
+  if (ordered && !o.tape && !o.inline_peels && walked > 0 && (o.peel_emission || o.peel_scatter)) {
     // a launch being captured into a graph can neither size the pass's buffers nor
     // read its count: its peel-offs walk in place
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) cudaGetLastError();
-    else if (capture != cudaStreamCaptureStatusNone) ordered = false;
-  }
-  if (ordered && !o.tape && !o.inline_peels && walked > 0 && (o.peel_emission || o.peel_scatter)) {
-    st = prepare_peel_pass(c, p, n_total, walked, o.records != nullptr,
-                           o.part_records > 0 ? (unsigned long long)o.part_records : 0, &part);
-    if (st != RT_OK) return st;
+    if (capture == cudaStreamCaptureStatusNone) {
+      st = prepare_peel_pass(c, p, n_total, walked, o.records != nullptr,
+                             o.part_records > 0 ? (unsigned long long)o.part_records : 0, &part);
+      if (st != RT_OK) return st;
+    }
   }
   const unsigned long long keys = (unsigned long long)c->instr.size() * (unsigned long long)(c->n_cells + 1);
   cudaError_t e = cudaSuccess;
