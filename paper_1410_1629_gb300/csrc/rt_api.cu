@@ -215,6 +215,7 @@ rt_status fail(rt_ctx ctx, rt_status code, const char* fmt, ...) {
 }
 
 rt_status cuda_fail(rt_ctx ctx, cudaError_t e, const char* what) {
+  cudaGetLastError();  // reported here: a later launch's check must not find it again
   return fail(ctx, e == cudaErrorMemoryAllocation ? RT_ERR_OOM : RT_ERR_CUDA, "%s: %s", what,
               cudaGetErrorString(e));
 }
