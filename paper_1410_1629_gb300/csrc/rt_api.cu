@@ -197,8 +197,9 @@ struct rt_ctx_s {
   cudaEvent_t part_ev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
   bool parts_timed = false;
   double emitted = 0.0;  // luminosity emitted since the last reset (host-side sum)
-  // device buffers released by the problem's set-up calls, for reuse
-  std::vector<std::pair<void*, size_t>> pool;
+  // device buffers released by the problem's set-up calls, for reuse, and those in
+  // use, each with its size
+  std::vector<std::pair<void*, size_t>> pool, pool_used;
   size_t pool_bytes = 0;
 };
 
@@ -237,7 +238,8 @@ void dfree(T*& p) {
 // size, so that a problem rebuilt with the same grid, wavelengths and
 // instruments (a fitting loop, an end-to-end run) allocates nothing.  At most
 // kPoolLimit bytes are kept; an allocation that fails empties the pool and
-// tries again.
+// tries again.  A buffer's size is the one it was allocated with: the problem's
+// dimensions say nothing about it after a set-up call that failed half-way.
 constexpr size_t kPoolLimit = size_t(16) << 30;
 
 void pool_flush(rt_ctx c) {
@@ -247,8 +249,15 @@ void pool_flush(rt_ctx c) {
 }
 
 template <class T>
-void pool_release(rt_ctx c, T*& p, size_t bytes) {
+void pool_release(rt_ctx c, T*& p) {
   if (!p) return;
+  size_t bytes = 0;
+  for (size_t i = 0; i < c->pool_used.size(); ++i) {
+    if (c->pool_used[i].first != static_cast<void*>(p)) continue;
+    bytes = c->pool_used[i].second;
+    c->pool_used.erase(c->pool_used.begin() + (long)i);
+    break;
+  }
   if (bytes == 0 || c->pool_bytes + bytes > kPoolLimit) {
     cudaFree(p);
   } else {
@@ -260,19 +269,23 @@ void pool_release(rt_ctx c, T*& p, size_t bytes) {
 
 template <class T>
 cudaError_t pool_alloc(rt_ctx c, T** p, size_t bytes) {
-  for (size_t i = 0; i < c->pool.size(); ++i) {
-    if (c->pool[i].second != bytes) continue;
+  cudaError_t e = cudaSuccess;
+  size_t i = 0;
+  while (i < c->pool.size() && c->pool[i].second != bytes) ++i;
+  if (i < c->pool.size()) {
     *p = static_cast<T*>(c->pool[i].first);
     c->pool_bytes -= bytes;
     c->pool.erase(c->pool.begin() + (long)i);
-    return cudaSuccess;
-  }
-  cudaError_t e = cudaMalloc(p, bytes);
-  if (e == cudaErrorMemoryAllocation && !c->pool.empty()) {
-    cudaGetLastError();
-    pool_flush(c);
+  } else {
     e = cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation && !c->pool.empty()) {
+      cudaGetLastError();
+      pool_flush(c);
+      e = cudaMalloc(p, bytes);
+    }
   }
+  if (e == cudaSuccess) c->pool_used.emplace_back(static_cast<void*>(*p), bytes);
+  else *p = nullptr;
   return e;
 }
 
@@ -290,30 +303,26 @@ void drop_order(rt_ctx c) {
 void free_grid(rt_ctx c) {
   c->tape_valid = false;
   cudaDeviceSynchronize();  // no kernel may still read the released buffers
-  pool_release(c, c->d_density, (size_t)c->n_cells * sizeof(float));
-  pool_release(c, c->d_child, (size_t)c->n_nodes * sizeof(int32_t));
-  if (c->grid_kind == RT_GRID_BINTREE) {
-    pool_release(c, c->d_rope, (size_t)c->n_cells * 6 * sizeof(int32_t));
-    pool_release(c, c->d_node_box, (size_t)c->n_nodes * 2 * sizeof(float4));
-  }
-  pool_release(c, c->d_cell_rank, (size_t)c->n_cells * sizeof(int));
-  pool_release(c, c->d_rank_cell, (size_t)c->n_cells * sizeof(float4));
+  pool_release(c, c->d_density);
+  pool_release(c, c->d_child);
+  pool_release(c, c->d_rope);
+  pool_release(c, c->d_node_box);
+  pool_release(c, c->d_cell_rank);
+  pool_release(c, c->d_rank_cell);
   drop_order(c);
-  pool_release(c, c->d_edges, (size_t)(c->nx + c->ny + c->nz + 3) * sizeof(float));
-  if (c->grid_kind == RT_GRID_VORONOI) {
-    pool_release(c, c->d_site, (size_t)c->n_cells * sizeof(float4));
-    pool_release(c, c->d_face_off, (size_t)(c->n_cells + 1) * sizeof(unsigned));
-    pool_release(c, c->d_face, (size_t)c->n_nodes * sizeof(float4));
-    pool_release(c, c->d_bucket_seed, (size_t)c->vb_n[0] * c->vb_n[1] * c->vb_n[2] * sizeof(int));
-  }
-  pool_release(c, c->d_density_s, (size_t)c->n_cells * sizeof(float));
-  pool_release(c, c->d_abs_tmp, (size_t)c->n_cells * sizeof(double));
-  pool_release(c, c->d_planes64, (size_t)(c->nx + c->ny + c->nz + 3) * sizeof(double));
-  pool_release(c, c->d_dust_T, (size_t)c->n_cells * sizeof(double));
+  pool_release(c, c->d_edges);
+  pool_release(c, c->d_site);
+  pool_release(c, c->d_face_off);
+  pool_release(c, c->d_face);
+  pool_release(c, c->d_bucket_seed);
+  pool_release(c, c->d_density_s);
+  pool_release(c, c->d_abs_tmp);
+  pool_release(c, c->d_planes64);
+  pool_release(c, c->d_dust_T);
   c->permuted = false;
-  pool_release(c, c->d_absorption, (size_t)c->n_lambda * c->n_cells * sizeof(double));
-  for (auto& p : c->d_columns) pool_release(c, p, (size_t)c->n_cells * sizeof(float));
-  for (auto& p : c->d_line_dep) pool_release(c, p, (size_t)c->n_cells * sizeof(double));
+  pool_release(c, c->d_absorption);
+  for (auto& p : c->d_columns) pool_release(c, p);
+  for (auto& p : c->d_line_dep) pool_release(c, p);
   c->tables_dirty = true;
   c->tape_valid = false;
   c->has_grid = false;
@@ -339,13 +348,13 @@ bool frame_axis(const DevInstr& I, int& axis, int& dir) {
 void free_problem(rt_ctx c) {
   c->tape_valid = false;
   cudaDeviceSynchronize();  // no kernel may still write the released buffers
-  for (auto& q : c->instr) pool_release(c, q.d_image, q.n_elems * sizeof(double));
+  for (auto& q : c->instr) pool_release(c, q.d_image);
   c->instr.clear();
   c->sources.clear();
-  pool_release(c, c->d_absorption, (size_t)c->n_lambda * c->n_cells * sizeof(double));
-  pool_release(c, c->d_dust_lum, (size_t)c->n_lambda * c->n_cells * sizeof(double));
-  pool_release(c, c->d_dust_cum, (size_t)c->n_lambda * c->n_cells * sizeof(double));
-  pool_release(c, c->d_dust_tiles, (size_t)c->n_lambda * dust_tiles(c->n_cells) * sizeof(double));
+  pool_release(c, c->d_absorption);
+  pool_release(c, c->d_dust_lum);
+  pool_release(c, c->d_dust_cum);
+  pool_release(c, c->d_dust_tiles);
   c->dust_ready = false;
   c->dust_total.clear();
   c->n_lambda = 0;
@@ -641,7 +650,6 @@ rt_status rt_context_destroy(rt_ctx c) {
   dfree(c->d_src); dfree(c->d_src_cum);
   dfree(c->d_stats); dfree(c->d_counters); dfree(c->d_work); dfree(c->d_flags);
   dfree(c->d_adj); dfree(c->d_adj_img); dfree(c->d_adj_max); dfree(c->d_tune_grad); dfree(c->d_tape);
-  for (auto& p : c->d_line_dep) dfree(p);
   dfree(c->d_dust_clamped); dfree(c->d_dust_table);
   dfree(c->d_peel); dfree(c->d_peel_perm); dfree(c->d_peel_hist); dfree(c->d_peel_tiles); dfree(c->d_peel_count);
   dfree(c->d_peel_tag);
@@ -1075,8 +1083,8 @@ rt_status prepare_cell_order(rt_ctx c) {
   }
   drop_order(c);
   if (e == cudaSuccess) return RT_OK;
-  dfree(c->d_cell_rank);
-  dfree(c->d_rank_cell);
+  pool_release(c, c->d_cell_rank);
+  pool_release(c, c->d_rank_cell);
   if (e != cudaErrorMemoryAllocation) return cuda_fail(c, e, "order of the cells");
   cudaGetLastError();
   return RT_OK;
