@@ -332,7 +332,7 @@ cudaError_t launch_walks(const FwdParams& p, const unsigned* perm, int num_sms, 
     kernel = k_peel_sorted<G>;
   }
   cudaError_t e = cudaSuccess;
-  if (smem) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (smem) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tr::kMaxScratch<G>);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, tr::kBlock, smem);

@@ -2002,6 +2002,15 @@ __device__ __forceinline__ OctGrid::Scratch lane_scratch<OctGrid>(size_t offset)
   return OctGrid::Scratch{reinterpret_cast<int*>(S_RAW + offset) + threadIdx.x};
 }
 
+// The most dynamic shared memory of lane_scratch, over all grids of a kind.  A
+// kernel's limit is set to this and not to a launch's own need: it belongs to the
+// kernel, and another context's launch of a shallower tree, in another thread,
+// would lower it between the setting and the launch.
+template <class G>
+constexpr size_t kMaxScratch = 0;
+template <>
+constexpr size_t kMaxScratch<OctGrid> = (size_t)kBlock * kOctStack * sizeof(int);
+
 template <class G>
 __device__ __forceinline__ void load_grid_cache(const FwdParams&) {}
 template <>
@@ -2170,7 +2179,7 @@ cudaError_t launch_body(void (*kernel)(const FwdParams), const FwdParams& p, int
   const size_t bytes = sizeof(Shared<G, kTape>) + extra;
   // static and dynamic shared memory together pass 48 KB: the launch needs
   // the dynamic part allowed explicitly
-  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(Shared<G, kTape>) + kMaxScratch<G>));
   if (e != cudaSuccess) return e;
   int per_sm = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kBlock, bytes);
