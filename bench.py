@@ -44,8 +44,8 @@ BYTES_COLUMN_PEEL = 8
 TRAFFIC_CAPTURE = {"sources_sha256_16": "416c7b865a0dea5c", "kernel": "k_forward_cartesian",
                    "bytes_per_packet": (37898666000 + 18077492000) / 2e6}
 KERNEL_SOURCES = ["paper_1410_1629_gb300/csrc/rt_forward.cu", "paper_1410_1629_gb300/csrc/rt_device.cuh",
-                  "paper_1410_1629_gb300/csrc/rt_internal.h", "paper_1410_1629_gb300/csrc/rt_transport.cuh",
-                  "paper_1410_1629_gb300/build.py"]
+                  "paper_1410_1629_gb300/csrc/rt_internal.h", "paper_1410_1629_gb300/csrc/rt_math.cuh",
+                  "paper_1410_1629_gb300/csrc/rt_transport.cuh", "include/rt.h", "paper_1410_1629_gb300/build.py"]
 
 
 def column_tables(prob):
@@ -76,18 +76,14 @@ def column_tables(prob):
 
 
 def source_code(text, name):
-    """The code of a CUDA source without its // comments and blank lines (a
-    comment edit leaves the kernel, and so its traffic, unchanged); other
+    """The code of a CUDA source or header without its comments and blank lines
+    (a comment edit leaves the kernel, and so its traffic, unchanged); other
     files whole."""
     if not name.endswith((".cu", ".cuh", ".h")):
         return text
-    out = []
-    for line in text.splitlines():
-        i = line.find("//")
-        line = (line if i < 0 else line[:i]).rstrip()
-        if line:
-            out.append(line)
-    return "\n".join(out)
+    import re
+    code = re.sub(r"//[^\n]*|/\*.*?\*/", "", text, flags=re.S)
+    return "\n".join(line.rstrip() for line in code.splitlines() if line.strip())
 
 
 def kernel_sources_hash(read=None):
