@@ -388,9 +388,13 @@ double host_emission(const DustArgs& A, double T) {
 }
 
 constexpr int kTableOctaves = 192;
-// Cells from which the table pays: building it costs as much as solving about
-// 28 k cells, in one wave.
-constexpr long long kTableCells = 1 << 16;
+// Cells from which the table pays: those of one wave of direct solves (a block of
+// 256 on each of 152 SMs, the FP64 pipe's share of each).  Up to there both take
+// the time of one root (484 us for 32768 cells by the table, 487 us solved by
+// themselves; 24 wavelengths, 4 to 60 K), and from there on the direct solves
+// take a second wave (46656 cells 495 against 868 us, 64000 cells 497 against 872
+// us).
+constexpr long long kTableCells = 152 * 256;
 
 }  // namespace
 

@@ -43,3 +43,29 @@ def test_rows_whose_last_coefficient_vanishes(strength):
     # ln T carries 2 ulp of a number below 9.3 on both sides, E's rounding over its slope (at least 1) adds less
     np.testing.assert_allclose(T_g, T_o, rtol=1e-14, atol=0)
     assert held_g == held_o == 0
+
+
+@pytest.mark.parametrize("shape", [(1, 127, 306), (1, 127, 307), (36, 36, 36)])  # 38862, 38989 (line: 38912) and 46656 cells
+def test_grids_around_the_table_s_line(shape):
+    from oracle import oracle as O
+    rng = np.random.default_rng(8)
+    nz, ny, nx = shape
+    grid = W.cartesian_grid([0.0, float(nx), 0.0, float(ny), 0.0, float(nz)], rng.lognormal(0.0, 1.0, shape).astype(np.float32))
+    n_lambda = 8
+    wl = np.geomspace(0.1, 1000.0, n_lambda)
+    kappa, albedo, g = W.panchromatic_optics(wl, 1.25)
+    base = W.panchromatic_disk(n_cells=4, n_lambda=n_lambda, n_pix=8)
+    prob = W.replace(base, grid=grid, wavelengths=wl, kappa=kappa, albedo=albedo, g=g,
+                     sources=[W.replace(base.sources[0], lum=np.ones(n_lambda))])
+    S = 1e11
+    total = O.dust_emission(prob, np.exp(rng.uniform(np.log(0.7), np.log(1.4e4), grid.n_cells)), S).sum(axis=0)
+    total[rng.uniform(size=total.size) < 0.05] = 0.0
+    ab = np.full((n_lambda, 1), 1.0 / n_lambda) * total[None, :]
+    T_o, held_o = O.dust_temperature(prob, ab, S)
+    sim = rt.Simulation(prob)
+    try:
+        T_g, held_g = sim.dust_temperature(S, absorption=ab)
+    finally:
+        sim.close()
+    np.testing.assert_allclose(T_g, T_o, rtol=1e-14, atol=0)  # (as above; exact planes and masses)
+    assert held_g == held_o and held_o > 0
