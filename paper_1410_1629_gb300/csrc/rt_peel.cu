@@ -30,13 +30,12 @@ namespace {
 // (frame and SED; the whole calculation) 10.3 -> 8.8 ms, ragged disk 2.53 ->
 // 2.44 ms.
 
-// Resident blocks per SM that the walks' register allocation aims at (disk
-// galaxy and panchromatic disk flat between 4 and 6; octree 3 / 4 / 5: 31.7 /
-// 27.8 / 29.2 ms, k-d tree 31.5 / 30.0 / 32.7, Voronoi 29.4 / 25.6 / 26.2).
-template <class G>
+// Resident blocks per SM that the walks' register allocation aims at (octree 3 /
+// 4 / 5: 31.7 / 27.8 / 29.2 ms, k-d tree 31.5 / 30.0 / 32.7, Voronoi 29.4 / 25.6 /
+// 26.2, before k_peel_together and the paired face planes; cartesian 4 / 5 / 6:
+// 7.45 / 7.44 / 7.51 ms per 4e6 packets of the disk galaxy, without spills only at
+// 4).
 constexpr int kPeelBlocks = 4;
-template <>
-constexpr int kPeelBlocks<tr::CartGrid> = 5;
 
 // Whether the walks of a warp are kept together crossing by crossing
 // (k_peel_together) or only start together (k_peel_sorted): trees.  On the other
@@ -170,7 +169,7 @@ __device__ __forceinline__ void add_counts(const FwdParams& P, const Counts& sum
 // The walks of the sorted records and their deposits; one record per thread,
 // consecutive threads on consecutive records of the order.
 template <class G>
-__global__ void __launch_bounds__(tr::kBlock, kPeelBlocks<G>) k_peel_sorted(const __grid_constant__ FwdParams P,
+__global__ void __launch_bounds__(tr::kBlock, kPeelBlocks) k_peel_sorted(const __grid_constant__ FwdParams P,
                                                                             const unsigned* __restrict__ perm) {
   tr::load_grid_cache<G>(P);
   __syncthreads();
@@ -235,7 +234,7 @@ constexpr int kSegment = 256, kRefill = 24;
 // walks spill: octree 18.7 -> 20.7 ms; saved 19.9 ms).  Without any the plain
 // kernel runs.
 template <class G, bool kShare>
-__global__ void __launch_bounds__(tr::kBlock, kPeelBlocks<G>) k_peel_together(const __grid_constant__ FwdParams P,
+__global__ void __launch_bounds__(tr::kBlock, kPeelBlocks) k_peel_together(const __grid_constant__ FwdParams P,
                                                                             const unsigned* __restrict__ perm) {
   tr::load_grid_cache<G>(P);
   __syncthreads();
