@@ -22,8 +22,6 @@
 #include "rt_internal.h"
 
 namespace rtk {
-// Zero entries after the Voronoi neighbour and face arrays.
-constexpr long long kVorPad = 2;
 // rt_layout.cu: n doubles from device memory to memory the device addresses.
 cudaError_t launch_copy_f64(const double* src, double* dst, long long n, cudaStream_t stream);
 }  // namespace rtk
@@ -925,21 +923,18 @@ rt_status rt_create_grid(rt_ctx c, const rt_grid_desc* d, int32_t* grid_id) {
                           cudaMemcpyHostToDevice));
   }
   if (d->kind == RT_GRID_VORONOI) {
-    // neighbour ids and face planes in pairs, with kVorPad zero entries after
-    // the last list
-    const size_t n_alloc = vor_face.size() + kVorPad;
+    // neighbour ids and face planes in pairs (none for a single cell)
+    const size_t n_faces = vor_face.size(), n_alloc = std::max<size_t>(1, n_faces);
     RT_CUDA(c, pool_alloc(c, &c->d_child, n_alloc * sizeof(int32_t)));
-    RT_CUDA(c, cudaMemset(c->d_child, 0, n_alloc * sizeof(int32_t)));
-    if (n_nodes > 0)
-      RT_CUDA(c, cudaMemcpy(c->d_child, vor_nbr.data(), vor_nbr.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
+    RT_CUDA(c, pool_alloc(c, &c->d_face, n_alloc * sizeof(float4)));
+    if (n_faces > 0) {
+      RT_CUDA(c, cudaMemcpy(c->d_child, vor_nbr.data(), n_faces * sizeof(int32_t), cudaMemcpyHostToDevice));
+      RT_CUDA(c, cudaMemcpy(c->d_face, vor_face.data(), n_faces * sizeof(float4), cudaMemcpyHostToDevice));
+    }
     RT_CUDA(c, pool_alloc(c, &c->d_site, vor_site.size() * sizeof(float4)));
     RT_CUDA(c, cudaMemcpy(c->d_site, vor_site.data(), vor_site.size() * sizeof(float4), cudaMemcpyHostToDevice));
     RT_CUDA(c, pool_alloc(c, &c->d_face_off, vor_off.size() * sizeof(unsigned)));
     RT_CUDA(c, cudaMemcpy(c->d_face_off, vor_off.data(), vor_off.size() * sizeof(unsigned), cudaMemcpyHostToDevice));
-    RT_CUDA(c, pool_alloc(c, &c->d_face, n_alloc * sizeof(float4)));
-    RT_CUDA(c, cudaMemset(c->d_face, 0, n_alloc * sizeof(float4)));
-    if (n_nodes > 0)
-      RT_CUDA(c, cudaMemcpy(c->d_face, vor_face.data(), vor_face.size() * sizeof(float4), cudaMemcpyHostToDevice));
     RT_CUDA(c, pool_alloc(c, &c->d_bucket_seed, vor_seed.size() * sizeof(int)));
     RT_CUDA(c, cudaMemcpy(c->d_bucket_seed, vor_seed.data(), vor_seed.size() * sizeof(int), cudaMemcpyHostToDevice));
     for (int a = 0; a < 3; ++a) c->vb_n[a] = vb_n[a];
@@ -984,7 +979,7 @@ rt_status rt_create_grid(rt_ctx c, const rt_grid_desc* d, int32_t* grid_id) {
   }
   std::memcpy(c->bounds, d->bounds, sizeof c->bounds);
   c->n_cells = n_cells;
-  c->n_nodes = d->kind == RT_GRID_VORONOI ? (long long)vor_face.size() + kVorPad : n_nodes;  // as allocated
+  c->n_nodes = n_nodes;
   if (d->kind == RT_GRID_OCTREE) c->order_child = std::move(child_host);
   c->order_site = std::move(vor_site);
   c->order = std::move(order);
