@@ -379,8 +379,8 @@ rt_status rt_read_absorption(rt_ctx ctx, double* dst, size_t n_elems, int32_t ds
  * Cartesian and rectilinear grids. */
 
 /* Equilibrium temperature of every cell: the T at which it emits the
- * luminosity it absorbed summed over the wavelengths, found by bisection in
- * ln T between t_min and t_max (64 halvings).  absorption: row-major float64
+ * luminosity it absorbed summed over the wavelengths, between t_min and t_max,
+ * to about 1e-15 (Newton steps in ln T, or on larger grids a tabulated inverse).  absorption: row-major float64
  * [n_lambda][n_cells] (host, or device with absorption_on_device = 1), or
  * NULL for the context's absorption tallies.  temperature: float64 [n_cells]
  * (host, or device with dst_on_device = 1): 0 for cells without dust or
@@ -577,7 +577,8 @@ rt_status rt_batch_read_stats(rt_ctx ctx, int32_t batch_id, rt_stats* out);
 /* Choose control_lanes and the packets per work-list run by timing launches
  * of a fraction (0 < fraction <= 1) of every model's packets for each
  * candidate (control_lanes 8, 12, ..., 32; runs of 64, 256, 1024, 4096
- * packets, without those far too short for the whole batch); the choice is kept for later launches with control_lanes 0 and
+ * packets, without those far too short for the whole batch); the choice is kept
+ * for later launches with control_lanes 0 and
  * written to *control_lanes and *run_packets if not NULL.  The images and
  * tallies are zeroed afterwards.  Synchronous.  Errors: RT_ERR_ARG,
  * RT_ERR_CUDA. */

@@ -89,8 +89,8 @@ struct rt_ctx_s {
   float* d_density = nullptr;
   int32_t* d_child = nullptr;
   float* d_edges = nullptr;  // rectilinear grids: FP32 edges, x then y then z (nx + ny + nz + 3)
-  // Voronoi grids: sites, face offsets, face planes (neighbour ids in
-  // d_child, n_nodes faces), bucket seeds
+  // Voronoi grids: sites, face offsets, face planes (neighbour ids in d_child), both
+  // in pairs, bucket seeds
   float4* d_site = nullptr;
   unsigned* d_face_off = nullptr;
   float4* d_face = nullptr;
@@ -170,7 +170,7 @@ struct rt_ctx_s {
   unsigned long long tape_n = 0, tape_first = 0, tape_seed = 0, tape_norm = 0;
   int tape_max_events = 0, tape_weight_cut = 0, tape_peel_e = 0, tape_peel_s = 0, tape_model = 0;
   double tape_w_min = 0.0;
-  // the sorted peel-off pass (cartesian launches): records, their order,
+  // the sorted peel-off pass: records, their order,
   // counts per sort key and per scan tile, the record counter; the count of
   // the last launch comes back through pinned memory without a wait and sizes
   // the buffer of later launches

@@ -19,10 +19,12 @@ namespace {
 // order of the FP64 image additions differs from walking the peel-off in place.
 //
 // On trees and Voronoi grids every frame's peel-offs walk (80 % of the
-// crossings): clumpy octree 52.0 -> 44.2 ms per 2e6 packets, k-d tree 70.0 ->
-// 50.0 ms, Voronoi disk 52.8 -> 38.3 ms per 1.5e6; 16, 10 and 14 lanes active
-// per instruction of the sorted walks against 9, 7 and 6 in place.  Bound by
-// instruction issue (63-68 % of cycles), trees in the descent to the next leaf.
+// crossings): clumpy octree 52.0 -> 35.2 ms per 2e6 packets, k-d tree 70.0 ->
+// 37.9 ms, Voronoi disk 52.8 -> 35.7 ms per 1.5e6 (the whole launch; the trees'
+// walks kept together crossing by crossing, below); 23, 21 and 14 lanes active per
+// instruction of the sorted walks against 9, 7 and 6 in place.  Bound by
+// instruction issue (61-64 % of cycles), trees in the descent to the next leaf,
+// Voronoi grids also by the face planes' wavefronts (74 % of the L1's).
 //
 // Instruments that look along the same direction (a frame and an SED of one
 // view) see the same optical depth and phase-function value: one record and one

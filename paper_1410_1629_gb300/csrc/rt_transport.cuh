@@ -841,7 +841,8 @@ struct BinGrid {
 
   // Into the neighbouring leaf through face `axis`: the exit point with the
   // other coordinates kept inside the current leaf (the walk never steps
-  // back across a face), located from the root.
+  // back across a face), located from the leaf's rope for that face, or from the
+  // root when it lies on an edge of the leaf.
   __device__ static __forceinline__ bool advance(const FwdParams& P, float3 x, float3 d, float3, int axis, Walk& w,
                                                  Scratch&) {
     const float da = pick(axis, d);
@@ -1053,7 +1054,7 @@ struct VorGrid {
   __device__ static __forceinline__ int id(const FwdParams&, const Walk& w) { return w.leaf; }
   __device__ static __forceinline__ int cell_id(const FwdParams&, const Cell& c) { return c.leaf; }
   __device__ static __forceinline__ int sort_place(const FwdParams& P, const Cell& c) { return __ldg(&P.cell_rank[c.leaf]); }
-  // (init only uses the middle of a known leaf's box)
+  // (init only uses the cell's id)
   __device__ static __forceinline__ Cell sorted_cell(const FwdParams& P, unsigned place) {
     const float4 c = __ldg(&P.rank_cell[place]);
     return Cell{__float_as_int(c.w), {c.x, c.y, c.z}, {c.x, c.y, c.z}};
