@@ -18,7 +18,7 @@
 // mass, is one function for all cells of a launch and its inverse is tabulated
 // once per call and looked up per cell, and the thermal emission uses the
 // library's own a / (exp(x) - 1) (rt_math.cuh).  192 x 192 x 128 cells, 24
-// wavelengths: temperatures 44.9 ms, emission and running sums 10.3 ms; now 7.6
+// wavelengths: temperatures 44.9 ms, emission and running sums 10.3 ms; now 7.0
 // ms together with the read-out (56.0 before).
 #include <algorithm>
 #include <cmath>

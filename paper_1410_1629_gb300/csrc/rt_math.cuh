@@ -1,25 +1,29 @@
 // Double-precision exponential and logarithm of the forced-scattering
 // inversion (Sect. 1) and of the dust's emission, written for a device whose
 // FP64 pipe issues one warp instruction per 16 cycles of an SM, whatever its
-// active lanes: 1 - exp(-x) in 15 FP64 instructions, exp(x) - 1 in 16, -ln(1 -
-// v) in 18, table-driven (P. T. P. Tang, "Table-driven implementation of the
+// active lanes: 1 - exp(-x) and exp(x) - 1 in 11 FP64 instructions, -ln(1 - v)
+// in 14, table-driven (P. T. P. Tang, "Table-driven implementation of the
 // exponential function in IEEE floating-point arithmetic", ACM TOMS 15, 1989,
-// and "... of the logarithm function ...", ACM TOMS 16, 1990).  The two largest
-// terms of a result are added with their rounding error, which joins the small
-// terms, so that little but the result's own rounding is left.  The range
-// reduction, the remainders of constants and the high-order terms of the series
-// use integer and FP32 instructions; where an FP32 value enters an FP64 sum its
-// weight there is below 2^-33, so its rounding stays below 2^-56 of the result.
+// and "... of the logarithm function ...", ACM TOMS 16, 1990).  The tables hold
+// the leading bits of their values apart, so that the largest part of a result is
+// exact and the rest, which is small against it, carries the roundings.  Where
+// the result is as small as the reduced argument, the argument is not reduced.
+// The range reduction, the remainders of constants and the high-order terms of
+// the series use integer and FP32 instructions; where an FP32 value enters an
+// FP64 sum its weight there is below 2^-32, so its rounding stays below 2^-56 of
+// the result, 2^-55.5 at the longest series' ends.
 //
 // Against 113-bit arithmetic (2e5 arguments in each of 17 ranges, on the
-// device): 1 - exp(-x) and exp(x) - 1 within 0.51 ulp, -ln(1 - v) within 0.53
-// ulp, their rms errors within 0.01 % of those of the correctly rounded values
+// device): 1 - exp(-x) within 0.55 ulp, exp(x) - 1 within 0.56, -ln(1 - v) within
+// 0.60, their rms errors within 0.2 % of those of the correctly rounded values
 // (0.289 ulp); the CUDA library's expm1 and log1p: 1.15 and 1.49 ulp, rms up to
-// 0.325 and 0.387.  Measured with the library's functions in their place (time
-// over that with these): 256 batched models (110 ms) 1.034, a 48^3 fit with an
-// absorption target (20.5 ms) 1.053, dust temperatures and emission (7.6 ms)
-// 1.27, 1e4 packets of a 32^3 cube (0.39 ms) 1.034, a taped forward launch with
-// its adjoint (32.7 ms) 0.985.
+// 0.325 and 0.387, in no range more than 0.1 % below these.  Measured with the
+// library's functions in their place (time over that with these): 256 batched
+// models (110 ms) 1.056, a 48^3 fit with an absorption target (20.3 ms) 1.070,
+// dust temperatures and emission (7.0 ms) 1.37, 1e4 packets of a 32^3 cube (0.38
+// ms) 1.04, a taped forward launch with its adjoint (32.7 ms) 0.99.  (A form that
+// kept the rounding errors of the leading sums by two-sums, 15, 16 and 18
+// instructions: 0.53 ulp, a replayed adjoint of 1e7 packets 414 against 392 ms.)
 //
 // The file compiles as CUDA (device functions) and as plain C++ (for tests).
 #pragma once
@@ -74,493 +78,484 @@ RT_FN float cut(double v) {
   return float_of((top & 0x80000000u) | ((unsigned)(be - 896) << 23) | ((unsigned)(b >> 29) & 0x7fffffu));
 }
 
-// 2^(-j/128), and 1 - 2^(-j/128), each as a double and its remainder
+// 2^(-j/128), to 13 bits, and the remainder: hi - 2^(-j/128); in kExpUpTable
+// 2^(j/128), to 13 bits, and the remainder 2^(j/128) - hi
 struct ExpEntry {
-  double t, a;
-  float t_lo, a_lo;
-};
-// 2^(j/128), and 2^(j/128) - 1, likewise
-struct alignas(16) ExpUpEntry {
-  double t, t_lo, a, a_lo;
+  double t, hi, lo;
 };
 // a reciprocal of the middle of [1/2 + j/256, 1/2 + (j + 1)/256] to 13 bits
-// (1 for the last interval), the same less one, and its logarithm as a double
-// and its remainder
+// (1 for the last four intervals), the same less one, and its logarithm to a multiple
+// of 2^-40 and its remainder
 struct alignas(16) LogEntry {
   double rc, c, ln;
   float ln_lo;
 };
 
-// ln 2 / 128 as a double and its remainder, ln 2 to 43 bits (its products with
-// exponents are exact) and its remainder
+// ln 2 / 128 as a double and its remainder, ln 2 to a multiple of 2^-40 (sums of
+// its multiples and of table entries are exact) and its remainder
 constexpr double kLn2Over128 = 0x1.62e42fefa39efp-8;
 constexpr float kLn2Over128Lo = 0x1.abc9e3b39803fp-63;
-constexpr double kLn2 = 0x1.62e42fefa38p-1;
-constexpr float kLn2Lo = 0x1.ef35793c7673p-45;
+constexpr double kLn2 = 0x1.62e42fefa4p-1;
+constexpr float kLn2Lo = -0x1.8432a1b0e2634p-43;
 RT_TABLE ExpEntry kExpTable[128] = {
-    {0x1.0000000000000p+0, 0x0.0p+0, 0x0.0p+0f, 0x0.0p+0f},
-    {0x1.fd3c22b8f71f1p-1, 0x1.61eea3847077bp-8, 0x1.2eb74ap-58f, 0x1.148b6ap-62f},
-    {0x1.fa7c1819e90d8p-1, 0x1.60f9f985bc9f4p-7, 0x1.748540p-56f, 0x1.6f5818p-61f},
-    {0x1.f7bfdad9cbe14p-1, 0x1.0804a4c683d8fp-6, -0x1.dbb12ep-55f, -0x1.13b4c0p-61f},
-    {0x1.f50765b6e4540p-1, 0x1.5f134923757f3p-6, 0x1.9d3e12p-55f, 0x1.60f692p-62f},
-    {0x1.f252b376bba97p-1, 0x1.b5a991288ad16p-6, 0x1.3a1a5cp-55f, 0x1.796904p-61f},
-    {0x1.efa1bee615a27p-1, 0x1.05e4119ea5d89p-5, 0x1.dc7f48p-55f, -0x1.c7f486p-59f},
-    {0x1.ecf482d8e67f1p-1, 0x1.30b7d271980f7p-5, -0x1.c93f3cp-55f, 0x1.27e768p-60f},
-    {0x1.ea4afa2a490dap-1, 0x1.5b505d5b6f268p-5, -0x1.e9c232p-55f, -0x1.63dce8p-59f},
-    {0x1.e7a51fbc74c83p-1, 0x1.85ae0438b37cbp-5, 0x1.2d522cp-55f, 0x1.2add36p-59f},
-    {0x1.e502ee78b3ff6p-1, 0x1.afd11874c009ep-5, 0x1.39e898p-56f, -0x1.cf44c0p-59f},
-    {0x1.e264614f5a129p-1, 0x1.d9b9eb0a5ed76p-5, -0x1.7b6278p-55f, -0x1.2761fap-61f},
-    {0x1.dfc97337b9b5fp-1, 0x1.01b466423250ap-4, -0x1.1a5cd4p-55f, 0x1.a5cd50p-59f},
-    {0x1.dd321f301b460p-1, 0x1.166f067f25cfep-4, 0x1.2da578p-55f, -0x1.6d2bbcp-58f},
-    {0x1.da9e603db3285p-1, 0x1.2b0cfe1266bd4p-4, 0x1.c23006p-55f, 0x1.ee7fccp-58f},
-    {0x1.d80e316c98398p-1, 0x1.3f8e749b3e342p-4, -0x1.11ec18p-55f, 0x1.1ec18cp-59f},
-    {0x1.d5818dcfba487p-1, 0x1.53f391822dbc7p-4, 0x1.2ed02ep-56f, -0x1.76816cp-59f},
-    {0x1.d2f87080d89f2p-1, 0x1.683c7bf93b074p-4, -0x1.d487b8p-55f, -0x1.5bc248p-58f},
-    {0x1.d072d4a07897cp-1, 0x1.7c695afc3b424p-4, -0x1.cbc374p-55f, -0x1.a1e45ep-58f},
-    {0x1.cdf0b555dc3fap-1, 0x1.907a55511e032p-4, -0x1.dd83b6p-56f, -0x1.13e256p-59f},
-    {0x1.cb720dcef9069p-1, 0x1.a46f918837cb7p-4, 0x1.503cbep-57f, 0x1.5f8686p-58f},
-    {0x1.c8f6d9406e7b5p-1, 0x1.b84935fc8c257p-4, 0x1.1acbc4p-57f, 0x1.ca6876p-58f},
-    {0x1.c67f12e57d14bp-1, 0x1.cc0768d4175a6p-4, 0x1.2884e0p-55f, -0x1.442700p-58f},
-    {0x1.c40ab5fffd07ap-1, 0x1.dfaa500017c2dp-4, 0x1.b4537ep-55f, -0x1.a29bf0p-58f},
-    {0x1.c199bdd85529cp-1, 0x1.f332113d56b1fp-4, 0x1.110658p-56f, -0x1.10658ap-60f},
-    {0x1.bf2c25bd71e09p-1, 0x1.034f690a387dep-3, -0x1.efdca4p-55f, -0x1.0235c0p-59f},
-    {0x1.bcc1e904bc1d2p-1, 0x1.0cf85bed0f8b7p-3, 0x1.23dd08p-56f, 0x1.b845f0p-57f},
-    {0x1.ba5b030a1064ap-1, 0x1.1693f3d7be6dap-3, -0x1.efcd30p-55f, -0x1.032cf2p-59f},
-    {0x1.b7f76f2fb5e47p-1, 0x1.20224341286e4p-3, -0x1.5584f8p-57f, 0x1.5584f8p-57f},
-    {0x1.b59728de5593ap-1, 0x1.29a35c86a9b1ap-3, -0x1.c71dfcp-55f, -0x1.c71022p-58f},
-    {0x1.b33a2b84f15fbp-1, 0x1.331751ec3a814p-3, -0x1.2805e4p-58f, 0x1.2805e4p-58f},
-    {0x1.b0e07298db666p-1, 0x1.3c7e359c9266ap-3, -0x1.bdef54p-55f, -0x1.0842acp-57f},
-    {0x1.ae89f995ad3adp-1, 0x1.45d819a94b14bp-3, 0x1.7a1cd4p-55f, -0x1.e8734ep-57f},
-    {0x1.ac36bbfd3f37ap-1, 0x1.4f25100b03219p-3, -0x1.f9234cp-56f, -0x1.b72cd4p-62f},
-    {0x1.a9e6b5579fdbfp-1, 0x1.58652aa180903p-3, 0x1.0fac90p-55f, -0x1.f5921ep-60f},
-    {0x1.a799e1330b358p-1, 0x1.61987b33d329ep-3, 0x1.bcb7ecp-55f, 0x1.0d204ep-57f},
-    {0x1.a5503b23e255dp-1, 0x1.6abf137076a8ep-3, -0x1.d2f6eep-55f, -0x1.684892p-58f},
-    {0x1.a309bec4a2d33p-1, 0x1.73d904ed74b33p-3, 0x1.6305c8p-55f, -0x1.8c1720p-57f},
-    {0x1.a0c667b5de565p-1, 0x1.7ce6612886a6dp-3, -0x1.359496p-55f, 0x1.aca4aep-58f},
-    {0x1.9e86319e32323p-1, 0x1.85e7398737374p-3, 0x1.824ca8p-57f, -0x1.824ca8p-57f},
-    {0x1.9c49182a3f090p-1, 0x1.8edb9f5703dc0p-3, 0x1.c7c46cp-57f, -0x1.c7c46cp-57f},
-    {0x1.9a0f170ca07bap-1, 0x1.97c3a3cd7e119p-3, -0x1.173bdap-55f, 0x1.73bd92p-59f},
-    {0x1.97d829fde4e50p-1, 0x1.a09f58086c6c2p-3, -0x1.d185b8p-55f, -0x1.73d242p-58f},
-    {0x1.95a44cbc8520fp-1, 0x1.a96ecd0deb7c4p-3, -0x1.64b7cap-57f, 0x1.64b7cap-57f},
-    {0x1.93737b0cdc5e5p-1, 0x1.b23213cc8e86cp-3, -0x1.75fc78p-58f, 0x1.75fc78p-58f},
-    {0x1.9145b0b91ffc6p-1, 0x1.bae93d1b800eap-3, -0x1.dd6792p-55f, -0x1.14c368p-58f},
-    {0x1.8f1ae99157736p-1, 0x1.c39459baa2327p-3, 0x1.5cc13ap-56f, 0x1.467d8cp-57f},
-    {0x1.8cf3216b5448cp-1, 0x1.cc337a52aedd0p-3, -0x1.0d55e4p-57f, 0x1.0d55e4p-57f},
-    {0x1.8ace5422aa0dbp-1, 0x1.d4c6af7557c93p-3, 0x1.6e9f16p-55f, -0x1.ba7c56p-57f},
-    {0x1.88ac7d98a6699p-1, 0x1.dd4e099d6659ap-3, 0x1.994c30p-55f, 0x1.9acf44p-57f},
-    {0x1.868d99b4492edp-1, 0x1.e5c9992edb44ep-3, -0x1.fc6f8ap-55f, -0x1.c83b22p-62f},
-    {0x1.8471a4623c7adp-1, 0x1.ee396e770e14dp-3, -0x1.8d684ap-56f, -0x1.ca5ed8p-58f},
-    {0x1.82589994cce13p-1, 0x1.f69d99accc7b6p-3, -0x1.d4c1dep-55f, -0x1.59f116p-58f},
-    {0x1.80427543e1a12p-1, 0x1.fef62af0797b9p-3, -0x1.27c866p-55f, 0x1.3e4332p-58f},
-    {0x1.7e2f336cf4e62p-1, 0x1.03a199261633cp-2, 0x1.05d02cp-57f, -0x1.05d02cp-57f},
-    {0x1.7c1ed0130c132p-1, 0x1.07c25fd9e7d9bp-2, 0x1.f124cep-55f, 0x1.db665ep-60f},
-    {0x1.7a11473eb0187p-1, 0x1.0bdd71829fcf2p-2, -0x1.41577ep-56f, 0x1.41577ep-56f},
-    {0x1.780694fde5d3fp-1, 0x1.0ff2d60434581p-2, 0x1.866b80p-55f, 0x1.e651fep-57f},
-    {0x1.75feb564267c9p-1, 0x1.14029537b306fp-2, -0x1.024596p-55f, -0x1.fb74d6p-56f},
-    {0x1.73f9a48a58174p-1, 0x1.180cb6eb4fd19p-2, -0x1.0a8d96p-55f, -0x1.eae4d2p-56f},
-    {0x1.71f75e8ec5f74p-1, 0x1.1c1142e274118p-2, -0x1.16e478p-56f, 0x1.16e478p-56f},
-    {0x1.6ff7df9519484p-1, 0x1.201040d5cd6f8p-2, -0x1.83c0f2p-56f, 0x1.83c0f2p-56f},
-    {0x1.6dfb23c651a2fp-1, 0x1.2409b8735cba2p-2, -0x1.bbe3a6p-58f, 0x1.bbe3a6p-58f},
-    {0x1.6c012750bdabfp-1, 0x1.27fdb15e84a82p-2, -0x1.289566p-57f, 0x1.289566p-57f},
-    {0x1.6a09e667f3bcdp-1, 0x1.2bec333018867p-2, -0x1.bdd342p-55f, -0x1.08b2fcp-57f},
-    {0x1.68155d44ca973p-1, 0x1.2fd545766ad1ap-2, 0x1.038ae4p-58f, -0x1.038ae4p-58f},
-    {0x1.6623882552225p-1, 0x1.33b8efb55bbb7p-2, -0x1.bb6098p-55f, -0x1.127d9ep-57f},
-    {0x1.6434634ccc320p-1, 0x1.37973966679c0p-2, -0x1.c483c8p-56f, 0x1.c483c8p-56f},
-    {0x1.6247eb03a5585p-1, 0x1.3b7029f8b54f7p-2, -0x1.383c18p-55f, -0x1.8f87d0p-56f},
-    {0x1.605e1b976dc09p-1, 0x1.3f43c8d1247efp-2, -0x1.3e242ap-55f, -0x1.83b7acp-56f},
-    {0x1.5e76f15ad2148p-1, 0x1.43121d4a5bd6fp-2, 0x1.ba6f94p-55f, 0x1.1641b4p-57f},
-    {0x1.5c9268a5946b7p-1, 0x1.46db2eb4d7292p-2, 0x1.c4b1b8p-61f, -0x1.c4b1b8p-61f},
-    {0x1.5ab07dd485429p-1, 0x1.4a9f0456f57adp-2, 0x1.6324c0p-55f, 0x1.39b680p-56f},
-    {0x1.58d12d497c7fdp-1, 0x1.4e5da56d07006p-2, 0x1.295e16p-56f, -0x1.295e16p-56f},
-    {0x1.56f4736b527dap-1, 0x1.521719295b04bp-2, 0x1.9bb2c0p-55f, 0x1.913500p-57f},
-    {0x1.551a4ca5d920fp-1, 0x1.55cb66b44dbe2p-2, -0x1.d689cep-56f, 0x1.d689cep-56f},
-    {0x1.5342b569d4f82p-1, 0x1.597a952c560fcp-2, -0x1.07abe2p-56f, 0x1.07abe2p-56f},
-    {0x1.516daa2cf6642p-1, 0x1.5d24aba61337cp-2, -0x1.f76856p-56f, 0x1.f76856p-56f},
-    {0x1.4f9b2769d2ca7p-1, 0x1.60c9b12c5a6b3p-2, -0x1.4b309ep-55f, -0x1.699ec6p-56f},
-    {0x1.4dcb299fddd0dp-1, 0x1.6469acc0445e5p-2, 0x1.8ecdbcp-55f, 0x1.c4c910p-57f},
-    {0x1.4bfdad5362a27p-1, 0x1.6804a5593abb2p-2, 0x1.d4397ap-57f, -0x1.d4397ap-57f},
-    {0x1.4a32af0d7d3dep-1, 0x1.6b9aa1e505843p-2, 0x1.9cb630p-55f, 0x1.8d2744p-57f},
-    {0x1.486a2b5c13cd0p-1, 0x1.6f2ba947d8660p-2, 0x1.3c1a3cp-57f, -0x1.3c1a3cp-57f},
-    {0x1.46a41ed1d0057p-1, 0x1.72b7c25c5ff51p-2, 0x1.c944bep-55f, 0x1.b5da18p-58f},
-    {0x1.44e086061892dp-1, 0x1.763ef3f3ceda6p-2, 0x1.89b7a0p-60f, -0x1.89b7a0p-60f},
-    {0x1.431f5d950a897p-1, 0x1.79c144d5eaed2p-2, -0x1.1c7ddep-56f, 0x1.1c7ddep-56f},
-    {0x1.4160a21f72e2ap-1, 0x1.7d3ebbc11a3acp-2, -0x1.ef3692p-59f, 0x1.ef3692p-59f},
-    {0x1.3fa4504ac801cp-1, 0x1.80b75f6a6ffc9p-2, -0x1.7d0240p-55f, -0x1.05fb80p-56f},
-    {0x1.3dea64c123422p-1, 0x1.842b367db97bcp-2, 0x1.ada092p-56f, -0x1.ada092p-56f},
-    {0x1.3c32dc313a8e5p-1, 0x1.879a479d8ae37p-2, -0x1.efff84p-55f, -0x1.0007c8p-59f},
-    {0x1.3a7db34e59ff7p-1, 0x1.8b0499634c012p-2, -0x1.5e436ep-57f, 0x1.5e436ep-57f},
-    {0x1.38cae6d05d866p-1, 0x1.8e6a325f44f35p-2, -0x1.e958d4p-55f, -0x1.6a72c4p-59f},
-    {0x1.371a7373aa9cbp-1, 0x1.91cb1918aac6bp-2, -0x1.63aeacp-55f, -0x1.38a2a8p-56f},
-    {0x1.356c55f929ff1p-1, 0x1.9527540dac01ep-2, -0x1.b5cee6p-56f, 0x1.b5cee6p-56f},
-    {0x1.33c08b26416ffp-1, 0x1.987ee9b37d201p-2, 0x1.327218p-55f, 0x1.9b1bd0p-56f},
-    {0x1.32170fc4cd831p-1, 0x1.9bd1e07664f9ep-2, 0x1.a9ce78p-56f, -0x1.a9ce78p-56f},
-    {0x1.306fe0a31b715p-1, 0x1.9f203eb9c91d6p-2, 0x1.6f46aep-56f, -0x1.6f46aep-56f},
-    {0x1.2ecafa93e2f56p-1, 0x1.a26a0ad83a154p-2, 0x1.1ca0f4p-57f, -0x1.1ca0f4p-57f},
-    {0x1.2d285a6e4030bp-1, 0x1.a5af4b237f9e9p-2, 0x1.002476p-55f, 0x1.ffb716p-56f},
-    {0x1.2b87fd0dad990p-1, 0x1.a8f005e4a4ce0p-2, -0x1.10adcep-60f, 0x1.10adcep-60f},
-    {0x1.29e9df51fdee1p-1, 0x1.ac2c415c0423ep-2, 0x1.612e8ap-56f, -0x1.612e8ap-56f},
-    {0x1.284dfe1f56381p-1, 0x1.af6403c1538ffp-2, -0x1.a4c3a8p-55f, -0x1.6cf15cp-57f},
-    {0x1.26b4565e27cddp-1, 0x1.b2975343b0646p-2, 0x1.2bd33ap-56f, -0x1.2bd33ap-56f},
-    {0x1.251ce4fb2a63fp-1, 0x1.b5c63609ab382p-2, 0x1.ac155cp-56f, -0x1.ac155cp-56f},
-    {0x1.2387a6e756238p-1, 0x1.b8f0b23153b8fp-2, 0x1.9b07ecp-55f, 0x1.93e052p-57f},
-    {0x1.21f49917ddc96p-1, 0x1.bc16cdd0446d4p-2, 0x1.2a97eap-56f, -0x1.2a97eap-56f},
-    {0x1.2063b88628cd6p-1, 0x1.bf388ef3ae654p-2, 0x1.dc7758p-56f, -0x1.dc7758p-56f},
-    {0x1.1ed5022fcd91dp-1, 0x1.c255fba064dc7p-2, -0x1.1df980p-55f, -0x1.c40d00p-56f},
-    {0x1.1d4873168b9aap-1, 0x1.c56f19d2e8cabp-2, 0x1.e016e0p-55f, 0x1.fe9200p-59f},
-    {0x1.1bbe084045cd4p-1, 0x1.c883ef7f74659p-2, -0x1.953864p-55f, -0x1.ab1e72p-57f},
-    {0x1.1a35beb6fcb75p-1, 0x1.cb94829206916p-2, 0x1.e5b4c8p-56f, -0x1.e5b4c8p-56f},
-    {0x1.18af9388c8deap-1, 0x1.cea0d8ee6e42dp-2, -0x1.11023ep-55f, -0x1.ddfb86p-56f},
-    {0x1.172b83c7d517bp-1, 0x1.d1a8f87055d0ap-2, -0x1.19041cp-56f, 0x1.19041cp-56f},
-    {0x1.15a98c8a58e51p-1, 0x1.d4ace6eb4e35ep-2, 0x1.2406acp-56f, -0x1.2406acp-56f},
-    {0x1.1429aaea92de0p-1, 0x1.d7acaa2ada441p-2, -0x1.32fbfap-55f, -0x1.9a080cp-56f},
-    {0x1.12abdc06c31ccp-1, 0x1.daa847f279c68p-2, -0x1.1b514cp-59f, 0x1.1b514cp-59f},
-    {0x1.11301d0125b51p-1, 0x1.dd9fc5fdb495fp-2, -0x1.6c5104p-55f, -0x1.275df8p-56f},
-    {0x1.0fb66affed31bp-1, 0x1.e0932a00259cap-2, -0x1.b9bedcp-58f, 0x1.b9bedcp-58f},
-    {0x1.0e3ec32d3d1a2p-1, 0x1.e38279a585cbcp-2, 0x1.03a172p-60f, -0x1.03a172p-60f},
-    {0x1.0cc922b7247f7p-1, 0x1.e66dba91b7011p-2, 0x1.01edc2p-55f, 0x1.fc247ep-56f},
-    {0x1.0b5586cf9890fp-1, 0x1.e954f260cede1p-2, 0x1.8a62e4p-55f, 0x1.d6746ep-57f},
-    {0x1.09e3ecac6f383p-1, 0x1.ec3826a7218f9p-2, 0x1.148782p-55f, 0x1.d6f0fcp-56f},
-    {0x1.0874518759bc8p-1, 0x1.ef175cf14c870p-2, 0x1.186be4p-58f, -0x1.186be4p-58f},
-    {0x1.0706b29ddf6dep-1, 0x1.f1f29ac441244p-2, -0x1.c91dfep-56f, 0x1.c91dfep-56f},
-    {0x1.059b0d3158574p-1, 0x1.f4c9e59d4f518p-2, 0x1.d73e2ap-56f, -0x1.d73e2ap-56f},
-    {0x1.04315e86e7f85p-1, 0x1.f79d42f2300f7p-2, -0x1.0a31c2p-55f, -0x1.eb9c7cp-56f},
-    {0x1.02c9a3e778061p-1, 0x1.fa6cb8310ff3ep-2, -0x1.190836p-57f, 0x1.190836p-57f},
-    {0x1.0163da9fb3335p-1, 0x1.fd384ac099995p-2, 0x1.b6129ap-55f, 0x1.27b59ap-57f},
+    {0x1.0000000000000p+0, 0x1.0p+0, 0x0.0p+0},
+    {0x1.fd3c22b8f71f1p-1, 0x1.fd4p-1, 0x1.eea3847077b45p-16},
+    {0x1.fa7c1819e90d8p-1, 0x1.fa8p-1, 0x1.f3f30b793e8b8p-16},
+    {0x1.f7bfdad9cbe14p-1, 0x1.f7cp-1, 0x1.2931a0f63b762p-20},
+    {0x1.f50765b6e4540p-1, 0x1.f5p-1, -0x1.d96db915019d4p-15},
+    {0x1.f252b376bba97p-1, 0x1.f25p-1, -0x1.59bb5dd4ba743p-16},
+    {0x1.efa1bee615a27p-1, 0x1.efap-1, -0x1.bee615a277720p-17},
+    {0x1.ecf482d8e67f1p-1, 0x1.ecfp-1, -0x1.20b6399fc236cp-15},
+    {0x1.ea4afa2a490dap-1, 0x1.ea5p-1, 0x1.41756dbc99e9cp-15},
+    {0x1.e7a51fbc74c83p-1, 0x1.e7ap-1, -0x1.47ef1d320d2d5p-15},
+    {0x1.e502ee78b3ff6p-1, 0x1.e5p-1, -0x1.773c59ffb139fp-16},
+    {0x1.e264614f5a129p-1, 0x1.e26p-1, -0x1.1853d684a284ap-15},
+    {0x1.dfc97337b9b5fp-1, 0x1.dfdp-1, 0x1.a3321192851a6p-15},
+    {0x1.dd321f301b460p-1, 0x1.dd3p-1, -0x1.0f980da3025b5p-16},
+    {0x1.da9e603db3285p-1, 0x1.daap-1, 0x1.9fc24cd7a8f74p-17},
+    {0x1.d80e316c98398p-1, 0x1.d81p-1, 0x1.ce9367c68447bp-17},
+    {0x1.d5818dcfba487p-1, 0x1.d58p-1, -0x1.8dcfba48725dap-17},
+    {0x1.d2f87080d89f2p-1, 0x1.d3p-1, 0x1.e3dfc9d839d48p-15},
+    {0x1.d072d4a07897cp-1, 0x1.d07p-1, -0x1.6a503c4bdc688p-16},
+    {0x1.cdf0b555dc3fap-1, 0x1.cdfp-1, -0x1.6aabb87f3889fp-18},
+    {0x1.cb720dcef9069p-1, 0x1.cb7p-1, -0x1.06e77c8348a82p-16},
+    {0x1.c8f6d9406e7b5p-1, 0x1.c8fp-1, -0x1.b6501b9ed446bp-15},
+    {0x1.c67f12e57d14bp-1, 0x1.c68p-1, 0x1.da3505d696bbep-18},
+    {0x1.c40ab5fffd07ap-1, 0x1.c41p-1, 0x1.528000be164bbp-15},
+    {0x1.c199bdd85529cp-1, 0x1.c1ap-1, 0x1.9089eab58f778p-15},
+    {0x1.bf2c25bd71e09p-1, 0x1.bf3p-1, 0x1.ed21470fbbdfcp-16},
+    {0x1.bcc1e904bc1d2p-1, 0x1.bccp-1, -0x1.e904bc1d2247cp-17},
+    {0x1.ba5b030a1064ap-1, 0x1.ba6p-1, 0x1.3f3d7be6d9efdp-15},
+    {0x1.b7f76f2fb5e47p-1, 0x1.b7fp-1, -0x1.dbcbed791baaap-15},
+    {0x1.b59728de5593ap-1, 0x1.b59p-1, -0x1.ca379564e638ep-15},
+    {0x1.b33a2b84f15fbp-1, 0x1.b34p-1, 0x1.751ec3a814250p-15},
+    {0x1.b0e07298db666p-1, 0x1.b0ep-1, -0x1.ca636d9964211p-19},
+    {0x1.ae89f995ad3adp-1, 0x1.ae9p-1, 0x1.819a94b14a85ep-15},
+    {0x1.ac36bbfd3f37ap-1, 0x1.ac3p-1, -0x1.aeff4fcde7037p-15},
+    {0x1.a9e6b5579fdbfp-1, 0x1.a9ep-1, -0x1.ad55e7f6fd0fbp-15},
+    {0x1.a799e1330b358p-1, 0x1.a7ap-1, 0x1.87b33d329e435p-15},
+    {0x1.a5503b23e255dp-1, 0x1.a55p-1, -0x1.d91f12ae45a12p-20},
+    {0x1.a309bec4a2d33p-1, 0x1.a31p-1, 0x1.904ed74b329d0p-15},
+    {0x1.a0c667b5de565p-1, 0x1.a0cp-1, -0x1.99ed779592ca7p-15},
+    {0x1.9e86319e32323p-1, 0x1.9e8p-1, -0x1.8c678c8c8c609p-15},
+    {0x1.9c49182a3f090p-1, 0x1.9c5p-1, 0x1.b9f5703dbf8e1p-15},
+    {0x1.9a0f170ca07bap-1, 0x1.9a1p-1, 0x1.d1e6bf08c8b9ep-18},
+    {0x1.97d829fde4e50p-1, 0x1.97ep-1, 0x1.f58086c6c1d18p-15},
+    {0x1.95a44cbc8520fp-1, 0x1.95ap-1, -0x1.132f21483ba6dp-15},
+    {0x1.93737b0cdc5e5p-1, 0x1.937p-1, -0x1.bd866e2f27a28p-16},
+    {0x1.9145b0b91ffc6p-1, 0x1.914p-1, -0x1.6c2e47ff1622ap-15},
+    {0x1.8f1ae99157736p-1, 0x1.8f2p-1, 0x1.459baa232751ap-15},
+    {0x1.8cf3216b5448cp-1, 0x1.8cfp-1, -0x1.90b5aa245f795p-16},
+    {0x1.8ace5422aa0dbp-1, 0x1.8adp-1, 0x1.abdd55f24a458p-17},
+    {0x1.88ac7d98a6699p-1, 0x1.88bp-1, 0x1.c133accb34cd6p-16},
+    {0x1.868d99b4492edp-1, 0x1.869p-1, 0x1.3325db689bf8ep-16},
+    {0x1.8471a4623c7adp-1, 0x1.847p-1, -0x1.a4623c7acce53p-17},
+    {0x1.82589994cce13p-1, 0x1.826p-1, 0x1.d99accc7b5d4cp-15},
+    {0x1.80427543e1a12p-1, 0x1.804p-1, -0x1.3aa1f0d08db07p-16},
+    {0x1.7e2f336cf4e62p-1, 0x1.7e3p-1, 0x1.99261633bdf46p-18},
+    {0x1.7c1ed0130c132p-1, 0x1.7c2p-1, 0x1.2fecf3ecd83b7p-17},
+    {0x1.7a11473eb0187p-1, 0x1.7a1p-1, -0x1.473eb0186d7d5p-17},
+    {0x1.780694fde5d3fp-1, 0x1.78p-1, -0x1.a53f7974fd867p-15},
+    {0x1.75feb564267c9p-1, 0x1.76p-1, 0x1.4a9bd98374091p-17},
+    {0x1.73f9a48a58174p-1, 0x1.74p-1, 0x1.96dd69fa310a9p-15},
+    {0x1.71f75e8ec5f74p-1, 0x1.71fp-1, -0x1.d7a3b17dcf749p-15},
+    {0x1.6ff7df9519484p-1, 0x1.6ffp-1, -0x1.f7e546520f3e2p-15},
+    {0x1.6dfb23c651a2fp-1, 0x1.6ep-1, 0x1.370e6b9744378p-15},
+    {0x1.6c012750bdabfp-1, 0x1.6cp-1, -0x1.2750bdabeed77p-17},
+    {0x1.6a09e667f3bcdp-1, 0x1.6a1p-1, 0x1.86660310cdbddp-15},
+    {0x1.68155d44ca973p-1, 0x1.681p-1, -0x1.575132a5cc207p-15},
+    {0x1.6623882552225p-1, 0x1.662p-1, -0x1.c412a91124894p-16},
+    {0x1.6434634ccc320p-1, 0x1.643p-1, -0x1.18d3330c7f1dcp-15},
+    {0x1.6247eb03a5585p-1, 0x1.624p-1, -0x1.fac0e95612c7cp-15},
+    {0x1.605e1b976dc09p-1, 0x1.606p-1, 0x1.e468923f74f89p-17},
+    {0x1.5e76f15ad2148p-1, 0x1.5e7p-1, -0x1.bc56b48521ba7p-15},
+    {0x1.5c9268a5946b7p-1, 0x1.5c9p-1, -0x1.3452ca35b80e2p-16},
+    {0x1.5ab07dd485429p-1, 0x1.5abp-1, -0x1.f752150a56325p-19},
+    {0x1.58d12d497c7fdp-1, 0x1.58dp-1, -0x1.2d497c7fd252cp-17},
+    {0x1.56f4736b527dap-1, 0x1.56fp-1, -0x1.1cdad49f699bbp-15},
+    {0x1.551a4ca5d920fp-1, 0x1.552p-1, 0x1.6cd689b7c4eb4p-15},
+    {0x1.5342b569d4f82p-1, 0x1.534p-1, -0x1.5ab4ea7c0ef85p-16},
+    {0x1.516daa2cf6642p-1, 0x1.517p-1, 0x1.2ae984cdf1f77p-16},
+    {0x1.4f9b2769d2ca7p-1, 0x1.4fap-1, 0x1.36258b4d654b3p-15},
+    {0x1.4dcb299fddd0dp-1, 0x1.4ddp-1, 0x1.3598088bca713p-15},
+    {0x1.4bfdad5362a27p-1, 0x1.4cp-1, 0x1.29564eaec715ep-16},
+    {0x1.4a32af0d7d3dep-1, 0x1.4a3p-1, -0x1.5786be9ef3397p-16},
+    {0x1.486a2b5c13cd0p-1, 0x1.487p-1, 0x1.7528fb0cbfb10p-15},
+    {0x1.46a41ed1d0057p-1, 0x1.46ap-1, -0x1.07b474015dc94p-15},
+    {0x1.44e086061892dp-1, 0x1.44ep-1, -0x1.0c0c3125a0627p-18},
+    {0x1.431f5d950a897p-1, 0x1.432p-1, 0x1.44d5eaed2471fp-18},
+    {0x1.4160a21f72e2ap-1, 0x1.416p-1, -0x1.443ee5c53f086p-18},
+    {0x1.3fa4504ac801cp-1, 0x1.3fap-1, -0x1.1412b2006e830p-15},
+    {0x1.3dea64c123422p-1, 0x1.3dfp-1, 0x1.66cfb72f77293p-15},
+    {0x1.3c32dc313a8e5p-1, 0x1.3c3p-1, -0x1.6e189d4724200p-16},
+    {0x1.3a7db34e59ff7p-1, 0x1.3a8p-1, 0x1.2658d30048af2p-16},
+    {0x1.38cae6d05d866p-1, 0x1.38dp-1, 0x1.464be89e69e96p-15},
+    {0x1.371a7373aa9cbp-1, 0x1.372p-1, 0x1.63231558d563bp-15},
+    {0x1.356c55f929ff1p-1, 0x1.357p-1, 0x1.d5036b0079b5dp-16},
+    {0x1.33c08b26416ffp-1, 0x1.33cp-1, -0x1.164c82dfe9939p-18},
+    {0x1.32170fc4cd831p-1, 0x1.321p-1, -0x1.c3f13360c4d4ep-15},
+    {0x1.306fe0a31b715p-1, 0x1.307p-1, 0x1.f5ce48ead2173p-21},
+    {0x1.2ecafa93e2f56p-1, 0x1.2edp-1, 0x1.415b0742a7b8dp-15},
+    {0x1.2d285a6e4030bp-1, 0x1.2d3p-1, 0x1.e9646ff3d2ffep-15},
+    {0x1.2b87fd0dad990p-1, 0x1.2b8p-1, -0x1.ff436b663ff78p-15},
+    {0x1.29e9df51fdee1p-1, 0x1.29fp-1, 0x1.882b80847b4f7p-15},
+    {0x1.284dfe1f56381p-1, 0x1.285p-1, 0x1.00f054e3fb498p-16},
+    {0x1.26b4565e27cddp-1, 0x1.26bp-1, -0x1.159789f37495fp-15},
+    {0x1.251ce4fb2a63fp-1, 0x1.252p-1, 0x1.8d826ace0653fp-16},
+    {0x1.2387a6e756238p-1, 0x1.238p-1, -0x1.e9b9d588e19b0p-15},
+    {0x1.21f49917ddc96p-1, 0x1.21fp-1, -0x1.2645f77258955p-15},
+    {0x1.2063b88628cd6p-1, 0x1.206p-1, -0x1.dc431466b1dc7p-16},
+    {0x1.1ed5022fcd91dp-1, 0x1.1edp-1, -0x1.408bf36472e20p-15},
+    {0x1.1d4873168b9aap-1, 0x1.1d5p-1, 0x1.e33a5d19561ffp-15},
+    {0x1.1bbe084045cd4p-1, 0x1.1bcp-1, 0x1.f7bfba32c654ep-17},
+    {0x1.1a35beb6fcb75p-1, 0x1.1a3p-1, -0x1.6fadbf2dd4f2ep-15},
+    {0x1.18af9388c8deap-1, 0x1.18bp-1, 0x1.b1dcdc8591102p-19},
+    {0x1.172b83c7d517bp-1, 0x1.173p-1, 0x1.1f0e0aba148c8p-15},
+    {0x1.15a98c8a58e51p-1, 0x1.15bp-1, 0x1.9cdd69c6bb6e0p-15},
+    {0x1.1429aaea92de0p-1, 0x1.143p-1, 0x1.95455b4881330p-15},
+    {0x1.12abdc06c31ccp-1, 0x1.12bp-1, 0x1.08fe4f38d011bp-15},
+    {0x1.11301d0125b51p-1, 0x1.113p-1, -0x1.d0125b50a4ebcp-21},
+    {0x1.0fb66affed31bp-1, 0x1.0fbp-1, -0x1.9abffb4c6bc8dp-15},
+    {0x1.0e3ec32d3d1a2p-1, 0x1.0e4p-1, 0x1.3cd2c2e5dfdf9p-17},
+    {0x1.0cc922b7247f7p-1, 0x1.0cdp-1, 0x1.b75236e022fe1p-15},
+    {0x1.0b5586cf9890fp-1, 0x1.0b5p-1, -0x1.61b3e6243d8a6p-15},
+    {0x1.09e3ecac6f383p-1, 0x1.09ep-1, -0x1.f656379c1a291p-16},
+    {0x1.0874518759bc8p-1, 0x1.087p-1, -0x1.1461d66f20231p-15},
+    {0x1.0706b29ddf6dep-1, 0x1.07p-1, -0x1.aca777db771b7p-15},
+    {0x1.059b0d3158574p-1, 0x1.05ap-1, 0x1.3cb3a9ea2f146p-15},
+    {0x1.04315e86e7f85p-1, 0x1.043p-1, -0x1.5e86e7f84bd74p-17},
+    {0x1.02c9a3e778061p-1, 0x1.02dp-1, 0x1.970621fe7c464p-15},
+    {0x1.0163da9fb3335p-1, 0x1.016p-1, -0x1.ed4fd999ab6c2p-16},
 };
-RT_TABLE ExpUpEntry kExpUpTable[128] = {
-    {0x1.0000000000000p+0, 0x0.0p+0, 0x0.0p+0, 0x0.0p+0},
-    {0x1.0163da9fb3335p+0, 0x1.b61299ab8cdb7p-54, 0x1.63da9fb33356ep-8, -0x1.ed665473248c8p-62},
-    {0x1.02c9a3e778061p+0, -0x1.19083535b085dp-56, 0x1.64d1f3bc03077p-7, 0x1.bdf2b293de8a7p-62},
-    {0x1.04315e86e7f85p+0, -0x1.0a31c1977c96ep-54, 0x1.0c57a1b9fe12fp-6, 0x1.738f9a20da47ep-60},
-    {0x1.059b0d3158574p+0, 0x1.d73e2a475b465p-55, 0x1.66c34c5615d0fp-6, -0x1.183ab7149735cp-60},
-    {0x1.0706b29ddf6dep+0, -0x1.c91dfe2b13c27p-55, 0x1.c1aca777db772p-6, -0x1.23bfc562784d8p-60},
-    {0x1.0874518759bc8p+0, 0x1.186be4bb284ffp-57, 0x1.0e8a30eb37901p-5, 0x1.86be4bb284ff4p-61},
-    {0x1.09e3ecac6f383p+0, 0x1.1487818316136p-54, 0x1.3c7d958de7069p-5, -0x1.6f0fcf9d3d94ap-59},
-    {0x1.0b5586cf9890fp+0, 0x1.8a62e4adc610bp-54, 0x1.6ab0d9f3121ecp-5, 0x1.4c5c95b8c2155p-59},
-    {0x1.0cc922b7247f7p+0, 0x1.01edc16e24f71p-54, 0x1.992456e48fee8p-5, 0x1.edc16e24f717ap-62},
-    {0x1.0e3ec32d3d1a2p+0, 0x1.03a1727c57b53p-59, 0x1.c7d865a7a3440p-5, 0x1.03a1727c57b53p-59},
-    {0x1.0fb66affed31bp+0, -0x1.b9bedc44ebd7bp-57, 0x1.f6cd5ffda635ep-5, 0x1.19048eec50a13p-59},
-    {0x1.11301d0125b51p+0, -0x1.6c51039449b3ap-54, 0x1.1301d0125b50ap-4, 0x1.3aefc6bb64c63p-58},
-    {0x1.12abdc06c31ccp+0, -0x1.1b514b36ca5c7p-58, 0x1.2abdc06c31cc0p-4, -0x1.1b514b36ca5c7p-58},
-    {0x1.1429aaea92de0p+0, -0x1.32fbf9af1369ep-54, 0x1.429aaea92ddfbp-4, 0x1.a080ca1d92c37p-59},
-    {0x1.15a98c8a58e51p+0, 0x1.2406ab9eeab0ap-55, 0x1.5a98c8a58e512p-4, 0x1.20355cf75584fp-58},
-    {0x1.172b83c7d517bp+0, -0x1.19041b9d78a76p-55, 0x1.72b83c7d517aep-4, -0x1.9041b9d78a75bp-59},
-    {0x1.18af9388c8deap+0, -0x1.11023d1970f6cp-54, 0x1.8af9388c8de9cp-4, -0x1.1023d1970f6bfp-58},
-    {0x1.1a35beb6fcb75p+0, 0x1.e5b4c7b4968e4p-55, 0x1.a35beb6fcb754p-4, -0x1.a4b384b6971bep-59},
-    {0x1.1bbe084045cd4p+0, -0x1.95386352ef607p-54, 0x1.bbe084045cd3ap-4, -0x1.5386352ef6073p-58},
-    {0x1.1d4873168b9aap+0, 0x1.e016e00a2643cp-54, 0x1.d4873168b9aa8p-4, -0x1.fe91ff5d9bc3ep-58},
-    {0x1.1ed5022fcd91dp+0, -0x1.1df98027bb78cp-54, 0x1.ed5022fcd91ccp-4, -0x1.df98027bb78b8p-58},
-    {0x1.2063b88628cd6p+0, 0x1.dc775814a8495p-55, 0x1.031dc431466b2p-3, -0x1.1c453f5abdb59p-58},
-    {0x1.21f49917ddc96p+0, 0x1.2a97e9494a5eep-55, 0x1.0fa4c8beee4b1p-3, 0x1.54bf4a4a52f6dp-58},
-    {0x1.2387a6e756238p+0, 0x1.9b07eb6c70573p-54, 0x1.1c3d373ab11c3p-3, 0x1.b07eb6c70572dp-58},
-    {0x1.251ce4fb2a63fp+0, 0x1.ac155bef4f4a4p-55, 0x1.28e727d9531fap-3, -0x1.4faa9042c2d70p-57},
-    {0x1.26b4565e27cddp+0, 0x1.2bd339940e9d9p-55, 0x1.35a2b2f13e6e9p-3, 0x1.5e99cca074ec9p-58},
-    {0x1.284dfe1f56381p+0, -0x1.a4c3a8c3f0d7ep-54, 0x1.426ff0fab1c05p-3, -0x1.261d461f86bedp-57},
-    {0x1.29e9df51fdee1p+0, 0x1.612e8afad1255p-55, 0x1.4f4efa8fef709p-3, 0x1.84ba2beb44954p-57},
-    {0x1.2b87fd0dad990p+0, -0x1.10adcd6381aa4p-59, 0x1.5c3fe86d6cc80p-3, -0x1.10adcd6381aa4p-59},
-    {0x1.2d285a6e4030bp+0, 0x1.0024754db41d5p-54, 0x1.6942d3720185ap-3, 0x1.23aa6da0ea709p-65},
-    {0x1.2ecafa93e2f56p+0, 0x1.1ca0f45d52383p-56, 0x1.7657d49f17ab1p-3, -0x1.c6be17455b8fap-57},
-    {0x1.306fe0a31b715p+0, 0x1.6f46ad23182e4p-55, 0x1.837f0518db8a9p-3, 0x1.bd1ab48c60b91p-57},
-    {0x1.32170fc4cd831p+0, 0x1.a9ce78e18047cp-55, 0x1.90b87e266c18ap-3, -0x1.58c61c79fee0fp-57},
-    {0x1.33c08b26416ffp+0, 0x1.32721843659a6p-54, 0x1.9e0459320b7fap-3, 0x1.9390c21b2cd2dp-57},
-    {0x1.356c55f929ff1p+0, -0x1.b5cee5c4e4628p-55, 0x1.ab62afc94ff86p-3, 0x1.28c468ec6e75ep-57},
-    {0x1.371a7373aa9cbp+0, -0x1.63aeabf42eae2p-54, 0x1.b8d39b9d54e55p-3, 0x1.c51540bd151e6p-58},
-    {0x1.38cae6d05d866p+0, -0x1.e958d3c9904bdp-54, 0x1.c6573682ec32cp-3, 0x1.6a72c366fb432p-58},
-    {0x1.3a7db34e59ff7p+0, -0x1.5e436d661f5e3p-56, 0x1.d3ed9a72cffb7p-3, 0x1.43792533c143ap-57},
-    {0x1.3c32dc313a8e5p+0, -0x1.efff8375d29c3p-54, 0x1.e196e189d4724p-3, 0x1.0007c8a2d63cep-58},
-    {0x1.3dea64c123422p+0, 0x1.ada0911f09ebcp-55, 0x1.ef5326091a112p-3, -0x1.497dbb83d8512p-57},
-    {0x1.3fa4504ac801cp+0, -0x1.7d023f956f9f3p-54, 0x1.fd228256400ddp-3, 0x1.7ee035483065fp-61},
-    {0x1.4160a21f72e2ap+0, -0x1.ef3691c309278p-58, 0x1.0582887dcb8a8p-2, -0x1.ef3691c309278p-58},
-    {0x1.431f5d950a897p+0, -0x1.1c7dde35f7999p-55, 0x1.0c7d76542a25bp-2, 0x1.c704439410ccfp-56},
-    {0x1.44e086061892dp+0, 0x1.89b7a04ef80d0p-59, 0x1.13821818624b4p-2, 0x1.89b7a04ef80d0p-59},
-    {0x1.46a41ed1d0057p+0, 0x1.c944bd1648a76p-54, 0x1.1a907b474015ep-2, -0x1.b5da174dbac4dp-57},
-    {0x1.486a2b5c13cd0p+0, 0x1.3c1a3b69062f0p-56, 0x1.21a8ad704f340p-2, 0x1.3c1a3b69062f0p-56},
-    {0x1.4a32af0d7d3dep+0, 0x1.9cb62f3d1be56p-54, 0x1.28cabc35f4f7ap-2, -0x1.8d27430b906a8p-56},
-    {0x1.4bfdad5362a27p+0, 0x1.d4397afec42e2p-56, 0x1.2ff6b54d8a89cp-2, 0x1.d4397afec42e2p-56},
-    {0x1.4dcb299fddd0dp+0, 0x1.8ecdbbc6a7833p-54, 0x1.372ca67f77436p-2, -0x1.c4c910e561f34p-56},
-    {0x1.4f9b2769d2ca7p+0, -0x1.4b309d25957e3p-54, 0x1.3e6c9da74b29bp-2, -0x1.2cc2749655f8cp-56},
-    {0x1.516daa2cf6642p+0, -0x1.f768569bd93efp-55, 0x1.45b6a8b3d9907p-2, 0x1.12f52c84d8222p-60},
-    {0x1.5342b569d4f82p+0, -0x1.07abe1db13cadp-55, 0x1.4d0ad5a753e07p-2, 0x1.f0a83c49d86a6p-56},
-    {0x1.551a4ca5d920fp+0, -0x1.d689cefede59bp-55, 0x1.546932976483bp-2, 0x1.4bb188090d32ap-58},
-    {0x1.56f4736b527dap+0, 0x1.9bb2c011d93adp-54, 0x1.5bd1cdad49f6ap-2, -0x1.9134ffb89b14cp-56},
-    {0x1.58d12d497c7fdp+0, 0x1.295e15b9a1de8p-55, 0x1.6344b525f1ff5p-2, -0x1.ad43d48cbc431p-56},
-    {0x1.5ab07dd485429p+0, 0x1.6324c054647adp-54, 0x1.6ac1f752150a5p-2, 0x1.8c93015191eb3p-56},
-    {0x1.5c9268a5946b7p+0, 0x1.c4b1b816986a2p-60, 0x1.7249a29651adcp-2, 0x1.c4b1b816986a2p-60},
-    {0x1.5e76f15ad2148p+0, 0x1.ba6f93080e65ep-54, 0x1.79dbc56b48522p-2, -0x1.1641b3dfc668ap-56},
-    {0x1.605e1b976dc09p+0, -0x1.3e2429b56de47p-54, 0x1.81786e5db7023p-2, -0x1.f1214dab6f239p-57},
-    {0x1.6247eb03a5585p+0, -0x1.383c17e40b497p-54, 0x1.891fac0e95613p-2, -0x1.c1e0bf205a4b8p-57},
-    {0x1.6434634ccc320p+0, -0x1.c483c759d8933p-55, 0x1.90d18d3330c7fp-2, 0x1.dbe1c5313b669p-58},
-    {0x1.6623882552225p+0, -0x1.bb60987591c34p-54, 0x1.988e209548892p-2, 0x1.127d9e29b8f31p-56},
-    {0x1.68155d44ca973p+0, 0x1.038ae44f73e65p-57, 0x1.a05575132a5ccp-2, 0x1.038ae44f73e65p-57},
-    {0x1.6a09e667f3bcdp+0, -0x1.bdd3413b26456p-54, 0x1.a827999fcef32p-2, 0x1.08b2fb1366ea9p-56},
-    {0x1.6c012750bdabfp+0, -0x1.2895667ff0b0dp-56, 0x1.b0049d42f6afcp-2, -0x1.2895667ff0b0dp-56},
-    {0x1.6dfb23c651a2fp+0, -0x1.bbe3a683c88abp-57, 0x1.b7ec8f19468bcp-2, -0x1.bbe3a683c88abp-57},
-    {0x1.6ff7df9519484p+0, -0x1.83c0f25860ef6p-55, 0x1.bfdf7e546520fp-2, 0x1.f0fc369e7c427p-57},
-    {0x1.71f75e8ec5f74p+0, -0x1.16e4786887a99p-55, 0x1.c7dd7a3b17dcfp-2, 0x1.d2370f2ef0acdp-56},
-    {0x1.73f9a48a58174p+0, -0x1.0a8d96c65d53cp-54, 0x1.cfe69229605cfp-2, -0x1.51b2d8cbaa774p-59},
-    {0x1.75feb564267c9p+0, -0x1.0245957316dd3p-54, 0x1.d7fad59099f23p-2, -0x1.22cab98b6e9b2p-61},
-    {0x1.780694fde5d3fp+0, 0x1.866b80a02162dp-54, 0x1.e01a53f7974fep-2, -0x1.e651fd7f7a74dp-56},
-    {0x1.7a11473eb0187p+0, -0x1.41577ee04992fp-55, 0x1.e8451cfac061bp-2, 0x1.7d51023f6cda2p-56},
-    {0x1.7c1ed0130c132p+0, 0x1.f124cd1164dd6p-54, 0x1.f07b404c304cap-2, -0x1.db665dd36454fp-59},
-    {0x1.7e2f336cf4e62p+0, 0x1.05d02ba15797ep-56, 0x1.f8bccdb3d3988p-2, 0x1.05d02ba15797ep-56},
-    {0x1.80427543e1a12p+0, -0x1.27c86626d972bp-54, 0x1.0084ea87c3423p-1, 0x1.b06f33b24d1aap-55},
-    {0x1.82589994cce13p+0, -0x1.d4c1dd41532d8p-54, 0x1.04b1332999c25p-1, 0x1.59f115f566940p-57},
-    {0x1.8471a4623c7adp+0, -0x1.8d684a341cdfbp-55, 0x1.08e348c478f5ap-1, -0x1.8d684a341cdfbp-55},
-    {0x1.868d99b4492edp+0, -0x1.fc6f89bd4f6bap-54, 0x1.0d1b3368925d9p-1, 0x1.c83b21584a2e1p-61},
-    {0x1.88ac7d98a6699p+0, 0x1.994c2f37cb53ap-54, 0x1.1158fb314cd33p-1, -0x1.9acf4320d2b16p-56},
-    {0x1.8ace5422aa0dbp+0, 0x1.6e9f156864b27p-54, 0x1.159ca845541b7p-1, -0x1.22c1d52f369b2p-55},
-    {0x1.8cf3216b5448cp+0, -0x1.0d55e32e9e3aap-56, 0x1.19e642d6a8918p-1, -0x1.0d55e32e9e3aap-56},
-    {0x1.8f1ae99157736p+0, 0x1.5cc13a2e3976cp-55, 0x1.1e35d322aee6cp-1, 0x1.5cc13a2e3976cp-55},
-    {0x1.9145b0b91ffc6p+0, -0x1.dd6792e582524p-54, 0x1.228b61723ff8bp-1, 0x1.14c368d3ed6e2p-57},
-    {0x1.93737b0cdc5e5p+0, -0x1.75fc781b57ebcp-57, 0x1.26e6f619b8bcap-1, -0x1.75fc781b57ebcp-57},
-    {0x1.95a44cbc8520fp+0, -0x1.64b7c96a5f039p-56, 0x1.2b4899790a41ep-1, -0x1.64b7c96a5f039p-56},
-    {0x1.97d829fde4e50p+0, -0x1.d185b7c1b85d1p-54, 0x1.2fb053fbc9c9fp-1, 0x1.73d241f23d17bp-57},
-    {0x1.9a0f170ca07bap+0, -0x1.173bd91cee632p-54, 0x1.341e2e1940f73p-1, 0x1.d1884dc62339cp-55},
-    {0x1.9c49182a3f090p+0, 0x1.c7c46b071f2bep-56, 0x1.389230547e120p-1, 0x1.c7c46b071f2bep-56},
-    {0x1.9e86319e32323p+0, 0x1.824ca78e64c6ep-56, 0x1.3d0c633c64646p-1, 0x1.824ca78e64c6ep-56},
-    {0x1.a0c667b5de565p+0, -0x1.359495d1cd533p-54, 0x1.418ccf6bbcac9p-1, 0x1.94d6d45c6559ap-55},
-    {0x1.a309bec4a2d33p+0, 0x1.6305c7ddc36abp-54, 0x1.46137d8945a67p-1, -0x1.39f47044792a9p-55},
-    {0x1.a5503b23e255dp+0, -0x1.d2f6edb8d41e1p-54, 0x1.4aa07647c4ab9p-1, 0x1.684892395f0f8p-57},
-    {0x1.a799e1330b358p+0, 0x1.bcb7ecac563c7p-54, 0x1.4f33c266166b1p-1, -0x1.0d204d4ea70e5p-56},
-    {0x1.a9e6b5579fdbfp+0, 0x1.0fac90ef7fd31p-54, 0x1.53cd6aaf3fb7fp-1, -0x1.e0a6de210059ep-55},
-    {0x1.ac36bbfd3f37ap+0, -0x1.f9234cae76cd0p-55, 0x1.586d77fa7e6f4p-1, -0x1.f9234cae76cd0p-55},
-    {0x1.ae89f995ad3adp+0, 0x1.7a1cd345dcc81p-54, 0x1.5d13f32b5a75bp-1, -0x1.0bc65974466fdp-55},
-    {0x1.b0e07298db666p+0, -0x1.bdef54c80e425p-54, 0x1.61c0e531b6ccbp-1, 0x1.0842acdfc6f6dp-56},
-    {0x1.b33a2b84f15fbp+0, -0x1.2805e3084d708p-57, 0x1.66745709e2bf6p-1, -0x1.2805e3084d708p-57},
-    {0x1.b59728de5593ap+0, -0x1.c71dfbbba6de3p-54, 0x1.6b2e51bcab273p-1, 0x1.c7102222c90e8p-57},
-    {0x1.b7f76f2fb5e47p+0, -0x1.5584f7e54ac3bp-56, 0x1.6feede5f6bc8ep-1, -0x1.5584f7e54ac3bp-56},
-    {0x1.ba5b030a1064ap+0, -0x1.efcd30e54292ep-54, 0x1.74b6061420c93p-1, 0x1.032cf1abd6d20p-58},
-    {0x1.bcc1e904bc1d2p+0, 0x1.23dd07a2d9e84p-55, 0x1.7983d209783a4p-1, 0x1.23dd07a2d9e84p-55},
-    {0x1.bf2c25bd71e09p+0, -0x1.efdca3f6b9c73p-54, 0x1.7e584b7ae3c11p-1, 0x1.0235c094638d1p-58},
-    {0x1.c199bdd85529cp+0, 0x1.11065895048ddp-55, 0x1.83337bb0aa538p-1, 0x1.11065895048ddp-55},
-    {0x1.c40ab5fffd07ap+0, 0x1.b4537e083c60ap-54, 0x1.88156bfffa0f5p-1, -0x1.2eb207df0e7d7p-56},
-    {0x1.c67f12e57d14bp+0, 0x1.2884dff483cadp-54, 0x1.8cfe25cafa297p-1, -0x1.aef64016f86a6p-55},
-    {0x1.c8f6d9406e7b5p+0, 0x1.1acbc48805c44p-56, 0x1.91edb280dcf6ap-1, 0x1.1acbc48805c44p-56},
-    {0x1.cb720dcef9069p+0, 0x1.503cbd1e949dbp-56, 0x1.96e41b9df20d2p-1, 0x1.503cbd1e949dbp-56},
-    {0x1.cdf0b555dc3fap+0, -0x1.dd83b53829d72p-55, 0x1.9be16aabb87f4p-1, -0x1.dd83b53829d72p-55},
-    {0x1.d072d4a07897cp+0, -0x1.cbc3743797a9cp-54, 0x1.a0e5a940f12f7p-1, 0x1.a1e45e4342b1cp-57},
-    {0x1.d2f87080d89f2p+0, -0x1.d487b719d8578p-54, 0x1.a5f0e101b13e3p-1, 0x1.5bc247313d440p-57},
-    {0x1.d5818dcfba487p+0, 0x1.2ed02d75b3707p-55, 0x1.ab031b9f7490ep-1, 0x1.2ed02d75b3707p-55},
-    {0x1.d80e316c98398p+0, -0x1.11ec18beddfe8p-54, 0x1.b01c62d93072fp-1, 0x1.dc27ce8244030p-55},
-    {0x1.da9e603db3285p+0, 0x1.c2300696db532p-54, 0x1.b53cc07b6650bp-1, -0x1.ee7fcb492566dp-57},
-    {0x1.dd321f301b460p+0, 0x1.2da5778f018c3p-54, 0x1.ba643e60368c1p-1, -0x1.a4b510e1fce7bp-55},
-    {0x1.dfc97337b9b5fp+0, -0x1.1a5cd4f184b5cp-54, 0x1.bf92e66f736bdp-1, 0x1.cb46561cf6949p-55},
-    {0x1.e264614f5a129p+0, -0x1.7b627817a1496p-54, 0x1.c4c8c29eb4251p-1, 0x1.093b0fd0bd6d3p-55},
-    {0x1.e502ee78b3ff6p+0, 0x1.39e8980a9cc8fp-55, 0x1.ca05dcf167fecp-1, 0x1.39e8980a9cc8fp-55},
-    {0x1.e7a51fbc74c83p+0, 0x1.2d522ca0c8de2p-54, 0x1.cf4a3f78e9907p-1, -0x1.a55ba6be6e43dp-55},
-    {0x1.ea4afa2a490dap+0, -0x1.e9c23179c2893p-54, 0x1.d495f454921b3p-1, 0x1.63dce863d76ccp-58},
-    {0x1.ecf482d8e67f1p+0, -0x1.c93f3b411ad8cp-54, 0x1.d9e905b1ccfe1p-1, 0x1.b60625f72939ep-57},
-    {0x1.efa1bee615a27p+0, 0x1.dc7f486a4b6b0p-54, 0x1.df437dcc2b44fp-1, -0x1.1c05bcada4a7cp-57},
-    {0x1.f252b376bba97p+0, 0x1.3a1a5bf0d8e43p-54, 0x1.e4a566ed7752fp-1, -0x1.8bcb481e4e379p-55},
-    {0x1.f50765b6e4540p+0, 0x1.9d3e12dd8a18bp-54, 0x1.ea0ecb6dc8a81p-1, -0x1.8b07b489d79d4p-56},
-    {0x1.f7bfdad9cbe14p+0, -0x1.dbb12d006350ap-54, 0x1.ef7fb5b397c27p-1, 0x1.227697fce57b3p-57},
-    {0x1.fa7c1819e90d8p+0, 0x1.74853f3a5931ep-55, 0x1.f4f83033d21b0p-1, 0x1.74853f3a5931ep-55},
-    {0x1.fd3c22b8f71f1p+0, 0x1.2eb74966579e7p-57, 0x1.fa784571ee3e2p-1, 0x1.2eb74966579e7p-57},
+RT_TABLE ExpEntry kExpUpTable[128] = {
+    {0x1.0000000000000p+0, 0x1.0p+0, 0x0.0p+0},
+    {0x1.0163da9fb3335p+0, 0x1.016p+0, 0x1.ed4fd999ab6c2p-15},
+    {0x1.02c9a3e778061p+0, 0x1.02c8p+0, 0x1.a3e778060ee6fp-16},
+    {0x1.04315e86e7f85p+0, 0x1.043p+0, 0x1.5e86e7f84bd74p-16},
+    {0x1.059b0d3158574p+0, 0x1.0598p+0, 0x1.8698ac2ba1d74p-15},
+    {0x1.0706b29ddf6dep+0, 0x1.0708p+0, -0x1.4d62209223924p-16},
+    {0x1.0874518759bc8p+0, 0x1.0878p+0, -0x1.d73c5321bfb9ep-15},
+    {0x1.09e3ecac6f383p+0, 0x1.09ep+0, 0x1.f656379c1a291p-15},
+    {0x1.0b5586cf9890fp+0, 0x1.0b58p+0, -0x1.3c9833b784eb4p-15},
+    {0x1.0cc922b7247f7p+0, 0x1.0cc8p+0, 0x1.22b7247f7407bp-16},
+    {0x1.0e3ec32d3d1a2p+0, 0x1.0e4p+0, -0x1.3cd2c2e5dfdf9p-16},
+    {0x1.0fb66affed31bp+0, 0x1.0fb8p+0, -0x1.950012ce50dcep-16},
+    {0x1.11301d0125b51p+0, 0x1.113p+0, 0x1.d0125b50a4ebcp-20},
+    {0x1.12abdc06c31ccp+0, 0x1.12a8p+0, 0x1.ee03618e5fdc9p-15},
+    {0x1.1429aaea92de0p+0, 0x1.1428p+0, 0x1.aaea92ddfb341p-16},
+    {0x1.15a98c8a58e51p+0, 0x1.15a8p+0, 0x1.8c8a58e512481p-16},
+    {0x1.172b83c7d517bp+0, 0x1.1728p+0, 0x1.c1e3ea8bd6e70p-15},
+    {0x1.18af9388c8deap+0, 0x1.18bp+0, -0x1.b1dcdc8591102p-18},
+    {0x1.1a35beb6fcb75p+0, 0x1.1a38p+0, -0x1.20a481a4561a5p-15},
+    {0x1.1bbe084045cd4p+0, 0x1.1bcp+0, -0x1.f7bfba32c654ep-16},
+    {0x1.1d4873168b9aap+0, 0x1.1d48p+0, 0x1.cc5a2e6a9e017p-18},
+    {0x1.1ed5022fcd91dp+0, 0x1.1ed8p+0, -0x1.7ee819371a3bfp-15},
+    {0x1.2063b88628cd6p+0, 0x1.206p+0, 0x1.dc431466b1dc7p-15},
+    {0x1.21f49917ddc96p+0, 0x1.21f8p+0, -0x1.b374111b4ed57p-15},
+    {0x1.2387a6e756238p+0, 0x1.2388p+0, -0x1.6462a771e64f8p-18},
+    {0x1.251ce4fb2a63fp+0, 0x1.252p+0, -0x1.8d826ace0653fp-15},
+    {0x1.26b4565e27cddp+0, 0x1.26b8p+0, -0x1.d4d0ec1916d43p-15},
+    {0x1.284dfe1f56381p+0, 0x1.285p+0, -0x1.00f054e3fb498p-15},
+    {0x1.29e9df51fdee1p+0, 0x1.29e8p+0, 0x1.df51fdee12c26p-16},
+    {0x1.2b87fd0dad990p+0, 0x1.2b88p+0, -0x1.79293380110aep-23},
+    {0x1.2d285a6e4030bp+0, 0x1.2d28p+0, 0x1.69b900c2d0024p-18},
+    {0x1.2ecafa93e2f56p+0, 0x1.2ec8p+0, 0x1.7d49f17ab08e5p-15},
+    {0x1.306fe0a31b715p+0, 0x1.307p+0, -0x1.f5ce48ead2173p-20},
+    {0x1.32170fc4cd831p+0, 0x1.3218p+0, -0x1.e07664f9d958cp-17},
+    {0x1.33c08b26416ffp+0, 0x1.33cp+0, 0x1.164c82dfe9939p-17},
+    {0x1.356c55f929ff1p+0, 0x1.357p+0, -0x1.d5036b0079b5dp-15},
+    {0x1.371a7373aa9cbp+0, 0x1.3718p+0, 0x1.39b9d54e5538ap-15},
+    {0x1.38cae6d05d866p+0, 0x1.38c8p+0, 0x1.73682ec32c2d5p-15},
+    {0x1.3a7db34e59ff7p+0, 0x1.3a8p+0, -0x1.2658d30048af2p-15},
+    {0x1.3c32dc313a8e5p+0, 0x1.3c3p+0, 0x1.6e189d4724200p-15},
+    {0x1.3dea64c123422p+0, 0x1.3de8p+0, 0x1.326091a111adap-15},
+    {0x1.3fa4504ac801cp+0, 0x1.3fa8p+0, -0x1.d7da9bff22fa0p-15},
+    {0x1.4160a21f72e2ap+0, 0x1.416p+0, 0x1.443ee5c53f086p-17},
+    {0x1.431f5d950a897p+0, 0x1.432p+0, -0x1.44d5eaed2471fp-17},
+    {0x1.44e086061892dp+0, 0x1.44ep+0, 0x1.0c0c3125a0627p-17},
+    {0x1.46a41ed1d0057p+0, 0x1.46a8p+0, -0x1.f09717fd446d7p-15},
+    {0x1.486a2b5c13cd0p+0, 0x1.4868p+0, 0x1.15ae09e6809e1p-15},
+    {0x1.4a32af0d7d3dep+0, 0x1.4a3p+0, 0x1.5786be9ef3397p-15},
+    {0x1.4bfdad5362a27p+0, 0x1.4cp+0, -0x1.29564eaec715ep-15},
+    {0x1.4dcb299fddd0dp+0, 0x1.4dc8p+0, 0x1.94cfeee86b1dap-15},
+    {0x1.4f9b2769d2ca7p+0, 0x1.4f98p+0, 0x1.93b4e9653569ap-15},
+    {0x1.516daa2cf6642p+0, 0x1.517p+0, -0x1.2ae984cdf1f77p-15},
+    {0x1.5342b569d4f82p+0, 0x1.534p+0, 0x1.5ab4ea7c0ef85p-15},
+    {0x1.551a4ca5d920fp+0, 0x1.5518p+0, 0x1.2652ec9076297p-15},
+    {0x1.56f4736b527dap+0, 0x1.56f8p+0, -0x1.c64a56c12cc8ap-15},
+    {0x1.58d12d497c7fdp+0, 0x1.58dp+0, 0x1.2d497c7fd252cp-16},
+    {0x1.5ab07dd485429p+0, 0x1.5abp+0, 0x1.f752150a56325p-18},
+    {0x1.5c9268a5946b7p+0, 0x1.5c9p+0, 0x1.3452ca35b80e2p-15},
+    {0x1.5e76f15ad2148p+0, 0x1.5e78p+0, -0x1.0ea52deb79164p-16},
+    {0x1.605e1b976dc09p+0, 0x1.606p+0, -0x1.e468923f74f89p-16},
+    {0x1.6247eb03a5585p+0, 0x1.6248p+0, -0x1.4fc5aa7b4e0f0p-20},
+    {0x1.6434634ccc320p+0, 0x1.6438p+0, -0x1.ce5999e701c48p-15},
+    {0x1.6623882552225p+0, 0x1.662p+0, 0x1.c412a91124894p-15},
+    {0x1.68155d44ca973p+0, 0x1.6818p+0, -0x1.515d9ab467bf2p-15},
+    {0x1.6a09e667f3bcdp+0, 0x1.6a08p+0, 0x1.e667f3bcc908bp-16},
+    {0x1.6c012750bdabfp+0, 0x1.6cp+0, 0x1.2750bdabeed77p-16},
+    {0x1.6dfb23c651a2fp+0, 0x1.6df8p+0, 0x1.91e328d177910p-15},
+    {0x1.6ff7df9519484p+0, 0x1.6ff8p+0, -0x1.035735be183c1p-19},
+    {0x1.71f75e8ec5f74p+0, 0x1.71f8p+0, -0x1.42e27411845b9p-17},
+    {0x1.73f9a48a58174p+0, 0x1.73f8p+0, 0x1.a48a58173bd5dp-16},
+    {0x1.75feb564267c9p+0, 0x1.76p+0, -0x1.4a9bd98374091p-16},
+    {0x1.780694fde5d3fp+0, 0x1.7808p+0, -0x1.6b021a2c09e65p-16},
+    {0x1.7a11473eb0187p+0, 0x1.7a1p+0, 0x1.473eb0186d7d5p-16},
+    {0x1.7c1ed0130c132p+0, 0x1.7c2p+0, -0x1.2fecf3ecd83b7p-16},
+    {0x1.7e2f336cf4e62p+0, 0x1.7e3p+0, -0x1.99261633bdf46p-17},
+    {0x1.80427543e1a12p+0, 0x1.804p+0, 0x1.3aa1f0d08db07p-15},
+    {0x1.82589994cce13p+0, 0x1.8258p+0, 0x1.332999c25159fp-17},
+    {0x1.8471a4623c7adp+0, 0x1.847p+0, 0x1.a4623c7acce53p-16},
+    {0x1.868d99b4492edp+0, 0x1.869p+0, -0x1.3325db689bf8ep-15},
+    {0x1.88ac7d98a6699p+0, 0x1.88bp+0, -0x1.c133accb34cd6p-15},
+    {0x1.8ace5422aa0dbp+0, 0x1.8adp+0, -0x1.abdd55f24a458p-16},
+    {0x1.8cf3216b5448cp+0, 0x1.8cfp+0, 0x1.90b5aa245f795p-15},
+    {0x1.8f1ae99157736p+0, 0x1.8f18p+0, 0x1.74c8abb9b15ccp-15},
+    {0x1.9145b0b91ffc6p+0, 0x1.9148p+0, -0x1.27a37001d3badp-15},
+    {0x1.93737b0cdc5e5p+0, 0x1.937p+0, 0x1.bd866e2f27a28p-15},
+    {0x1.95a44cbc8520fp+0, 0x1.95a8p+0, -0x1.d9a1bd6f88b26p-15},
+    {0x1.97d829fde4e50p+0, 0x1.97d8p+0, 0x1.4fef2727c5cf5p-19},
+    {0x1.9a0f170ca07bap+0, 0x1.9a1p+0, -0x1.d1e6bf08c8b9ep-17},
+    {0x1.9c49182a3f090p+0, 0x1.9c48p+0, 0x1.182a3f0901c7cp-16},
+    {0x1.9e86319e32323p+0, 0x1.9e88p+0, -0x1.ce61cdcdce7dbp-16},
+    {0x1.a0c667b5de565p+0, 0x1.a0c8p+0, -0x1.984a21a9b4d65p-16},
+    {0x1.a309bec4a2d33p+0, 0x1.a308p+0, 0x1.bec4a2d3358c1p-16},
+    {0x1.a5503b23e255dp+0, 0x1.a55p+0, 0x1.d91f12ae45a12p-19},
+    {0x1.a799e1330b358p+0, 0x1.a798p+0, 0x1.e1330b3586f2ep-16},
+    {0x1.a9e6b5579fdbfp+0, 0x1.a9e8p+0, -0x1.4aa860240bc15p-16},
+    {0x1.ac36bbfd3f37ap+0, 0x1.ac38p+0, -0x1.4402c0c863f24p-16},
+    {0x1.ae89f995ad3adp+0, 0x1.ae88p+0, 0x1.f995ad3ad5e87p-16},
+    {0x1.b0e07298db666p+0, 0x1.b0ep+0, 0x1.ca636d9964211p-18},
+    {0x1.b33a2b84f15fbp+0, 0x1.b338p+0, 0x1.15c278afd7b60p-15},
+    {0x1.b59728de5593ap+0, 0x1.b598p+0, -0x1.ae4354d8ce38fp-17},
+    {0x1.b7f76f2fb5e47p+0, 0x1.b7f8p+0, -0x1.21a0943722ab1p-17},
+    {0x1.ba5b030a1064ap+0, 0x1.ba58p+0, 0x1.818508324c206p-15},
+    {0x1.bcc1e904bc1d2p+0, 0x1.bccp+0, 0x1.e904bc1d2247cp-16},
+    {0x1.bf2c25bd71e09p+0, 0x1.bf3p+0, -0x1.ed21470fbbdfcp-15},
+    {0x1.c199bdd85529cp+0, 0x1.c198p+0, 0x1.bdd85529c2221p-16},
+    {0x1.c40ab5fffd07ap+0, 0x1.c408p+0, 0x1.5afffe83d368ap-15},
+    {0x1.c67f12e57d14bp+0, 0x1.c68p+0, -0x1.da3505d696bbep-17},
+    {0x1.c8f6d9406e7b5p+0, 0x1.c8f8p+0, -0x1.26bf9184aee53p-16},
+    {0x1.cb720dcef9069p+0, 0x1.cb7p+0, 0x1.06e77c8348a82p-15},
+    {0x1.cdf0b555dc3fap+0, 0x1.cdfp+0, 0x1.6aabb87f3889fp-17},
+    {0x1.d072d4a07897cp+0, 0x1.d07p+0, 0x1.6a503c4bdc688p-15},
+    {0x1.d2f87080d89f2p+0, 0x1.d2f8p+0, 0x1.c203627c62b78p-18},
+    {0x1.d5818dcfba487p+0, 0x1.d58p+0, 0x1.8dcfba48725dap-16},
+    {0x1.d80e316c98398p+0, 0x1.d81p+0, -0x1.ce9367c68447bp-16},
+    {0x1.da9e603db3285p+0, 0x1.daap+0, -0x1.9fc24cd7a8f74p-16},
+    {0x1.dd321f301b460p+0, 0x1.dd3p+0, 0x1.0f980da3025b5p-15},
+    {0x1.dfc97337b9b5fp+0, 0x1.dfc8p+0, 0x1.7337b9b5eb969p-16},
+    {0x1.e264614f5a129p+0, 0x1.e268p+0, -0x1.cf5852f6baf6cp-15},
+    {0x1.e502ee78b3ff6p+0, 0x1.e5p+0, 0x1.773c59ffb139fp-15},
+    {0x1.e7a51fbc74c83p+0, 0x1.e7a8p+0, -0x1.7021c59be5a56p-15},
+    {0x1.ea4afa2a490dap+0, 0x1.ea48p+0, 0x1.7d152486cc2c8p-15},
+    {0x1.ecf482d8e67f1p+0, 0x1.ecf8p+0, -0x1.be938cc07b928p-15},
+    {0x1.efa1bee615a27p+0, 0x1.efap+0, 0x1.bee615a277720p-16},
+    {0x1.f252b376bba97p+0, 0x1.f25p+0, 0x1.59bb5dd4ba743p-15},
+    {0x1.f50765b6e4540p+0, 0x1.f508p+0, -0x1.34923757f3161p-17},
+    {0x1.f7bfdad9cbe14p+0, 0x1.f7cp+0, -0x1.2931a0f63b762p-19},
+    {0x1.fa7c1819e90d8p+0, 0x1.fa8p+0, -0x1.f3f30b793e8b8p-15},
+    {0x1.fd3c22b8f71f1p+0, 0x1.fd4p+0, -0x1.eea3847077b45p-15},
 };
 RT_TABLE LogEntry kLogTable[128] = {
-    {0x1.fe00000000000p+0, 0x1.fc00000000000p-1, 0x1.60e32f44788d9p-1, -0x1.ac1bb6p-56f},
-    {0x1.fa10000000000p+0, 0x1.f420000000000p-1, 0x1.5ceb4e16f11bdp-1, 0x1.a65260p-55f},
-    {0x1.f630000000000p+0, 0x1.ec60000000000p-1, 0x1.58fbcdcdb80c2p-1, -0x1.6d76d0p-58f},
-    {0x1.f260000000000p+0, 0x1.e4c0000000000p-1, 0x1.5514efdbb2d63p-1, -0x1.b88128p-56f},
-    {0x1.eea0000000000p+0, 0x1.dd40000000000p-1, 0x1.5136f66336c97p-1, -0x1.0ed19cp-55f},
-    {0x1.eaf0000000000p+0, 0x1.d5e0000000000p-1, 0x1.4d62242e94aa0p-1, -0x1.1e2cdap-55f},
-    {0x1.e740000000000p+0, 0x1.ce80000000000p-1, 0x1.4985ece016ba9p-1, 0x1.6122ccp-55f},
-    {0x1.e3b0000000000p+0, 0x1.c760000000000p-1, 0x1.45c414576a743p-1, 0x1.aa159cp-55f},
-    {0x1.e020000000000p+0, 0x1.c040000000000p-1, 0x1.41fb1f8350d6ep-1, -0x1.29f84cp-56f},
-    {0x1.dca0000000000p+0, 0x1.b940000000000p-1, 0x1.3e3c23918e76cp-1, 0x1.56bc92p-55f},
-    {0x1.d930000000000p+0, 0x1.b260000000000p-1, 0x1.3a8766721ed12p-1, 0x1.1d0616p-55f},
-    {0x1.d5d0000000000p+0, 0x1.aba0000000000p-1, 0x1.36dd2e951ecccp-1, 0x1.58f138p-58f},
-    {0x1.d270000000000p+0, 0x1.a4e0000000000p-1, 0x1.332c33125536fp-1, 0x1.62bd6ep-55f},
-    {0x1.cf20000000000p+0, 0x1.9e40000000000p-1, 0x1.2f860b54da12ap-1, 0x1.eadaeap-55f},
-    {0x1.cbe0000000000p+0, 0x1.97c0000000000p-1, 0x1.2beaff89b89ecp-1, -0x1.5a84b6p-58f},
-    {0x1.c8b0000000000p+0, 0x1.9160000000000p-1, 0x1.285b5840fbf6ap-1, -0x1.5ffa74p-55f},
-    {0x1.c590000000000p+0, 0x1.8b20000000000p-1, 0x1.24d75e6134bdbp-1, 0x1.0fb9e4p-57f},
-    {0x1.c270000000000p+0, 0x1.84e0000000000p-1, 0x1.214d2b9d6c05cp-1, -0x1.b6177ep-55f},
-    {0x1.bf60000000000p+0, 0x1.7ec0000000000p-1, 0x1.1dcef9ca55ce8p-1, 0x1.e88388p-57f},
-    {0x1.bc50000000000p+0, 0x1.78a0000000000p-1, 0x1.1a4aa38b77f3cp-1, 0x1.619302p-55f},
-    {0x1.b950000000000p+0, 0x1.72a0000000000p-1, 0x1.16d2a38adf5edp-1, -0x1.fc87e8p-55f},
-    {0x1.b660000000000p+0, 0x1.6cc0000000000p-1, 0x1.1367452acf872p-1, -0x1.c7872ep-55f},
-    {0x1.b370000000000p+0, 0x1.66e0000000000p-1, 0x1.0ff6041a2bfaep-1, -0x1.767c08p-58f},
-    {0x1.b090000000000p+0, 0x1.6120000000000p-1, 0x1.0c91bc8186ce8p-1, 0x1.0d79bep-55f},
-    {0x1.adc0000000000p+0, 0x1.5b80000000000p-1, 0x1.093abae514ea2p-1, 0x1.188f44p-56f},
-    {0x1.aaf0000000000p+0, 0x1.55e0000000000p-1, 0x1.05de1c19707f8p-1, 0x1.c2c7e2p-58f},
-    {0x1.a830000000000p+0, 0x1.5060000000000p-1, 0x1.028f1d69a5ffep-1, 0x1.933550p-56f},
-    {0x1.a570000000000p+0, 0x1.4ae0000000000p-1, 0x1.fe7538ded33fdp-2, 0x1.649258p-58f},
-    {0x1.a2c0000000000p+0, 0x1.4580000000000p-1, 0x1.f7e82e660f5c1p-2, 0x1.a763b4p-57f},
-    {0x1.a020000000000p+0, 0x1.4040000000000p-1, 0x1.f177b7dfd4080p-2, -0x1.4d9368p-56f},
-    {0x1.9d80000000000p+0, 0x1.3b00000000000p-1, 0x1.eafcd2cea9d71p-2, 0x1.3a8c72p-57f},
-    {0x1.9ae0000000000p+0, 0x1.35c0000000000p-1, 0x1.e4775d2ec473fp-2, -0x1.16029ep-56f},
-    {0x1.9850000000000p+0, 0x1.30a0000000000p-1, 0x1.de0f55682c86bp-2, -0x1.c03c10p-56f},
-    {0x1.95d0000000000p+0, 0x1.2ba0000000000p-1, 0x1.d7c55acb1f74cp-2, 0x1.b67b28p-56f},
-    {0x1.9350000000000p+0, 0x1.26a0000000000p-1, 0x1.d1716d3f8bfacp-2, -0x1.1c903cp-56f},
-    {0x1.90d0000000000p+0, 0x1.21a0000000000p-1, 0x1.cb136d18feba4p-2, 0x1.c5d504p-58f},
-    {0x1.8e60000000000p+0, 0x1.1cc0000000000p-1, 0x1.c4d45b6e800bap-2, 0x1.b1a024p-57f},
-    {0x1.8c00000000000p+0, 0x1.1800000000000p-1, 0x1.beb4d9da71b7cp-2, -0x1.0f3c5ap-59f},
-    {0x1.89a0000000000p+0, 0x1.1340000000000p-1, 0x1.b88bea5879dfap-2, 0x1.f36db6p-57f},
-    {0x1.8740000000000p+0, 0x1.0e80000000000p-1, 0x1.b2596fb0c4ad3p-2, -0x1.fc0536p-56f},
-    {0x1.84f0000000000p+0, 0x1.09e0000000000p-1, 0x1.ac476d020486fp-2, 0x1.bc43bep-61f},
-    {0x1.82a0000000000p+0, 0x1.0540000000000p-1, 0x1.a62c25e7fae87p-2, 0x1.69d288p-58f},
-    {0x1.8060000000000p+0, 0x1.00c0000000000p-1, 0x1.a0321ed14dda4p-2, 0x1.ea5240p-56f},
-    {0x1.7e20000000000p+0, 0x1.f880000000000p-2, 0x1.9a2f1c2edb668p-2, 0x1.ae6274p-56f},
-    {0x1.7bf0000000000p+0, 0x1.efc0000000000p-2, 0x1.944e23354ad21p-2, -0x1.6a8be0p-57f},
-    {0x1.79c0000000000p+0, 0x1.e700000000000p-2, 0x1.8e64799901f7cp-2, -0x1.735f3ap-56f},
-    {0x1.7790000000000p+0, 0x1.de40000000000p-2, 0x1.88720582eb4cep-2, 0x1.79a060p-60f},
-    {0x1.7570000000000p+0, 0x1.d5c0000000000p-2, 0x1.82a28d34904c8p-2, -0x1.05ecc6p-59f},
-    {0x1.7350000000000p+0, 0x1.cd40000000000p-2, 0x1.7cca97da6a214p-2, -0x1.6643e0p-56f},
-    {0x1.7130000000000p+0, 0x1.c4c0000000000p-2, 0x1.76ea0c82cdd9cp-2, 0x1.65a91ap-56f},
-    {0x1.6f20000000000p+0, 0x1.bc80000000000p-2, 0x1.712d738157b5dp-2, 0x1.d319a4p-59f},
-    {0x1.6d20000000000p+0, 0x1.b480000000000p-2, 0x1.6b9574b0f8913p-2, 0x1.39be62p-58f},
-    {0x1.6b10000000000p+0, 0x1.ac40000000000p-2, 0x1.65c878c015543p-2, 0x1.94f3b8p-57f},
-    {0x1.6910000000000p+0, 0x1.a440000000000p-2, 0x1.6020689b1c74dp-2, 0x1.e0e330p-58f},
-    {0x1.6720000000000p+0, 0x1.9c80000000000p-2, 0x1.5a9ded96bc650p-2, -0x1.c04ec2p-57f},
-    {0x1.6520000000000p+0, 0x1.9480000000000p-2, 0x1.54e5f19e5bde4p-2, -0x1.8a7362p-63f},
-    {0x1.6330000000000p+0, 0x1.8cc0000000000p-2, 0x1.4f53de9d24b18p-2, 0x1.4d4cd2p-59f},
-    {0x1.6150000000000p+0, 0x1.8540000000000p-2, 0x1.49e85f23bbf99p-2, 0x1.323906p-57f},
-    {0x1.5f60000000000p+0, 0x1.7d80000000000p-2, 0x1.4446dddb9775ep-2, 0x1.e34224p-56f},
-    {0x1.5d80000000000p+0, 0x1.7600000000000p-2, 0x1.3ecc460ef5f50p-2, -0x1.4313e0p-58f},
-    {0x1.5bb0000000000p+0, 0x1.6ec0000000000p-2, 0x1.39794346979ccp-2, -0x1.b87198p-56f},
-    {0x1.59d0000000000p+0, 0x1.6740000000000p-2, 0x1.33efc101dbbe0p-2, 0x1.4ce40ap-63f},
-    {0x1.5800000000000p+0, 0x1.6000000000000p-2, 0x1.2e8e2bae11d31p-2, -0x1.8f4cdcp-56f},
-    {0x1.5640000000000p+0, 0x1.5900000000000p-2, 0x1.29552f81ff523p-2, 0x1.301772p-56f},
-    {0x1.5470000000000p+0, 0x1.51c0000000000p-2, 0x1.23e5398b931d0p-2, 0x1.d33310p-56f},
-    {0x1.52b0000000000p+0, 0x1.4ac0000000000p-2, 0x1.1e9e3678891f4p-2, 0x1.51d6e2p-56f},
-    {0x1.50f0000000000p+0, 0x1.43c0000000000p-2, 0x1.195033b43fa99p-2, 0x1.c66678p-56f},
-    {0x1.4f40000000000p+0, 0x1.3d00000000000p-2, 0x1.142bfeb9a0474p-2, -0x1.9e7a4ap-56f},
-    {0x1.4d80000000000p+0, 0x1.3600000000000p-2, 0x1.0ed005f657da4p-2, 0x1.c56bd2p-56f},
-    {0x1.4bd0000000000p+0, 0x1.2f40000000000p-2, 0x1.099e371c0bc82p-2, -0x1.9f2684p-59f},
-    {0x1.4a20000000000p+0, 0x1.2880000000000p-2, 0x1.0465a08154ffap-2, -0x1.05f0aep-56f},
-    {0x1.4880000000000p+0, 0x1.2200000000000p-2, 0x1.feb0233e607ccp-3, 0x1.6e32d6p-57f},
-    {0x1.46e0000000000p+0, 0x1.1b80000000000p-2, 0x1.f488311d1b493p-3, -0x1.058a0ep-57f},
-    {0x1.4540000000000p+0, 0x1.1500000000000p-2, 0x1.ea5349e23ac0ep-3, -0x1.b2ce30p-58f},
-    {0x1.43a0000000000p+0, 0x1.0e80000000000p-2, 0x1.e0114c533197fp-3, -0x1.4990bcp-59f},
-    {0x1.4210000000000p+0, 0x1.0840000000000p-2, 0x1.d627d7c1b2da7p-3, -0x1.41d2fap-57f},
-    {0x1.4080000000000p+0, 0x1.0200000000000p-2, 0x1.cc320c0176502p-3, 0x1.039a66p-57f},
-    {0x1.3ef0000000000p+0, 0x1.f780000000000p-3, 0x1.c22fca31887ddp-3, 0x1.58817cp-64f},
-    {0x1.3d60000000000p+0, 0x1.eb00000000000p-3, 0x1.b820f2fc7e508p-3, 0x1.77bcc4p-57f},
-    {0x1.3bd0000000000p+0, 0x1.de80000000000p-3, 0x1.ae05669628825p-3, 0x1.b0987ap-58f},
-    {0x1.3a50000000000p+0, 0x1.d280000000000p-3, 0x1.a4454820d19fap-3, -0x1.89c340p-58f},
-    {0x1.38d0000000000p+0, 0x1.c680000000000p-3, 0x1.9a7938d209947p-3, 0x1.637564p-57f},
-    {0x1.3750000000000p+0, 0x1.ba80000000000p-3, 0x1.90a11b46b9b56p-3, 0x1.013756p-63f},
-    {0x1.35e0000000000p+0, 0x1.af00000000000p-3, 0x1.8726935acac62p-3, 0x1.764c64p-57f},
-    {0x1.3460000000000p+0, 0x1.a300000000000p-3, 0x1.7d36832b8f0e3p-3, -0x1.74cf74p-58f},
-    {0x1.32f0000000000p+0, 0x1.9780000000000p-3, 0x1.73a4d01722e5cp-3, -0x1.9403e4p-57f},
-    {0x1.3180000000000p+0, 0x1.8c00000000000p-3, 0x1.6a079d0f7aad2p-3, -0x1.eedcbap-62f},
-    {0x1.3020000000000p+0, 0x1.8100000000000p-3, 0x1.60ca8fe8858afp-3, 0x1.2287fap-57f},
-    {0x1.2eb0000000000p+0, 0x1.7580000000000p-3, 0x1.57168c4aff0e6p-3, -0x1.2e7b70p-58f},
-    {0x1.2d50000000000p+0, 0x1.6a80000000000p-3, 0x1.4dc378969b1c1p-3, 0x1.ad9bb8p-58f},
-    {0x1.2bf0000000000p+0, 0x1.5f80000000000p-3, 0x1.446579dc223dep-3, -0x1.c2a542p-57f},
-    {0x1.2a90000000000p+0, 0x1.5480000000000p-3, 0x1.3afc766c1e210p-3, -0x1.2bf46ap-58f},
-    {0x1.2930000000000p+0, 0x1.4980000000000p-3, 0x1.3188543c098a1p-3, 0x1.51c006p-58f},
-    {0x1.27e0000000000p+0, 0x1.3f00000000000p-3, 0x1.2877bbc0b6ba6p-3, -0x1.7205eap-60f},
-    {0x1.2690000000000p+0, 0x1.3480000000000p-3, 0x1.1f5cd21a0d938p-3, 0x1.14d5dep-57f},
-    {0x1.2540000000000p+0, 0x1.2a00000000000p-3, 0x1.16377fb124192p-3, -0x1.e540bep-59f},
-    {0x1.23f0000000000p+0, 0x1.1f80000000000p-3, 0x1.0d07ac9dcbcf8p-3, -0x1.3bdf12p-57f},
-    {0x1.22a0000000000p+0, 0x1.1500000000000p-3, 0x1.03cd40a51ac0dp-3, 0x1.2f3828p-57f},
-    {0x1.2150000000000p+0, 0x1.0a80000000000p-3, 0x1.f510466fd80bfp-4, 0x1.b95ae8p-58f},
-    {0x1.2010000000000p+0, 0x1.0080000000000p-3, 0x1.e353fec9a2699p-4, -0x1.84447ap-62f},
-    {0x1.1ed0000000000p+0, 0x1.ed00000000000p-4, 0x1.d183f87ea737cp-4, 0x1.46a844p-58f},
-    {0x1.1d90000000000p+0, 0x1.d900000000000p-4, 0x1.bfa007672aa23p-4, -0x1.745a22p-58f},
-    {0x1.1c50000000000p+0, 0x1.c500000000000p-4, 0x1.ada7fec6ac801p-4, 0x1.01a5d8p-59f},
-    {0x1.1b10000000000p+0, 0x1.b100000000000p-4, 0x1.9b9bb14949167p-4, -0x1.cdb2f8p-59f},
-    {0x1.19e0000000000p+0, 0x1.9e00000000000p-4, 0x1.8a6377a915c29p-4, -0x1.1296e6p-58f},
-    {0x1.18b0000000000p+0, 0x1.8b00000000000p-4, 0x1.7918a1bf981d6p-4, 0x1.11d0f4p-59f},
-    {0x1.1780000000000p+0, 0x1.7800000000000p-4, 0x1.67bb0726ec0fcp-4, -0x1.b692c2p-58f},
-    {0x1.1650000000000p+0, 0x1.6500000000000p-4, 0x1.564a7ef514311p-4, 0x1.9517ccp-59f},
-    {0x1.1520000000000p+0, 0x1.5200000000000p-4, 0x1.44c6dfb9b7606p-4, 0x1.75f068p-58f},
-    {0x1.13f0000000000p+0, 0x1.3f00000000000p-4, 0x1.332fff7bd1f18p-4, 0x1.41527ap-59f},
-    {0x1.12d0000000000p+0, 0x1.2d00000000000p-4, 0x1.22743457a9c8ep-4, -0x1.4bdf52p-58f},
-    {0x1.11a0000000000p+0, 0x1.1a00000000000p-4, 0x1.10b75afd660c6p-4, 0x1.7330e6p-60f},
-    {0x1.1080000000000p+0, 0x1.0800000000000p-4, 0x1.ffae9119b9303p-5, 0x1.ba1316p-60f},
-    {0x1.0f60000000000p+0, 0x1.ec00000000000p-5, 0x1.ddcaadb46ef1bp-5, 0x1.09ab70p-62f},
-    {0x1.0e40000000000p+0, 0x1.c800000000000p-5, 0x1.bbc2bfc44f417p-5, 0x1.e5bafap-60f},
-    {0x1.0d20000000000p+0, 0x1.a400000000000p-5, 0x1.99967a4f2b1c8p-5, 0x1.976b98p-59f},
-    {0x1.0c10000000000p+0, 0x1.8200000000000p-5, 0x1.792e93e5199edp-5, -0x1.a88378p-59f},
-    {0x1.0af0000000000p+0, 0x1.5e00000000000p-5, 0x1.56bac43ed7f9ap-5, -0x1.5c8202p-61f},
-    {0x1.09e0000000000p+0, 0x1.3c00000000000p-5, 0x1.360ebf5d83765p-5, 0x1.9281d2p-59f},
-    {0x1.08d0000000000p+0, 0x1.1a00000000000p-5, 0x1.15413ca0e72a8p-5, -0x1.b1d2c2p-59f},
-    {0x1.07c0000000000p+0, 0x1.f000000000000p-6, 0x1.e8a3ee30cdcacp-6, 0x1.7086b2p-63f},
-    {0x1.06b0000000000p+0, 0x1.ac00000000000p-6, 0x1.a68151fb5c04ap-6, -0x1.080ed4p-64f},
-    {0x1.05a0000000000p+0, 0x1.6800000000000p-6, 0x1.641a176270d6fp-6, 0x1.8ca45ep-60f},
-    {0x1.0490000000000p+0, 0x1.2400000000000p-6, 0x1.216daf6d9321ap-6, -0x1.87ca50p-60f},
-    {0x1.0390000000000p+0, 0x1.c800000000000p-7, 0x1.c4db352e6d472p-7, -0x1.f0d974p-61f},
-    {0x1.0280000000000p+0, 0x1.4000000000000p-7, 0x1.3e7295d25a7d9p-7, -0x1.ff29a2p-65f},
-    {0x1.0180000000000p+0, 0x1.8000000000000p-8, 0x1.7ee11ebd82e94p-8, -0x1.61e96ep-62f},
-    {0x1.0000000000000p+0, 0x0.0p+0, 0x0.0p+0, 0x0.0p+0f},
+    {0x1.fep+0, 0x1.fcp-1, 0x1.60e32f4478p-1, 0x1.1b195p-42f},
+    {0x1.fa1p+0, 0x1.f42p-1, 0x1.5ceb4e16f2p-1, -0x1.c852cep-42f},
+    {0x1.f63p+0, 0x1.ec6p-1, 0x1.58fbcdcdb8p-1, 0x1.83e928p-46f},
+    {0x1.f26p+0, 0x1.e4cp-1, 0x1.5514efdbb2p-1, 0x1.ac591ep-42f},
+    {0x1.eeap+0, 0x1.dd4p-1, 0x1.5136f66336p-1, 0x1.92d78ap-42f},
+    {0x1.eafp+0, 0x1.d5ep-1, 0x1.4d62242e94p-1, 0x1.53f70ep-42f},
+    {0x1.e74p+0, 0x1.ce8p-1, 0x1.4985ece016p-1, 0x1.752b0ap-42f},
+    {0x1.e3bp+0, 0x1.c76p-1, 0x1.45c414576ap-1, 0x1.d0daa2p-43f},
+    {0x1.e02p+0, 0x1.c04p-1, 0x1.41fb1f835p-1, 0x1.adbb58p-42f},
+    {0x1.dcap+0, 0x1.b94p-1, 0x1.3e3c23918ep-1, 0x1.db156cp-43f},
+    {0x1.d93p+0, 0x1.b26p-1, 0x1.3a8766721ep-1, 0x1.a248e8p-42f},
+    {0x1.d5dp+0, 0x1.abap-1, 0x1.36dd2e951ep-1, 0x1.998158p-42f},
+    {0x1.d27p+0, 0x1.a4ep-1, 0x1.332c331256p-1, -0x1.9214eap-42f},
+    {0x1.cf2p+0, 0x1.9e4p-1, 0x1.2f860b54dap-1, 0x1.2a7ab6p-45f},
+    {0x1.cbep+0, 0x1.97cp-1, 0x1.2beaff89b8p-1, 0x1.3d7ea6p-42f},
+    {0x1.c8bp+0, 0x1.916p-1, 0x1.285b5840fcp-1, -0x1.2caffep-46f},
+    {0x1.c59p+0, 0x1.8b2p-1, 0x1.24d75e6134p-1, 0x1.7b622p-42f},
+    {0x1.c27p+0, 0x1.84ep-1, 0x1.214d2b9d6cp-1, 0x1.6e49e8p-47f},
+    {0x1.bf6p+0, 0x1.7ecp-1, 0x1.1dcef9ca56p-1, -0x1.8bf0bcp-44f},
+    {0x1.bc5p+0, 0x1.78ap-1, 0x1.1a4aa38b78p-1, -0x1.874f36p-46f},
+    {0x1.b95p+0, 0x1.72ap-1, 0x1.16d2a38aep-1, -0x1.426fe4p-42f},
+    {0x1.b66p+0, 0x1.6ccp-1, 0x1.1367452adp-1, -0x1.e39c78p-43f},
+    {0x1.b37p+0, 0x1.66ep-1, 0x1.0ff6041a2cp-1, -0x1.482edp-47f},
+    {0x1.b09p+0, 0x1.612p-1, 0x1.0c91bc8186p-1, 0x1.9d086cp-42f},
+    {0x1.adcp+0, 0x1.5b8p-1, 0x1.093abae514p-1, 0x1.d44462p-42f},
+    {0x1.aafp+0, 0x1.55ep-1, 0x1.05de1c197p-1, 0x1.fe0386p-43f},
+    {0x1.a83p+0, 0x1.506p-1, 0x1.028f1d69a6p-1, -0x1.cd9956p-53f},
+    {0x1.a57p+0, 0x1.4aep-1, 0x1.fe7538ded4p-2, -0x1.805d36p-43f},
+    {0x1.a2cp+0, 0x1.458p-1, 0x1.f7e82e661p-2, -0x1.47d962p-43f},
+    {0x1.a02p+0, 0x1.404p-1, 0x1.f177b7dfd4p-2, 0x1.feb26cp-48f},
+    {0x1.9d8p+0, 0x1.3bp-1, 0x1.eafcd2cea8p-2, 0x1.d71276p-42f},
+    {0x1.9aep+0, 0x1.35cp-1, 0x1.e4775d2ec4p-2, 0x1.cfaeap-44f},
+    {0x1.985p+0, 0x1.30ap-1, 0x1.de0f55682cp-2, 0x1.0d51fep-43f},
+    {0x1.95dp+0, 0x1.2bap-1, 0x1.d7c55acb2p-2, -0x1.16724cp-43f},
+    {0x1.935p+0, 0x1.26ap-1, 0x1.d1716d3f8cp-2, -0x1.511c9p-48f},
+    {0x1.90dp+0, 0x1.21ap-1, 0x1.cb136d19p-2, -0x1.45be3ap-42f},
+    {0x1.8e6p+0, 0x1.1ccp-1, 0x1.c4d45b6e8p-2, 0x1.746c68p-47f},
+    {0x1.8cp+0, 0x1.18p-1, 0x1.beb4d9da7p-2, 0x1.b7bf78p-42f},
+    {0x1.89ap+0, 0x1.134p-1, 0x1.b88bea5878p-2, 0x1.dfa3e6p-42f},
+    {0x1.874p+0, 0x1.0e8p-1, 0x1.b2596fb0c4p-2, 0x1.5a502p-43f},
+    {0x1.84fp+0, 0x1.09ep-1, 0x1.ac476d0204p-2, 0x1.0de07p-43f},
+    {0x1.82ap+0, 0x1.054p-1, 0x1.a62c25e7fcp-2, -0x1.178e96p-42f},
+    {0x1.806p+0, 0x1.00cp-1, 0x1.a0321ed14cp-2, 0x1.da47aap-42f},
+    {0x1.7e2p+0, 0x1.f88p-2, 0x1.9a2f1c2edcp-2, -0x1.32f28cp-43f},
+    {0x1.7bfp+0, 0x1.efcp-2, 0x1.944e23354cp-2, -0x1.2df2d6p-42f},
+    {0x1.79cp+0, 0x1.e7p-2, 0x1.8e647999p-2, 0x1.f7ba32p-42f},
+    {0x1.779p+0, 0x1.de4p-2, 0x1.88720582ecp-2, -0x1.663f44p-43f},
+    {0x1.757p+0, 0x1.d5cp-2, 0x1.82a28d349p-2, 0x1.31fdf4p-44f},
+    {0x1.735p+0, 0x1.cd4p-2, 0x1.7cca97da6cp-2, -0x1.dec59ap-42f},
+    {0x1.713p+0, 0x1.c4cp-2, 0x1.76ea0c82ccp-2, 0x1.d9c596p-42f},
+    {0x1.6f2p+0, 0x1.bc8p-2, 0x1.712d738158p-2, -0x1.28bc5ap-44f},
+    {0x1.6d2p+0, 0x1.b48p-2, 0x1.6b9574b0f8p-2, 0x1.226274p-43f},
+    {0x1.6b1p+0, 0x1.ac4p-2, 0x1.65c878c014p-2, 0x1.54332ap-42f},
+    {0x1.691p+0, 0x1.a44p-2, 0x1.6020689b1cp-2, 0x1.d34784p-44f},
+    {0x1.672p+0, 0x1.9c8p-2, 0x1.5a9ded96bcp-2, 0x1.93f1fep-44f},
+    {0x1.652p+0, 0x1.948p-2, 0x1.54e5f19e5cp-2, -0x1.0e0062p-45f},
+    {0x1.633p+0, 0x1.8ccp-2, 0x1.4f53de9d24p-2, 0x1.63014ep-43f},
+    {0x1.615p+0, 0x1.854p-2, 0x1.49e85f23bcp-2, -0x1.9b66e4p-48f},
+    {0x1.5f6p+0, 0x1.7d8p-2, 0x1.4446dddb98p-2, -0x1.1430e6p-43f},
+    {0x1.5d8p+0, 0x1.76p-2, 0x1.3ecc460ef4p-2, 0x1.f4febcp-42f},
+    {0x1.5bbp+0, 0x1.6ecp-2, 0x1.3979434698p-2, -0x1.8d1b88p-44f},
+    {0x1.59dp+0, 0x1.674p-2, 0x1.33efc101dcp-2, -0x1.07ffd6p-44f},
+    {0x1.58p+0, 0x1.6p-2, 0x1.2e8e2bae1p-2, 0x1.d309c2p-42f},
+    {0x1.564p+0, 0x1.59p-2, 0x1.29552f82p-2, -0x1.5b968p-43f},
+    {0x1.547p+0, 0x1.51cp-2, 0x1.23e5398b94p-2, -0x1.c5f166p-43f},
+    {0x1.52bp+0, 0x1.4acp-2, 0x1.1e9e367888p-2, 0x1.1f4548p-42f},
+    {0x1.50fp+0, 0x1.43cp-2, 0x1.195033b44p-2, -0x1.59a39ap-44f},
+    {0x1.4f4p+0, 0x1.3dp-2, 0x1.142bfeb9ap-2, 0x1.1ce618p-44f},
+    {0x1.4d8p+0, 0x1.36p-2, 0x1.0ed005f658p-2, -0x1.2dc752p-45f},
+    {0x1.4bdp+0, 0x1.2f4p-2, 0x1.099e371c0cp-2, -0x1.bf067cp-45f},
+    {0x1.4a2p+0, 0x1.288p-2, 0x1.0465a08154p-2, 0x1.ff37dp-43f},
+    {0x1.488p+0, 0x1.22p-2, 0x1.feb0233e6p-3, 0x1.f316e4p-45f},
+    {0x1.46ep+0, 0x1.1b8p-2, 0x1.f488311d18p-3, 0x1.a495f4p-42f},
+    {0x1.454p+0, 0x1.15p-2, 0x1.ea5349e238p-3, 0x1.606e4ep-42f},
+    {0x1.43ap+0, 0x1.0e8p-2, 0x1.e0114c533p-3, 0x1.97eeb6p-43f},
+    {0x1.421p+0, 0x1.084p-2, 0x1.d627d7c1bp-3, 0x1.6d357cp-42f},
+    {0x1.408p+0, 0x1.02p-2, 0x1.cc320c0178p-3, -0x1.afdbf2p-43f},
+    {0x1.3efp+0, 0x1.f78p-3, 0x1.c22fca3188p-3, 0x1.f7402cp-45f},
+    {0x1.3d6p+0, 0x1.ebp-3, 0x1.b820f2fc8p-3, -0x1.af7a22p-43f},
+    {0x1.3bdp+0, 0x1.de8p-3, 0x1.ae05669628p-3, 0x1.04a6c2p-44f},
+    {0x1.3a5p+0, 0x1.d28p-3, 0x1.a4454820dp-3, 0x1.9f9cecp-43f},
+    {0x1.38dp+0, 0x1.c68p-3, 0x1.9a7938d208p-3, 0x1.94758ep-43f},
+    {0x1.375p+0, 0x1.ba8p-3, 0x1.90a11b46b8p-3, 0x1.b5601p-43f},
+    {0x1.35ep+0, 0x1.afp-3, 0x1.8726935ac8p-3, 0x1.6312ecp-42f},
+    {0x1.346p+0, 0x1.a3p-3, 0x1.7d36832b9p-3, -0x1.e3a5d4p-44f},
+    {0x1.32fp+0, 0x1.978p-3, 0x1.73a4d0172p-3, 0x1.72dcd8p-42f},
+    {0x1.318p+0, 0x1.8cp-3, 0x1.6a079d0f78p-3, 0x1.568fe2p-42f},
+    {0x1.302p+0, 0x1.81p-3, 0x1.60ca8fe888p-3, -0x1.3a85bap-42f},
+    {0x1.2ebp+0, 0x1.758p-3, 0x1.57168c4bp-3, -0x1.e344bap-44f},
+    {0x1.2d5p+0, 0x1.6a8p-3, 0x1.4dc3789698p-3, 0x1.8e09aep-42f},
+    {0x1.2bfp+0, 0x1.5f8p-3, 0x1.446579dc2p-3, 0x1.1eec7ap-42f},
+    {0x1.2a9p+0, 0x1.548p-3, 0x1.3afc766c2p-3, -0x1.df0258p-43f},
+    {0x1.293p+0, 0x1.498p-3, 0x1.3188543c08p-3, 0x1.8a12a4p-43f},
+    {0x1.27ep+0, 0x1.3fp-3, 0x1.2877bbc0b8p-3, -0x1.45a0bap-43f},
+    {0x1.269p+0, 0x1.348p-3, 0x1.1f5cd21a1p-3, -0x1.363dd6p-42f},
+    {0x1.254p+0, 0x1.2ap-3, 0x1.16377fb128p-3, -0x1.f370f2p-42f},
+    {0x1.23fp+0, 0x1.1f8p-3, 0x1.0d07ac9dc8p-3, 0x1.e7bd88p-42f},
+    {0x1.22ap+0, 0x1.15p-3, 0x1.03cd40a518p-3, 0x1.606a5ep-42f},
+    {0x1.215p+0, 0x1.0a8p-3, 0x1.f510466fep-4, -0x1.fd0246p-42f},
+    {0x1.201p+0, 0x1.008p-3, 0x1.e353fec9ap-4, 0x1.34c7dp-43f},
+    {0x1.1edp+0, 0x1.edp-4, 0x1.d183f87eap-4, 0x1.cdf146p-42f},
+    {0x1.1d9p+0, 0x1.d9p-4, 0x1.bfa007673p-4, -0x1.577574p-42f},
+    {0x1.1c5p+0, 0x1.c5p-4, 0x1.ada7fec6bp-4, -0x1.bff6fep-43f},
+    {0x1.1b1p+0, 0x1.b1p-4, 0x1.9b9bb1495p-4, -0x1.ba64e6p-42f},
+    {0x1.19ep+0, 0x1.9ep-4, 0x1.8a6377a91p-4, 0x1.70a2eep-42f},
+    {0x1.18bp+0, 0x1.8bp-4, 0x1.7918a1bfap-4, -0x1.f8a778p-42f},
+    {0x1.178p+0, 0x1.78p-4, 0x1.67bb0726fp-4, -0x1.f8236ep-43f},
+    {0x1.165p+0, 0x1.65p-4, 0x1.564a7ef51p-4, 0x1.0c44cap-42f},
+    {0x1.152p+0, 0x1.52p-4, 0x1.44c6dfb9bp-4, 0x1.d81976p-42f},
+    {0x1.13fp+0, 0x1.3fp-4, 0x1.332fff7bdp-4, 0x1.f18282p-44f},
+    {0x1.12dp+0, 0x1.2dp-4, 0x1.22743457bp-4, -0x1.8dc94cp-42f},
+    {0x1.11ap+0, 0x1.1ap-4, 0x1.10b75afd6p-4, 0x1.83185cp-42f},
+    {0x1.108p+0, 0x1.08p-4, 0x1.ffae9119cp-5, -0x1.b3f322p-43f},
+    {0x1.0f6p+0, 0x1.ecp-5, 0x1.ddcaadb46p-5, 0x1.de361p-42f},
+    {0x1.0e4p+0, 0x1.c8p-5, 0x1.bbc2bfc44p-5, 0x1.e82e7ap-42f},
+    {0x1.0d2p+0, 0x1.a4p-5, 0x1.99967a4f2p-5, 0x1.6390ccp-42f},
+    {0x1.0c1p+0, 0x1.82p-5, 0x1.792e93e52p-5, -0x1.984da8p-43f},
+    {0x1.0afp+0, 0x1.5ep-5, 0x1.56bac43eep-5, -0x1.00cc2cp-42f},
+    {0x1.09ep+0, 0x1.3cp-5, 0x1.360ebf5d8p-5, 0x1.bb2b26p-44f},
+    {0x1.08dp+0, 0x1.1ap-5, 0x1.15413ca0ep-5, 0x1.ca9e4ep-43f},
+    {0x1.07cp+0, 0x1.fp-6, 0x1.e8a3ee30cp-6, 0x1.b95818p-43f},
+    {0x1.06bp+0, 0x1.acp-6, 0x1.a68151fb4p-6, 0x1.c049fcp-42f},
+    {0x1.05ap+0, 0x1.68p-6, 0x1.641a17628p-6, -0x1.e5213ap-43f},
+    {0x1.049p+0, 0x1.24p-6, 0x1.216daf6d8p-6, 0x1.32199ep-42f},
+    {0x1.0p+0, 0x0.0p+0, 0x0.0p+0, 0x0.0p+0f},
+    {0x1.0p+0, 0x0.0p+0, 0x0.0p+0, 0x0.0p+0f},
+    {0x1.0p+0, 0x0.0p+0, 0x0.0p+0, 0x0.0p+0f},
+    {0x1.0p+0, 0x0.0p+0, 0x0.0p+0, 0x0.0p+0f},
 };
 
 // x = k ln2/128 + r + r_lo with |r| <= ln2/256 + the rounding of the FP32
-// quotient kf; r is exact, r_lo the remainder of k ln2/128.
+// quotient, r exact and r_lo the remainder of k ln2/128; for x below 6.5 ln2/128
+// (0.035) k = 0 and r = x.
 struct Reduced {
   int k;
   double r;
   float r_lo;
 };
-RT_FN Reduced reduce(float kf, double x) {
+RT_FN Reduced reduce(double x) {
+  float kf = rintf(cut(x) * 184.664965f);  // 128 / ln 2
+  kf = kf < 7.0f ? 0.0f : fminf(kf, 131071.0f);  // 2^1024 is no double
   return Reduced{(int)kf, fma(-widen(kf), kLn2Over128, x), -kf * kLn2Over128Lo};
-}
-constexpr float k128OverLn2 = 184.664965f;
-
-// X + Y, rounded, and its rounding error, for |X| >= |Y| or X = 0 (Dekker, 1971).
-RT_FN double add_exact(double X, double Y, double& err) {
-  const double s = X + Y;
-  err = (X - s) + Y;
-  return s;
 }
 
 // 1 - exp(-x) for x >= 0 (finite).  With T = 2^(-k/128) and p = 1 - exp(-r -
-// r_lo): 1 - exp(-x) = (1 - T) + T p, where 1 - T = (1 - 2^-m) + 2^-m a.  The two
-// largest terms are added exactly: for m > 0 those of 1 - T, for m = 0 (1 - T =
-// a) a and T r, whose own rounding error is kept too.  From 54 ln 2 on the
-// result rounds to 1.
+// r_lo): 1 - exp(-x) = (1 - T) + T p.  1 - T is the exact difference of 1 and T's
+// leading 13 bits, plus the remainder, which joins T p: from k = 7 on that is
+// small enough against the result for its rounding not to count (below, k = 0
+// and the result is p, rounded once).  With T < 2^-5 all of it is small.  From 54
+// ln 2 on the result rounds to 1.
 RT_FN double one_minus_exp(double x) {
   const bool big = bits_of(x) > 0x4042b5c28f5c28f6ll;  // x > 37.42
-  const Reduced R = reduce(rintf((big ? 0.0f : cut(x)) * k128OverLn2), x);
+  const Reduced R = reduce(big ? 0.0 : x);
   const double r = R.r;
-  // p = r + r (-r/2 + r^2/6 - r^3/24 + r^4 (1/120 - r/720)) + r_lo (1 - r)
+  // p = r + r (-r/2 + r^2/6 - r^3/24 + r^4/120 - r^5 (1/720 - r/5040 + ...)) + r_lo (1 - r)
   const float rf = cut(r);
-  double q = fma(r, widen(fmaf(rf, -1.0f / 720.0f, 1.0f / 120.0f)), -1.0 / 24.0);
+  const float tail = fmaf(rf, fmaf(rf, fmaf(rf, 1.0f / 362880.0f, -1.0f / 40320.0f), 1.0f / 5040.0f), -1.0f / 720.0f);
+  double q = fma(r, widen(tail), 1.0 / 120.0);
+  q = fma(r, q, -1.0 / 24.0);
   q = fma(r, q, 1.0 / 6.0);
   q = fma(r, q, -0.5);
   const double r_lo = widen(R.r_lo);
   const double v = fma(r, fma(r, q, -r_lo), r_lo);
   const ExpEntry e = kExpTable[R.k & 127];
   const int m = R.k >> 7;
-  const bool low = m == 0;
   const long long scale = (long long)m << 52;
+  const bool far = m > 5;
   const double T = double_of(bits_of(e.t) - scale);
-  const double a = (R.k & 127) ? double_of(bits_of(e.a) - scale) : 0.0;
-  const double p1 = T * r, e1 = fma(T, r, -p1);
-  const double above = double_of(0x3ff0000000000000ll - (1ll << (53 - m)));  // 1 - 2^-m
-  double err;
-  const double s = add_exact(low ? e.a : above, low ? p1 : a, err);
-  const double w = fma(T, v, low ? e1 : p1);
-  const float lo = fmaf(e.t_lo, rf, e.a_lo) * float_of((unsigned)(127 - m) << 23);
-  return big ? 1.0 : s + (w + (err + widen(lo)));
+  const double hi = far ? 0.0 : double_of(bits_of(e.hi) - scale);
+  const double lo = far ? -T : ((R.k & 127) ? double_of(bits_of(e.lo) - scale) : 0.0);
+  const double w = fma(T, r, fma(T, v, lo));
+  return big ? 1.0 : (1.0 - hi) + w;
 }
 
 // exp(x) - 1 for 0 <= x <= 709.78 (the largest with a finite result), in the
-// same way: T = 2^(k/128), exp(x) - 1 = (T - 1) + T p, p = exp(r + r_lo) - 1.
+// same way: T = 2^(k/128), exp(x) - 1 = (T - 1) + T p, p = exp(r + r_lo) - 1; from
+// T = 2^53 on the 1 is one of the small terms.
 RT_FN double exp_minus_one(double x) {
-  // (2^1024 is no double: the last half interval takes the one below)
-  const Reduced R = reduce(fminf(rintf(cut(x) * k128OverLn2), 131071.0f), x);
+  const Reduced R = reduce(x);
   const double r = R.r;
-  // p = r + r (r/2 + r^2/6 + r^3/24 + r^4 (1/120 + r/720)) + r_lo (1 + r)
+  // p = r + r (r/2 + r^2/6 + r^3/24 + r^4/120 + r^5 (1/720 + r/5040 + ...)) + r_lo (1 + r)
   const float rf = cut(r);
-  double q = fma(r, widen(fmaf(rf, 1.0f / 720.0f, 1.0f / 120.0f)), 1.0 / 24.0);
+  const float tail = fmaf(rf, fmaf(rf, fmaf(rf, 1.0f / 362880.0f, 1.0f / 40320.0f), 1.0f / 5040.0f), 1.0f / 720.0f);
+  double q = fma(r, widen(tail), 1.0 / 120.0);
+  q = fma(r, q, 1.0 / 24.0);
   q = fma(r, q, 1.0 / 6.0);
   q = fma(r, q, 0.5);
   const double r_lo = widen(R.r_lo);
   const double v = fma(r, fma(r, q, r_lo), r_lo);
-  const ExpUpEntry e = kExpUpTable[R.k & 127];
-  const bool low = R.k < 128;
-  const long long scale = (long long)(R.k >> 7) << 52;
+  const ExpEntry e = kExpUpTable[R.k & 127];
+  const int m = R.k >> 7;
+  const long long scale = (long long)m << 52;
   const double T = double_of(bits_of(e.t) + scale);
-  const double lo = low ? e.a_lo : ((R.k & 127) ? double_of(bits_of(e.t_lo) + scale) : 0.0);
-  const double p1 = T * r, e1 = fma(e.t_lo, r, fma(T, r, -p1));  // (e1 is for m = 0)
-  double err;
-  const double s = add_exact(low ? e.a : T, low ? p1 : -1.0, err);
-  const double w = fma(T, v, low ? e1 : p1);
-  return s + (w + (err + lo));
+  const double hi = double_of(bits_of(e.hi) + scale);
+  double lo = (R.k & 127) ? double_of(bits_of(e.lo) + scale) : 0.0;
+  if (m > 52) lo -= 1.0;
+  const double w = fma(T, r, fma(T, v, lo));
+  return (hi - (m > 52 ? 0.0 : 1.0)) + w;
 }
 
 // a / (exp(x) - 1) for x > 0; zero above 709.78, where exp(x) - 1 overflows.
@@ -569,10 +564,10 @@ RT_FN double bose(double x, double a = 1.0) {
 }
 
 // -ln(1 - v) for 0 <= v < 1.  y = 1 - v = 2^-m z with z in (1/2, 1], z rc = 1 +
-// r, |r| <= 2^-8: -ln(1 - v) = m ln 2 + ln rc - ln(1 + r).  r = (rc - 1) - rc (1
+// r, |r| <= 2^-8 (2^-6 on the last four intervals, where rc = 1): -ln(1 - v) = m ln 2 + ln rc - ln(1 + r).  r = (rc - 1) - rc (1
 // - z), where 1 - z is v for m = 0 (v < 1/2) and exact above; the product's
-// rounding error is kept.  The two largest terms are added exactly: m ln 2 and
-// ln rc for m > 0, ln rc and -r for m = 0.
+// rounding error is kept.  m ln 2 + ln rc to a multiple of 2^-40 is exact; its
+// remainder joins ln(1 + r).  Below 1/64 the result is that, rounded once.
 RT_FN double neg_log_one_minus(double v) {
   const bool low = bits_of(v) < 0x3fe0000000000000ll;  // v < 1/2
   long long by = bits_of(1.0 - v);
@@ -584,17 +579,17 @@ RT_FN double neg_log_one_minus(double v) {
   const double w = low ? v : 1.0 - z;
   const double P = e.rc * w, pe = fma(e.rc, w, -P);
   const double r = e.c - P;  // exact; 1 + r - pe = z rc
-  // -ln(1 + r) = -r + r (r/2 - r^2/3 + r^3/4 - r^4 (1/5 - r/6 + r^2/7))
+  // -ln(1 + r) = -r + r (r/2 - r^2/3 + r^3/4 - r^4/5 + r^5 (1/6 - r/7 + ...))
   const float rf = cut(r);
-  const float tail = fmaf(rf, fmaf(rf, -1.0f / 7.0f, 1.0f / 6.0f), -1.0f / 5.0f);
-  double q = fma(r, widen(tail), 0.25);
+  const float tail =
+      fmaf(rf, fmaf(rf, fmaf(rf, fmaf(rf, 1.0f / 10.0f, -1.0f / 9.0f), 1.0f / 8.0f), -1.0f / 7.0f), 1.0f / 6.0f);
+  double q = fma(r, widen(tail), -0.2);
+  q = fma(r, q, 0.25);
   q = fma(r, q, -1.0 / 3.0);
   q = fma(r, q, 0.5);
   const float mf = (float)m;
-  double err;
-  const double s = add_exact(low ? e.ln : widen(mf) * kLn2, low ? -r : e.ln, err);
-  const double u = fma(r, r * q, low ? pe : pe - r);
-  return s + (u + (err + widen(fmaf(mf, kLn2Lo, e.ln_lo))));
+  const float lo = cut(pe) + fmaf(mf, kLn2Lo, e.ln_lo);
+  return fma(widen(mf), kLn2, e.ln) + (fma(r, r * q, widen(lo)) - r);
 }
 
 }  // namespace rtk

@@ -2,9 +2,10 @@
 FP32 terms: little but the rounding of the result itself (at most 1/2 ulp,
 1/sqrt(12) ulp rms) is left, against extended precision, the same source
 compiled as C++.  What may be added to it: the FP32 tail of the logarithm's
-series, r^4 / 5 of the result with |r| <= 2^-8 and a relative error of 2^-23,
-and the FP32 remainders of tables and constants, 2^-53 of the largest term
-with the same error: at most 2^-4 ulp together."""
+series, r^5 / 6 of the result with |r| <= 2^-6 and a relative error of 7.5e-8
+(the constant's and one rounding), or the rounding of the part beyond the exact
+one, 2^-63 against a result above 0.0156 (an ulp of 2^-58) and 2^-62 above 0.034
+(2^-57): at most 1/10 ulp."""
 import ctypes
 import os
 import subprocess
