@@ -250,8 +250,8 @@ typedef struct {
                            more with debug records): beyond it a launch goes part by part, on
                            cartesian grids its last peel-offs walk in place.  0 (default): 4e9 on
                            cartesian grids, else 2^28 (9.7 GB), or in place when memory is too
-                           short for the records of 2^20 packets.  The buffer is sized from the
-                           last launch's count, takes at most 40 % of the free device memory,
+                           short for 2^23 (0.3 GB).  The buffer is sized from the last
+                           launch's count, takes at most 40 % of the free device memory,
                            and is kept until the context is destroyed                         */
 } rt_launch_opts;
 

@@ -1139,14 +1139,15 @@ namespace {
 // records the buffer holds by the estimate.
 constexpr unsigned long long kPeelPart = 1ull << 28;
 constexpr unsigned long long kPeelMost = 4000000000ull;
-// The fewest packets of a part: each part clears and scans the counts of all
-// keys and ends with its last packets' walks.  When memory is too short for that
-// many packets' records, the launch walks its peel-offs in place.  2e6 packets
-// whole / in parts of 2^20, 2^19, 2^18, 2^16 / in place: octree of 4e5 leaves 35 /
-// 47, 61, 102, 299 / 51 ms, of 3e6 leaves 69 / 99, 135, 223, 657 / 95 ms, k-d tree
-// of 2e5 leaves 38 / 54, 71, 125, 379 / 69 ms, 3e4 Voronoi cells (1.5e6 packets)
-// 36 / 39, 45, 66, 125 / 48 ms.
-constexpr unsigned long long kMinPart = 1ull << 20;
+// The fewest records of a part: each part clears and scans the counts of all
+// keys and ends with its last packets' walks, about 10 ms together.  When memory
+// is too short for them the launch walks its peel-offs in place.  2e6 packets (5 to
+// 15 records each) whole / in parts of 2^20, 2^19, 2^18, 2^16 packets / in place:
+// octree of 4e5 leaves 35 / 47, 61, 102, 299 / 51 ms, of 3e6 leaves 69 / 99, 135,
+// 223, 657 / 95 ms, k-d tree of 2e5 leaves 38 / 54, 71, 125, 379 / 69 ms, power-law
+// grid (4e6) 36 / 43, 53, 90, 190 / 47 ms, 3e4 Voronoi cells (1.5e6) 36 / 39, 45,
+// 66, 125 / 48 ms: the two meet between 5e6 and 1e7 records.
+constexpr unsigned long long kMinPart = 1ull << 23;
 rt_status prepare_peel_pass(rt_ctx c, FwdParams& p, unsigned long long n_total, int walked, bool tags,
                             unsigned long long limit, unsigned long long* part) {
   const unsigned long long keys = (unsigned long long)c->instr.size() * (unsigned long long)(c->n_cells + 1);
@@ -1172,10 +1173,10 @@ rt_status prepare_peel_pass(rt_ctx c, FwdParams& p, unsigned long long n_total, 
   // eight per walked instrument (a packet peels off once per event)
   const double per = c->peel_per_packet > 0.0 ? 1.25 * c->peel_per_packet + 0.05 : 8.0 * walked;
   const bool parts = c->grid_kind != RT_GRID_CARTESIAN;
-  const unsigned long long least = parts && !limit ? std::min(n_total, kMinPart) : 1;  // packets of a part
+  const unsigned long long all = (unsigned long long)std::min(per * (double)n_total, (double)kPeelMost);
+  const unsigned long long least = parts && !limit ? std::min(all, kMinPart) : 1;
   if (!limit) limit = parts ? kPeelPart : kPeelMost;
-  unsigned long long want = std::min((unsigned long long)std::min(per * (double)n_total, (double)kPeelMost), limit);
-  want = std::max(want, std::min(4096ull, limit));
+  unsigned long long want = std::min(std::max(all, 4096ull), limit);
   if (want > c->peel_cap) {
     size_t free_b = 0, total_b = 0;
     RT_CUDA(c, cudaMemGetInfo(&free_b, &total_b));
@@ -1183,7 +1184,7 @@ rt_status prepare_peel_pass(rt_ctx c, FwdParams& p, unsigned long long n_total, 
     const size_t record = sizeof(PeelRecord) + sizeof(unsigned);
     want = std::min(want, (unsigned long long)(0.4 * ((double)free_b + (double)(c->peel_cap * record))) / record);
   }
-  if (std::max(want, c->peel_cap) < (unsigned long long)std::min(per * (double)least, (double)kPeelMost)) return RT_OK;
+  if (std::max(want, c->peel_cap) < std::max(least, std::min(4096ull, limit))) return RT_OK;
   if (want > c->peel_cap) {
     dfree(c->d_peel);
     dfree(c->d_peel_perm);

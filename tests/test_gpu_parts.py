@@ -106,8 +106,8 @@ def test_buffer_sized_by_a_launch_of_fewer_records(grid, shared):
 
 
 def test_no_small_parts_when_memory_is_short():
-    """With memory for the records of fewer than 2^20 packets a launch of more
-    walks its peel-offs in place; with memory given back it sorts them again."""
+    """With memory for fewer than 2^23 of its records a launch walks its peel-offs in
+    place; with memory given back it sorts them again."""
     prob = _problem("octree", False)
     n = 400_000  # of 3 wavelengths: 1.2e6 packets, 0.7 GB of records at the first estimate
     sim = rt.Simulation(prob)
