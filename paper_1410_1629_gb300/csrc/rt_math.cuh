@@ -11,11 +11,11 @@
 // The range reduction, the remainders of constants and the high-order terms of
 // the series use integer and FP32 instructions; where an FP32 value enters an
 // FP64 sum its weight there is below 2^-32, so its rounding stays below 2^-56 of
-// the result, 2^-55.5 at the longest series' ends.
+// the result.
 //
 // Against 113-bit arithmetic (2e5 arguments in each of 17 ranges, on the
 // device): 1 - exp(-x) within 0.55 ulp, exp(x) - 1 within 0.56, -ln(1 - v) within
-// 0.60, their rms errors within 0.2 % of those of the correctly rounded values
+// 0.58, their rms errors within 0.2 % of those of the correctly rounded values
 // (0.289 ulp); the CUDA library's expm1 and log1p: 1.15 and 1.49 ulp, rms up to
 // 0.325 and 0.387, in no range more than 0.1 % below these.  Measured with the
 // library's functions in their place (time over that with these): 256 batched
@@ -84,8 +84,9 @@ struct ExpEntry {
   double t, hi, lo;
 };
 // a reciprocal of the middle of [1/2 + j/256, 1/2 + (j + 1)/256] to 13 bits
-// (1 for the last four intervals), the same less one, and its logarithm to a multiple
-// of 2^-40 and its remainder
+// (1 for the last three intervals, and for the one before them a value that
+// keeps its |r| below 2^-9 wherever the result is below 2^-6), the same less one,
+// and its logarithm to a multiple of 2^-40 and its remainder
 struct alignas(16) LogEntry {
   double rc, c, ln;
   float ln_lo;
@@ -482,7 +483,7 @@ RT_TABLE LogEntry kLogTable[128] = {
     {0x1.06bp+0, 0x1.acp-6, 0x1.a68151fb4p-6, 0x1.c049fcp-42f},
     {0x1.05ap+0, 0x1.68p-6, 0x1.641a17628p-6, -0x1.e5213ap-43f},
     {0x1.049p+0, 0x1.24p-6, 0x1.216daf6d8p-6, 0x1.32199ep-42f},
-    {0x1.0p+0, 0x0.0p+0, 0x0.0p+0, 0x0.0p+0f},
+    {0x1.0388p+0, 0x1.c4p-7, 0x1.c0e9338cp-7, 0x1.210b9ap-42f},
     {0x1.0p+0, 0x0.0p+0, 0x0.0p+0, 0x0.0p+0f},
     {0x1.0p+0, 0x0.0p+0, 0x0.0p+0, 0x0.0p+0f},
     {0x1.0p+0, 0x0.0p+0, 0x0.0p+0, 0x0.0p+0f},
@@ -564,10 +565,11 @@ RT_FN double bose(double x, double a = 1.0) {
 }
 
 // -ln(1 - v) for 0 <= v < 1.  y = 1 - v = 2^-m z with z in (1/2, 1], z rc = 1 +
-// r, |r| <= 2^-8 (2^-6 on the last four intervals, where rc = 1): -ln(1 - v) = m ln 2 + ln rc - ln(1 + r).  r = (rc - 1) - rc (1
-// - z), where 1 - z is v for m = 0 (v < 1/2) and exact above; the product's
-// rounding error is kept.  m ln 2 + ln rc to a multiple of 2^-40 is exact; its
-// remainder joins ln(1 + r).  Below 1/64 the result is that, rounded once.
+// r, |r| <= 2^-8 (3/256 on the last three intervals, where rc = 1): -ln(1 - v) =
+// m ln 2 + ln rc - ln(1 + r).  r = (rc - 1) - rc (1 - z), where 1 - z is v for m =
+// 0 (v < 1/2) and exact above; the product's rounding error is kept.  m ln 2 + ln
+// rc to a multiple of 2^-40 is exact; its remainder joins ln(1 + r).  Below 3/256
+// the result is that, rounded once.
 RT_FN double neg_log_one_minus(double v) {
   const bool low = bits_of(v) < 0x3fe0000000000000ll;  // v < 1/2
   long long by = bits_of(1.0 - v);
@@ -581,8 +583,7 @@ RT_FN double neg_log_one_minus(double v) {
   const double r = e.c - P;  // exact; 1 + r - pe = z rc
   // -ln(1 + r) = -r + r (r/2 - r^2/3 + r^3/4 - r^4/5 + r^5 (1/6 - r/7 + ...))
   const float rf = cut(r);
-  const float tail =
-      fmaf(rf, fmaf(rf, fmaf(rf, fmaf(rf, 1.0f / 10.0f, -1.0f / 9.0f), 1.0f / 8.0f), -1.0f / 7.0f), 1.0f / 6.0f);
+  const float tail = fmaf(rf, fmaf(rf, fmaf(rf, -1.0f / 9.0f, 1.0f / 8.0f), -1.0f / 7.0f), 1.0f / 6.0f);
   double q = fma(r, widen(tail), -0.2);
   q = fma(r, q, 0.25);
   q = fma(r, q, -1.0 / 3.0);

@@ -1,11 +1,11 @@
 """The FP64 functions of csrc/rt_math.cuh lose no precision to their tables and
 FP32 terms: little but the rounding of the result itself (at most 1/2 ulp,
 1/sqrt(12) ulp rms) is left, against extended precision, the same source
-compiled as C++.  What may be added to it: the FP32 tail of the logarithm's
-series, r^5 / 6 of the result with |r| <= 2^-6 and a relative error of 7.5e-8
-(the constant's and one rounding), or the rounding of the part beyond the exact
-one, 2^-63 against a result above 0.0156 (an ulp of 2^-58) and 2^-62 above 0.034
-(2^-57): at most 1/10 ulp."""
+compiled as C++.  What may be added to it: the rounding of the part beyond the
+exact one, 2^-63 against a result above 0.0117 (an ulp of 2^-59) or 2^-62 above
+0.0156 (2^-58) and above 0.034 (2^-57), and the FP32 tails of the series, 7.5e-8
+of r^5 / 6 with |r| <= 3/256 and of r^5 / 720 with |r| <= 0.035 (0.03 ulp): at
+most 1/10 ulp."""
 import ctypes
 import os
 import subprocess
