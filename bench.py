@@ -38,11 +38,11 @@ BYTES_PATH_CROSSING, BYTES_PEEL_CROSSING, BYTES_DEPOSIT = 20, 4, 16
 BYTES_COLUMN_PEEL = 8
 # DRAM bytes (read + write) per packet of the transport kernel, from an ncu
 # capture of one 2e6-packet launch of this workload (dram__bytes_read.sum
-# 37.920 GB + dram__bytes_write.sum 18.083 GB), valid only for the kernel
+# 37.651 GB + dram__bytes_write.sum 17.864 GB), valid only for the kernel
 # code whose hash is given (kernel_sources_hash: the sources without their
 # comments); the per-launch traffic is this figure times the packets.
-TRAFFIC_CAPTURE = {"sources_sha256_16": "7ebce241d82d7cf3", "kernel": "k_forward_cartesian",
-                   "bytes_per_packet": (37919683000 + 18082974000) / 2e6}
+TRAFFIC_CAPTURE = {"sources_sha256_16": "d2e20a20aec171d9", "kernel": "k_forward_cartesian",
+                   "bytes_per_packet": (37651125000 + 17863537000) / 2e6}
 KERNEL_SOURCES = ["paper_1410_1629_gb300/csrc/rt_forward.cu", "paper_1410_1629_gb300/csrc/rt_device.cuh",
                   "paper_1410_1629_gb300/csrc/rt_internal.h", "paper_1410_1629_gb300/csrc/rt_math.cuh",
                   "paper_1410_1629_gb300/csrc/rt_transport.cuh", "include/rt.h", "paper_1410_1629_gb300/build.py"]
